@@ -32,7 +32,7 @@ def listed():
         dict(name="step_batched", kind="step", family="batched", functions=1000, samples=120_000_000, graph=True,
              launch_stats=True),
         # One very large kernel, loop nests and many global loads.
-        dict(name="step_large", kind="step", family="large", functions=1, instructions=100_000, samples=20_000_000,
+        dict(name="step_large", kind="step", family="large", functions=1, instructions=120_000, samples=20_000_000,
              graph=False, launch_stats=False),
         # Serving: a program nobody has seen, from host arrays to advice and out again.
         dict(name="session_small", kind="session", family="batched", functions=3, samples=100_003),
@@ -67,7 +67,7 @@ def draw(rng):
         family = rng.choice(["rodinia", "batched", "batched", "large"])
         c = dict(kind=kind, family=family, graph=rng.random() < 0.5, launch_stats=rng.random() < 0.5)
         if family == "large":
-            c.update(functions=1, instructions=_loguniform(rng, 20_000, 90_000), samples=_loguniform(rng, 10**5, 10**7))
+            c.update(functions=1, instructions=_loguniform(rng, 20_000, 45_000), samples=_loguniform(rng, 10**5, 10**7))
         else:
             c.update(functions=_loguniform(rng, 1, 60 if family == "rodinia" else 900),
                      samples=_loguniform(rng, 10**4, 10**8))
