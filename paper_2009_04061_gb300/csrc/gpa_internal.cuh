@@ -187,6 +187,7 @@ struct SearchArena {
   int32_t nodes, src, layers, warps;  // warps: search groups (the fourth tier's are CTAs)
   int64_t bytes;   // per group
   char* global;    // global-memory tiers: warps * bytes
+  int* hash;       // third tier: warps * 2 * nodes ints, empty (-1) between searches; else nullptr
 };
 
 __device__ __forceinline__ void set_status(const Prog& P, unsigned long long bits) {
@@ -346,7 +347,7 @@ void launch_search(const Prog& P, const Arch& A, const SearchArena* tiers, const
                    int sms, int64_t* launches);
 void launch_coverage(const Prog& P, const Arch& A, const SearchArena* tiers, const SearchFork* fork, cudaStream_t st,
                      int sms, int64_t* launches);
-int64_t search_arena_bytes(int nodes, int src, int layers);
+int64_t search_arena_bytes(int nodes, int src, int layers, bool own_hash);
 int search_warps_per_sm();  // resident one-warp CTAs of the search kernel per SM (global-memory tiers)
 void launch_build_meta(const Prog& P, int4* meta, cudaStream_t st, int sms, int64_t* launches);
 void launch_build_events(const Prog& P, int32_t* ev_off, uint32_t* events, int32_t* tmp, cudaStream_t st, int sms,

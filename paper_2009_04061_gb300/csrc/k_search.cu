@@ -48,13 +48,16 @@ struct Arena {
   int* ctr;  // 0 nodes, 1 edges, 2 occurrences, 3 hash slots used, 4 overflow, 5 scratch
 };
 
-__host__ __device__ inline int64_t arena_bytes(int N, int SRC, int L) {
+// own_hash: the node hash (2 * N ints) lies in the arena; otherwise it is kept
+// apart (SearchArena::hash).
+__host__ __device__ inline int64_t arena_bytes(int N, int SRC, int L, bool own_hash) {
   const int64_t E = 2 * (int64_t)N, O = N;
-  int64_t ints = 12 * (int64_t)N + (int64_t)L * N + 2 * (int64_t)N + N + E + 3 * O + 3 * (int64_t)N + 4 * (int64_t)SRC + 8;
+  int64_t ints = 12 * (int64_t)N + (int64_t)L * N + (own_hash ? 2 * (int64_t)N : 0) + N + E + 3 * O + 3 * (int64_t)N +
+                 4 * (int64_t)SRC + 8;
   return 8 * (int64_t)N + 8 * (int64_t)SRC + ((ints * 4 + 15) & ~(int64_t)15);
 }
 
-__device__ Arena carve(char* base, int N, int SRC, int L, int* ctr) {
+__device__ Arena carve(char* base, int* hash, int N, int SRC, int L, int* ctr) {
   Arena a;
   a.N = N; a.E = 2 * N; a.O = N; a.SRC = SRC; a.L = L;
   a.dpk = reinterpret_cast<unsigned long long*>(base);
@@ -63,7 +66,8 @@ __device__ Arena carve(char* base, int N, int SRC, int L, int* ctr) {
   int** node_arrays[12] = {&a.blk, &a.S, &a.wall, &a.k, &a.e0, &a.e1, &a.fl, &a.seen, &a.ord, &a.tmp, &a.grp, &a.q};
   for (int t = 0; t < 12; ++t) { *node_arrays[t] = p; p += N; }
   a.dl = p; p += (int64_t)L * N;
-  a.ht = p; p += 2 * N;
+  a.ht = hash;
+  if (!hash) { a.ht = p; p += 2 * N; }
   a.hused = p; p += N;
   a.eto = p; p += a.E;
   a.on = p; p += a.O; a.ox = p; p += a.O; a.onext = p; p += a.O;
@@ -1090,9 +1094,11 @@ __device__ bool group_search(const G& g, const Prog& P, const Arch& A, const Are
 // of the first queue, part 2 the second overflow, which reuses the first
 // queue's storage; tier 4 the third overflow (bottom of the first overflow
 // queue's storage) and its top region. A search that outgrows its tier is
-// queued for the next one; the last tier records why it ran out.
+// queued for the next one; the last tier records why it ran out. An arena
+// that holds its own hash (`clear`) has it emptied when the group's first task
+// arrives, so a group that finds none touches no memory.
 template <class G>
-__device__ void run_tasks(const G& g, const Prog& P, const Arch& A, const Arena& a, int tier, int part) {
+__device__ void run_tasks(const G& g, const Prog& P, const Arch& A, const Arena& a, int tier, int part, bool clear) {
   const int me = g.rank();
   // The tasks of this launch, in order: nl of the large list, n0 read up
   // from the bottom of q0, n1 read down from the top of q1.
@@ -1120,6 +1126,11 @@ __device__ void run_tasks(const G& g, const Prog& P, const Arch& A, const Arena&
     if (me == 0) t = atomicAdd(&P.stats[h_slot], 1ull);
     t = g.broadcast(t);
     if (t >= nl + n0 + n1) break;
+    if (clear) {
+      for (int k = me; k < 2 * a.N; k += G::kSize) a.ht[k] = -1;
+      g.sync();
+      clear = false;
+    }
     const int4 task = t < nl        ? P.large_queue[t]
                       : t < nl + n0 ? q0[t - nl]
                                     : q1[cap - 1 - (t - nl - n0)];
@@ -1167,16 +1178,21 @@ __device__ void run_tasks(const G& g, const Prog& P, const Arch& A, const Arena&
 __global__ void __launch_bounds__(kWarpsPerCta * 32, GPA_SEARCH_MIN_CTAS)
     k_search_warp(Prog P, Arch A, SearchArena SA, int tier, int part) {
   extern __shared__ __align__(16) char smem[];
-  const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
+  const int wid = threadIdx.x >> 5;
   const int gw = blockIdx.x * (blockDim.x >> 5) + wid;
   char* base = tier < 3 ? smem + (int64_t)wid * SA.bytes : SA.global + (int64_t)gw * SA.bytes;
   // The search counters live in shared memory in every tier (the arena of
   // tier 3 is in global memory): frontier sizes are read after every round.
   __shared__ int s_ctr[kWarpsPerCta][8];
-  const Arena a = carve(base, SA.nodes, SA.src, SA.layers, s_ctr[wid]);
-  for (int t = lane; t < 2 * SA.nodes; t += 32) a.ht[t] = -1;
-  __syncwarp();
-  run_tasks(WarpGroup{}, P, A, a, tier, part);
+  // The third tier's hashes lie apart from its arenas (whose pool the fourth
+  // tier lays out anew) and are empty between searches: every search empties
+  // the slots it used, also when it outgrew its arena. They were cleared with
+  // the context, so a launch clears nothing. (A launch that began by clearing
+  // its warps' 256 KB hashes wrote 956 MB and took 145 us with no search to
+  // run, 4 us now; the launch appears twice in a step.)
+  int* hash = SA.hash ? SA.hash + (int64_t)gw * 2 * SA.nodes : nullptr;
+  const Arena a = carve(base, hash, SA.nodes, SA.src, SA.layers, s_ctr[wid]);
+  run_tasks(WarpGroup{}, P, A, a, tier, part, hash == nullptr);
 }
 
 // The fourth tier: a CTA per search, over a global-memory arena of its own
@@ -1188,15 +1204,15 @@ __global__ void __launch_bounds__(kCtaThreads, 1) k_search_cta(Prog P, Arch A, S
   __shared__ int s_red[CtaGroup::kWarps];
   __shared__ unsigned long long s_cast;
   const CtaGroup g{s_red, &s_cast};
-  const Arena a = carve(SA.global + (int64_t)blockIdx.x * SA.bytes, SA.nodes, SA.src, SA.layers, s_ctr);
-  for (int t = threadIdx.x; t < 2 * SA.nodes; t += kCtaThreads) a.ht[t] = -1;
-  __syncthreads();
-  run_tasks(g, P, A, a, 4, 0);
+  const Arena a = carve(SA.global + (int64_t)blockIdx.x * SA.bytes, nullptr, SA.nodes, SA.src, SA.layers, s_ctr);
+  run_tasks(g, P, A, a, 4, 0, true);
 }
 
 }  // namespace
 
-int64_t search_arena_bytes(int nodes, int src, int layers) { return arena_bytes(nodes, src, layers); }
+int64_t search_arena_bytes(int nodes, int src, int layers, bool own_hash) {
+  return arena_bytes(nodes, src, layers, own_hash);
+}
 
 int search_warps_per_sm() {
   int n = 0;
@@ -1222,18 +1238,22 @@ void launch_search(const Prog& P, const Arch& A, const SearchArena* tiers, const
     cudaStreamWaitEvent(fork->side, fork->fork, 0);
     s3 = fork->side;
   }
-  k_search_warp<<<tiers[0].warps / kWarpsPerCta, kWarpsPerCta * 32, smem1, st>>>(P, A, tiers[0], 1, 0);
-  k_search_warp<<<tiers[2].warps, 32, 0, s3>>>(P, A, tiers[2], 3, 1);
+  // No launch takes more groups than there can be tasks (one per use entry).
+  const int most = (int)std::min<int64_t>(P.queue_cap, INT32_MAX);
+  const int g1 = std::max(1, std::min(tiers[0].warps, most) / kWarpsPerCta);
+  const int g2 = std::min(tiers[1].warps, most), g3 = std::min(tiers[2].warps, most);
+  k_search_warp<<<g1, kWarpsPerCta * 32, smem1, st>>>(P, A, tiers[0], 1, 0);
+  k_search_warp<<<g3, 32, 0, s3>>>(P, A, tiers[2], 3, 1);
   if (fork) cudaEventRecord(fork->join, fork->side);
-  k_search_warp<<<tiers[1].warps, 32, smem2, st>>>(P, A, tiers[1], 2, 0);
+  k_search_warp<<<g2, 32, smem2, st>>>(P, A, tiers[1], 2, 0);
   if (fork) cudaStreamWaitEvent(st, fork->join, 0);
-  k_search_warp<<<tiers[2].warps, 32, 0, st>>>(P, A, tiers[2], 3, 2);
+  k_search_warp<<<g3, 32, 0, st>>>(P, A, tiers[2], 3, 2);
   *launches += 4;
   if (P.t4_nodes > 0) {
     // The fourth tier runs after the third on this stream, so the third tier's
     // arena pool is free by then: when it holds more fourth-tier arenas than the
     // program's own, the CTAs carve theirs from it (at most one CTA per SM).
-    SearchArena t4{P.t4_nodes, P.t4_src, kMaxLayers, P.t4_ctas, P.t4_bytes, P.t4_arena};
+    SearchArena t4{P.t4_nodes, P.t4_src, kMaxLayers, P.t4_ctas, P.t4_bytes, P.t4_arena, nullptr};
     const int64_t in_pool = (int64_t)tiers[2].warps * tiers[2].bytes / P.t4_bytes;
     if (in_pool > t4.warps && tiers[2].global) {
       t4.warps = (int)std::min<int64_t>(in_pool, std::max(sms, 1));

@@ -320,8 +320,9 @@ gpa_status gpa_create(const gpa_arch_desc* arch, const gpa_options* opts, gpa_ct
   T[1].nodes = n2; T[1].src = std::min(n2, 256); T[1].layers = 4; T[1].warps = (n2 <= 512 ? 3 : 1) * c->sms;
   T[2].nodes = n3; T[2].src = std::min(n3, 1024); T[2].layers = kMaxLayers; T[2].warps = o.search_slots;
   for (int t = 0; t < 3; ++t) {
-    T[t].bytes = search_arena_bytes(T[t].nodes, T[t].src, T[t].layers);
+    T[t].bytes = search_arena_bytes(T[t].nodes, T[t].src, T[t].layers, t < 2);
     T[t].global = nullptr;
+    T[t].hash = nullptr;
   }
   gpa_status s = GPA_OK;
   if (T[0].bytes * 4 > 220 * 1024 || T[1].bytes > 220 * 1024) s = GPA_ERR_INVALID_ARG;
@@ -330,6 +331,13 @@ gpa_status gpa_create(const gpa_arch_desc* arch, const gpa_options* opts, gpa_ct
     s = GPA_ERR_OOM;
   }
   if (!s && cudaMemset(T[2].global, 0, (size_t)T[2].bytes * T[2].warps) != cudaSuccess) s = GPA_ERR_CUDA;
+  // The third tier's node hashes start empty (-1); every search leaves them so.
+  const size_t hash_bytes = sizeof(int32_t) * 2 * (size_t)T[2].nodes * T[2].warps;
+  if (!s && cudaMalloc(&T[2].hash, hash_bytes) != cudaSuccess) {
+    T[2].hash = nullptr;
+    s = GPA_ERR_OOM;
+  }
+  if (!s && cudaMemset(T[2].hash, 0xFF, hash_bytes) != cudaSuccess) s = GPA_ERR_CUDA;
   if (!s && cudaEventCreateWithFlags(&c->scratch_ev, cudaEventDisableTiming) != cudaSuccess) s = GPA_ERR_CUDA;
   if (!s && cudaStreamCreateWithFlags(&c->build_stream, cudaStreamNonBlocking) != cudaSuccess) s = GPA_ERR_CUDA;
   if (!s && cudaStreamCreateWithFlags(&c->fork.side, cudaStreamNonBlocking) != cudaSuccess) s = GPA_ERR_CUDA;
@@ -337,6 +345,7 @@ gpa_status gpa_create(const gpa_arch_desc* arch, const gpa_options* opts, gpa_ct
   if (!s && cudaEventCreateWithFlags(&c->fork.join, cudaEventDisableTiming) != cudaSuccess) s = GPA_ERR_CUDA;
   if (s) {
     if (c->tier[2].global) cudaFree(c->tier[2].global);
+    if (c->tier[2].hash) cudaFree(c->tier[2].hash);
     if (c->scratch_ev) cudaEventDestroy(c->scratch_ev);
     if (c->build_stream) cudaStreamDestroy(c->build_stream);
     if (c->fork.side) cudaStreamDestroy(c->fork.side);
@@ -354,6 +363,7 @@ gpa_status gpa_destroy(gpa_ctx* ctx) {
   cudaDeviceSynchronize();
   for (auto& kv : ctx->progs) free_program(kv.second);
   if (ctx->tier[2].global) cudaFree(ctx->tier[2].global);
+  if (ctx->tier[2].hash) cudaFree(ctx->tier[2].hash);
   for (int k = 0; k < 2; ++k) {
     if (ctx->stage[k]) cudaFree(ctx->stage[k]);
     if (ctx->ev_copied[k]) cudaEventDestroy(ctx->ev_copied[k]);
@@ -583,7 +593,7 @@ static gpa_status alloc_program(const gpa_program_desc* d, ProgramRec* R, int ti
       P.t4_nodes = (int32_t)n4;
       P.t4_src = (int32_t)std::min<int64_t>(n4, 4096);
       P.t4_ctas = n4 <= ((int64_t)1 << 18) ? 16 : n4 <= ((int64_t)1 << 20) ? 8 : 4;
-      P.t4_bytes = search_arena_bytes(P.t4_nodes, P.t4_src, kMaxLayers);
+      P.t4_bytes = search_arena_bytes(P.t4_nodes, P.t4_src, kMaxLayers, true);
       TRY(dev_alloc(R, &P.t4_arena, (size_t)P.t4_bytes * P.t4_ctas));
     }
   }
