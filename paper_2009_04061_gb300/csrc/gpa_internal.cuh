@@ -16,6 +16,7 @@ constexpr int kEvBuckets = 16;   // event segments per block: resources by r mod
 __host__ __device__ inline int ev_bucket(int r) { return r & (kEvBuckets - 1); }
 constexpr int kCnt = 24;         // counters per instruction: class * 2 + latency flag
 constexpr uint16_t kAllLits = 0xFFFF;
+constexpr int kLaneNodes = 128;  // most nodes of a one-lane search (first and second tier)
 constexpr int kMaxLayers = 8;    // back-edge layers for longest paths (K <= 7)
 constexpr int kMaxSrc = 64;      // merged sources per stalled use in the thread-per-use kernels
 constexpr int kBigSrc = 2048;    // merged sources per stalled use (hard upper bound; beyond kMaxSrc
@@ -182,10 +183,11 @@ struct Prog {
   int32_t* a_par_limit;           // nf
 };
 
-// Per-warp arenas of the general (multi-block) search.
+// Arenas of the general (multi-block) search: one search a lane in the first
+// two tiers (bytes: shared memory of a warp), per group in the others.
 struct SearchArena {
   int32_t nodes, src, layers, warps;  // warps: search groups (the fourth tier's are CTAs)
-  int64_t bytes;   // per group
+  int64_t bytes;   // per warp or group
   char* global;    // global-memory tiers: warps * bytes
   int* hash;       // third tier: warps * 2 * nodes ints, empty (-1) between searches; else nullptr
 };
@@ -348,6 +350,10 @@ void launch_search(const Prog& P, const Arch& A, const SearchArena* tiers, const
 void launch_coverage(const Prog& P, const Arch& A, const SearchArena* tiers, const SearchFork* fork, cudaStream_t st,
                      int sms, int64_t* launches);
 int64_t search_arena_bytes(int nodes, int src, int layers, bool own_hash);
+int search_lane_width(int nodes);      // lanes of a warp that search, for arenas of so many nodes
+int64_t search_lane_bytes(int nodes);  // their arenas, in bytes a warp
+void launch_search_lanes(const Prog& P, const Arch& A, const SearchArena& T, int tier, cudaStream_t st,
+                         int64_t* launches);
 int search_warps_per_sm();  // resident one-warp CTAs of the search kernel per SM (global-memory tiers)
 void launch_build_meta(const Prog& P, int4* meta, cudaStream_t st, int sms, int64_t* launches);
 void launch_build_events(const Prog& P, int32_t* ev_off, uint32_t* events, int32_t* tmp, cudaStream_t st, int sms,

@@ -2,19 +2,16 @@
 // stalled use j through resource r whose value may come from outside j's
 // block, with the three pruning rules evaluated over the set of source paths.
 //
-// One search group per (use, resource) task: a warp in the first three tiers,
-// a whole CTA in the fourth (searches of tens of thousands to millions of
-// nodes). The graph of (block, literal set) nodes lives in the group's arena:
-// shared memory for the common small searches, global memory for the few that
-// outgrow it (same code). The group's threads scan node blocks in parallel
+// The third and fourth search tier: one search group per (use, resource) task, a
+// warp in the third tier, a whole CTA in the fourth (searches of tens of
+// thousands to millions of nodes); searches of up to 128 nodes run one to a lane
+// before them (k_search_lanes.cu). The graph of (block, literal set) nodes lives
+// in the group's arena in global memory. The group's threads scan node blocks in parallel
 // through per-block event lists (defs and unguarded reads, bottom-up), insert
 // nodes and sources into open-addressing hashes together, relax distances and
 // propagate reachability bits over frontiers with atomics, and run the
 // layered longest paths as level-synchronous frontiers; rank 0 only resets
-// counters between steps. The first tier's searches (at most 64 nodes, two or
-// three nodes a wave) run pass A, rule 2's reachability and the longest paths
-// on one thread instead (worklist queues reaching the same fixpoints): there
-// the warp-wide protocol of a wave cost more than the work it spread.
+// counters between steps.
 //
 // Node 0 is the part of j's block above j, already scanned by the local pass
 // (its sources are settled there). A node's d is the shortest distance from
@@ -35,7 +32,6 @@ namespace {
 constexpr int kInf = 0x3FFFFFFF;
 constexpr uint32_t kBackBit = 0x80000000u;
 constexpr int kExpanded = 1;
-constexpr int kWarpsPerCta = 4;
 
 struct Arena {
   int N, E, O, SRC, L;
@@ -92,7 +88,7 @@ __device__ __forceinline__ void prefetch_l1(const void* p) {
 __device__ __forceinline__ int dist_of(const Arena& a, int u) { return (int)(a.dpk[u] >> 32); }
 __device__ __forceinline__ int par_of(const Arena& a, int u) { return (int)(a.dpk[u] & 0xFFFFFFFFull); }
 
-// The threads that run one search together: a warp (tiers 1-3) or a whole
+// The threads that run one search together: a warp (third tier) or a whole
 // CTA (the fourth tier's very large searches). Both give the search the same
 // steps: a barrier, an any-vote, exclusive prefix counts, inclusive sums and
 // reductions over the group, a read of a shared flag that every thread takes
@@ -545,118 +541,14 @@ __device__ bool group_search(const G& g, const Prog& P, const Arch& A, const Are
     return cnt;
   };
 
-  // Pass A by one thread, for the first tier's small searches: a
-  // label-correcting queue (a node is queued when its distance improves and it
-  // is expanded or within the bound; a node is expanded once, when first taken
-  // within the bound; an expanded node taken again relaxes its edges from its
-  // better distance). It reaches the fixpoint of the waves below (every node
-  // whose shortest distance over the expanded nodes' edges is within the bound
-  // is expanded), without a vote, a prefix count or a claim round per node: a
-  // small search's waves are two or three nodes wide, so the warp-wide
-  // protocol cost more than the work it spread. The queue is a ring over q
-  // (a node is in it at most once at a time).
-  auto serial_pass_a = [&]() {
-    int* ring = a.q;
-    int head = 0, tail = 0, inq = 0;
-    int nn = ctr[0], ne = ctr[1], nh = ctr[3];
-    auto push = [&](int v) {
-      if (a.fl[v] & 8) return;
-      a.fl[v] |= 8;
-      ring[tail] = v;
-      tail = tail + 1 == a.N ? 0 : tail + 1;
-      ++inq;
-    };
-    push(0);
-    while (inq > 0) {
-      const int u = ring[head];
-      head = head + 1 == a.N ? 0 : head + 1;
-      --inq;
-      a.fl[u] &= ~8;
-      const int du = dist_of(a, u);
-      if (!(a.fl[u] & kExpanded)) {
-        if (du > bound) continue;
-        const int B = a.blk[u];
-        const int4 pm = __ldg(&P.block_meta[2 * (size_t)B + 1]);
-        const int first = __ldg(&P.block_meta[2 * (size_t)B].x);
-        const uint32_t tw = __ldg(&P.touch_mask[(size_t)B * kWords + w]);
-        const size_t seg = (size_t)B * kEvBuckets + ev_bucket(r);
-        const int ev_beg = __ldg(&P.ev_off[seg]);
-        int ev_end = __ldg(&P.ev_off[seg + 1]);
-        ev_end = (tw & bit) ? ev_end : ev_beg;
-        scan(u, first, ev_beg, ev_end);
-        if (ctr[4]) break;
-        const int Sout = (a.S[u] >> 16) & 0xFFFF;
-        a.e0[u] = ne;
-        for (int q = (a.fl[u] & 4) ? pm.y : pm.x; q < pm.y; ++q) {
-          const int p = q == pm.x ? pm.z : q == pm.x + 1 ? pm.w : __ldg(&P.pred[q]);
-          if (!(P.rout[(size_t)p * kWords + w] & bit)) continue;
-          if (ne >= a.E) { ctr[4] = 2; break; }
-          uint32_t h = node_hash(p, Sout) & hmask;
-          int v = -1;
-          for (int probe = 0; probe <= (int)hmask; ++probe) {
-            const int c = a.ht[h];
-            if (c < 0) break;
-            if (a.blk[c] == p && (a.S[c] & 0xFFFF) == Sout) { v = c; break; }
-            h = (h + 1) & hmask;
-          }
-          if (v < 0) {
-            if (a.ht[h] >= 0) { ctr[4] = 6; break; }  // not reached: 2N slots for at most N nodes
-            if (nn >= a.N) { ctr[4] = 1; break; }
-            v = nn++;
-            a.blk[v] = p; a.S[v] = Sout; a.wall[v] = -1; a.fl[v] = 0; a.k[v] = kInf;
-            a.e0[v] = 0; a.e1[v] = 0;
-            a.dpk[v] = ((unsigned long long)kInf << 32) | 0xFFFFFFFFull;
-            a.hused[nh++] = (int)h;
-            a.ht[h] = v;
-          }
-          a.eto[ne++] = v | (p >= B ? (int)kBackBit : 0);
-        }
-        a.e1[u] = ne;
-        if (ctr[4]) break;
-      }
-      if (du >= kInf) continue;
-      // distance with parent, and fewest back edges, relaxed together
-      const unsigned long long nd = ((unsigned long long)(du + wout(u)) << 32) | (unsigned)u;
-      const int ku = a.k[u];
-      for (int e = a.e0[u]; e < a.e1[u]; ++e) {
-        const int v = a.eto[e] & 0x7FFFFFFF;
-        const int nk = ku + (int)((uint32_t)a.eto[e] >> 31);
-        bool better = false;
-        if (nd < a.dpk[v]) { a.dpk[v] = nd; better = true; }
-        if (nk < a.k[v]) { a.k[v] = nk; better = true; }
-        if (better && ((a.fl[v] & kExpanded) || dist_of(a, v) <= bound)) push(v);
-      }
-    }
-    ctr[0] = nn; ctr[1] = ne; ctr[3] = nh;
-  };
-
   // Pass A expands in waves the nodes within the bound, relaxing as they
-  // link (or by one thread, above); pass B, only if some source is within its
+  // link; pass B, only if some source is within its
   // latency, completes the graph. Both run in this one loop, so the wave code
   // exists once in the kernel (the search kernel is bound by instruction fetch
   // when its warps spread over a larger body).
   bool cand = false, pass_b = false, grew_b = false;
-  const bool serial_a = G::kSize == 32 && tier == 1;
-  if (serial_a) {
-    if (me == 0) serial_pass_a();
-    g.sync();
-    // pass B starts from the nodes pass A left unexpanded
-    const int n_now = ctr[0];
-    int m = 0;
-    for (int i0 = 0; i0 < n_now; i0 += G::kSize) {
-      const int i = i0 + me;
-      const bool un = i < n_now && !(a.fl[i] & kExpanded);
-      int tot;
-      const int at = g.slot(un, &tot);
-      if (un) ubuf[m + at] = i;
-      m += tot;
-    }
-    g.sync();
-    if (me == 0) ctr[6] = m;
-    g.sync();
-  }
   while (!ctr[4]) {
-    const int cnt = serial_a && !pass_b ? 0 : take_wave(pass_b ? -1 : bound);
+    const int cnt = take_wave(pass_b ? -1 : bound);
     if (cnt > 0) {
       grew_b |= pass_b;
       expand_list(list, cnt, !pass_b);
@@ -709,18 +601,17 @@ __device__ bool group_search(const G& g, const Prog& P, const Arch& A, const Are
   // Shortest distance with parents, and fewest back edges, over the whole
   // graph. When pass B expanded no node, every edge of the graph was relaxed
   // to the fixpoint in pass A, whose (distance, parent) minimum over the same
-  // edges is this one; the one-thread pass A relaxes the back-edge counts
-  // along with the distances, so its searches then need neither.
-  const bool fresh_d = grew_b, fresh_k = grew_b || !serial_a;
+  // edges is this one.
+  const bool fresh_d = grew_b;
   for (int u = me; u < n; u += G::kSize) {
     if (fresh_d) a.dpk[u] = u == 0 ? 0ull : (((unsigned long long)kInf << 32) | 0xFFFFFFFFull);
-    if (fresh_k) a.k[u] = u == 0 ? 0 : kInf;
+    a.k[u] = u == 0 ? 0 : kInf;
     a.fl[u] &= ~8;
   }
   if (me == 0) a.q[0] = 0;
   g.sync();
 #pragma unroll 1
-  for (int mode = fresh_d ? 0 : 1; mode < (fresh_k ? 2 : 1); ++mode) relax_from(a.q, 1, mode);
+  for (int mode = fresh_d ? 0 : 1; mode < 2; ++mode) relax_from(a.q, 1, mode);
   phase(1);
 
   // Sources: a warp-synchronous hash keyed by instruction gives each source an
@@ -883,40 +774,10 @@ __device__ bool group_search(const G& g, const Prog& P, const Arch& A, const Are
       const int b = wg >= 0 ? a.wneed[wg] : 0;
       return b ? ~(1u << (b - 1)) : 0xFFFFFFFFu;
     };
-    // A first-tier search propagates by one thread with a worklist ring over
-    // q (a node is in it at most once at a time, flag 8): the same fixpoint
-    // as the frontier rounds below, without a round's barriers and counters.
-    if (serial_a && me == 0) {
-      int* ring = a.q;
-      int head = 0, tail = 1, inq = 1;
-      ring[0] = 0;
-      a.fl[0] |= 8;
-      while (inq > 0) {
-        const int u = ring[head];
-        head = head + 1 == a.N ? 0 : head + 1;
-        --inq;
-        a.fl[u] &= ~8;
-        const unsigned m = (unsigned)reach[u] & pass_mask(u);
-        if (!m || !edges_ok(u, n)) continue;
-        for (int e = a.e0[u]; e < a.e1[u]; ++e) {
-          const int v = a.eto[e] & 0x7FFFFFFF;
-          if (!target_ok(v, n)) break;
-          const unsigned add = m & ~(unsigned)reach[v];
-          if (!add) continue;
-          reach[v] |= (int)add;
-          if (!(a.fl[v] & 8)) {
-            a.fl[v] |= 8;
-            ring[tail] = v;
-            tail = tail + 1 == a.N ? 0 : tail + 1;
-            ++inq;
-          }
-        }
-      }
-    }
     int* cur = a.q;
     int* nxt = a.tmp;
     if (me == 0) { cur[0] = 0; ctr[5] = 0; }
-    int fsize = serial_a ? 0 : 1;
+    int fsize = 1;
     g.sync();
     while (fsize > 0) {
       // Clear the queued flags of the whole frontier first: bits that arrive
@@ -994,80 +855,45 @@ __device__ bool group_search(const G& g, const Prog& P, const Arch& A, const Are
       if (!((uint32_t)a.eto[e] >> 31)) atomicAdd(&a.ord[a.eto[e] & 0x7FFFFFFF], 1);
   if (me == 0) a.dl[0] = 0;
   g.sync();
-  if (serial_a) {
-    // A first-tier search runs the layers by one thread: Kahn's order with a
-    // queue over q (each node enters a layer's queue once, when its last
-    // forward in-edge is taken), the nodes' lengths read once into tmp.
-    for (int u = me; u < n; u += G::kSize) a.tmp[u] = wout(u);
+  for (int l = 0; l <= maxK; ++l) {
+    int* dll = a.dl + (int64_t)l * a.N;
+    if (me == 0) ctr[5] = 0;
     g.sync();
-    if (me == 0) {
-      int* ring = a.q;
-      for (int l = 0; l <= maxK; ++l) {
-        int* dll = a.dl + (int64_t)l * a.N;
-        int head = 0, tail = 0;
-        for (int u = 0; u < n; ++u) {
-          a.seen[u] = a.ord[u];  // remaining forward in-edges
-          if (a.ord[u] == 0) ring[tail++] = u;
-        }
-        while (head < tail) {
-          const int u = ring[head++];
-          const int cv = dll[u];
-          const int nd = cv + a.tmp[u];
-          for (int e = a.e0[u]; e < a.e1[u]; ++e) {
-            const int v = a.eto[e] & 0x7FFFFFFF;
-            if ((uint32_t)a.eto[e] >> 31) {
-              int* t = &a.dl[(int64_t)(l + 1) * a.N + v];
-              if (cv >= 0 && l + 1 <= maxK && nd > *t) *t = nd;
-            } else {
-              if (cv >= 0 && nd > dll[v]) dll[v] = nd;
-              if (--a.seen[v] == 0 && tail < a.N) ring[tail++] = v;
-            }
-          }
-        }
-      }
+    for (int u = me; u < n; u += G::kSize) {
+      a.seen[u] = a.ord[u];  // remaining forward in-edges
+      if (a.ord[u] == 0) a.q[atomicAdd((int*)&a.ctr[5], 1)] = u;
     }
     g.sync();
-  } else {
-    for (int l = 0; l <= maxK; ++l) {
-      int* dll = a.dl + (int64_t)l * a.N;
-      if (me == 0) ctr[5] = 0;
-      g.sync();
-      for (int u = me; u < n; u += G::kSize) {
-        a.seen[u] = a.ord[u];  // remaining forward in-edges
-        if (a.ord[u] == 0) a.q[atomicAdd((int*)&a.ctr[5], 1)] = u;
-      }
-      g.sync();
-      int fsize = ctr[5];
-      int* cur = a.q;
-      int* nxt = a.tmp;
-      g.sync();
-      if (me == 0) ctr[5] = 0;
-      g.sync();
-      while (fsize > 0) {
-        for (int f0 = 0; f0 < fsize; f0 += G::kSize) {
-          if (f0 + me < fsize) {
-            const int u = cur[f0 + me];
-            const int cv = dll[u];
-            const int nd = cv + wout(u);
-            for (int e = a.e0[u]; e < a.e1[u]; ++e) {
-              const int v = a.eto[e] & 0x7FFFFFFF;
-              const bool back = (uint32_t)a.eto[e] >> 31;
-              if (back) {
-                if (cv >= 0 && l + 1 <= maxK) atomicMax(&a.dl[(int64_t)(l + 1) * a.N + v], nd);
-              } else {
-                if (cv >= 0) atomicMax(&dll[v], nd);
-                if (atomicSub(&a.seen[v], 1) == 1) nxt[atomicAdd((int*)&a.ctr[5], 1)] = v;
-              }
+    int fsize = ctr[5];
+    int* cur = a.q;
+    int* nxt = a.tmp;
+    g.sync();
+    if (me == 0) ctr[5] = 0;
+    g.sync();
+    while (fsize > 0) {
+      for (int f0 = 0; f0 < fsize; f0 += G::kSize) {
+        if (f0 + me < fsize) {
+          const int u = cur[f0 + me];
+          const int cv = dll[u];
+          const int nd = cv + wout(u);
+          for (int e = a.e0[u]; e < a.e1[u]; ++e) {
+            const int v = a.eto[e] & 0x7FFFFFFF;
+            const bool back = (uint32_t)a.eto[e] >> 31;
+            if (back) {
+              if (cv >= 0 && l + 1 <= maxK) atomicMax(&a.dl[(int64_t)(l + 1) * a.N + v], nd);
+            } else {
+              if (cv >= 0) atomicMax(&dll[v], nd);
+              if (atomicSub(&a.seen[v], 1) == 1) nxt[atomicAdd((int*)&a.ctr[5], 1)] = v;
             }
           }
         }
-        g.sync();
-        fsize = ctr[5];
-        g.sync();
-        if (me == 0) ctr[5] = 0;
-        int* sw = cur; cur = nxt; nxt = sw;
-        g.sync();
       }
+      g.sync();
+      fsize = ctr[5];
+      g.sync();
+      if (me == 0) ctr[5] = 0;
+      int* sw = cur; cur = nxt; nxt = sw;
+      g.sync();
     }
   }
   for (int m = me; m < nsrc; m += G::kSize) {
@@ -1089,9 +915,8 @@ __device__ bool group_search(const G& g, const Prog& P, const Arch& A, const Are
 }
 
 // The task loop of a search group: claim (use, resource) tasks from one
-// queue until it is empty. Tier 1 reads the local pass's queue; tier 2 the
-// first overflow queue; tier 3 part 1 the large list and the region at the top
-// of the first queue, part 2 the second overflow, which reuses the first
+// queue until it is empty. Tier 3 part 1 reads the large list and the region at
+// the top of the first queue, part 2 the second overflow, which reuses the first
 // queue's storage; tier 4 the third overflow (bottom of the first overflow
 // queue's storage) and its top region. A search that outgrows its tier is
 // queued for the next one; the last tier records why it ran out. An arena
@@ -1106,12 +931,8 @@ __device__ void run_tasks(const G& g, const Prog& P, const Arch& A, const Arena&
   const int4* q0 = P.queue;
   const int4* q1 = P.queue;
   unsigned long long nl = 0, n0 = 0, n1 = 0;
-  int h_slot = SS_QUEUE_HEAD;
-  if (tier == 1) {
-    n0 = P.stats[SS_QUEUE_N];
-  } else if (tier == 2) {
-    q0 = P.ovf_queue, n0 = P.stats[SS_OVF_N], h_slot = SS_OVF_HEAD;
-  } else if (tier == 3 && part == 1) {
+  int h_slot = 0;
+  if (tier == 3 && part == 1) {
     nl = min(P.stats[SS_LARGE_N], (unsigned long long)kLargeQueue);
     n1 = P.stats[SS_HINT3_N], h_slot = SS_HINT3_HEAD;
   } else if (tier == 3) {
@@ -1147,52 +968,38 @@ __device__ void run_tasks(const G& g, const Prog& P, const Arch& A, const Arena&
     }
     if (me != 0) continue;
     if (!P.diag) atomicMax(&P.tier_hint[task.w], (unsigned)(tier + 1));  // later steps queue it for a bigger tier
-    if (tier < 3 || (tier == 3 && P.t4_nodes > 0)) {
-      // tier 1 -> bottom of ovf_queue; tier 2 -> bottom of queue; tier 3 part 2
-      // -> bottom of ovf_queue (after tier 2 read it); part 1, which may run
-      // beside tier 1, -> top of ovf_queue
-      const bool top = tier == 3 && part == 1;
-      const int o_slot = tier == 1 ? SS_OVF_N : tier == 2 ? SS_OVF2_N : top ? SS_OVF3H_N : SS_OVF3_N;
-      int4* oq = tier == 2 ? P.queue : P.ovf_queue;
-      const unsigned long long o = atomicAdd(&P.stats[o_slot], 1ull);
-      if (o < cap) oq[top ? cap - 1 - o : o] = task; else capacity(P, 8);
+    if (tier == 3 && P.t4_nodes > 0) {
+      // part 2 -> bottom of ovf_queue (after tier 2 read it); part 1, which may
+      // run beside tier 1, -> top of ovf_queue
+      const bool top = part == 1;
+      const unsigned long long o = atomicAdd(&P.stats[top ? SS_OVF3H_N : SS_OVF3_N], 1ull);
+      if (o < cap) P.ovf_queue[top ? cap - 1 - o : o] = task; else capacity(P, 8);
     } else {
       capacity(P, a.ctr[7] > 0 ? a.ctr[7] : 1);  // the last tier: why it ran out
     }
   }
 }
 
-// Persistent work-stealing warps, one search each. Tiers 1 and 2 keep the
-// arena in shared memory (tier 1: several warps per CTA, small arenas; tier 2:
-// one warp per CTA, a large arena); tier 3 uses global-memory arenas. Tier 3
-// runs in two parts: part 1 takes the searches queued straight for it (the
-// large list first) and may run beside tiers 1 and 2; part 2 takes the second
-// tier's overflow.
-// Registers: at least six 128-thread CTAs per SM, i.e. 80 registers a thread
-// (96 without the bound). The first tier and the third tier's hinted part run
-// side by side and together fill the SM's registers, so fewer registers a warp
-// keep more warps in flight (measured: 40.7 against 41.9 ms a step).
-#ifndef GPA_SEARCH_MIN_CTAS
-#define GPA_SEARCH_MIN_CTAS 6
-#endif
-__global__ void __launch_bounds__(kWarpsPerCta * 32, GPA_SEARCH_MIN_CTAS)
-    k_search_warp(Prog P, Arch A, SearchArena SA, int tier, int part) {
-  extern __shared__ __align__(16) char smem[];
-  const int wid = threadIdx.x >> 5;
-  const int gw = blockIdx.x * (blockDim.x >> 5) + wid;
-  char* base = tier < 3 ? smem + (int64_t)wid * SA.bytes : SA.global + (int64_t)gw * SA.bytes;
-  // The search counters live in shared memory in every tier (the arena of
-  // tier 3 is in global memory): frontier sizes are read after every round.
-  __shared__ int s_ctr[kWarpsPerCta][8];
-  // The third tier's hashes lie apart from its arenas (whose pool the fourth
-  // tier lays out anew) and are empty between searches: every search empties
-  // the slots it used, also when it outgrew its arena. They were cleared with
-  // the context, so a launch clears nothing. (A launch that began by clearing
-  // its warps' 256 KB hashes wrote 956 MB and took 145 us with no search to
-  // run, 4 us now; the launch appears twice in a step.)
-  int* hash = SA.hash ? SA.hash + (int64_t)gw * 2 * SA.nodes : nullptr;
-  const Arena a = carve(base, hash, SA.nodes, SA.src, SA.layers, s_ctr[wid]);
-  run_tasks(WarpGroup{}, P, A, a, tier, part, hash == nullptr);
+// The third tier: persistent work-stealing warps, one search each, over
+// global-memory arenas, in two parts: part 1 takes the searches queued straight
+// for it (the large list first) and may run beside tiers 1 and 2; part 2 takes the
+// second tier's overflow.
+// Registers: 80 a thread (96 without the bound), so 24 one-warp CTAs fit an SM:
+// the searches are chains of dependent loads, and more warps in flight finish
+// more of them (measured: 40.7 against 41.9 ms a step).
+__global__ void __launch_bounds__(32, 24) k_search_warp(Prog P, Arch A, SearchArena SA, int part) {
+  // The search counters live in shared memory (the arena is in global memory):
+  // frontier sizes are read after every round.
+  __shared__ int s_ctr[8];
+  // The node hashes lie apart from the arenas (whose pool the fourth tier lays
+  // out anew) and are empty between searches: every search empties the slots
+  // it used, also when it outgrew its arena. They were cleared with the context,
+  // so a launch clears nothing. (A launch that began by clearing its warps'
+  // 256 KB hashes wrote 956 MB and took 145 us with no search to run; the launch
+  // appears twice in a step.)
+  const Arena a = carve(SA.global + (int64_t)blockIdx.x * SA.bytes, SA.hash + (int64_t)blockIdx.x * 2 * SA.nodes,
+                        SA.nodes, SA.src, SA.layers, s_ctr);
+  run_tasks(WarpGroup{}, P, A, a, 3, part, false);
 }
 
 // The fourth tier: a CTA per search, over a global-memory arena of its own
@@ -1222,10 +1029,6 @@ int search_warps_per_sm() {
 
 void launch_search(const Prog& P, const Arch& A, const SearchArena* tiers, const SearchFork* fork, cudaStream_t st,
                    int sms, int64_t* launches) {
-  // Each launch requests its own tier's arena size.
-  const size_t smem1 = (size_t)tiers[0].bytes * kWarpsPerCta;
-  const size_t smem2 = (size_t)tiers[1].bytes;
-  allow_max_smem(k_search_warp);
   // The searches queued straight for the third tier depend on nothing the
   // first two tiers do: with a second stream they run beside them (no kernel
   // waits on another; the join only orders the third tier's second part,
@@ -1239,16 +1042,14 @@ void launch_search(const Prog& P, const Arch& A, const SearchArena* tiers, const
     s3 = fork->side;
   }
   // No launch takes more groups than there can be tasks (one per use entry).
-  const int most = (int)std::min<int64_t>(P.queue_cap, INT32_MAX);
-  const int g1 = std::max(1, std::min(tiers[0].warps, most) / kWarpsPerCta);
-  const int g2 = std::min(tiers[1].warps, most), g3 = std::min(tiers[2].warps, most);
-  k_search_warp<<<g1, kWarpsPerCta * 32, smem1, st>>>(P, A, tiers[0], 1, 0);
-  k_search_warp<<<g3, 32, 0, s3>>>(P, A, tiers[2], 3, 1);
+  const int g3 = (int)std::min<int64_t>(tiers[2].warps, P.queue_cap);
+  launch_search_lanes(P, A, tiers[0], 1, st, launches);
+  k_search_warp<<<g3, 32, 0, s3>>>(P, A, tiers[2], 1);
   if (fork) cudaEventRecord(fork->join, fork->side);
-  k_search_warp<<<g2, 32, smem2, st>>>(P, A, tiers[1], 2, 0);
+  launch_search_lanes(P, A, tiers[1], 2, st, launches);
   if (fork) cudaStreamWaitEvent(st, fork->join, 0);
-  k_search_warp<<<g3, 32, 0, st>>>(P, A, tiers[2], 3, 2);
-  *launches += 4;
+  k_search_warp<<<g3, 32, 0, st>>>(P, A, tiers[2], 2);
+  *launches += 2;
   if (P.t4_nodes > 0) {
     // The fourth tier runs after the third on this stream, so the third tier's
     // arena pool is free by then: when it holds more fourth-tier arenas than the

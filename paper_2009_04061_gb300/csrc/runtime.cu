@@ -296,36 +296,33 @@ gpa_status gpa_create(const gpa_arch_desc* arch, const gpa_options* opts, gpa_ct
   if (o.search_slots == 0) o.search_slots = search_warps_per_sm() * c->sms;
   if (o.max_sources_per_use == 0) o.max_sources_per_use = kBigSrc;
   if (o.large_search_nodes == 0) o.large_search_nodes = kLargeNodes;
-  if (o.small_search_nodes == 0) o.small_search_nodes = 64;
+  if (o.small_search_nodes == 0) o.small_search_nodes = 16;
   if (o.small_search_warps == 0) o.small_search_warps = 24;
   c->opts = o;
-  // Tier 1: four warps per CTA with small shared-memory arenas, six CTAs per
-  // SM by default (small_search_warps): as many warps as the search kernel's
-  // registers allow. The searches are chains of dependent steps, so more warps
-  // in flight finish more of them (on the batched workload, 64-node arenas at
-  // 24 warps per SM take the first tier from 26.0 to 22.2 ms against 128-node
-  // arenas at 12, while the third tier's hinted part runs beside it). Tier 2: three one-warp CTAs per SM with larger shared-memory arenas
-  // (one per SM beyond 512 nodes). Tier 3: warps
-  // with global-memory arenas for the rare searches beyond that. Node
-  // capacities are powers of two (hash masks).
+  // Tiers 1 and 2: one search a lane over shared-memory arenas, as many one-warp
+  // CTAs per SM as their arenas fit. Tier 3: warps with global-memory arenas
+  // for the searches beyond that. Node capacities are powers of two (hash
+  // masks); a lane's arena holds at most 128 (byte indices).
   int n1 = 2, n3 = 2;
-  while (n1 < o.small_search_nodes && n1 < 1024) n1 <<= 1;
+  while (n1 < o.small_search_nodes && n1 < kLaneNodes) n1 <<= 1;
   while (n3 < o.max_search_nodes) n3 <<= 1;
-  int n2 = 2;
-  const int want2 = o.mid_search_nodes ? o.mid_search_nodes : n1;
-  while (n2 < want2 && n2 < 1024) n2 <<= 1;
-  n2 = std::max(n1, n2);
+  int n2 = n1;
+  const int want2 = o.mid_search_nodes ? o.mid_search_nodes : 64;
+  while (n2 < want2 && n2 < kLaneNodes) n2 <<= 1;
   SearchArena* T = c->tier;
-  T[0].nodes = n1; T[0].src = std::min(n1, 64); T[0].layers = 4; T[0].warps = o.small_search_warps * c->sms;
-  T[1].nodes = n2; T[1].src = std::min(n2, 256); T[1].layers = 4; T[1].warps = (n2 <= 512 ? 3 : 1) * c->sms;
+  auto lane_tier = [&](int nodes, int most) {
+    SearchArena t{};
+    t.nodes = nodes;
+    t.bytes = search_lane_bytes(nodes);
+    // a CTA's arena and the 1 KB the system reserves for it, in 227 KB of an SM
+    t.warps = c->sms * (int)std::max<int64_t>(1, std::min<int64_t>(most, 227 * 1024 / (t.bytes + 1024)));
+    return t;
+  };
+  T[0] = lane_tier(n1, o.small_search_warps);
+  T[1] = lane_tier(n2, 32);
   T[2].nodes = n3; T[2].src = std::min(n3, 1024); T[2].layers = kMaxLayers; T[2].warps = o.search_slots;
-  for (int t = 0; t < 3; ++t) {
-    T[t].bytes = search_arena_bytes(T[t].nodes, T[t].src, T[t].layers, t < 2);
-    T[t].global = nullptr;
-    T[t].hash = nullptr;
-  }
+  T[2].bytes = search_arena_bytes(T[2].nodes, T[2].src, T[2].layers, false);
   gpa_status s = GPA_OK;
-  if (T[0].bytes * 4 > 220 * 1024 || T[1].bytes > 220 * 1024) s = GPA_ERR_INVALID_ARG;
   if (!s && cudaMalloc(&T[2].global, (size_t)T[2].bytes * T[2].warps) != cudaSuccess) {
     T[2].global = nullptr;
     s = GPA_ERR_OOM;
