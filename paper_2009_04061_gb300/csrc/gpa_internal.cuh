@@ -41,9 +41,9 @@ enum {
   // cycles of its five phases.
   SS_PHASE = 13, SS_SIZES = 31, SS_PASSB = 47, SS_SLOW = 48,
   // 55: unused
-  SS_OVF3_N = 56, SS_OVF3_HEAD = 57,  // searches handed on to the program's own fourth tier
+  SS_OVF3_N = 56, SS_OVF3_HEAD = 57,  // searches that outgrew the shared-memory warps (bottom of queue[3])
   SS_SIZE_CYC = 58,  // with -DGPA_PHASE_TIMING: cycles of the searches by log2 of their node count (16)
-  SS_HINT3_N = 74,   // searches queued straight for the third tier (from the top of `queue`)
+  SS_HINT3_N = 74,   // searches queued straight for the global-memory warps (from the top of queue[3])
   SS_FAILBITS = 75,  // why a step reported GPA_ERR_CAPACITY: the last search tier ran out of
                      // 1 nodes, 2 edges, 3 occurrences, 4 sources, 5 back-edge layers,
                      // 6 hash rounds; 8 queue, 9 sources per use, 10 merged edges,
@@ -53,14 +53,17 @@ enum {
   SS_COV_ALL = 80,   // the counting pass's total of sources before pruning
   SS_XN = 81,        // unpruned edges written by the export pass
   SS_HIST_HEAD = 82, // next chunk of the run-aware aggregation kernel (reset before each launch)
-  SS_HINT3_HEAD = 83,  // next of the searches queued straight for the third tier
-  SS_OVF3H_N = 84,     // searches for the fourth tier stored from the top of `ovf_queue`
-  SS_LARGE_N = 85,     // entries of large_queue
+  SS_HINT3_HEAD = 83,  // next of them
+  SS_T4_N = 84, SS_T4_HEAD = 85,  // searches for the fourth tier (queue[4])
   SS_REACH_CLS = 86,   // next entry of reach_order for each of the staged fixpoint's 4 launches
   SS_SUSE_N = 90,      // entries of suse (the stalled uses of this step)
   SS_ADV_HEAD = 91,    // next entry of reach_order for the advice kernel's CTAs
-  SS_N = 92
+  // searches queued straight for a size class of the shared-memory warps
+  SS_A1_N = 92, SS_A2_N = 93, SS_A3_N = 94, SS_A1_HEAD = 95,  // (heads 95-97)
+  SS_N = 98
 };
+// Values of tier_hint: the queue that a use entry's search belongs to.
+enum { kHintLane2 = 2, kHintA1 = 3, kHintA3 = 5, kHintWarp = 6, kHintCta = 7 };
 
 struct Arch {
   int32_t n_op;
@@ -141,13 +144,17 @@ struct Prog {
   int32_t* head;                  // ni: raw-edge list head per use (-1 = none)
   int4* raw;                      // raw edges: def, next, dmin, dlong | flags << 24
   int64_t raw_cap;
-  int4* queue;                    // general searches: use, resource, start literal set, use entry
-  int32_t large_nodes;            // node count from which a third-tier search is started early
-  uint8_t* large_hint;            // n_use: 1 when the entry's last third-tier search had large_nodes nodes or more
-  int4* large_queue;              // kLargeQueue: such searches, started before the other third-tier ones
-  uint32_t* tier_hint;            // n_use: smallest search tier known to hold the entry's search (0: none);
+  // General searches. A task is named by its use entry e; tasks[e] = {use,
+  // resource | start literal set << 9 | blocked << 25}. Each queue has queue_cap
+  // entries: 0 first tier from the bottom (after it the second tier's overflow),
+  // first size class of the shared-memory warps from the top; 1 second tier,
+  // second class; 2 third class; 3 overflow to the global-memory warps, searches
+  // queued straight for them; 4 fourth tier. An entry is in one region of a
+  // queue at a time, so the two regions never meet.
+  int2* tasks;                    // n_use
+  int32_t* queue[5];
+  uint32_t* tier_hint;            // n_use: the queue known to hold the entry's search (0: none);
                                   // kept across steps (a search's size depends only on the program)
-  int4* ovf_queue;                // general searches that outgrew a small scratch slot
   int64_t queue_cap;
   int32_t* edge_cnt;              // ni + 1 (exclusive scan in place -> offsets)
   int32_t* big_use;               // ni: uses with more than kMaxSrc sources (SS_BIG_N of them)
@@ -335,14 +342,13 @@ __host__ __device__ inline int64_t reach_smem_need(int64_t nbf, int64_t ne, int6
 // the larger a function, the fewer warps per SM its launch runs.
 constexpr int64_t kReachClassCap[4] = {200 * 1024, 64 * 1024, 28 * 1024, 12 * 1024};
 constexpr int64_t kReachSmemCap = 200 * 1024;
-// A second stream (and two events) on which the searches queued straight for
-// the third tier run beside the first two tiers.
+// Two more streams (and their events) on which the searches queued straight
+// for the shared-memory and the global-memory warps run beside the first two
+// tiers.
 struct SearchFork {
-  cudaStream_t side;
-  cudaEvent_t fork, join;
+  cudaStream_t side[2];
+  cudaEvent_t fork, join[2];
 };
-constexpr int kLargeQueue = 4096;  // capacity of large_queue
-constexpr int kLargeNodes = 1024;  // default of large_nodes
 void launch_blame(const Prog& P, const Arch& A, const SearchArena* tiers, const SearchFork* fork, int max_src,
                   int32_t* scan_tmp, cudaStream_t st, int sms, int64_t* launches);
 void launch_search(const Prog& P, const Arch& A, const SearchArena* tiers, const SearchFork* fork, cudaStream_t st,
@@ -354,6 +360,8 @@ int search_lane_width(int nodes);      // lanes of a warp that search, for arena
 int64_t search_lane_bytes(int nodes);  // their arenas, in bytes a warp
 void launch_search_lanes(const Prog& P, const Arch& A, const SearchArena& T, int tier, cudaStream_t st,
                          int64_t* launches);
+void launch_search_smem(const Prog& P, const Arch& A, int most_nodes, int part, cudaStream_t st, int sms,
+                        int64_t* launches);
 int search_warps_per_sm();  // resident one-warp CTAs of the search kernel per SM (global-memory tiers)
 void launch_build_meta(const Prog& P, int4* meta, cudaStream_t st, int sms, int64_t* launches);
 void launch_build_events(const Prog& P, int32_t* ev_off, uint32_t* events, int32_t* tmp, cudaStream_t st, int sms,

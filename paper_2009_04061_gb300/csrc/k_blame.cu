@@ -182,38 +182,19 @@ __global__ void k_search_local(Prog P, Arch A) {
         continue;
       }
       if (P.diag) cov_add(P, e, n_all, n_kept);  // the in-block part; the search adds the rest
-      // A search known to outgrow the first tier goes straight to the tier
-      // that held it before: the second tier's queue; the third tier's large
-      // list (searches that had large_nodes nodes or more, started first) or
-      // its region at the top of the first queue; or the fourth tier's region
-      // at the top of the overflow queue.
+      // A search known to outgrow the first tier goes straight to the queue
+      // that held it before (see Prog::queue).
       const uint32_t hint = P.tier_hint[e];
-      const int4 task = make_int4(j, r, (int)S | (blocked ? 1 << 20 : 0), e);
-      if (hint >= 4 && P.t4_nodes > 0) {
-        const unsigned long long t = atomicAdd(&P.stats[SS_OVF3H_N], 1ull);
-        if (t < (unsigned long long)P.queue_cap) P.ovf_queue[P.queue_cap - 1 - (int64_t)t] = task;
-        else capacity(P, 8);
-      } else if (hint >= 3) {
-        bool placed = false;
-        if (P.large_hint[e]) {
-          const unsigned long long t = atomicAdd(&P.stats[SS_LARGE_N], 1ull);
-          if (t < (unsigned long long)kLargeQueue) {
-            P.large_queue[t] = task;
-            placed = true;
-          }
-        }
-        if (!placed) {
-          const unsigned long long t = atomicAdd(&P.stats[SS_HINT3_N], 1ull);
-          if (t < (unsigned long long)P.queue_cap) P.queue[P.queue_cap - 1 - (int64_t)t] = task;
-          else capacity(P, 8);
-        }
-      } else {
-        const int slot = hint == 2 ? SS_OVF_N : SS_QUEUE_N;
-        int4* q = hint == 2 ? P.ovf_queue : P.queue;
-        const unsigned long long t = atomicAdd(&P.stats[slot], 1ull);
-        if (t < (unsigned long long)P.queue_cap) q[t] = task;
-        else capacity(P, 8);
-      }
+      P.tasks[e] = make_int2(j, r | ((int)S << 9) | (blocked ? 1 << 25 : 0));
+      int slot = SS_QUEUE_N, q = 0;
+      bool top = false;
+      if (hint >= kHintCta && P.t4_nodes > 0) { slot = SS_T4_N; q = 4; }
+      else if (hint >= kHintWarp) { slot = SS_HINT3_N; q = 3; top = true; }
+      else if (hint >= kHintA1) { slot = SS_A1_N + (int)hint - kHintA1; q = (int)hint - kHintA1; top = hint < kHintA3; }
+      else if (hint == kHintLane2) { slot = SS_OVF_N; q = 1; }
+      const unsigned long long t = atomicAdd(&P.stats[slot], 1ull);
+      if (t < (unsigned long long)P.queue_cap) P.queue[q][top ? P.queue_cap - 1 - (int64_t)t : (int64_t)t] = e;
+      else capacity(P, 8);
     }
   }
 }

@@ -4,8 +4,9 @@
 //
 // The third and fourth search tier: one search group per (use, resource) task, a
 // warp in the third tier, a whole CTA in the fourth (searches of tens of
-// thousands to millions of nodes); searches of up to 128 nodes run one to a lane
-// before them (k_search_lanes.cu). The graph of (block, literal set) nodes lives
+// thousands to millions of nodes); searches of up to 64 nodes run one to a lane
+// before them (k_search_lanes.cu), those of up to 5,632 one to a warp in shared
+// memory (k_search_smem.cu). The graph of (block, literal set) nodes lives
 // in the group's arena in global memory. The group's threads scan node blocks in parallel
 // through per-block event lists (defs and unguarded reads, bottom-up), insert
 // nodes and sources into open-addressing hashes together, relax distances and
@@ -915,65 +916,44 @@ __device__ bool group_search(const G& g, const Prog& P, const Arch& A, const Are
 }
 
 // The task loop of a search group: claim (use, resource) tasks from one
-// queue until it is empty. Tier 3 part 1 reads the large list and the region at
-// the top of the first queue, part 2 the second overflow, which reuses the first
-// queue's storage; tier 4 the third overflow (bottom of the first overflow
-// queue's storage) and its top region. A search that outgrows its tier is
-// queued for the next one; the last tier records why it ran out. An arena
-// that holds its own hash (`clear`) has it emptied when the group's first task
-// arrives, so a group that finds none touches no memory.
+// queue until it is empty. A search that outgrows the third tier is queued for
+// the fourth; the last tier records why it ran out. An arena that holds its own
+// hash (`clear`) has it emptied when the group's first task arrives, so a group
+// that finds none touches no memory.
 template <class G>
 __device__ void run_tasks(const G& g, const Prog& P, const Arch& A, const Arena& a, int tier, int part, bool clear) {
   const int me = g.rank();
-  // The tasks of this launch, in order: nl of the large list, n0 read up
-  // from the bottom of q0, n1 read down from the top of q1.
+  // part 1: the searches queued straight for these warps; part 2: the
+  // shared-memory warps' overflow
   const unsigned long long cap = (unsigned long long)P.queue_cap;
-  const int4* q0 = P.queue;
-  const int4* q1 = P.queue;
-  unsigned long long nl = 0, n0 = 0, n1 = 0;
-  int h_slot = 0;
-  if (tier == 3 && part == 1) {
-    nl = min(P.stats[SS_LARGE_N], (unsigned long long)kLargeQueue);
-    n1 = P.stats[SS_HINT3_N], h_slot = SS_HINT3_HEAD;
-  } else if (tier == 3) {
-    n0 = P.stats[SS_OVF2_N], h_slot = SS_OVF2_HEAD;
-  } else {
-    q0 = q1 = P.ovf_queue, n0 = P.stats[SS_OVF3_N], n1 = P.stats[SS_OVF3H_N], h_slot = SS_OVF3_HEAD;
-  }
-  n0 = min(n0, cap);
-  n1 = min(n1, cap - n0);
+  const int32_t* q = P.queue[tier];
+  const bool top = tier == 3 && part == 1;
+  const unsigned long long nt = min(P.stats[tier == 4 ? SS_T4_N : top ? SS_HINT3_N : SS_OVF3_N], cap);
+  const int h_slot = tier == 4 ? SS_T4_HEAD : top ? SS_HINT3_HEAD : SS_OVF3_HEAD;
   while (true) {
     unsigned long long t = 0;
     if (me == 0) t = atomicAdd(&P.stats[h_slot], 1ull);
     t = g.broadcast(t);
-    if (t >= nl + n0 + n1) break;
+    if (t >= nt) break;
     if (clear) {
       for (int k = me; k < 2 * a.N; k += G::kSize) a.ht[k] = -1;
       g.sync();
       clear = false;
     }
-    const int4 task = t < nl        ? P.large_queue[t]
-                      : t < nl + n0 ? q0[t - nl]
-                                    : q1[cap - 1 - (t - nl - n0)];
+    const int e = q[top ? cap - 1 - t : t];
+    const int2 packed = P.tasks[e];
+    const int4 task = make_int4(packed.x, packed.y & 0x1FF, (int)((uint32_t)packed.y >> 9 & 0xFFFFu), e);
     const int f = P.block_func[P.instr_block[task.x]];
     // The coverage count needs every source: no latency bound.
     const int bound = P.diag ? kInf - 1 : P.res_maxlat[(size_t)f * kNumRes + task.y];
     const uint16_t live = live_literals(P.res_guards[(size_t)f * kNumRes + task.y], P.guard[task.x]);
     const bool ok = group_search(g, P, A, a, task.x, task.y, (uint16_t)task.z, bound, live, tier, task.w,
-                                 (task.z >> 20) & 1);
-    if (ok) {
-      // later steps start a large third-tier search before the others
-      if (me == 0 && tier == 3 && !P.diag && ((volatile int*)a.ctr)[0] >= P.large_nodes) P.large_hint[task.w] = 1;
-      continue;
-    }
-    if (me != 0) continue;
-    if (!P.diag) atomicMax(&P.tier_hint[task.w], (unsigned)(tier + 1));  // later steps queue it for a bigger tier
+                                 (packed.y >> 25) & 1);
+    if (ok || me != 0) continue;
     if (tier == 3 && P.t4_nodes > 0) {
-      // part 2 -> bottom of ovf_queue (after tier 2 read it); part 1, which may
-      // run beside tier 1, -> top of ovf_queue
-      const bool top = part == 1;
-      const unsigned long long o = atomicAdd(&P.stats[top ? SS_OVF3H_N : SS_OVF3_N], 1ull);
-      if (o < cap) P.ovf_queue[top ? cap - 1 - o : o] = task; else capacity(P, 8);
+      if (!P.diag) atomicMax(&P.tier_hint[e], (unsigned)kHintCta);  // later steps queue it there
+      const unsigned long long o = atomicAdd(&P.stats[SS_T4_N], 1ull);
+      if (o < cap) P.queue[4][o] = e; else capacity(P, 8);
     } else {
       capacity(P, a.ctr[7] > 0 ? a.ctr[7] : 1);  // the last tier: why it ran out
     }
@@ -982,8 +962,8 @@ __device__ void run_tasks(const G& g, const Prog& P, const Arch& A, const Arena&
 
 // The third tier: persistent work-stealing warps, one search each, over
 // global-memory arenas, in two parts: part 1 takes the searches queued straight
-// for it (the large list first) and may run beside tiers 1 and 2; part 2 takes the
-// second tier's overflow.
+// for it and runs beside the other tiers; part 2 takes the shared-memory warps'
+// overflow.
 // Registers: 80 a thread (96 without the bound), so 24 one-warp CTAs fit an SM:
 // the searches are chains of dependent loads, and more warps in flight finish
 // more of them (measured: 40.7 against 41.9 ms a step).
@@ -1029,25 +1009,32 @@ int search_warps_per_sm() {
 
 void launch_search(const Prog& P, const Arch& A, const SearchArena* tiers, const SearchFork* fork, cudaStream_t st,
                    int sms, int64_t* launches) {
-  // The searches queued straight for the third tier depend on nothing the
-  // first two tiers do: with a second stream they run beside them (no kernel
-  // waits on another; the join only orders the third tier's second part,
-  // which shares its arenas, after them).
-  // Tier 1 is submitted first, so its CTAs take their share of each SM and the
-  // third tier's warps fill the registers left beside them.
-  cudaStream_t s3 = st;
+  // The searches queued straight for the larger tiers depend on nothing the
+  // first two tiers do: with further streams they run beside them (no kernel
+  // waits on another; the joins only order the parts that share arenas or
+  // storage after them). They are submitted first, so that the largest searches
+  // start first and the first tiers' CTAs fill the SMs as they come free.
+  cudaStream_t s1 = st, s3 = st;
   if (fork) {
     cudaEventRecord(fork->fork, st);
-    cudaStreamWaitEvent(fork->side, fork->fork, 0);
-    s3 = fork->side;
+    s3 = fork->side[0];
+    s1 = fork->side[1];
+    cudaStreamWaitEvent(s3, fork->fork, 0);
+    cudaStreamWaitEvent(s1, fork->fork, 0);
   }
   // No launch takes more groups than there can be tasks (one per use entry).
   const int g3 = (int)std::min<int64_t>(tiers[2].warps, P.queue_cap);
-  launch_search_lanes(P, A, tiers[0], 1, st, launches);
   k_search_warp<<<g3, 32, 0, s3>>>(P, A, tiers[2], 1);
-  if (fork) cudaEventRecord(fork->join, fork->side);
+  launch_search_smem(P, A, tiers[2].nodes, 1, s1, sms, launches);
+  launch_search_lanes(P, A, tiers[0], 1, st, launches);
   launch_search_lanes(P, A, tiers[1], 2, st, launches);
-  if (fork) cudaStreamWaitEvent(st, fork->join, 0);
+  if (fork) {
+    cudaEventRecord(fork->join[0], s3);
+    cudaEventRecord(fork->join[1], s1);
+    cudaStreamWaitEvent(st, fork->join[0], 0);
+    cudaStreamWaitEvent(st, fork->join[1], 0);
+  }
+  launch_search_smem(P, A, tiers[2].nodes, 2, st, sms, launches);
   k_search_warp<<<g3, 32, 0, st>>>(P, A, tiers[2], 2);
   *launches += 2;
   if (P.t4_nodes > 0) {

@@ -97,16 +97,17 @@ struct LaneSearch {
   LaneArena<LPW> a;
   int state;
   int j, r, gj, e_use, b0, fb, bound, low;  // low: pass B's least block
-  uint16_t live, S0;
+  uint16_t live;
   bool blocked, pass_b, back;               // back: the graph has a back edge
   int nn, ne, no, nl;                       // nodes, edges, occurrences, unexpanded nodes
   int over;                                 // why the arena is too small (0: it is not)
 
-  __device__ __forceinline__ void begin(const Prog& P, const int4& task) {
+  __device__ __forceinline__ void begin(const Prog& P, int e) {
+    const int2 task = P.tasks[e];
+    e_use = e;
     j = task.x;
-    r = task.y;
-    e_use = task.w;
-    blocked = (task.z >> 20) & 1;
+    r = task.y & 0x1FF;
+    blocked = (task.y >> 25) & 1;
     gj = P.guard[j];
     b0 = P.instr_block[j];
     const int f = P.block_func[b0];
@@ -114,7 +115,7 @@ struct LaneSearch {
     const size_t fr = (size_t)f * kNumRes + r;
     bound = P.diag ? 0x7FFFFFFF : P.res_maxlat[fr];  // the coverage count needs every source
     live = live_literals(P.res_guards[fr], gj);
-    S0 = keep_literals((uint16_t)task.z, live);
+    const uint16_t S0 = keep_literals((uint16_t)((uint32_t)task.y >> 9), live);
     over = P.func_block_off[f + 1] - fb > 0xFFFF ? 1 : 0;
     for (int h = 0; h < a.occ - a.hash; ++h) a.word(a.hash + h) = 0u;
     a.node(0, W_KEY) = (uint32_t)(b0 - fb) | ((uint32_t)S0 << 16);
@@ -226,9 +227,6 @@ struct LaneSearch {
     a.byte(u, W_EDGE, 1) = (uint8_t)(ne - ne0);
     if (over) state = L_FINISH;
   }
-
-  // The task again, for the next tier's queue.
-  __device__ __forceinline__ int4 task() const { return make_int4(j, r, (int)S0 | (blocked ? 1 << 20 : 0), e_use); }
 
   __device__ __forceinline__ int wall_of(int u) const { return a.half(u, W_INFO, 0); }
   __device__ __forceinline__ int len_of(int u) const { return a.half(u, W_LEN, 0); }
@@ -488,7 +486,7 @@ __global__ void __launch_bounds__(32) k_search_lanes(Prog P, Arch A, int nodes, 
   extern __shared__ __align__(16) uint32_t lane_sm[];
   const int lane = threadIdx.x;
   const unsigned long long cap = (unsigned long long)P.queue_cap;
-  const int4* tasks = tier == 1 ? P.queue : P.ovf_queue;
+  const int32_t* queue = P.queue[tier - 1];
   const unsigned long long n_tasks = min(P.stats[tier == 1 ? SS_QUEUE_N : SS_OVF_N], cap);
   unsigned long long* head = &P.stats[tier == 1 ? SS_QUEUE_HEAD : SS_OVF_HEAD];
   if (n_tasks == 0) return;
@@ -525,12 +523,10 @@ __global__ void __launch_bounds__(32) k_search_lanes(Prog P, Arch A, int nodes, 
 #endif
           if (s.over) {
             if (!P.diag) atomicMax(&P.tier_hint[s.e_use], (unsigned)(tier + 1));  // later steps queue it there
-            // first tier -> bottom of ovf_queue; second tier -> bottom of queue
+            // first tier -> bottom of queue 1; second tier -> bottom of queue 0
             const unsigned long long o = atomicAdd(&P.stats[tier == 1 ? SS_OVF_N : SS_OVF2_N], 1ull);
-            if (o < cap)
-              (tier == 1 ? P.ovf_queue : P.queue)[o] = s.task();
-            else
-              capacity(P, 8);
+            if (o < cap) P.queue[2 - tier][o] = s.e_use;
+            else capacity(P, 8);
           }
         }
       }
@@ -543,7 +539,7 @@ __global__ void __launch_bounds__(32) k_search_lanes(Prog P, Arch A, int nodes, 
       more = t + (unsigned long long)__popc(idle) < n_tasks;
       if (s.state == L_IDLE) {
         t += (unsigned long long)__popc(idle & ((1u << lane) - 1u));
-        if (t < n_tasks) s.begin(P, tasks[t]);
+        if (t < n_tasks) s.begin(P, queue[t]);
       }
       __syncwarp();
     } else if (growing) {

@@ -1,0 +1,805 @@
+// Step (b)/(c), general backward searches (Sec. 4), the middle tier: one search
+// per warp over an arena in shared memory, up to 5,632 (block, literal set)
+// nodes.
+//
+// These searches grow four or five nodes a wave over hundreds of waves, and
+// each of their later steps (fewest back edges, rule 2's reachability, longest
+// paths) walks the graph's depth level by level, so a search is a chain of
+// thousands of dependent accesses to its own arena and the largest one decides
+// how long a step takes. What bounds it is the latency of that arena: in global
+// memory (k_search_warp, 700 cycles an access) a search of 227 nodes took 650 us
+// and one of 5,269 took 6.4 ms. So the arena is laid out small enough for shared
+// memory: 36.5 bytes a node (16-bit node, edge and list indices; distance and
+// parent in one word; words that later steps reuse) plus the hash, and holds the
+// block lengths that the global-memory search reads from the program again and
+// again.
+//
+// One CTA of 16 warps per SM gives its 227 KB to one size class after another:
+// 1 search of 5,632 nodes, 4 of 1,280, 16 of 320. Searches that an earlier step
+// of the program found to be of a class are queued for it and run largest class
+// first; a search that outgrows its class goes on a list of its CTA, which works
+// off its lists in ascending order at the end. Beyond the last class (or a full
+// list) the global-memory tier takes over.
+//
+// The graph, the passes and the rules are those of k_search.cu's group search;
+// like the one-lane search (k_search_lanes.cu) it ends early when its only
+// unexpanded node meets an unguarded reader of r before any def was met.
+#include <algorithm>
+
+#include "gpa_internal.cuh"
+
+namespace gpa {
+
+namespace {
+
+constexpr int kWarps = 16;
+constexpr int kClasses = 3;
+constexpr int kLocalList = 256;      // searches a CTA keeps for its own next class
+constexpr int kDistBits = 19, kIdxBits = 13;
+constexpr uint32_t kFar = (1u << kDistBits) - 1u;  // no distance yet
+constexpr uint32_t kIdxMask = (1u << kIdxBits) - 1u;
+constexpr uint32_t kNoWall = 0xFFFFu;
+constexpr uint32_t F_EXP = 1u << 24, F_QUE = 1u << 25, F_NEED = 1u << 26, F_BACK = 1u << 27;
+constexpr int kSearchInf = 0x7FFFFFFF;
+
+__host__ __device__ inline int class_nodes(int c, int most) {
+  const int n = c == 0 ? 320 : c == 1 ? 1280 : 5632;
+  return n < most ? n : most;
+}
+__host__ __device__ inline int class_warps(int c) { return c == 0 ? 16 : c == 1 ? 4 : 1; }
+__host__ __device__ inline int hash_slots(int n) {  // a power of two, at least 1.4 n
+  int h = 16;
+  while (5 * h < 7 * n) h <<= 1;
+  return h;
+}
+__host__ __device__ inline int n_occ(int n) { return n / 4 < 8 ? 8 : (n / 4 + 1) & ~1; }
+__host__ __device__ inline int n_src(int n) { return n / 8 < 8 ? 8 : n / 8; }
+__host__ __device__ inline int n_edge(int n) { return (3 * n / 2 + 3) & ~1; }
+__host__ __device__ inline int64_t warp_arena_bytes(int n) {
+  const int64_t nn = (n + 1) & ~1;
+  const int64_t b = 4 * (6 * nn + n_occ(n) + 4 * (int64_t)n_src(n)) +
+                    2 * (3 * nn + n_edge(n) + hash_slots(n) + n_occ(n));
+  return (b + 15) & ~(int64_t)15;
+}
+
+struct WArena {
+  int n, occs, srcs, edges;
+  uint32_t hmask;
+  uint32_t *key;   // block (relative to the function) | literal set << 16
+  uint32_t *dp;    // distance << 13 | parent; then the reach mask; then a layer's longest distance
+  uint32_t *wl;    // wall position (kNoWall: none) | instructions of the block << 16
+  uint32_t *ef;    // first edge | edges << 16 | flags << 24
+  uint32_t *kk;    // fewest back edges; then forward in-edges | in-edges left << 16
+  uint32_t *gx;    // two 16-bit lists; then the wall group + 1; then the next layer's longest distance
+  uint32_t *oc;    // per occurrence: position | node << 16 | def kind << 29
+  uint32_t *si, *sd, *sk, *sh;  // per source: block | position << 16; distance << 13 | nearest occurrence;
+                                // fewest back edges | cut << 31; first occurrence
+  uint16_t *l0, *l1, *l2;  // node lists
+  uint16_t *ed;    // edges: target | back << 15
+  uint16_t *ht;    // node (or source) hash: 0xFFFF empty, 0xFFFE being filled
+  uint16_t *on;    // per occurrence: the next of its source
+  volatile int *ctr;  // 0 nodes, 1 edges, 2 occurrences, 3 unexpanded nodes, 4 too small, 5-6 list lengths, 7 back edges
+  uint16_t *wpos;  // 32 wall positions
+};
+
+__device__ WArena carve(char* base, int n, int* ctr, uint16_t* wpos) {
+  WArena a;
+  const int nn = (n + 1) & ~1;
+  a.n = n; a.occs = n_occ(n); a.srcs = n_src(n); a.edges = n_edge(n);
+  const int hs = hash_slots(n);
+  a.hmask = (uint32_t)hs - 1u;
+  uint32_t* p = reinterpret_cast<uint32_t*>(base);
+  a.key = p; p += nn; a.dp = p; p += nn; a.wl = p; p += nn;
+  a.ef = p; p += nn; a.kk = p; p += nn; a.gx = p; p += nn;
+  a.oc = p; p += a.occs;
+  a.si = p; p += a.srcs; a.sd = p; p += a.srcs; a.sk = p; p += a.srcs; a.sh = p; p += a.srcs;
+  uint16_t* q = reinterpret_cast<uint16_t*>(p);
+  a.l0 = q; q += nn; a.l1 = q; q += nn; a.l2 = q; q += nn;
+  a.ed = q; q += a.edges;
+  a.ht = q; q += hs;
+  a.on = q;
+  a.ctr = ctr;
+  a.wpos = wpos;
+  return a;
+}
+
+__device__ __forceinline__ uint32_t mix(uint32_t k) {
+  uint32_t h = (k & 0xFFFFu) * 0x9E3779B1u ^ ((k >> 16) * 0x85EBCA77u);
+  return h ^ (h >> 15);
+}
+__device__ __forceinline__ void prefetch_l1(const void* p) {
+  asm volatile("prefetch.global.L1 [%0];" ::"l"(__cvta_generic_to_global(p)));
+}
+
+// One search by one warp. Returns 0 when it is done, else why its arena is too
+// small (nothing was emitted).
+__device__ int warp_search(const Prog& P, const Arch& A, const WArena& a, int j, int r, uint16_t S0, int e_use,
+                           bool blocked) {
+  const int lane = threadIdx.x & 31;
+  const unsigned lt = (1u << lane) - 1u;
+  volatile int* ctr = a.ctr;
+  const int gj = P.guard[j];
+  const int b0 = P.instr_block[j];
+  const int f = P.block_func[b0];
+  const int fb = P.func_block_off[f];
+  if (P.func_block_off[f + 1] - fb > 0xFFFF) {  // its blocks need more than the arena's 16 bits
+    if (lane == 0) ctr[0] = 0;
+    __syncwarp();
+    return 1;
+  }
+  const size_t fr = (size_t)f * kNumRes + r;
+  const int bound = P.diag ? kSearchInf : P.res_maxlat[fr];
+  const uint16_t live = live_literals(P.res_guards[fr], gj);
+  const int w = r >> 5;
+  const uint32_t bit = 1u << (r & 31);
+  S0 = keep_literals(S0, live);
+  auto clear_hash = [&]() {
+    uint32_t* h = reinterpret_cast<uint32_t*>(a.ht);
+    for (uint32_t i = lane; i <= a.hmask / 2; i += 32) h[i] = 0xFFFFFFFFu;
+  };
+  auto fail = [&](int why) { if (ctr[4] == 0) ctr[4] = why; };
+  // every lane reads the flag before any of them may set it again
+  auto failed = [&]() -> int {
+    __syncwarp();
+    const int x = ctr[4];
+    __syncwarp();
+    return x;
+  };
+  auto dist_of = [&](int u) { return a.dp[u] >> kIdxBits; };
+  auto len_of = [&](int u) { return a.wl[u] >> 16; };
+  auto wall_of = [&](int u) { return a.wl[u] & 0xFFFFu; };
+  auto occ_node = [&](int o) { return (int)((a.oc[o] >> 16) & kIdxMask); };
+  auto occ_pos = [&](int o) { return (int)(a.oc[o] & 0xFFFFu); };
+
+  clear_hash();
+  if (lane == 0) {
+    ctr[0] = 1; ctr[1] = 0; ctr[2] = 0; ctr[3] = 1; ctr[4] = 0; ctr[5] = 0; ctr[6] = 0; ctr[7] = 0;
+    a.key[0] = (uint32_t)(b0 - fb) | ((uint32_t)S0 << 16);
+    a.dp[0] = 0u; a.wl[0] = kNoWall; a.ef[0] = 0u;
+    a.l0[0] = 0;
+  }
+  __syncwarp();
+  uint16_t* ub = a.l0;   // unexpanded nodes: ctr[3] of them
+  uint16_t* uk = a.l1;
+  uint16_t* const d0 = reinterpret_cast<uint16_t*>(a.gx);  // nodes to relax from: ctr[5] of them
+  uint16_t* const d1 = d0 + a.n;
+
+  // Expands the nodes of l2, 32 at a time: parallel scans, then linking. With
+  // `only`, the single node dominates everything beyond it and no def was met
+  // yet: returns true when it meets an unguarded reader before any def.
+  auto expand = [&](int cnt, bool only) -> bool {
+    for (int c0 = 0; c0 < cnt; c0 += 32) {
+      const bool mine = c0 + lane < cnt;
+      const int u = mine ? a.l2[c0 + lane] : 0;
+      const uint32_t key = a.key[u];
+      const int B = fb + (int)(key & 0xFFFFu);
+      uint16_t S = (uint16_t)(key >> 16);
+      int4 pm = make_int4(0, 0, -1, -1);
+      uint32_t ro0 = 0u, ro1 = 0u;
+      bool stop = !mine, cut = false;
+      int len = 0;
+      if (mine) {
+        const int4 m0 = __ldg(&P.block_meta[2 * (size_t)B]);
+        pm = __ldg(&P.block_meta[2 * (size_t)B + 1]);
+        const uint32_t tw = __ldg(&P.touch_mask[(size_t)B * kWords + w]);
+        const size_t seg = (size_t)B * kEvBuckets + ev_bucket(r);
+        const int ev_beg = __ldg(&P.ev_off[seg]);
+        int ev_end = __ldg(&P.ev_off[seg + 1]);
+        if (!(tw & bit) || u == 0) ev_end = ev_beg;
+        if (pm.z >= 0) {
+          ro0 = P.rout[(size_t)pm.z * kWords + w];
+          prefetch_l1(&P.block_meta[2 * (size_t)pm.z]);
+          prefetch_l1(&P.touch_mask[(size_t)pm.z * kWords + w]);
+          prefetch_l1(&P.ev_off[(size_t)pm.z * kEvBuckets + ev_bucket(r)]);
+        }
+        if (pm.w >= 0) {
+          ro1 = P.rout[(size_t)pm.w * kWords + w];
+          prefetch_l1(&P.block_meta[2 * (size_t)pm.w]);
+          prefetch_l1(&P.touch_mask[(size_t)pm.w * kWords + w]);
+          prefetch_l1(&P.ev_off[(size_t)pm.w * kEvBuckets + ev_bucket(r)]);
+        }
+        uint32_t wall = kNoWall;
+        int last_def = -1;
+        bool any_def = false;
+        for (int e0 = ev_beg; e0 < ev_end && !stop; e0 += 4) {
+          uint32_t evs[4];
+#pragma unroll
+          for (int q = 0; q < 4; ++q) evs[q] = e0 + q < ev_end ? __ldg(&P.events[e0 + q]) : 0x1FFu;
+#pragma unroll
+          for (int q = 0; q < 4; ++q) {
+            const uint32_t ev = evs[q];
+            if (stop || (int)(ev & 0x1FFu) != r) continue;
+            const int pos = (int)(ev >> 16), x = m0.x + pos;
+            if (ev & 0x200u) {  // def of r
+              last_def = pos;
+              if (!contains(S, gj) && !(B == b0 && x < j)) {  // sources above j in its block are settled
+                any_def = true;
+                const int o = atomicAdd((int*)&ctr[2], 1);
+                if (o < a.occs) a.oc[o] = (uint32_t)pos | ((uint32_t)u << 16) | (((ev >> 10) & 3u) << 29);
+                else fail(3);
+              }
+              S = add_literal(S, (int)((ev >> 12) & 0xFu));
+              if (contains(S, gj)) stop = true;
+            } else if (wall == kNoWall && pos != last_def && x != j) {  // unguarded reader of r
+              wall = (uint32_t)pos;
+              cut |= only && !any_def;
+            }
+          }
+        }
+        len = u == 0 ? j - m0.x + 1 : m0.y - m0.x;
+        a.wl[u] = wall | ((uint32_t)len << 16);
+        if (stop) pm = make_int4(0, 0, -1, -1);
+      }
+      if (__any_sync(0xffffffffu, cut)) return true;
+      // Linking: the edge range from a prefix sum, then each lane finds or adds
+      // the nodes of its predecessors that a def of r leaves; a lane claims an
+      // empty slot, fills it in the same round, and lanes that met the claim look
+      // again in the next.
+      auto reaches = [&](int q) -> bool {
+        const int k = q - pm.x;
+        if (k == 0) return ro0 & bit;
+        if (k == 1) return ro1 & bit;
+        return P.rout[(size_t)__ldg(&P.pred[q]) * kWords + w] & bit;
+      };
+      int deg = 0;
+      for (int q = pm.x; q < pm.y; ++q) deg += reaches(q) ? 1 : 0;
+      int incl = deg;
+#pragma unroll
+      for (int o = 1; o < 32; o <<= 1) {
+        const int y = __shfl_up_sync(0xffffffffu, incl, o);
+        if (lane >= o) incl += y;
+      }
+      const int total = __shfl_sync(0xffffffffu, incl, 31);
+      const int maxdeg = __reduce_max_sync(0xffffffffu, deg);
+      const int ne = ctr[1];
+      if (ne + total > a.edges || maxdeg > 255) fail(2);
+      if (failed()) return false;
+      const int at = ne + incl - deg;
+      if (mine) a.ef[u] = (uint32_t)at | ((uint32_t)deg << 16) | F_EXP;
+      __syncwarp();
+      const int Sout = (int)keep_literals(S, live);
+      uint32_t nd = 0xFFFFFFFFu;
+      if (mine) {
+        const uint32_t d = dist_of(u) + (uint32_t)len;
+        if (d >= kFar) fail(1);
+        nd = (d << kIdxBits) | (uint32_t)u;
+      }
+      int qp = pm.x;
+      bool back = false;
+      for (int kk = 0; kk < maxdeg; ++kk) {
+        bool pending = kk < deg;
+        int p = -1;
+        if (pending) {
+          while (!reaches(qp)) ++qp;
+          const int k = qp - pm.x;
+          p = k == 0 ? pm.z : k == 1 ? pm.w : __ldg(&P.pred[qp]);
+          ++qp;
+        }
+        const uint32_t pk = (uint32_t)(p - fb) | ((uint32_t)Sout << 16);
+        uint32_t h = mix(pk) & a.hmask;
+        int v = -1;
+        for (int round = 0; round < 4 * (int)a.hmask + 64; ++round) {
+          if (!__any_sync(0xffffffffu, pending)) break;
+          if (pending) {
+            const uint32_t c = *(volatile uint16_t*)&a.ht[h];
+            if (c < 0xFFFEu) {
+              if (*(volatile uint32_t*)&a.key[c] == pk) { v = (int)c; pending = false; }
+              else h = (h + 1) & a.hmask;
+            } else if (c == 0xFFFFu) {
+              if (atomicCAS((unsigned short*)&a.ht[h], (unsigned short)0xFFFF, (unsigned short)0xFFFE) == 0xFFFF) {
+                const int nv = atomicAdd((int*)&ctr[0], 1);
+                pending = false;
+                if (nv >= a.n) {
+                  fail(1);
+                  *(volatile uint16_t*)&a.ht[h] = 0xFFFF;
+                } else {
+                  a.key[nv] = pk; a.wl[nv] = kNoWall; a.ef[nv] = 0u;
+                  a.dp[nv] = 0xFFFFFFFFu;
+                  ub[atomicAdd((int*)&ctr[3], 1)] = (uint16_t)nv;
+                  __threadfence_block();
+                  *(volatile uint16_t*)&a.ht[h] = (uint16_t)nv;
+                  v = nv;
+                }
+              }
+            }  // 0xFFFE: another lane is filling this slot
+          }
+          __syncwarp();
+        }
+        if (pending) fail(6);  // the round limit is a bound, not expected to be reached
+        if (kk < deg && v >= 0) {
+          back |= p >= B;
+          a.ed[at + kk] = (uint16_t)(v | (p >= B ? 0x8000 : 0));
+          if (nd < *(volatile uint32_t*)&a.dp[v] && atomicMin(&a.dp[v], nd) > nd &&
+              (*(volatile uint32_t*)&a.ef[v] & F_EXP) && !(atomicOr(&a.ef[v], F_QUE) & F_QUE))
+            d0[atomicAdd((int*)&ctr[5], 1)] = (uint16_t)v;
+        }
+      }
+      if (back) ctr[7] = 1;
+      __syncwarp();
+      if (lane == 0) ctr[1] = ne + total;
+      if (failed()) return false;
+    }
+    return false;
+  };
+
+  // Carries improved distances on from the listed expanded nodes (d0, ctr[5]).
+  auto relax = [&]() {
+    uint16_t* cur = d0;
+    uint16_t* nxt = d1;
+    int fs = ctr[5];
+    __syncwarp();
+    while (fs > 0) {
+      if (lane == 0) ctr[5] = 0;
+      __syncwarp();
+      for (int i = lane; i < fs; i += 32) {
+        const int u = cur[i];
+        const uint32_t ef = atomicAnd(&a.ef[u], ~F_QUE);
+        const uint32_t d = (*(volatile uint32_t*)&a.dp[u] >> kIdxBits) + len_of(u);
+        if (d >= kFar) { fail(1); continue; }
+        const uint32_t nd = (d << kIdxBits) | (uint32_t)u;
+        const int e0 = (int)(ef & 0xFFFFu), e1 = e0 + (int)((ef >> 16) & 0xFFu);
+        for (int e = e0; e < e1; ++e) {
+          const int v = a.ed[e] & 0x7FFF;
+          if (nd < *(volatile uint32_t*)&a.dp[v] && atomicMin(&a.dp[v], nd) > nd &&
+              (*(volatile uint32_t*)&a.ef[v] & F_EXP) && !(atomicOr(&a.ef[v], F_QUE) & F_QUE))
+            nxt[atomicAdd((int*)&ctr[5], 1)] = (uint16_t)v;
+        }
+      }
+      __syncwarp();
+      fs = ctr[5];
+      uint16_t* sw = cur; cur = nxt; nxt = sw;
+      __syncwarp();
+    }
+    if (lane == 0) ctr[5] = 0;
+    __syncwarp();
+  };
+
+  bool cand = false, pass_b = false;
+  int low = 0;
+  while (true) {
+    // A wave: the unexpanded nodes within the bound (pass B: those that can lie
+    // on a path from a source within its latency; the others are dropped).
+    const int m = ctr[3];
+    const bool only = m == 1 && ctr[2] == 0 && !pass_b && !P.diag;
+    int cnt = 0, kept = 0;
+    for (int i0 = 0; i0 < m; i0 += 32) {
+      const int i = i0 + lane;
+      const int u = i < m ? ub[i] : 0;
+      const bool now = i < m && (pass_b ? fb + (int)(a.key[u] & 0xFFFFu) >= low : (int)dist_of(u) <= bound);
+      const bool keep = i < m && !now && !pass_b;
+      const unsigned mn = __ballot_sync(0xffffffffu, now), mk = __ballot_sync(0xffffffffu, keep);
+      if (now) a.l2[cnt + __popc(mn & lt)] = (uint16_t)u;
+      if (keep) uk[kept + __popc(mk & lt)] = (uint16_t)u;
+      cnt += __popc(mn);
+      kept += __popc(mk);
+    }
+    __syncwarp();
+    uint16_t* sw = ub; ub = uk; uk = sw;
+    if (lane == 0) ctr[3] = kept;
+    __syncwarp();
+    if (cnt > 0) {
+      if (expand(cnt, only)) return 0;  // every source lies beyond one unguarded reader
+      if (const int why = failed()) return why;
+      relax();
+      if (const int why = failed()) return why;
+      continue;
+    }
+    if (pass_b) break;
+    // End of pass A: a source within its latency? (A source farther than the
+    // bound fails rule 3.)
+    const int no = ctr[2];
+    int lo = kSearchInf;
+    for (int o = lane; o < no; o += 32) {
+      const int u = occ_node(o);
+      const int d = (int)dist_of(u) + (int)len_of(u) - 1 - occ_pos(o);
+      if (d > bound) continue;
+      const int B = fb + (int)(a.key[u] & 0xFFFFu);
+      if (d <= A.lat[P.opclass[P.block_meta[2 * (size_t)B].x + occ_pos(o)]]) lo = min(lo, P.block_minreach[B]);
+    }
+    low = __reduce_min_sync(0xffffffffu, lo);
+    cand = low != kSearchInf;
+    if (!cand) break;
+    pass_b = true;
+  }
+  if (!cand && !P.diag) return 0;
+  const int n = ctr[0], no = ctr[2];
+
+  // Fewest back edges from j: layer by layer, forward edges within a layer,
+  // back edges into the next (every node is listed once).
+  if (ctr[7]) {
+    for (int u = lane; u < n; u += 32) a.kk[u] = u == 0 ? 0u : 0xFFFFu;
+    if (lane == 0) { a.l0[0] = 0; ctr[5] = 0; ctr[6] = 0; }
+    __syncwarp();
+    int fs = 1;
+    uint16_t* cur = a.l0;
+    uint16_t* nxt = a.l1;
+    for (uint32_t k = 0; fs > 0; ++k) {
+      while (fs > 0) {
+        for (int i = lane; i < fs; i += 32) {
+          const int u = cur[i];
+          const uint32_t ef = *(volatile uint32_t*)&a.ef[u];
+          const int e0 = (int)(ef & 0xFFFFu), e1 = e0 + (int)((ef >> 16) & 0xFFu);
+          for (int e = e0; e < e1; ++e) {
+            const int ed = a.ed[e], v = ed & 0x7FFF;
+            if (*(volatile uint32_t*)&a.kk[v] <= k) continue;
+            if (ed & 0x8000) {
+              if (!(atomicOr(&a.ef[v], F_BACK) & F_BACK)) a.l2[atomicAdd((int*)&ctr[6], 1)] = (uint16_t)v;
+            } else if (atomicMin(&a.kk[v], k) > k) {
+              nxt[atomicAdd((int*)&ctr[5], 1)] = (uint16_t)v;
+            }
+          }
+        }
+        __syncwarp();
+        fs = ctr[5];
+        uint16_t* sw = cur; cur = nxt; nxt = sw;
+        __syncwarp();
+        if (lane == 0) ctr[5] = 0;
+        __syncwarp();
+      }
+      // the back edges' targets that no fewer back edges reached
+      const int nb = ctr[6];
+      for (int i = lane; i < nb; i += 32) {
+        const int v = a.l2[i];
+        atomicAnd(&a.ef[v], ~F_BACK);
+        if (atomicMin(&a.kk[v], k + 1) > k + 1) cur[atomicAdd((int*)&ctr[5], 1)] = (uint16_t)v;
+      }
+      __syncwarp();
+      fs = ctr[5];
+      __syncwarp();
+      if (lane == 0) { ctr[5] = 0; ctr[6] = 0; }
+      __syncwarp();
+    }
+  }
+  const bool has_back = ctr[7];
+
+  // Sources: a hash keyed by (block, position) gives each an index; per source
+  // the shortest distance with its occurrence, the fewest back edges, and its
+  // occurrences chained.
+  clear_hash();
+  if (lane == 0) ctr[5] = 0;
+  __syncwarp();
+  for (int o0 = 0; o0 < no; o0 += 32) {
+    const int o = o0 + lane;
+    bool pending = o < no;
+    const int u = pending ? occ_node(o) : 0;
+    const uint32_t id = pending ? (a.key[u] & 0xFFFFu) | ((uint32_t)occ_pos(o) << 16) : 0u;
+    uint32_t h = mix(id) & a.hmask;
+    int m = -1;
+    for (int round = 0; round < 4 * (int)a.hmask + 64; ++round) {
+      if (!__any_sync(0xffffffffu, pending)) break;
+      if (pending) {
+        const uint32_t c = *(volatile uint16_t*)&a.ht[h];
+        if (c < 0xFFFEu) {
+          if (*(volatile uint32_t*)&a.si[c] == id) { m = (int)c; pending = false; }
+          else h = (h + 1) & a.hmask;
+        } else if (c == 0xFFFFu) {
+          if (atomicCAS((unsigned short*)&a.ht[h], (unsigned short)0xFFFF, (unsigned short)0xFFFE) == 0xFFFF) {
+            const int nm = atomicAdd((int*)&ctr[5], 1);
+            pending = false;
+            if (nm >= a.srcs) {
+              fail(4);
+              *(volatile uint16_t*)&a.ht[h] = 0xFFFF;
+            } else {
+              a.si[nm] = id; a.sd[nm] = 0xFFFFFFFFu; a.sk[nm] = 0xFFFFu; a.sh[nm] = 0xFFFFu;
+              __threadfence_block();
+              *(volatile uint16_t*)&a.ht[h] = (uint16_t)nm;
+              m = nm;
+            }
+          }
+        }
+      }
+      __syncwarp();
+    }
+    if (pending) fail(6);
+    if (m >= 0) {
+      const uint32_t d = dist_of(u) + len_of(u) - 1u - (uint32_t)occ_pos(o);
+      atomicMin(&a.sd[m], (d << kIdxBits) | (uint32_t)o);
+      atomicMin(&a.sk[m], has_back ? a.kk[u] : 0u);
+      a.on[o] = (uint16_t)atomicExch(&a.sh[m], (uint32_t)o);
+    }
+    __syncwarp();
+  }
+  if (const int why = failed()) return why;
+  const int nsrc = ctr[5];
+  auto src_instr = [&](int m) {
+    return P.block_meta[2 * (size_t)(fb + (int)(a.si[m] & 0xFFFFu))].x + (int)(a.si[m] >> 16);
+  };
+  int alive = 0;
+  for (int m = lane; m < nsrc; m += 32) {
+    const int op = P.opclass[src_instr(m)];
+    bool drop = (int)(a.sd[m] >> kIdxBits) > A.lat[op];                    // rule 3
+    if (P.diag == 1 && (blocked || !keeps_any(P, A, j, op))) drop = true;  // rule 2 above j, rule 1
+    if (P.diag == 2) drop = false;                                         // export: rule 2 for every source
+    if (drop) a.sk[m] |= 1u << 31;
+    alive += drop ? 0 : 1;
+  }
+  alive = __reduce_add_sync(0xffffffffu, alive);
+  if (alive == 0) {
+    if (P.diag == 1 && lane == 0) cov_add(P, e_use, nsrc, 0);
+    return 0;
+  }
+
+  // Rule 2. The walls that can cut a source lie on the parent chain of its
+  // nearest occurrence: mark their nodes.
+  __syncwarp();
+  for (int m = lane; m < nsrc; m += 32) {
+    if (a.sk[m] >> 31) continue;
+    const int o = (int)(a.sd[m] & kIdxMask), u = occ_node(o);
+    if (wall_of(u) != kNoWall && (int)wall_of(u) > occ_pos(o)) atomicOr(&a.ef[u], F_NEED);
+    for (int v = (int)(a.dp[u] & kIdxMask), hops = 0; v > 0 && hops < n; v = (int)(a.dp[v] & kIdxMask), ++hops)
+      if (wall_of(v) != kNoWall) atomicOr(&a.ef[v], F_NEED);
+  }
+  __syncwarp();
+  for (int u = lane; u < n; u += 32) a.gx[u] = 0u;
+  __syncwarp();
+  // Up to 32 wall groups at a time, one per block (the reader met first from
+  // the bottom over the block's nodes): bit g of a node's mask says it is reached
+  // without passing group g's wall; a node of the group passes every bit on but
+  // its own.
+  int scan0 = 0;
+  while (alive > 0) {
+    int ng = 0;
+    while (scan0 < n && ng < 32) {
+      const int u = scan0 + lane;
+      const unsigned need = __ballot_sync(0xffffffffu, u < n && (*(volatile uint32_t*)&a.ef[u] & F_NEED));
+      if (!need) { scan0 += 32; continue; }
+      const uint32_t B = a.key[scan0 + __ffs(need) - 1] & 0xFFFFu;
+      int wp = 0;
+      for (int v = lane; v < n; v += 32) {
+        if (v == 0 || (a.key[v] & 0xFFFFu) != B || wall_of(v) == kNoWall) continue;
+        a.gx[v] = (uint32_t)(ng + 1);
+        atomicAnd(&a.ef[v], ~F_NEED);
+        wp = max(wp, (int)wall_of(v));
+      }
+      wp = __reduce_max_sync(0xffffffffu, wp);
+      if (lane == 0) a.wpos[ng] = (uint16_t)wp;
+      ++ng;
+      __syncwarp();
+    }
+    if (ng == 0) break;
+    const uint32_t full = ng == 32 ? 0xFFFFFFFFu : (1u << ng) - 1u;
+    for (int u = lane; u < n; u += 32) a.dp[u] = u == 0 ? full : 0u;
+    if (lane == 0) { a.l0[0] = 0; ctr[5] = 0; }
+    __syncwarp();
+    uint16_t* cur = a.l0;
+    uint16_t* nxt = a.l1;
+    int fs = 1;
+    while (fs > 0) {
+      // The whole frontier's queued flags first: bits that reach a frontier node
+      // during this round queue it again.
+      for (int i = lane; i < fs; i += 32) atomicAnd(&a.ef[cur[i]], ~F_QUE);
+      __syncwarp();
+      for (int i = lane; i < fs; i += 32) {
+        const int u = cur[i];
+        const uint32_t g = a.gx[u];
+        const uint32_t mk = *(volatile uint32_t*)&a.dp[u] & (g ? ~(1u << (g - 1)) : 0xFFFFFFFFu);
+        if (!mk) continue;
+        const uint32_t ef = *(volatile uint32_t*)&a.ef[u];
+        const int e0 = (int)(ef & 0xFFFFu), e1 = e0 + (int)((ef >> 16) & 0xFFu);
+        for (int e = e0; e < e1; ++e) {
+          const int v = a.ed[e] & 0x7FFF;
+          if (!(mk & ~*(volatile uint32_t*)&a.dp[v])) continue;
+          const uint32_t old = atomicOr(&a.dp[v], mk);
+          if ((old | mk) != old && !(atomicOr(&a.ef[v], F_QUE) & F_QUE))
+            nxt[atomicAdd((int*)&ctr[5], 1)] = (uint16_t)v;
+        }
+      }
+      __syncwarp();
+      fs = ctr[5];
+      uint16_t* sw = cur; cur = nxt; nxt = sw;
+      __syncwarp();
+      if (lane == 0) ctr[5] = 0;
+      __syncwarp();
+    }
+    // A source survives if, for every group, one of its occurrences is reached
+    // without passing that group's wall.
+    int dropped = 0;
+    for (int m = lane; m < nsrc; m += 32) {
+      if (a.sk[m] >> 31) continue;
+      uint32_t ok = 0u;
+      for (uint32_t o = a.sh[m]; o != 0xFFFFu && ok != full; o = a.on[o]) {
+        const int u = occ_node((int)o);
+        const uint32_t g = a.gx[u];
+        uint32_t rr = a.dp[u];
+        if (g && occ_pos((int)o) < (int)a.wpos[g - 1]) rr &= ~(1u << (g - 1));
+        ok |= rr;
+      }
+      if (ok != full) { a.sk[m] |= 1u << 31; ++dropped; }
+    }
+    alive -= __reduce_add_sync(0xffffffffu, dropped);
+    if (scan0 >= n) break;
+    __syncwarp();
+    for (int u = lane; u < n; u += 32) a.gx[u] = 0u;
+    __syncwarp();
+  }
+  if (P.diag == 1) {
+    if (lane == 0) cov_add(P, e_use, nsrc, alive);
+    return 0;
+  }
+  const bool every = P.diag == 2;  // the export keeps every source (the cut is its dom flag)
+  if (alive == 0 && !every) return 0;
+
+  // Longest path with exactly K back edges: one layer per back edge, each a DAG
+  // of forward edges processed in Kahn's order; back edges feed the next layer.
+  __syncwarp();
+  int maxk = 0;
+  for (int m = lane; m < nsrc; m += 32)
+    if (!(a.sk[m] >> 31) || every) maxk = max(maxk, (int)(a.sk[m] & 0xFFFFu));
+  maxk = __reduce_max_sync(0xffffffffu, maxk);
+  if (maxk >= kMaxLayers) return 5;
+  for (int u = lane; u < n; u += 32) {
+    a.kk[u] = 0u;
+    a.dp[u] = u == 0 ? 0u : 0xFFFFFFFFu;
+    a.gx[u] = 0xFFFFFFFFu;
+  }
+  __syncwarp();
+  const int ne = ctr[1];
+  for (int e = lane; e < ne; e += 32) {
+    const int ed = a.ed[e];
+    if (!(ed & 0x8000)) atomicAdd(&a.kk[ed], 1u);
+  }
+  __syncwarp();
+  for (int l = 0; l <= maxk; ++l) {
+    int fs = 0;
+    for (int u0 = 0; u0 < n; u0 += 32) {
+      const int u = u0 + lane;
+      const uint32_t in = u < n ? a.kk[u] & 0xFFFFu : 1u;
+      const unsigned z = __ballot_sync(0xffffffffu, in == 0u);
+      if (u < n) a.kk[u] = in | (in << 16);
+      if (in == 0u) a.l0[fs + __popc(z & lt)] = (uint16_t)u;
+      fs += __popc(z);
+    }
+    uint16_t* cur = a.l0;
+    uint16_t* nxt = a.l1;
+    if (lane == 0) ctr[5] = 0;
+    __syncwarp();
+    while (fs > 0) {
+      for (int i = lane; i < fs; i += 32) {
+        const int u = cur[i];
+        const int cv = *(volatile int*)&a.dp[u];
+        const int nd = cv + (int)len_of(u);
+        const uint32_t ef = a.ef[u];
+        const int e0 = (int)(ef & 0xFFFFu), e1 = e0 + (int)((ef >> 16) & 0xFFu);
+        for (int e = e0; e < e1; ++e) {
+          const int ed = a.ed[e], v = ed & 0x7FFF;
+          if (ed & 0x8000) {
+            if (cv >= 0 && l < maxk) atomicMax((int*)&a.gx[v], nd);
+          } else {
+            if (cv >= 0) atomicMax((int*)&a.dp[v], nd);
+            if ((atomicSub(&a.kk[v], 1u << 16) >> 16) == 1u) nxt[atomicAdd((int*)&ctr[5], 1)] = (uint16_t)v;
+          }
+        }
+      }
+      __syncwarp();
+      fs = ctr[5];
+      uint16_t* sw = cur; cur = nxt; nxt = sw;
+      __syncwarp();
+      if (lane == 0) ctr[5] = 0;
+      __syncwarp();
+    }
+    for (int m = lane; m < nsrc; m += 32) {
+      const bool cut = a.sk[m] >> 31;
+      if ((cut && !every) || (int)(a.sk[m] & 0xFFFFu) != l) continue;
+      int best = -1;
+      uint32_t kind = 0;
+      for (uint32_t o = a.sh[m]; o != 0xFFFFu; o = a.on[o]) {
+        const int u = occ_node((int)o), d = *(volatile int*)&a.dp[u];
+        kind = (a.oc[o] >> 29) & 3u;
+        if (d >= 0) best = max(best, d + (int)len_of(u) - 1 - occ_pos((int)o));
+      }
+      if (best < 1) { capacity(P, 13); continue; }
+      const int dmin = (int)(a.sd[m] >> kIdxBits);
+      if (every) xemit(P, j, src_instr(m), r, dmin, l, best, cut || blocked);
+      else emit_raw(P, A, j, src_instr(m), r, (int)kind, dmin, best);
+    }
+    __syncwarp();
+    if (l < maxk) {
+      for (int u = lane; u < n; u += 32) {
+        a.dp[u] = a.gx[u];
+        a.gx[u] = 0xFFFFFFFFu;
+      }
+      __syncwarp();
+    }
+  }
+  return 0;
+}
+
+// part 1: the searches queued for a class, largest class first (beside tiers 1
+// and 2); part 2: the second tier's overflow, from the first class up.
+__global__ void __launch_bounds__(kWarps * 32, 1) k_search_smem(Prog P, Arch A, int most_nodes, int part) {
+  extern __shared__ __align__(16) char smem[];
+  __shared__ int s_ctr[kWarps][8];
+  __shared__ uint16_t s_wpos[kWarps][32];
+  __shared__ int s_local[kClasses][kLocalList];  // use entries to redo in class c
+  __shared__ int s_nlocal[kClasses], s_hlocal[kClasses];
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  const unsigned long long cap = (unsigned long long)P.queue_cap;
+  unsigned long long n_tasks[kClasses] = {0, 0, 0};
+  if (part == 1) {
+    n_tasks[0] = min(P.stats[SS_A1_N], cap);
+    n_tasks[1] = min(P.stats[SS_A2_N], cap);
+    n_tasks[2] = min(P.stats[SS_A3_N], cap);
+  } else {
+    n_tasks[0] = min(P.stats[SS_OVF2_N], cap);
+  }
+  if (n_tasks[0] + n_tasks[1] + n_tasks[2] == 0) return;
+  if (threadIdx.x < kClasses) { s_nlocal[threadIdx.x] = 0; s_hlocal[threadIdx.x] = 0; }
+  __syncthreads();
+  unsigned long long runs = 0, most = 0, most_task = 0;
+
+  auto run_class = [&](int c, bool local) {
+    const int n = class_nodes(c, most_nodes);
+    if (warp < class_warps(c)) {
+      const WArena a = carve(smem + warp * warp_arena_bytes(n), n, s_ctr[warp], s_wpos[warp]);
+      // queue 0 top, queue 1 top, queue 2; the second tier's overflow: queue 0
+      const int32_t* q = c == 0 ? P.queue[0] : c == 1 ? P.queue[1] : P.queue[2];
+      const bool top = part == 1 && c < 2;
+      const int head = part == 1 ? SS_A1_HEAD + c : SS_OVF2_HEAD;
+      while (true) {
+        int e = -1;
+        if (lane == 0) {
+          if (local) {
+            const int t = atomicAdd(&s_hlocal[c], 1);
+            if (t < min(s_nlocal[c], kLocalList)) e = s_local[c][t];
+          } else {
+            const unsigned long long t = atomicAdd(&P.stats[head], 1ull);
+            if (t < n_tasks[c]) e = q[top ? cap - 1 - t : t];
+          }
+        }
+        e = __shfl_sync(0xffffffffu, e, 0);
+        if (e < 0) break;
+        const int2 task = P.tasks[e];
+        const int j = task.x, r = task.y & 0x1FF;
+        const int over = warp_search(P, A, a, j, r, (uint16_t)((uint32_t)task.y >> 9), e, (task.y >> 25) & 1);
+        const unsigned long long nn = (unsigned long long)max(min(s_ctr[warp][0], n), 0);
+        __syncwarp();
+        ++runs;
+        most = max(most, nn);
+        most_task = max(most_task, (nn << 40) | ((unsigned long long)r << 31) | (unsigned)j);
+        if (lane != 0) continue;
+#ifdef GPA_PHASE_TIMING
+        atomicAdd(&P.stats[SS_SIZES + min(15, 31 - __clz(max((int)nn, 1)))], 1ull);
+#endif
+        if (!over) continue;
+        int next = c + 1;  // the next class that is larger than this one
+        if (next < kClasses && class_nodes(next, most_nodes) == n) next = kClasses;
+        if (!P.diag) atomicMax(&P.tier_hint[e], (unsigned)(kHintA1 + next));
+        if (next < kClasses) {
+          const int t = atomicAdd(&s_nlocal[next], 1);
+          if (t < kLocalList) { s_local[next][t] = e; continue; }
+        }
+        const unsigned long long o = atomicAdd(&P.stats[SS_OVF3_N], 1ull);
+        if (o < cap) P.queue[3][o] = e; else capacity(P, 8);
+      }
+    }
+    __syncthreads();
+  };
+  if (part == 1) {
+    for (int c = kClasses - 1; c >= 0; --c)
+      if (n_tasks[c]) run_class(c, false);
+  } else {
+    run_class(0, false);
+  }
+  for (int c = 1; c < kClasses; ++c)
+    if (s_nlocal[c]) run_class(c, true);
+  if (lane == 0 && runs) {
+    atomicAdd(&P.stats[SS_GENERAL], runs);
+    atomicMax(&P.stats[SS_MAX_NODES], most);
+    atomicMax(&P.stats[SS_MAX_TASK], most_task);
+  }
+}
+
+}  // namespace
+
+void launch_search_smem(const Prog& P, const Arch& A, int most_nodes, int part, cudaStream_t st, int sms,
+                        int64_t* launches) {
+  size_t smem = 0;
+  for (int c = 0; c < kClasses; ++c)
+    smem = std::max(smem, (size_t)(class_warps(c) * warp_arena_bytes(class_nodes(c, most_nodes))));
+  allow_max_smem(k_search_smem);
+  const int grid = (int)std::max<int64_t>(1, std::min<int64_t>(sms, P.queue_cap));
+  k_search_smem<<<grid, kWarps * 32, smem, st>>>(P, A, most_nodes, part);
+  ++*launches;
+}
+
+}  // namespace gpa

@@ -55,7 +55,7 @@ struct gpa_ctx {
   cudaStream_t capture_stream = nullptr;  // private stream for gpa_step_capture
   cudaStream_t build_stream = nullptr;    // program allocation, copies and layout builds
   cudaEvent_t ev_copied[2] = {nullptr, nullptr}, ev_used[2] = {nullptr, nullptr};
-  gpa::SearchFork fork{nullptr, nullptr, nullptr};  // third-tier searches beside tiers 1-2
+  gpa::SearchFork fork{};  // larger searches beside tiers 1-2
 };
 
 namespace {
@@ -295,7 +295,6 @@ gpa_status gpa_create(const gpa_arch_desc* arch, const gpa_options* opts, gpa_ct
   // global-memory arenas hide latency better than few on shared memory.
   if (o.search_slots == 0) o.search_slots = search_warps_per_sm() * c->sms;
   if (o.max_sources_per_use == 0) o.max_sources_per_use = kBigSrc;
-  if (o.large_search_nodes == 0) o.large_search_nodes = kLargeNodes;
   if (o.small_search_nodes == 0) o.small_search_nodes = 16;
   if (o.small_search_warps == 0) o.small_search_warps = 24;
   c->opts = o;
@@ -337,17 +336,21 @@ gpa_status gpa_create(const gpa_arch_desc* arch, const gpa_options* opts, gpa_ct
   if (!s && cudaMemset(T[2].hash, 0xFF, hash_bytes) != cudaSuccess) s = GPA_ERR_CUDA;
   if (!s && cudaEventCreateWithFlags(&c->scratch_ev, cudaEventDisableTiming) != cudaSuccess) s = GPA_ERR_CUDA;
   if (!s && cudaStreamCreateWithFlags(&c->build_stream, cudaStreamNonBlocking) != cudaSuccess) s = GPA_ERR_CUDA;
-  if (!s && cudaStreamCreateWithFlags(&c->fork.side, cudaStreamNonBlocking) != cudaSuccess) s = GPA_ERR_CUDA;
   if (!s && cudaEventCreateWithFlags(&c->fork.fork, cudaEventDisableTiming) != cudaSuccess) s = GPA_ERR_CUDA;
-  if (!s && cudaEventCreateWithFlags(&c->fork.join, cudaEventDisableTiming) != cudaSuccess) s = GPA_ERR_CUDA;
+  for (int k = 0; k < 2; ++k) {
+    if (!s && cudaStreamCreateWithFlags(&c->fork.side[k], cudaStreamNonBlocking) != cudaSuccess) s = GPA_ERR_CUDA;
+    if (!s && cudaEventCreateWithFlags(&c->fork.join[k], cudaEventDisableTiming) != cudaSuccess) s = GPA_ERR_CUDA;
+  }
   if (s) {
     if (c->tier[2].global) cudaFree(c->tier[2].global);
     if (c->tier[2].hash) cudaFree(c->tier[2].hash);
     if (c->scratch_ev) cudaEventDestroy(c->scratch_ev);
     if (c->build_stream) cudaStreamDestroy(c->build_stream);
-    if (c->fork.side) cudaStreamDestroy(c->fork.side);
     if (c->fork.fork) cudaEventDestroy(c->fork.fork);
-    if (c->fork.join) cudaEventDestroy(c->fork.join);
+    for (int k = 0; k < 2; ++k) {
+      if (c->fork.side[k]) cudaStreamDestroy(c->fork.side[k]);
+      if (c->fork.join[k]) cudaEventDestroy(c->fork.join[k]);
+    }
     delete c;
     return s;
   }
@@ -370,9 +373,11 @@ gpa_status gpa_destroy(gpa_ctx* ctx) {
   if (ctx->capture_stream) cudaStreamDestroy(ctx->capture_stream);
   if (ctx->build_stream) cudaStreamDestroy(ctx->build_stream);
   if (ctx->scratch_ev) cudaEventDestroy(ctx->scratch_ev);
-  if (ctx->fork.side) cudaStreamDestroy(ctx->fork.side);
   if (ctx->fork.fork) cudaEventDestroy(ctx->fork.fork);
-  if (ctx->fork.join) cudaEventDestroy(ctx->fork.join);
+  for (int k = 0; k < 2; ++k) {
+    if (ctx->fork.side[k]) cudaStreamDestroy(ctx->fork.side[k]);
+    if (ctx->fork.join[k]) cudaEventDestroy(ctx->fork.join[k]);
+  }
   delete ctx;
   return GPA_OK;
 }
@@ -541,11 +546,9 @@ static gpa_status alloc_program(const gpa_program_desc* d, ProgramRec* R, int ti
   P.raw_cap = 2 * (int64_t)d->n_use + 1024;
   TRY(dev_alloc(R, &P.raw, (size_t)P.raw_cap));
   P.queue_cap = (int64_t)d->n_use + 1;
-  TRY(dev_alloc(R, &P.queue, (size_t)P.queue_cap));
-  TRY(dev_alloc(R, &P.ovf_queue, (size_t)P.queue_cap));
+  for (int k = 0; k < 5; ++k) TRY(dev_alloc(R, &P.queue[k], (size_t)P.queue_cap));
+  TRY(dev_alloc(R, &P.tasks, (size_t)std::max<int64_t>(d->n_use, 1)));
   TRY(dev_alloc(R, &P.tier_hint, (size_t)std::max<int64_t>(d->n_use, 1)));
-  TRY(dev_alloc(R, &P.large_hint, (size_t)std::max<int64_t>(d->n_use, 1)));
-  TRY(dev_alloc(R, &P.large_queue, (size_t)kLargeQueue));
   TRY(dev_alloc(R, &P.cov_cnt, (size_t)std::max<int64_t>(d->n_use, 1)));
   P.diag = 0;
   TRY(dev_alloc(R, &P.edge_off, ni + 1));
@@ -629,7 +632,6 @@ gpa_status gpa_load_program(gpa_ctx* ctx, const gpa_program_desc* d, gpa_pid* ou
   s = alloc_program(d, R, ctx->tier[2].nodes);
   if (s) { free_program(R); return s; }
   Prog& P = R->P;
-  P.large_nodes = ctx->opts.large_search_nodes;
   const size_t ni = P.ni;
   int32_t *pred_off = R->pred_off, *cursor = R->cursor, *ev_off = R->ev_off;
   uint32_t* events = R->events;
@@ -642,8 +644,7 @@ gpa_status gpa_load_program(gpa_ctx* ctx, const gpa_program_desc* d, gpa_pid* ou
     free_program(R);
     return GPA_ERR_CUDA;
   }
-  if (cudaMemsetAsync(P.tier_hint, 0, sizeof(uint32_t) * (size_t)std::max<int64_t>(R->n_use, 1), st) != cudaSuccess ||
-      cudaMemsetAsync(P.large_hint, 0, (size_t)std::max<int64_t>(R->n_use, 1), st) != cudaSuccess) {
+  if (cudaMemsetAsync(P.tier_hint, 0, sizeof(uint32_t) * (size_t)std::max<int64_t>(R->n_use, 1), st) != cudaSuccess) {
     free_program(R);
     return GPA_ERR_CUDA;
   }
@@ -1059,7 +1060,7 @@ gpa_status gpa_sync_status(gpa_ctx* ctx, gpa_pid pid, gpa_stream stream, int64_t
     info[2] = (int64_t)h[SS_MAX_NODES];
     info[3] = (int64_t)h[SS_SWEEPS];
     info[4] = (int64_t)h[SS_OVF_N];
-    info[5] = (int64_t)(h[SS_OVF2_N] + h[SS_HINT3_N] + std::min<unsigned long long>(h[SS_LARGE_N], kLargeQueue));
+    info[5] = (int64_t)(h[SS_OVF2_N] + h[SS_A1_N] + h[SS_A2_N] + h[SS_A3_N] + h[SS_HINT3_N]);
     info[6] = (int64_t)(h[SS_MAX_TASK] & 0x7FFFFFFFull);     // use of the largest search
     info[7] = (int64_t)((h[SS_MAX_TASK] >> 31) & 0x1FFull);  // its resource
   }
