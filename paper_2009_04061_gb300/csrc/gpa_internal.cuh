@@ -57,7 +57,7 @@ enum {
   SS_T4_N = 84, SS_T4_HEAD = 85,  // searches for the fourth tier (queue[4])
   SS_REACH_CLS = 86,   // next entry of reach_order for each of the staged fixpoint's 4 launches
   SS_SUSE_N = 90,      // entries of suse (the stalled uses of this step)
-  SS_ADV_HEAD = 91,    // next entry of reach_order for the advice kernel's CTAs
+  // 91: unused
   // searches queued straight for a size class of the shared-memory warps
   SS_A1_N = 92, SS_A2_N = 93, SS_A3_N = 94, SS_A1_HEAD = 95,  // (heads 95-97)
   SS_N = 98
@@ -77,6 +77,13 @@ struct Arch {
 struct LaunchRec {
   long long blocks;
   int32_t threads, regs, smem, reserved;
+};
+constexpr int kAdvTile = 1024;  // instructions of an advice tile
+constexpr int kAdvAcc = 14;     // per-function sums of the advice kernel, and its tiles that are done
+// A hotspot candidate of a tile.
+struct AdvCand {
+  unsigned long long v;
+  int32_t def, use, dist, pad;
 };
 struct SmModel {
   int32_t n_sms, schedulers, max_warps, max_blocks, regs, reg_unit, smem, smem_unit, smem_reserved;
@@ -168,7 +175,16 @@ struct Prog {
   unsigned long long* e_share;    // edges * 8
   int64_t edge_cap;
   unsigned long long* blame;      // ni * 24
-  // advice
+  // advice: tiles of at most kAdvTile instructions of one function
+  int32_t adv_tiles;
+  const int32_t* adv_tile_off;    // nf + 1: first tile of each function
+  const int32_t* adv_tile_func;   // adv_tiles
+  AdvCand* adv_tops;              // adv_tiles * 9 * 5
+  // one block of adv_zero counters, cleared at once: adv_acc, the loops' own
+  // samples, then a_loop_active, a_loop_matched, a_line_stall, a_line_lat
+  int64_t adv_zero;
+  unsigned long long* adv_acc;    // nf * kAdvAcc
+  unsigned long long *adv_own_active, *adv_own_matched;
   unsigned long long* a_totals;   // nf * 4
   unsigned long long* a_matched;  // nf * 8
   double* a_speedup;              // nf * 8
@@ -366,7 +382,7 @@ int search_warps_per_sm();  // resident one-warp CTAs of the search kernel per S
 void launch_build_meta(const Prog& P, int4* meta, cudaStream_t st, int sms, int64_t* launches);
 void launch_build_events(const Prog& P, int32_t* ev_off, uint32_t* events, int32_t* tmp, cudaStream_t st, int sms,
                          int64_t* launches);
-void launch_advise(const Prog& P, const Arch& A, cudaStream_t st, int sms, int64_t* launches);
+void launch_advise(const Prog& P, const Arch& A, cudaStream_t st, int64_t* launches);
 // Exclusive scan of n int32 values in place over buf[0..n], buf[n] receives the total.
 void scan_exclusive_inplace(int32_t* buf, int n, int32_t* tmp, cudaStream_t st, int64_t* launches);
 size_t scan_tmp_ints(int n);

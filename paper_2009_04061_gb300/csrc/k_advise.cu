@@ -5,22 +5,26 @@
 // pick each optimizer's top five hotspots (def, use, distance); with launch
 // statistics, the parallel optimizers (Eqs. 6-10).
 //
-// One CTA per function: threads stride over the function's instructions and
-// its merged edges (contiguous, since edges are ordered by use), reduce the
-// sums in shared memory, and thread 0 finishes the per-function results
-// (warp 0 merges the hotspot lists). The
-// CTAs take functions largest first from a counter, so the largest ones start
-// at once and the rest fill in behind them.
+// One CTA per tile of 1,024 instructions of one function, so that a large
+// function is spread over the chip (one CTA a function left a 20,000-instruction
+// function 880 us behind the others and a 120,000-instruction one 4.3 ms). A tile
+// reads its instructions' counters and blame and its edges (contiguous, since
+// edges are ordered by use) once: sums, loop and line roll-ups, and all nine
+// optimizers' top five together, each kept by a warp in its first five lanes
+// (a candidate that beats the fifth is inserted by a ballot and a shift). The
+// function's last tile to finish merges the tiles' lists and writes its results.
+// What bounds it is the counters' and blame's 384 bytes an instruction.
 #include "gpa_internal.cuh"
 
 namespace gpa {
 
 namespace {
 
-constexpr int kThreads = 512;
+constexpr int kThreads = 128;
+constexpr int kWarpsA = kThreads / 32;
 constexpr int kHot = 5;
 enum { O_RR = 0, O_SR, O_FS, O_FM, O_WB, O_MT, O_LU, O_CR, O_FI, N_O = 9 };
-constexpr int kAcc = 13;  // per-function sums, see k_advise
+constexpr int kAcc = kAdvAcc - 1;  // per-function sums, see k_advise; then the tiles that are done
 
 struct Cand { unsigned long long v; int def, use, dist; };
 
@@ -29,12 +33,38 @@ __device__ __forceinline__ bool better(const Cand& a, const Cand& b) {  // a ran
   if (a.def != b.def) return a.def < b.def;
   return a.use < b.use;
 }
-__device__ __forceinline__ void top_insert(Cand* top, int& n, const Cand& c) {
-  if (c.v == 0) return;
-  if (n == kHot && !better(c, top[kHot - 1])) return;
-  int p = n < kHot ? n++ : kHot - 1;
-  while (p > 0 && better(c, top[p - 1])) { top[p] = top[p - 1]; --p; }
-  top[p] = c;
+__device__ __forceinline__ Cand shfl_cand(const Cand& c, int src) {
+  return Cand{__shfl_sync(0xffffffffu, c.v, src), __shfl_sync(0xffffffffu, c.def, src),
+              __shfl_sync(0xffffffffu, c.use, src), __shfl_sync(0xffffffffu, c.dist, src)};
+}
+// A warp's top five, best first, in lanes 0-4 (v == 0: none): takes in every
+// lane's candidate (v == 0: none). Candidates are distinct, so the order is total.
+__device__ __forceinline__ void top_insert(Cand& top, const Cand& c) {
+  const int lane = threadIdx.x & 31;
+  const Cand fifth = shfl_cand(top, kHot - 1);
+  unsigned m = __ballot_sync(0xffffffffu, c.v != 0ull && better(c, fifth));
+  while (m) {
+    const Cand x = shfl_cand(c, __ffs(m) - 1);
+    m &= m - 1;
+    const int rank = __popc(__ballot_sync(0xffffffffu, lane < kHot && better(top, x)));
+    const Cand up{__shfl_up_sync(0xffffffffu, top.v, 1), __shfl_up_sync(0xffffffffu, top.def, 1),
+                  __shfl_up_sync(0xffffffffu, top.use, 1), __shfl_up_sync(0xffffffffu, top.dist, 1)};
+    if (lane > rank) top = up;  // (lanes past the fifth hold what fell out; they never rank)
+    if (lane == rank) top = x;
+  }
+}
+// Adds v to dst[l] for every lane with l >= 0, one atomic per distinct l of the
+// warp (neighbouring instructions mostly share their loop).
+__device__ __forceinline__ void add_by_loop(unsigned long long* dst, int l, unsigned long long v) {
+  unsigned m = __ballot_sync(0xffffffffu, l >= 0 && v != 0ull);
+  while (m) {
+    const int L = __shfl_sync(0xffffffffu, l, __ffs(m) - 1);
+    const bool mine = l == L;
+    unsigned long long s = mine ? v : 0ull;
+    for (int o = 16; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
+    if ((threadIdx.x & 31) == 0) atomicAdd(&dst[L], s);
+    m &= ~__ballot_sync(0xffffffffu, mine);
+  }
 }
 
 __device__ __forceinline__ double est(unsigned long long T, unsigned long long M) {
@@ -56,22 +86,20 @@ __device__ int lca_loop(const Prog& P, int a, int b) {
 
 // Matched samples of an edge per edge-based optimizer. Shares are indexed
 // class slot (exec, memory, sync, constant memory) * 2 + latency flag. The
-// def and use's innermost common loop (a walk up the loop nest) is found
-// only with `loops` (lu is 0 without it); `lca` receives it.
+// def and use's innermost common loop goes to `lca`.
 struct EdgeMatch { unsigned long long rr, sr, lu, cr; };
-__device__ __forceinline__ EdgeMatch edge_match(const Prog& P, const Arch& A, int64_t e, bool loops = true,
-                                                int* lca = nullptr) {
-  const unsigned long long* sh = P.e_share + e * 8;
-  const uint32_t fl = A.flags[P.opclass[P.e_def[e]]];
+__device__ __forceinline__ EdgeMatch edge_match(const Prog& P, const Arch& A, int64_t e, int def, int use, int* lca) {
+  const ulonglong2* sh = reinterpret_cast<const ulonglong2*>(P.e_share + e * 8);
+  const ulonglong2 s0 = sh[0], s1 = sh[1], s3 = sh[3];
+  const uint32_t fl = A.flags[P.opclass[def]];
   const bool local = fl & GPA_F_LOCAL;
   const bool global_mem = !local && !(fl & GPA_F_CONST);  // constant-memory stalls are never global
   EdgeMatch m;
-  m.rr = local ? (sh[2] + sh[3] + sh[6] + sh[7]) : 0ull;                       // Register Reuse
-  m.sr = (fl & GPA_F_LONG_ARITH) ? (sh[0] + sh[1]) : 0ull;                    // Strength Reduction
-  m.cr = sh[1] + (global_mem ? sh[3] : 0ull);                                 // latency samples
-  const int q = loops && m.cr ? lca_loop(P, innermost_loop(P, P.e_def[e]), innermost_loop(P, P.e_use[e])) : -1;
-  m.lu = q >= 0 ? m.cr : 0ull;
-  if (lca) *lca = q;
+  m.rr = local ? (s1.x + s1.y + s3.x + s3.y) : 0ull;           // Register Reuse
+  m.sr = (fl & GPA_F_LONG_ARITH) ? (s0.x + s0.y) : 0ull;      // Strength Reduction
+  m.cr = s0.y + (global_mem ? s1.y : 0ull);                   // latency samples
+  *lca = m.cr ? lca_loop(P, innermost_loop(P, def), innermost_loop(P, use)) : -1;
+  m.lu = *lca >= 0 ? m.cr : 0ull;
   return m;
 }
 
@@ -155,200 +183,212 @@ __device__ void parallel_advice(const Prog& P, int f, unsigned long long T, unsi
 }
 
 __global__ void __launch_bounds__(kThreads) k_advise(Prog P, Arch A) {
-  __shared__ unsigned long long red[kAcc][kThreads / 32];
+  __shared__ unsigned long long red[kAcc][kWarpsA];
   __shared__ unsigned long long tot[kAcc];
-  // each warp's top five (v == 0: none), two sets: warp 0 merges one optimizer's
-  // while the other warps fill the other with the next optimizer's
-  __shared__ Cand wtop[2][kThreads / 32][kHot];
-  __shared__ int s_f;
+  __shared__ Cand wtop[N_O][kWarpsA][kHot];  // each warp's top five (v == 0: none)
+  __shared__ bool s_last;
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-
-  while (true) {
-    __syncthreads();  // every thread has read s_f
-    if (tid == 0) {
-      const unsigned long long q = atomicAdd(&P.stats[SS_ADV_HEAD], 1ull);
-      s_f = q < (unsigned long long)P.nf ? P.reach_order[q] : -1;
-    }
-    __syncthreads();
-    const int f = s_f;
-    if (f < 0) break;
-    const int i0 = P.func_instr_off[f], i1 = P.func_instr_off[f + 1];
-    // Edge ranges are clamped to the edge capacity (overflow is reported in the status word).
-    const int64_t e0 = min((int64_t)P.edge_off[i0], P.edge_cap), e1 = min((int64_t)P.edge_off[i1], P.edge_cap);
-    unsigned long long acc[kAcc];
+  const int f = P.adv_tile_func[blockIdx.x];
+  const int t0 = P.adv_tile_off[f], nt = P.adv_tile_off[f + 1] - t0;
+  const int i0 = P.func_instr_off[f];
+  const int x0 = i0 + ((int)blockIdx.x - t0) * kAdvTile, x1 = min(P.func_instr_off[f + 1], x0 + kAdvTile);
+  // Edge ranges are clamped to the edge capacity (overflow is reported in the status word).
+  const int64_t e0 = min((int64_t)P.edge_off[x0], P.edge_cap), e1 = min((int64_t)P.edge_off[x1], P.edge_cap);
+  unsigned long long acc[kAcc];
 #pragma unroll
-    for (int q = 0; q < kAcc; ++q) acc[q] = 0ull;
-    // acc: 0 T, 1 A, 2 L, 3 issued, 4 FS, 5 FM, 6 WB, 7 MT, 8 RR, 9 SR, 10 LU, 11 CR, 12 FI
-    for (int x = i0 + tid; x < i1; x += kThreads) {
-      const unsigned long long* c = P.cnt + (size_t)x * kCnt;
-      unsigned long long a = 0, l = 0, stall = 0;
+  for (int q = 0; q < kAcc; ++q) acc[q] = 0ull;
+  Cand top[N_O];
 #pragma unroll
-      for (int e = 0; e < kCnt; ++e) {
-        if (e & 1) l += c[e]; else a += c[e];
-        if (e >= 2) stall += c[e];
+  for (int o = 0; o < N_O; ++o) top[o] = Cand{0ull, 0, 0, 0};
+  // acc: 0 T, 1 A, 2 L, 3 issued, 4 FS, 5 FM, 6 WB, 7 MT, 8 RR, 9 SR, 10 LU, 11 CR, 12 FI
+  for (int xb = x0 + warp * 32; xb < x1; xb += kThreads) {
+    const int x = xb + lane;
+    const bool in = x < x1;
+    unsigned long long a = 0, l = 0, stall = 0, fs = 0, wb = 0, mt = 0, bs = 0, bl = 0, c0 = 0, c1 = 0;
+    int loop = -1;
+    uint32_t ifl = 0, fl = 0;
+    if (in) {
+      const ulonglong2* c = reinterpret_cast<const ulonglong2*>(P.cnt + (size_t)x * kCnt);
+      const ulonglong2* b = reinterpret_cast<const ulonglong2*>(P.blame + (size_t)x * kCnt);
+      ifl = P.iflags[x];
+      fl = A.flags[P.opclass[x]];
+      loop = innermost_loop(P, x);
+#pragma unroll
+      for (int k = 0; k < kCnt / 2; ++k) {
+        const ulonglong2 v = c[k];
+        a += v.x;
+        l += v.y;
+        if (k == 0) c0 = v.x, c1 = v.y;
+        else stall += v.x + v.y;
+        if (k == 1) fs = v.x + v.y;
+        if (k == 5) wb = v.x + v.y;
+        if (k == 8) mt = v.x + v.y;
       }
-      acc[0] += a + l; acc[1] += a; acc[2] += l; acc[3] += c[0];
-      acc[4] += c[2] + c[3];
-      if (P.iflags[x] & 1) acc[5] += stall;
-      acc[6] += c[10] + c[11];
-      if (A.flags[P.opclass[x]] & GPA_F_GLOBAL) acc[7] += c[16] + c[17];
-      if (P.iflags[x] & 6) acc[12] += l;  // latency stalls in a device function or at a call site
-      for (int lp = innermost_loop(P, x); lp >= 0; lp = P.loop_parent[lp])
-        if (a) atomicAdd(&P.a_loop_active[lp], a);
-      const unsigned long long* b = P.blame + (size_t)x * kCnt;
-      unsigned long long bs = 0, bl = 0;
 #pragma unroll
-      for (int e = 2; e < kCnt; ++e) { bs += b[e]; if (e & 1) bl += b[e]; }
+      for (int k = 1; k < kCnt / 2; ++k) {
+        const ulonglong2 v = b[k];
+        bs += v.x + v.y;
+        bl += v.y;
+      }
+      acc[0] += a + l; acc[1] += a; acc[2] += l; acc[3] += c0;
       if (bs) atomicAdd(&P.a_line_stall[P.line[x]], bs);
       if (bl) atomicAdd(&P.a_line_lat[P.line[x]], bl);
     }
-    for (int64_t e = e0 + tid; e < e1; e += kThreads) {
-      int q;
-      const EdgeMatch m = edge_match(P, A, e, true, &q);
-      acc[8] += m.rr; acc[9] += m.sr; acc[10] += m.lu; acc[11] += m.cr;
-      if (m.lu)
-        for (int lp = q; lp >= 0; lp = P.loop_parent[lp]) atomicAdd(&P.a_loop_matched[lp], m.lu);
+    const unsigned long long fm = (ifl & 1) ? stall : 0ull;
+    const unsigned long long fi = (ifl & 6) ? l : 0ull;  // latency stalls in a device function or at a call site
+    if (!(fl & GPA_F_GLOBAL)) mt = 0ull;
+    acc[4] += fs; acc[5] += fm; acc[6] += wb; acc[7] += mt; acc[12] += fi;
+    add_by_loop(P.adv_own_active, loop, a);
+    const int pc = x - i0;
+    top_insert(top[O_FS], Cand{fs, pc, pc, 0});
+    top_insert(top[O_FM], Cand{fm, pc, pc, 0});
+    top_insert(top[O_WB], Cand{wb, pc, pc, 0});
+    top_insert(top[O_MT], Cand{mt, pc, pc, 0});
+    top_insert(top[O_FI], Cand{fi ? fi - c1 : 0ull, pc, pc, 0});  // a hotspot counts no SELECTED samples
+  }
+  for (int64_t eb = e0 + warp * 32; eb < e1; eb += kThreads) {
+    const int64_t e = eb + lane;
+    EdgeMatch m{0ull, 0ull, 0ull, 0ull};
+    int q = -1, def = 0, use = 0, dist = 0;
+    if (e < e1) {
+      def = P.e_def[e];
+      use = P.e_use[e];
+      dist = P.e_dmin[e];
+      m = edge_match(P, A, e, def, use, &q);
     }
+    acc[8] += m.rr; acc[9] += m.sr; acc[10] += m.lu; acc[11] += m.cr;
+    add_by_loop(P.adv_own_matched, q, m.lu);
+    def -= i0;
+    use -= i0;
+    top_insert(top[O_RR], Cand{m.rr, def, use, dist});
+    top_insert(top[O_SR], Cand{m.sr, def, use, dist});
+    top_insert(top[O_LU], Cand{m.lu, def, use, dist});
+    top_insert(top[O_CR], Cand{m.cr, def, use, dist});
+  }
 #pragma unroll
-    for (int q = 0; q < kAcc; ++q) {
-      unsigned long long v = acc[q];
-      for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
-      if (lane == 0) red[q][warp] = v;
+  for (int q = 0; q < kAcc; ++q) {
+    unsigned long long v = acc[q];
+    for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
+    if (lane == 0) red[q][warp] = v;
+  }
+#pragma unroll
+  for (int o = 0; o < N_O; ++o)
+    if (lane < kHot) wtop[o][warp][lane] = top[o];
+  __syncthreads();
+  if (tid < kAcc) {
+    unsigned long long v = 0;
+    for (int w = 0; w < kWarpsA; ++w) v += red[tid][w];
+    tot[tid] = v;
+  }
+  // The tile's top five, a warp per optimizer in turn.
+  for (int o = warp; o < N_O; o += kWarpsA) {
+    static_assert(kWarpsA * kHot <= 32, "one lane per entry of the warps' lists");
+    Cand best{0ull, 0, 0, 0};
+    top_insert(best, lane < kWarpsA * kHot ? wtop[o][lane / kHot][lane % kHot] : Cand{0ull, 0, 0, 0});
+    if (nt == 1) {
+      __syncwarp();  // (read before it is overwritten)
+      if (lane < kHot) wtop[o][0][lane] = best;
+    } else if (lane < kHot) {
+      AdvCand* out = P.adv_tops + ((size_t)blockIdx.x * N_O + o) * kHot + lane;
+      *out = AdvCand{best.v, best.def, best.use, best.dist, 0};
     }
+  }
+  __syncthreads();
+  if (nt > 1) {
+    // The last of the function's tiles finishes it.
+    unsigned long long* fa = P.adv_acc + (size_t)f * kAdvAcc;
+    if (tid < kAcc && tot[tid]) atomicAdd(&fa[tid], tot[tid]);
+    __threadfence();
     __syncthreads();
-    if (tid < kAcc) {
-      unsigned long long v = 0;
-      for (int w = 0; w < kThreads / 32; ++w) v += red[tid][w];
-      tot[tid] = v;
-    }
+    if (tid == 0) s_last = atomicAdd(&fa[kAcc], 1ull) == (unsigned long long)(nt - 1);
     __syncthreads();
-    const unsigned long long T = tot[0], Aact = tot[1];
-    if (tid == 0) {
-      unsigned long long M[N_O];
-      M[O_RR] = tot[8]; M[O_SR] = tot[9]; M[O_FS] = tot[4]; M[O_FM] = tot[5];
-      M[O_WB] = tot[6]; M[O_MT] = tot[7]; M[O_LU] = tot[10]; M[O_CR] = tot[11]; M[O_FI] = tot[12];
-      double sp[N_O];
-      for (int o = 0; o < N_O; ++o) {
-        const bool hide = (o == O_LU || o == O_CR || o == O_FI);
-        sp[o] = est(T, hide ? min(Aact, M[o]) : M[o]);
-        P.a_matched[(size_t)f * N_O + o] = M[o];
-        P.a_speedup[(size_t)f * N_O + o] = sp[o];
-      }
-      int ord[N_O];
-      for (int o = 0; o < N_O; ++o) ord[o] = o;
-      for (int a = 1; a < N_O; ++a) {  // stable: ties keep the lower id first
-        int v = ord[a], b = a - 1;
-        while (b >= 0 && sp[ord[b]] < sp[v]) { ord[b + 1] = ord[b]; --b; }
-        ord[b + 1] = v;
-      }
-      for (int o = 0; o < N_O; ++o) P.a_rank[(size_t)f * N_O + o] = ord[o];
-      for (int q = 0; q < 4; ++q) P.a_totals[(size_t)f * 4 + q] = tot[q];
-      parallel_advice(P, f, T, tot[3]);
-    }
-    // Hotspots, one optimizer at a time: thread-local top five, a warp-level
-    // merge, then thread 0 merges the warps' lists.
-    for (int o = 0; o < N_O; ++o) {
-      Cand top[kHot];
-      int nt = 0;
-      const bool edge_based = (o == O_RR || o == O_SR || o == O_LU || o == O_CR);
-      if (edge_based) {
-        for (int64_t e = e0 + tid; e < e1; e += kThreads) {
-          const EdgeMatch m = edge_match(P, A, e, o == O_LU);
-          const unsigned long long v = o == O_RR ? m.rr : o == O_SR ? m.sr : o == O_LU ? m.lu : m.cr;
-          top_insert(top, nt, Cand{v, P.e_def[e] - i0, P.e_use[e] - i0, P.e_dmin[e]});
+    if (!s_last) return;
+    __threadfence();
+    if (tid < kAcc) tot[tid] = __ldcg(&fa[tid]);
+    for (int o = warp; o < N_O; o += kWarpsA) {
+      Cand best{0ull, 0, 0, 0};
+      for (int k = 0; k < nt * kHot; k += 32) {
+        Cand c{0ull, 0, 0, 0};
+        const int q = k + lane;
+        if (q < nt * kHot) {
+          const int4* in = reinterpret_cast<const int4*>(P.adv_tops + ((size_t)(t0 + q / kHot) * N_O + o) * kHot + q % kHot);
+          const int2 v = __ldcg(reinterpret_cast<const int2*>(in));
+          const int2 du = __ldcg(reinterpret_cast<const int2*>(in) + 1);
+          c.v = (unsigned long long)(uint32_t)v.x | ((unsigned long long)(uint32_t)v.y << 32);
+          c.def = du.x;
+          c.use = du.y;
+          c.dist = __ldcg(reinterpret_cast<const int*>(in) + 4);
         }
-      } else {
-        for (int x = i0 + tid; x < i1; x += kThreads) {
-          const unsigned long long* c = P.cnt + (size_t)x * kCnt;
-          unsigned long long v = 0;
-          if (o == O_FS) v = c[2] + c[3];
-          else if (o == O_FM) { if (P.iflags[x] & 1) for (int e = 2; e < kCnt; ++e) v += c[e]; }
-          else if (o == O_WB) v = c[10] + c[11];
-          else if (o == O_FI) { if (P.iflags[x] & 6) for (int e = 3; e < kCnt; e += 2) v += c[e]; }
-          else if (A.flags[P.opclass[x]] & GPA_F_GLOBAL) v = c[16] + c[17];
-          top_insert(top, nt, Cand{v, x - i0, x - i0, 0});
-        }
+        top_insert(best, c);
       }
-      // The warp's top five: five rounds of a butterfly maximum over the lanes'
-      // next candidates (candidates are distinct, so the order is total; lanes
-      // out of candidates offer v = 0, ties between those go to the lower lane).
-      int ptr = 0;
-      for (int h = 0; h < kHot; ++h) {
-        Cand b = ptr < nt ? top[ptr] : Cand{0ull, 0, 0, 0};
-        int owner = lane;
-        for (int sh = 16; sh > 0; sh >>= 1) {
-          Cand y;
-          y.v = __shfl_xor_sync(0xffffffffu, b.v, sh);
-          y.def = __shfl_xor_sync(0xffffffffu, b.def, sh);
-          y.use = __shfl_xor_sync(0xffffffffu, b.use, sh);
-          y.dist = __shfl_xor_sync(0xffffffffu, b.dist, sh);
-          const int yo = __shfl_xor_sync(0xffffffffu, owner, sh);
-          if (better(y, b) || (!better(b, y) && yo < owner)) { b = y; owner = yo; }
-        }
-        if (lane == owner && b.v != 0ull) ++ptr;
-        if (lane == 0) wtop[o & 1][warp][h] = b;
-      }
-      __syncthreads();
-      // The CTA's top five: warp 0 merges the warps' sorted lists the same way
-      // (lane w offers the next entry of warp w's list).
-      if (warp == 0) {
-        static_assert(kThreads / 32 <= 32, "one lane per warp's list");
-        long long* out = P.a_hot + ((size_t)f * N_O + o) * kHot * 6;
-        int wp = 0, nb = 0;
-        for (int h = 0; h < kHot; ++h) {
-          Cand b = lane < kThreads / 32 && wp < kHot ? wtop[o & 1][lane][wp] : Cand{0ull, 0, 0, 0};
-          int owner = lane;
-          for (int sh = 16; sh > 0; sh >>= 1) {
-            Cand y;
-            y.v = __shfl_xor_sync(0xffffffffu, b.v, sh);
-            y.def = __shfl_xor_sync(0xffffffffu, b.def, sh);
-            y.use = __shfl_xor_sync(0xffffffffu, b.use, sh);
-            y.dist = __shfl_xor_sync(0xffffffffu, b.dist, sh);
-            const int yo = __shfl_xor_sync(0xffffffffu, owner, sh);
-            if (better(y, b) || (!better(b, y) && yo < owner)) { b = y; owner = yo; }
-          }
-          if (lane == owner && b.v != 0ull) ++wp;
-          if (lane == 0) {
-            if (b.v != 0ull) {
-              out[h * 6 + 0] = b.def; out[h * 6 + 1] = b.use;
-              out[h * 6 + 2] = P.line[i0 + b.def]; out[h * 6 + 3] = P.line[i0 + b.use];
-              out[h * 6 + 4] = b.dist; out[h * 6 + 5] = (long long)b.v;
-              ++nb;
-            } else {
-              for (int q = 0; q < 6; ++q) out[h * 6 + q] = -1;
-            }
-          }
-        }
-        if (lane == 0) P.a_nhot[(size_t)f * N_O + o] = nb;
-      }
-      // No barrier here: the next pass fills the other set, and warp 0 reaches
-      // the barrier after that pass only once this merge is done, before the
-      // pass after next fills this set again.
-    }
-    // Eq. 5 per loop scope of this function (its loop counters were only touched by this CTA).
-    __threadfence_block();
-    __syncthreads();
-    for (int lp = P.func_loop_off[f] + tid; lp < P.func_loop_off[f + 1]; lp += kThreads) {
-      const unsigned long long al = __ldcg(&P.a_loop_active[lp]);
-      const unsigned long long ml = __ldcg(&P.a_loop_matched[lp]);
-      P.a_loop_speedup[lp] = est(T, min(al, ml));
+      if (lane < kHot) wtop[o][0][lane] = best;
     }
     __syncthreads();
   }
+  const unsigned long long T = tot[0], Aact = tot[1];
+  // Results: the hotspots, a thread per entry; the estimates and the ranking, one
+  // thread; the parallel optimizers, another.
+  if (tid < N_O * kHot) {
+    const int o = tid / kHot, h = tid % kHot;
+    const Cand b = wtop[o][0][h];
+    long long* out = P.a_hot + ((size_t)f * N_O + o) * kHot * 6 + h * 6;
+    if (b.v != 0ull) {
+      out[0] = b.def; out[1] = b.use;
+      out[2] = P.line[i0 + b.def]; out[3] = P.line[i0 + b.use];
+      out[4] = b.dist; out[5] = (long long)b.v;
+    } else {
+      for (int q = 0; q < 6; ++q) out[q] = -1;
+    }
+    if (h == 0) {
+      int nb = 0;
+      while (nb < kHot && wtop[o][0][nb].v != 0ull) ++nb;
+      P.a_nhot[(size_t)f * N_O + o] = nb;
+    }
+  }
+  if (tid == 64) {
+    unsigned long long M[N_O];
+    M[O_RR] = tot[8]; M[O_SR] = tot[9]; M[O_FS] = tot[4]; M[O_FM] = tot[5];
+    M[O_WB] = tot[6]; M[O_MT] = tot[7]; M[O_LU] = tot[10]; M[O_CR] = tot[11]; M[O_FI] = tot[12];
+    double sp[N_O];
+    for (int o = 0; o < N_O; ++o) {
+      const bool hide = (o == O_LU || o == O_CR || o == O_FI);
+      sp[o] = est(T, hide ? min(Aact, M[o]) : M[o]);
+      P.a_matched[(size_t)f * N_O + o] = M[o];
+      P.a_speedup[(size_t)f * N_O + o] = sp[o];
+    }
+    int ord[N_O];
+    for (int o = 0; o < N_O; ++o) ord[o] = o;
+    for (int a = 1; a < N_O; ++a) {  // stable: ties keep the lower id first
+      int v = ord[a], b = a - 1;
+      while (b >= 0 && sp[ord[b]] < sp[v]) { ord[b + 1] = ord[b]; --b; }
+      ord[b + 1] = v;
+    }
+    for (int o = 0; o < N_O; ++o) P.a_rank[(size_t)f * N_O + o] = ord[o];
+    for (int q = 0; q < 4; ++q) P.a_totals[(size_t)f * 4 + q] = tot[q];
+  }
+  if (tid == 96) parallel_advice(P, f, T, tot[3]);
+  // Eq. 5 per loop scope: each loop's own samples go to it and to the loops
+  // around it (this CTA alone reads and writes the function's loop counters now).
+  const int l0 = P.func_loop_off[f], l1 = P.func_loop_off[f + 1];
+  for (int lp = l0 + tid; lp < l1; lp += kThreads) {
+    const unsigned long long al = __ldcg(&P.adv_own_active[lp]), ml = __ldcg(&P.adv_own_matched[lp]);
+    for (int q = lp; q >= 0; q = P.loop_parent[q]) {
+      if (al) atomicAdd(&P.a_loop_active[q], al);
+      if (ml) atomicAdd(&P.a_loop_matched[q], ml);
+    }
+  }
+  __threadfence_block();
+  __syncthreads();
+  for (int lp = l0 + tid; lp < l1; lp += kThreads)
+    P.a_loop_speedup[lp] = est(T, min(__ldcg(&P.a_loop_active[lp]), __ldcg(&P.a_loop_matched[lp])));
 }
 
 }  // namespace
 
-void launch_advise(const Prog& P, const Arch& A, cudaStream_t st, int sms, int64_t* launches) {
-  if (P.nl > 0) {
-    cudaMemsetAsync(P.a_loop_active, 0, sizeof(unsigned long long) * P.nl, st);
-    cudaMemsetAsync(P.a_loop_matched, 0, sizeof(unsigned long long) * P.nl, st);
-  }
-  cudaMemsetAsync(P.a_line_stall, 0, sizeof(unsigned long long) * P.n_lines, st);
-  cudaMemsetAsync(P.a_line_lat, 0, sizeof(unsigned long long) * P.n_lines, st);
-  cudaMemsetAsync(&P.stats[SS_ADV_HEAD], 0, sizeof(unsigned long long), st);
-  int blocks = P.nf < sms * 2 ? P.nf : sms * 2;
-  k_advise<<<blocks > 0 ? blocks : 1, kThreads, 0, st>>>(P, A);
+void launch_advise(const Prog& P, const Arch& A, cudaStream_t st, int64_t* launches) {
+  // every counter that is added to, in one block
+  cudaMemsetAsync(P.adv_acc, 0, sizeof(unsigned long long) * (size_t)P.adv_zero, st);
+  k_advise<<<P.adv_tiles, kThreads, 0, st>>>(P, A);
   ++*launches;
 }
 

@@ -569,11 +569,27 @@ static gpa_status alloc_program(const gpa_program_desc* d, ProgramRec* R, int ti
   TRY(dev_alloc(R, &P.a_rank, nf * GPA_NUM_OPT));
   TRY(dev_alloc(R, &P.a_nhot, nf * GPA_NUM_OPT));
   TRY(dev_alloc(R, &P.a_hot, nf * GPA_NUM_OPT * 5 * 6));
-  TRY(dev_alloc(R, &P.a_loop_active, nl));
-  TRY(dev_alloc(R, &P.a_loop_matched, nl));
   TRY(dev_alloc(R, &P.a_loop_speedup, nl));
-  TRY(dev_alloc(R, &P.a_line_stall, (size_t)P.n_lines));
-  TRY(dev_alloc(R, &P.a_line_lat, (size_t)P.n_lines));
+  {
+    std::vector<int32_t> off(nf + 1, 0), func;
+    for (size_t f = 0; f < nf; ++f) {
+      const int n = (d->func_instr_off[f + 1] - d->func_instr_off[f] + kAdvTile - 1) / kAdvTile;
+      off[f + 1] = off[f] + n;
+      func.insert(func.end(), (size_t)n, (int32_t)f);
+    }
+    P.adv_tiles = off[nf];
+    TRY(dev_copy(R, &P.adv_tile_off, off.data(), nf + 1));
+    TRY(dev_copy(R, &P.adv_tile_func, func.data(), func.size()));
+    TRY(dev_alloc(R, &P.adv_tops, (size_t)P.adv_tiles * GPA_NUM_OPT * 5));
+    P.adv_zero = (int64_t)(nf * kAdvAcc + 4 * nl + 2 * (size_t)P.n_lines);
+    TRY(dev_alloc(R, &P.adv_acc, (size_t)P.adv_zero));
+    P.adv_own_active = P.adv_acc + nf * kAdvAcc;
+    P.adv_own_matched = P.adv_own_active + nl;
+    P.a_loop_active = P.adv_own_matched + nl;
+    P.a_loop_matched = P.a_loop_active + nl;
+    P.a_line_stall = P.a_loop_matched + nl;
+    P.a_line_lat = P.a_line_stall + P.n_lines;
+  }
   TRY(dev_alloc(R, &P.a_par_match, nf * 2));
   TRY(dev_alloc(R, &P.a_par_speedup, nf * 2));
   TRY(dev_alloc(R, &P.a_par_warps, nf * 4));
@@ -914,7 +930,7 @@ gpa_status gpa_step_capture(gpa_ctx* ctx, gpa_pid pid, const uint64_t* dev_sampl
     launch_histogram(R->P, dev_samples, n, cs, ctx->sms, &ctx->launches, ctx->opts.hist_variant,
                      ctx->opts.hist_chunk);
   if (!s) s = blame_body(ctx, R, cs, false);
-  if (!s) launch_advise(R->P, ctx->arch, cs, ctx->sms, &ctx->launches);
+  if (!s) launch_advise(R->P, ctx->arch, cs, &ctx->launches);
   cudaGraph_t g = nullptr;
   const cudaError_t e = cudaStreamEndCapture(cs, &g);
   const int64_t kernels = ctx->launches - l0;
@@ -1034,7 +1050,7 @@ gpa_status gpa_advise(gpa_ctx* ctx, gpa_pid pid, const gpa_advice* out, gpa_stre
   ProgramRec* R = find(ctx, pid);
   if (!R) return GPA_ERR_NO_PROGRAM;
   cudaStream_t st = (cudaStream_t)stream;
-  launch_advise(R->P, ctx->arch, st, ctx->sms, &ctx->launches);
+  launch_advise(R->P, ctx->arch, st, &ctx->launches);
   CK(cudaGetLastError());
   if (out) return copy_advice(R, out, st);
   return GPA_OK;
