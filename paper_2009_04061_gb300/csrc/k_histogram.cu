@@ -11,6 +11,7 @@
 // that finds no slot within a few probes goes straight to its 64-bit global
 // counter. The hash is flushed to the global counters when three quarters
 // full and at the end. With Zipf-skewed hotness most samples stay on chip.
+#include <algorithm>
 #include <type_traits>
 
 #include "gpa_internal.cuh"
@@ -356,7 +357,12 @@ __global__ void __launch_bounds__(kRunThreads, 1) k_histogram_runs(Prog P, const
   };
   // Flush the window and place it for kernel id `want` (>= nf: none), from the
   // 32 samples starting at stream index m. CTA-uniform: every thread takes part.
+  // A kernel that holds fewer than 8 of them (kernels interleaved sample by
+  // sample: no run to count) is not worth a flush of the window: its samples are
+  // missed ones (5e6 interleaved samples of 100 kernels: see launch_histogram).
   auto place = [&](uint32_t want, int64_t m) {
+    const uint64_t x = __ldg(reinterpret_cast<const unsigned long long*>(s2 + m + lane));
+    if (want < (uint32_t)P.nf && __popc(__ballot_sync(0xffffffffu, (uint32_t)(x >> 48) == want)) < 8) return;
     __syncthreads();
     flush_win();
     __syncthreads();
@@ -366,7 +372,7 @@ __global__ void __launch_bounds__(kRunThreads, 1) k_histogram_runs(Prog P, const
       const uint32_t n_instr = (uint32_t)(foff[want + 1] - foff[want]);
       mode_first = (uint32_t)foff[want];
       mode_n = n_instr;
-      const uint32_t lo = window_start(__ldg(reinterpret_cast<const unsigned long long*>(s2 + m + lane)), want, n_instr);
+      const uint32_t lo = window_start(x, want, n_instr);
       mode_hi = want << 16;
       first5 = (want << 29) | (lo << 5);
       span5 = min(n_instr, kWinInstr) << 5;
@@ -537,8 +543,13 @@ void launch_histogram(const Prog& P, const uint64_t* samples, size_t n, cudaStre
   if (variant == 0) {
     const int head = (reinterpret_cast<uintptr_t>(samples) & 15u) ? 1 : 0;
     const int64_t vecs = ((int64_t)n - head) / 2;
-    const int chunk_tiles = hist_chunk > 0 ? hist_chunk : 24;
-    int64_t grid = (vecs + (int64_t)kRunTile * chunk_tiles - 1) / ((int64_t)kRunTile * chunk_tiles);
+    // Tiles per chunk: 24 for long streams (fewer claims and more tiles with a
+    // prefetch), down to one so that a short stream still gives every SM about
+    // four chunks to take.
+    const int64_t n_tiles = vecs / kRunTile;
+    const int chunk_tiles = hist_chunk > 0 ? hist_chunk
+                                           : (int)std::max<int64_t>(1, std::min<int64_t>(24, n_tiles / (4 * (int64_t)sms)));
+    int64_t grid = (n_tiles + chunk_tiles - 1) / chunk_tiles;
     if (grid > sms) grid = sms;
     if (grid < 1) grid = 1;
     cudaMemsetAsync(&P.stats[SS_HIST_HEAD], 0, sizeof(unsigned long long), st);
