@@ -59,11 +59,16 @@ enum {
   SS_SUSE_N = 90,      // entries of suse (the stalled uses of this step)
   // 91: unused
   // searches queued straight for a size class of the shared-memory warps
-  SS_A1_N = 92, SS_A2_N = 93, SS_A3_N = 94, SS_A1_HEAD = 95,  // (heads 95-97)
-  SS_N = 98
+  SS_A1_N = 92, SS_A1_HEAD = 97,  // kClasses of each
+  SS_N = 102
 };
+// Size classes of the shared-memory search warps (k_search_smem.cu), and the
+// queue and region of each class's searches known from an earlier step.
+constexpr int kClasses = 5;
+__host__ __device__ constexpr int class_queue(int c) { return c < 3 ? c : c == 3 ? 2 : 5; }
+__host__ __device__ constexpr bool class_top(int c) { return c != 2 && c != 4; }
 // Values of tier_hint: the queue that a use entry's search belongs to.
-enum { kHintLane2 = 2, kHintA1 = 3, kHintA3 = 5, kHintWarp = 6, kHintCta = 7 };
+enum { kHintLane2 = 2, kHintA1 = 3, kHintWarp = kHintA1 + kClasses, kHintCta };
 
 struct Arch {
   int32_t n_op;
@@ -155,11 +160,12 @@ struct Prog {
   // resource | start literal set << 9 | blocked << 25}. Each queue has queue_cap
   // entries: 0 first tier from the bottom (after it the second tier's overflow),
   // first size class of the shared-memory warps from the top; 1 second tier,
-  // second class; 2 third class; 3 overflow to the global-memory warps, searches
-  // queued straight for them; 4 fourth tier. An entry is in one region of a
+  // second class; 2 third class, fourth class; 3 overflow to the global-memory
+  // warps, searches queued straight for them; 4 fourth tier; 5 fifth class. An entry is in one region of a
   // queue at a time, so the two regions never meet.
   int2* tasks;                    // n_use
-  int32_t* queue[5];
+  int32_t* queue[6];
+  int32_t class_limit[kClasses];  // searches a class takes in a step; the rest go to the global-memory warps
   uint32_t* tier_hint;            // n_use: the queue known to hold the entry's search (0: none);
                                   // kept across steps (a search's size depends only on the program)
   int64_t queue_cap;
@@ -376,6 +382,7 @@ int search_lane_width(int nodes);      // lanes of a warp that search, for arena
 int64_t search_lane_bytes(int nodes);  // their arenas, in bytes a warp
 void launch_search_lanes(const Prog& P, const Arch& A, const SearchArena& T, int tier, cudaStream_t st,
                          int64_t* launches);
+int smem_class_limit(int c, int sms);
 void launch_search_smem(const Prog& P, const Arch& A, int most_nodes, int part, cudaStream_t st, int sms,
                         int64_t* launches);
 int search_warps_per_sm();  // resident one-warp CTAs of the search kernel per SM (global-memory tiers)

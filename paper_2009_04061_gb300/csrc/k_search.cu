@@ -1024,8 +1024,8 @@ void launch_search(const Prog& P, const Arch& A, const SearchArena* tiers, const
   }
   // No launch takes more groups than there can be tasks (one per use entry).
   const int g3 = (int)std::min<int64_t>(tiers[2].warps, P.queue_cap);
-  k_search_warp<<<g3, 32, 0, s3>>>(P, A, tiers[2], 1);
   launch_search_smem(P, A, tiers[2].nodes, 1, s1, sms, launches);
+  k_search_warp<<<g3, 32, 0, s3>>>(P, A, tiers[2], 1);
   launch_search_lanes(P, A, tiers[0], 1, st, launches);
   launch_search_lanes(P, A, tiers[1], 2, st, launches);
   if (fork) {

@@ -15,16 +15,21 @@
 // again.
 //
 // One CTA of 16 warps per SM gives its 227 KB to one size class after another:
-// 1 search of 5,632 nodes, 4 of 1,280, 16 of 320. Searches that an earlier step
-// of the program found to be of a class are queued for it and run largest class
-// first; a search that outgrows its class goes on a list of its CTA, which works
-// off its lists in ascending order at the end. Beyond the last class (or a full
-// list) the global-memory tier takes over.
+// 1 search of 5,632 nodes, 2 of 2,560, 4 of 1,280, 8 of 640, 16 of 320. Searches
+// that an earlier step of the program found to be of a class are queued for it
+// and run largest class first; a search that outgrows its class goes on a list of
+// its CTA, which works off its lists in ascending order at the end. Beyond the
+// last class the global-memory tier takes over. It also takes what the three
+// largest classes have beyond three rounds of the chip: there a search takes three
+// times as long, but 3,648 run at once (see smem_class_limit).
+// Registers: 80 a thread, so that global-memory searches (which use no shared
+// memory) find room beside this CTA.
 //
 // The graph, the passes and the rules are those of k_search.cu's group search;
 // like the one-lane search (k_search_lanes.cu) it ends early when its only
 // unexpanded node meets an unguarded reader of r before any def was met.
 #include <algorithm>
+#include <climits>
 
 #include "gpa_internal.cuh"
 
@@ -33,7 +38,6 @@ namespace gpa {
 namespace {
 
 constexpr int kWarps = 16;
-constexpr int kClasses = 3;
 constexpr int kLocalList = 256;      // searches a CTA keeps for its own next class
 constexpr int kDistBits = 19, kIdxBits = 13;
 constexpr uint32_t kFar = (1u << kDistBits) - 1u;  // no distance yet
@@ -43,10 +47,10 @@ constexpr uint32_t F_EXP = 1u << 24, F_QUE = 1u << 25, F_NEED = 1u << 26, F_BACK
 constexpr int kSearchInf = 0x7FFFFFFF;
 
 __host__ __device__ inline int class_nodes(int c, int most) {
-  const int n = c == 0 ? 320 : c == 1 ? 1280 : 5632;
+  const int n = c < 4 ? 320 << c : 5632;
   return n < most ? n : most;
 }
-__host__ __device__ inline int class_warps(int c) { return c == 0 ? 16 : c == 1 ? 4 : 1; }
+__host__ __device__ inline int class_warps(int c) { return 16 >> c; }
 __host__ __device__ inline int hash_slots(int n) {  // a power of two, at least 1.4 n
   int h = 16;
   while (5 * h < 7 * n) h <<= 1;
@@ -706,7 +710,7 @@ __device__ int warp_search(const Prog& P, const Arch& A, const WArena& a, int j,
 
 // part 1: the searches queued for a class, largest class first (beside tiers 1
 // and 2); part 2: the second tier's overflow, from the first class up.
-__global__ void __launch_bounds__(kWarps * 32, 1) k_search_smem(Prog P, Arch A, int most_nodes, int part) {
+__global__ void __launch_bounds__(768, 1) k_search_smem(Prog P, Arch A, int most_nodes, int part) {
   extern __shared__ __align__(16) char smem[];
   __shared__ int s_ctr[kWarps][8];
   __shared__ uint16_t s_wpos[kWarps][32];
@@ -714,15 +718,15 @@ __global__ void __launch_bounds__(kWarps * 32, 1) k_search_smem(Prog P, Arch A, 
   __shared__ int s_nlocal[kClasses], s_hlocal[kClasses];
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   const unsigned long long cap = (unsigned long long)P.queue_cap;
-  unsigned long long n_tasks[kClasses] = {0, 0, 0};
-  if (part == 1) {
-    n_tasks[0] = min(P.stats[SS_A1_N], cap);
-    n_tasks[1] = min(P.stats[SS_A2_N], cap);
-    n_tasks[2] = min(P.stats[SS_A3_N], cap);
-  } else {
-    n_tasks[0] = min(P.stats[SS_OVF2_N], cap);
-  }
-  if (n_tasks[0] + n_tasks[1] + n_tasks[2] == 0) return;
+  // tasks of class c: queued by the local pass (at most its limit, the rest went
+  // to the global-memory warps), or the second tier's overflow for the first class
+  auto n_tasks = [&](int c) -> unsigned long long {
+    if (part == 1) return min(P.stats[SS_A1_N + c], min(cap, (unsigned long long)P.class_limit[c]));
+    return c == 0 ? min(P.stats[SS_OVF2_N], cap) : 0ull;
+  };
+  unsigned long long any = 0;
+  for (int c = 0; c < kClasses; ++c) any |= n_tasks(c);
+  if (!any) return;
   if (threadIdx.x < kClasses) { s_nlocal[threadIdx.x] = 0; s_hlocal[threadIdx.x] = 0; }
   __syncthreads();
   unsigned long long runs = 0, most = 0, most_task = 0;
@@ -731,19 +735,21 @@ __global__ void __launch_bounds__(kWarps * 32, 1) k_search_smem(Prog P, Arch A, 
     const int n = class_nodes(c, most_nodes);
     if (warp < class_warps(c)) {
       const WArena a = carve(smem + warp * warp_arena_bytes(n), n, s_ctr[warp], s_wpos[warp]);
-      // queue 0 top, queue 1 top, queue 2; the second tier's overflow: queue 0
-      const int32_t* q = c == 0 ? P.queue[0] : c == 1 ? P.queue[1] : P.queue[2];
-      const bool top = part == 1 && c < 2;
+      const int32_t* q = P.queue[part == 1 ? class_queue(c) : 0];  // (queue 0: the second tier's overflow)
+      const bool top = part == 1 && class_top(c);
       const int head = part == 1 ? SS_A1_HEAD + c : SS_OVF2_HEAD;
+      const unsigned long long nt = n_tasks(c);
+      // what a list holds: the largest classes at most three rounds
+      const int list = c < 2 ? kLocalList : 3 * class_warps(c);
       while (true) {
         int e = -1;
         if (lane == 0) {
           if (local) {
             const int t = atomicAdd(&s_hlocal[c], 1);
-            if (t < min(s_nlocal[c], kLocalList)) e = s_local[c][t];
+            if (t < min(s_nlocal[c], list)) e = s_local[c][t];
           } else {
             const unsigned long long t = atomicAdd(&P.stats[head], 1ull);
-            if (t < n_tasks[c]) e = q[top ? cap - 1 - t : t];
+            if (t < nt) e = q[top ? cap - 1 - t : t];
           }
         }
         e = __shfl_sync(0xffffffffu, e, 0);
@@ -762,11 +768,11 @@ __global__ void __launch_bounds__(kWarps * 32, 1) k_search_smem(Prog P, Arch A, 
 #endif
         if (!over) continue;
         int next = c + 1;  // the next class that is larger than this one
-        if (next < kClasses && class_nodes(next, most_nodes) == n) next = kClasses;
+        while (next < kClasses && class_nodes(next, most_nodes) == n) ++next;
         if (!P.diag) atomicMax(&P.tier_hint[e], (unsigned)(kHintA1 + next));
         if (next < kClasses) {
           const int t = atomicAdd(&s_nlocal[next], 1);
-          if (t < kLocalList) { s_local[next][t] = e; continue; }
+          if (t < (next < 2 ? kLocalList : 3 * class_warps(next))) { s_local[next][t] = e; continue; }
         }
         const unsigned long long o = atomicAdd(&P.stats[SS_OVF3_N], 1ull);
         if (o < cap) P.queue[3][o] = e; else capacity(P, 8);
@@ -776,7 +782,7 @@ __global__ void __launch_bounds__(kWarps * 32, 1) k_search_smem(Prog P, Arch A, 
   };
   if (part == 1) {
     for (int c = kClasses - 1; c >= 0; --c)
-      if (n_tasks[c]) run_class(c, false);
+      if (n_tasks(c)) run_class(c, false);
   } else {
     run_class(0, false);
   }
@@ -791,11 +797,14 @@ __global__ void __launch_bounds__(kWarps * 32, 1) k_search_smem(Prog P, Arch A, 
 
 }  // namespace
 
+int smem_class_limit(int c, int sms) { return c < 2 ? INT_MAX : 3 * class_warps(c) * sms; }
+
 void launch_search_smem(const Prog& P, const Arch& A, int most_nodes, int part, cudaStream_t st, int sms,
                         int64_t* launches) {
   size_t smem = 0;
   for (int c = 0; c < kClasses; ++c)
     smem = std::max(smem, (size_t)(class_warps(c) * warp_arena_bytes(class_nodes(c, most_nodes))));
+  static_assert(kWarps * 32 <= 768, "the launch bound (768 threads: at most 80 registers each)");
   allow_max_smem(k_search_smem);
   const int grid = (int)std::max<int64_t>(1, std::min<int64_t>(sms, P.queue_cap));
   k_search_smem<<<grid, kWarps * 32, smem, st>>>(P, A, most_nodes, part);

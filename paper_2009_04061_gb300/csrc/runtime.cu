@@ -546,7 +546,7 @@ static gpa_status alloc_program(const gpa_program_desc* d, ProgramRec* R, int ti
   P.raw_cap = 2 * (int64_t)d->n_use + 1024;
   TRY(dev_alloc(R, &P.raw, (size_t)P.raw_cap));
   P.queue_cap = (int64_t)d->n_use + 1;
-  for (int k = 0; k < 5; ++k) TRY(dev_alloc(R, &P.queue[k], (size_t)P.queue_cap));
+  for (int k = 0; k < 6; ++k) TRY(dev_alloc(R, &P.queue[k], (size_t)P.queue_cap));
   TRY(dev_alloc(R, &P.tasks, (size_t)std::max<int64_t>(d->n_use, 1)));
   TRY(dev_alloc(R, &P.tier_hint, (size_t)std::max<int64_t>(d->n_use, 1)));
   TRY(dev_alloc(R, &P.cov_cnt, (size_t)std::max<int64_t>(d->n_use, 1)));
@@ -648,6 +648,7 @@ gpa_status gpa_load_program(gpa_ctx* ctx, const gpa_program_desc* d, gpa_pid* ou
   s = alloc_program(d, R, ctx->tier[2].nodes);
   if (s) { free_program(R); return s; }
   Prog& P = R->P;
+  for (int c = 0; c < kClasses; ++c) P.class_limit[c] = smem_class_limit(c, ctx->sms);
   const size_t ni = P.ni;
   int32_t *pred_off = R->pred_off, *cursor = R->cursor, *ev_off = R->ev_off;
   uint32_t* events = R->events;
@@ -1076,7 +1077,9 @@ gpa_status gpa_sync_status(gpa_ctx* ctx, gpa_pid pid, gpa_stream stream, int64_t
     info[2] = (int64_t)h[SS_MAX_NODES];
     info[3] = (int64_t)h[SS_SWEEPS];
     info[4] = (int64_t)h[SS_OVF_N];
-    info[5] = (int64_t)(h[SS_OVF2_N] + h[SS_A1_N] + h[SS_A2_N] + h[SS_A3_N] + h[SS_HINT3_N]);
+    info[5] = (int64_t)(h[SS_OVF2_N] + h[SS_HINT3_N]);
+    for (int c = 0; c < kClasses; ++c)
+      info[5] += (int64_t)std::min<unsigned long long>(h[SS_A1_N + c], (unsigned long long)R->P.class_limit[c]);
     info[6] = (int64_t)(h[SS_MAX_TASK] & 0x7FFFFFFFull);     // use of the largest search
     info[7] = (int64_t)((h[SS_MAX_TASK] >> 31) & 0x1FFull);  // its resource
   }
