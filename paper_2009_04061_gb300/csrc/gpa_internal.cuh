@@ -106,7 +106,8 @@ struct Prog {
   int32_t reach_cls[5];           // the staged fixpoint's launches: reach_order[reach_cls[c], reach_cls[c + 1])
   int32_t reach_cls_smem[4];      // and the largest need among them (0: no launch)
   const uint8_t* func_natural;    // nf: 1 when every loop body of the function is a natural loop
-                                  // (functions needing more use the global-memory fixpoint)
+  int32_t reach_windowed;         // functions that only the windowed kernel takes (too large for the other two,
+                                  // or large with other loops)
   // Fourth search tier, sized for this program's largest function (0 nodes:
   // none): searches that outgrow the context's third tier, a CTA each.
   int32_t t4_nodes, t4_src, t4_ctas;
@@ -150,7 +151,7 @@ struct Prog {
   uint32_t* uuse_mask;            // nb * 9: resources read by an unguarded instruction
   uint32_t* touch_mask;           // nb * 9: DEF | UUSE (blocks a search must scan)
   int32_t* res_maxlat;            // nf * 268: largest latency of any def of the resource in the function
-  uint32_t* res_guards;           // nf * 268: guard literals of the resource's defs in the function
+  uint32_t* res_guards;           // nf * 268, right behind res_maxlat: guard literals of the resource's defs in the function
   uint32_t* rin;                  // nb * 9
   uint32_t* rout;                 // nb * 9
   int32_t* head;                  // ni: raw-edge list head per use (-1 = none)
@@ -335,8 +336,6 @@ void launch_build_preds(const Prog& P, int n_succ, int32_t* pred_off, int32_t* c
                         int sms, int64_t* launches);
 void launch_histogram(const Prog& P, const uint64_t* samples, size_t n, cudaStream_t st, int sms, int64_t* launches,
                       int variant, int hist_chunk);
-void launch_dataflow(const Prog& P, const Arch& A, int max_sweeps, int schedule, cudaStream_t st, int sms,
-                     int64_t* launches);
 
 // Lets kernel func take up to the device's opt-in shared memory per block.
 // Every launch and captured graph node of a kernel then sees the same limit
@@ -353,17 +352,24 @@ inline void allow_max_smem(F func) {
 }
 
 // Shared memory of the staged fixpoint for a function of nbf blocks, ne
-// predecessor entries and nlf loops: ROUT (9 words a block), a 16-byte record
-// per block (16-byte aligned: up to 12 bytes of padding), the predecessor CSR,
-// each block's innermost loop, and per loop its parent and two 9-word masks (the
-// definitions in its body; those of its body and enclosing loops).
+// predecessor entries and nlf loops: ROUT (9 words a block) and a row of zeros,
+// a 16-byte record per block (16-byte aligned: up to 12 bytes of padding), the
+// predecessor CSR, each block's innermost loop, and per loop its parent and two
+// 9-word masks (the definitions in its body; those of its body and enclosing
+// loops; of the latter also a row of zeros).
 __host__ __device__ inline int64_t reach_smem_need(int64_t nbf, int64_t ne, int64_t nlf) {
-  return 4 * kWords * nbf + 12 + 16 * nbf + 4 * (nbf + 1) + 4 * ne + 4 * nbf + 4 * nlf + 2 * 4 * kWords * nlf;
+  return 4 * kWords * (nbf + 1) + 12 + 16 * nbf + 4 * (nbf + 1) + 4 * ne + 4 * nbf + 4 * nlf +
+         2 * 4 * kWords * nlf + 4 * kWords;
+}
+// Shared memory of the fixpoint by function and word: two chunks of 512 records,
+// a word per block and a zero, two per loop.
+__host__ __device__ inline int64_t reach_words_need(int64_t nbf, int64_t nlf) {
+  return 2 * 512 * 16 + 4 * (nbf + 1) + 8 * nlf;
 }
 // Size classes of the staged fixpoint's launches (upper bounds of the need):
 // the larger a function, the fewer warps per SM its launch runs.
 constexpr int64_t kReachClassCap[4] = {200 * 1024, 64 * 1024, 28 * 1024, 12 * 1024};
-constexpr int64_t kReachSmemCap = 200 * 1024;
+constexpr int64_t kReachSmemCap = 220 * 1024;  // of a CTA per function and word
 // Two more streams (and their events) on which the searches queued straight
 // for the shared-memory and the global-memory warps run beside the first two
 // tiers.
@@ -371,6 +377,8 @@ struct SearchFork {
   cudaStream_t side[2];
   cudaEvent_t fork, join[2];
 };
+void launch_dataflow(const Prog& P, const Arch& A, int max_sweeps, int schedule, const SearchFork* fork,
+                     cudaStream_t st, int sms, int64_t* launches);
 void launch_blame(const Prog& P, const Arch& A, const SearchArena* tiers, const SearchFork* fork, int max_src,
                   int32_t* scan_tmp, cudaStream_t st, int sms, int64_t* launches);
 void launch_search(const Prog& P, const Arch& A, const SearchArena* tiers, const SearchFork* fork, cudaStream_t st,

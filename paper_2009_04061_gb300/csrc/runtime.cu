@@ -473,6 +473,13 @@ static gpa_status alloc_program(const gpa_program_desc* d, ProgramRec* R, int ti
         }
     }
     TRY(dev_copy(R, &P.func_natural, natural.data(), nf));
+    P.reach_windowed = 0;
+    for (int k = 0; k < P.reach_cls[0]; ++k) {
+      const int f = order[k];
+      const int64_t nbf = d->func_block_off[f + 1] - d->func_block_off[f],
+                    nlf = d->func_loop_off[f + 1] - d->func_loop_off[f];
+      if (!natural[f] || reach_words_need(nbf, nlf) > kReachSmemCap) ++P.reach_windowed;
+    }
     // Smallest block reachable from each block: a min fixpoint over
     // successors, swept in descending block order (forward edges point up, so
     // each sweep settles every forward path; back edges need a few more).
@@ -529,8 +536,8 @@ static gpa_status alloc_program(const gpa_program_desc* d, ProgramRec* R, int ti
   TRY(dev_alloc(R, &ev_off, nb * kEvBuckets + 1));
   TRY(dev_alloc(R, &events, (size_t)d->n_def + (size_t)d->n_use));
   P.ev_off = ev_off; P.events = events;
-  TRY(dev_alloc(R, &P.res_maxlat, nf * kNumRes));
-  TRY(dev_alloc(R, &P.res_guards, nf * kNumRes));
+  TRY(dev_alloc(R, &P.res_maxlat, 2 * nf * kNumRes));
+  P.res_guards = reinterpret_cast<uint32_t*>(P.res_maxlat) + nf * kNumRes;
   P.pred_off = pred_off; P.pred = pred; P.loop_depth = ldepth; P.instr_block = iblock; P.block_func = bfunc;
   TRY(dev_alloc(R, &R->scan_tmp, scan_tmp_ints((int)std::max(ni, nb * kEvBuckets) + 1)));
   TRY(dev_alloc(R, &P.cnt, ni * kCnt));
@@ -814,10 +821,11 @@ static gpa_status blame_body(gpa_ctx* ctx, ProgramRec* R, cudaStream_t st, bool 
   // per-step counters: general searches, largest search, sweeps, raw edges, queues
   CK(cudaMemsetAsync(R->P.stats + SS_GENERAL, 0, sizeof(unsigned long long) * 3, st));
   CK(cudaMemsetAsync(R->P.stats + SS_RAW_N, 0, sizeof(unsigned long long) * (SS_N - SS_RAW_N), st));
-  launch_dataflow(R->P, ctx->arch, ctx->opts.max_fixpoint_sweeps, ctx->opts.reach_schedule, st, ctx->sms,
-                  &ctx->launches);
-  // The search scratch is shared by the context's programs: order its users.
+  // The search scratch and the side streams are shared by the context's
+  // programs: order their users.
   if (order_scratch) CK(cudaStreamWaitEvent(st, ctx->scratch_ev, 0));
+  launch_dataflow(R->P, ctx->arch, ctx->opts.max_fixpoint_sweeps, ctx->opts.reach_schedule, &ctx->fork, st, ctx->sms,
+                  &ctx->launches);
   launch_blame(R->P, ctx->arch, ctx->tier, &ctx->fork, ctx->opts.max_sources_per_use, R->scan_tmp, st, ctx->sms,
                &ctx->launches);
   if (order_scratch) CK(cudaEventRecord(ctx->scratch_ev, st));
@@ -841,9 +849,9 @@ static gpa_status coverage_run(gpa_ctx* ctx, ProgramRec* R, cudaStream_t st, int
   CK(cudaMemsetAsync(D.cov_cnt, 0, sizeof(uint32_t) * (size_t)std::max(R->n_use, 1), st));
   CK(cudaMemsetAsync(D.stats + SS_GENERAL, 0, sizeof(unsigned long long) * 3, st));
   CK(cudaMemsetAsync(D.stats + SS_RAW_N, 0, sizeof(unsigned long long) * (SS_N - SS_RAW_N), st));
-  launch_dataflow(D, ctx->arch, ctx->opts.max_fixpoint_sweeps, ctx->opts.reach_schedule, st, ctx->sms,
-                  &ctx->launches);
   CK(cudaStreamWaitEvent(st, ctx->scratch_ev, 0));
+  launch_dataflow(D, ctx->arch, ctx->opts.max_fixpoint_sweeps, ctx->opts.reach_schedule, &ctx->fork, st, ctx->sms,
+                  &ctx->launches);
   launch_coverage(D, ctx->arch, ctx->tier, &ctx->fork, st, ctx->sms, &ctx->launches);
   CK(cudaEventRecord(ctx->scratch_ev, st));
   CK(cudaGetLastError());
