@@ -126,7 +126,11 @@ struct WarpGroup {
     for (int o = 16; o > 0; o >>= 1) x = ::min(x, __shfl_xor_sync(0xffffffffu, x, o));
     return x;
   }
-  __device__ __forceinline__ int read(const volatile int* p) const { return *p; }
+  __device__ __forceinline__ int read(const volatile int* p) const {
+    const int v = *p;
+    __syncwarp();
+    return v;
+  }
   __device__ __forceinline__ unsigned long long broadcast(unsigned long long v) const {
     return __shfl_sync(0xffffffffu, v, 0);
   }
@@ -556,7 +560,8 @@ __device__ bool group_search(const G& g, const Prog& P, const Arch& A, const Are
       if (ctr[4]) break;
       // pass A relaxed the wave's edges as they were linked; carry on from the
       // expanded nodes that improved (queued in ord, counted in ctr[5])
-      const int n_dirty = pass_b ? 0 : ctr[5];
+      // (every thread reads the count before relax_from's rank 0 clears it)
+      const int n_dirty = pass_b ? 0 : g.read(&ctr[5]);
       if (n_dirty > 0) relax_from(a.ord, n_dirty, 0);
       continue;
     }
