@@ -41,9 +41,9 @@ enum {
   // cycles of its five phases.
   SS_PHASE = 13, SS_SIZES = 31, SS_PASSB = 47, SS_SLOW = 48,
   // 55: unused
-  SS_OVF3_N = 56, SS_OVF3_HEAD = 57,  // searches that outgrew the shared-memory warps (bottom of queue[3])
+  SS_OVF3_N = 56, SS_OVF3_HEAD = 57,  // searches of full lists of the shared-memory warps (bottom of queue[3])
   SS_SIZE_CYC = 58,  // with -DGPA_PHASE_TIMING: cycles of the searches by log2 of their node count (16)
-  SS_HINT3_N = 74,   // searches queued straight for the global-memory warps (from the top of queue[3])
+  SS_HINT3_N = 74,   // searches beyond a class's limit (from the top of queue[3])
   SS_FAILBITS = 75,  // why a step reported GPA_ERR_CAPACITY: the last search tier ran out of
                      // 1 nodes, 2 edges, 3 occurrences, 4 sources, 5 back-edge layers,
                      // 6 hash rounds; 8 queue, 9 sources per use, 10 merged edges,
@@ -60,15 +60,22 @@ enum {
   // 91: unused
   // searches queued straight for a size class of the shared-memory warps
   SS_A1_N = 92, SS_A1_HEAD = 97,  // kClasses of each
-  SS_N = 102
+  SS_WIDE_N = 102, SS_WIDE_HEAD = 103,    // searches for the CTAs of 128 threads: known ones (bottom of queue[6])
+  SS_WIDE2_N = 104, SS_WIDE2_HEAD = 105,  // and those that outgrew the shared-memory warps (its top)
+  SS_T5_N = 106, SS_T5_HEAD = 107,        // searches beyond 2^18 nodes (queue[7])
+  SS_N = 108
 };
 // Size classes of the shared-memory search warps (k_search_smem.cu), and the
 // queue and region of each class's searches known from an earlier step.
 constexpr int kClasses = 5;
+__host__ __device__ inline int class_nodes(int c, int most) {
+  const int n = c < 4 ? 320 << c : 5632;
+  return n < most ? n : most;
+}
 __host__ __device__ constexpr int class_queue(int c) { return c < 3 ? c : c == 3 ? 2 : 5; }
 __host__ __device__ constexpr bool class_top(int c) { return c != 2 && c != 4; }
 // Values of tier_hint: the queue that a use entry's search belongs to.
-enum { kHintLane2 = 2, kHintA1 = 3, kHintWarp = kHintA1 + kClasses, kHintCta };
+enum { kHintLane2 = 2, kHintA1 = 3, kHintWide = kHintA1 + kClasses, kHintCta, kHintGiant };
 
 struct Arch {
   int32_t n_op;
@@ -161,11 +168,13 @@ struct Prog {
   // resource | start literal set << 9 | blocked << 25}. Each queue has queue_cap
   // entries: 0 first tier from the bottom (after it the second tier's overflow),
   // first size class of the shared-memory warps from the top; 1 second tier,
-  // second class; 2 third class, fourth class; 3 overflow to the global-memory
-  // warps, searches queued straight for them; 4 fourth tier; 5 fifth class. An entry is in one region of a
+  // second class; 2 third class, fourth class; 3 full lists' overflow to the
+  // global-memory warps, what is beyond a class's limit; 4 CTAs of 512 threads; 5
+  // fifth class; 6 CTAs of 128 threads, the last class's overflow; 7 beyond 2^18
+  // nodes. An entry is in one region of a
   // queue at a time, so the two regions never meet.
   int2* tasks;                    // n_use
-  int32_t* queue[6];
+  int32_t* queue[8];
   int32_t class_limit[kClasses];  // searches a class takes in a step; the rest go to the global-memory warps
   uint32_t* tier_hint;            // n_use: the queue known to hold the entry's search (0: none);
                                   // kept across steps (a search's size depends only on the program)
@@ -370,12 +379,11 @@ __host__ __device__ inline int64_t reach_words_need(int64_t nbf, int64_t nlf) {
 // the larger a function, the fewer warps per SM its launch runs.
 constexpr int64_t kReachClassCap[4] = {200 * 1024, 64 * 1024, 28 * 1024, 12 * 1024};
 constexpr int64_t kReachSmemCap = 220 * 1024;  // of a CTA per function and word
-// Two more streams (and their events) on which the searches queued straight
-// for the shared-memory and the global-memory warps run beside the first two
-// tiers.
+// Three more streams (and their events) on which the searches queued straight
+// for the larger tiers run beside the first two.
 struct SearchFork {
-  cudaStream_t side[2];
-  cudaEvent_t fork, join[2];
+  cudaStream_t side[3];
+  cudaEvent_t fork, join[3];
 };
 void launch_dataflow(const Prog& P, const Arch& A, int max_sweeps, int schedule, const SearchFork* fork,
                      cudaStream_t st, int sms, int64_t* launches);

@@ -187,19 +187,23 @@ __global__ void k_search_local(Prog P, Arch A) {
       const uint32_t hint = P.tier_hint[e];
       P.tasks[e] = make_int2(j, r | ((int)S << 9) | (blocked ? 1 << 25 : 0));
       int slot = SS_QUEUE_N, q = 0;
-      bool top = false;
+      bool top = false, placed = false;
       unsigned long long t = 0;
-      if (hint >= kHintCta && P.t4_nodes > 0) { slot = SS_T4_N; q = 4; }
-      else if (hint >= kHintWarp) { slot = SS_HINT3_N; q = 3; top = true; }
+      if (hint >= kHintCta && P.t4_nodes > 0) {
+        const bool giant = hint >= kHintGiant;
+        slot = giant ? SS_T5_N : SS_T4_N;
+        q = giant ? 7 : 4;
+      } else if (hint >= kHintWide) { slot = SS_WIDE_N; q = 6; }
       else if (hint >= kHintA1) {
         const int c = (int)hint - kHintA1;
         slot = SS_A1_N + c;
         q = class_queue(c);
         top = class_top(c);
         t = atomicAdd(&P.stats[slot], 1ull);
-        if (t >= (unsigned long long)P.class_limit[c]) { slot = SS_HINT3_N; q = 3; top = true; }
+        placed = t < (unsigned long long)P.class_limit[c];
+        if (!placed) { slot = SS_HINT3_N; q = 3; top = true; }  // the warps
       } else if (hint == kHintLane2) { slot = SS_OVF_N; q = 1; }
-      if (slot < SS_A1_N) t = atomicAdd(&P.stats[slot], 1ull);
+      if (!placed) t = atomicAdd(&P.stats[slot], 1ull);
       if (t < (unsigned long long)P.queue_cap) P.queue[q][top ? P.queue_cap - 1 - (int64_t)t : (int64_t)t] = e;
       else capacity(P, 8);
     }

@@ -2,9 +2,10 @@
 // stalled use j through resource r whose value may come from outside j's
 // block, with the three pruning rules evaluated over the set of source paths.
 //
-// The third and fourth search tier: one search group per (use, resource) task, a
-// warp in the third tier, a whole CTA in the fourth (searches of tens of
-// thousands to millions of nodes); searches of up to 64 nodes run one to a lane
+// The search tiers in global memory: one search group per (use, resource) task, a
+// warp for what the shared-memory warps leave of their largest classes, a CTA of
+// 128 threads for up to 32,768 nodes (max_search_nodes), a CTA of 512 threads for
+// up to 2^18 nodes and for what is larger still; searches of up to 64 nodes run one to a lane
 // before them (k_search_lanes.cu), those of up to 5,632 one to a warp in shared
 // memory (k_search_smem.cu). The graph of (block, literal set) nodes lives
 // in the group's arena in global memory. The group's threads scan node blocks in parallel
@@ -89,8 +90,8 @@ __device__ __forceinline__ void prefetch_l1(const void* p) {
 __device__ __forceinline__ int dist_of(const Arena& a, int u) { return (int)(a.dpk[u] >> 32); }
 __device__ __forceinline__ int par_of(const Arena& a, int u) { return (int)(a.dpk[u] & 0xFFFFFFFFull); }
 
-// The threads that run one search together: a warp (third tier) or a whole
-// CTA (the fourth tier's very large searches). Both give the search the same
+// The threads that run one search together: a warp or a whole CTA
+// (the very large searches). Both give the search the same
 // steps: a barrier, an any-vote, exclusive prefix counts, inclusive sums and
 // reductions over the group, a read of a shared flag that every thread takes
 // before any of them may change it, and a broadcast from rank 0.
@@ -136,14 +137,13 @@ struct WarpGroup {
   }
 };
 
-constexpr int kCtaThreads = 512;  // threads of a fourth-tier search CTA
-
-// A CTA as one search group. `red` is shared scratch of kCtaThreads / 32
+// A CTA of NT threads as one search group. `red` is shared scratch of NT / 32
 // ints, `cast` a shared 64-bit slot for broadcasts. Every collective ends with
 // a barrier, so the scratch is free again when it returns.
+template <int NT>
 struct CtaGroup {
-  static constexpr int kSize = kCtaThreads;
-  static constexpr int kWarps = kCtaThreads / 32;
+  static constexpr int kSize = NT;
+  static constexpr int kWarps = NT / 32;
   int* red;
   unsigned long long* cast;
   __device__ __forceinline__ int rank() const { return threadIdx.x; }
@@ -920,24 +920,29 @@ __device__ bool group_search(const G& g, const Prog& P, const Arch& A, const Are
   return true;
 }
 
+// A queue region of searches and where those that outgrow the arenas go.
+struct Route {
+  int q, n_slot, h_slot;   // queue, its count and head
+  bool top;                // read down from the top of the queue
+  int next_q, next_slot;   // -1: the last tier (it records why it ran out)
+  bool next_top;
+  uint32_t next_hint;
+};
+
 // The task loop of a search group: claim (use, resource) tasks from one
-// queue until it is empty. A search that outgrows the third tier is queued for
-// the fourth; the last tier records why it ran out. An arena that holds its own
-// hash (`clear`) has it emptied when the group's first task arrives, so a group
-// that finds none touches no memory.
+// queue until it is empty. An arena that holds its own hash (`clear`) has it
+// emptied when the group's first task arrives, so a group that finds none touches
+// no memory.
 template <class G>
-__device__ void run_tasks(const G& g, const Prog& P, const Arch& A, const Arena& a, int tier, int part, bool clear) {
+__device__ void run_tasks(const G& g, const Prog& P, const Arch& A, const Arena& a, const Route& R, int tier,
+                          bool clear) {
   const int me = g.rank();
-  // part 1: the searches queued straight for these warps; part 2: the
-  // shared-memory warps' overflow
   const unsigned long long cap = (unsigned long long)P.queue_cap;
-  const int32_t* q = P.queue[tier];
-  const bool top = tier == 3 && part == 1;
-  const unsigned long long nt = min(P.stats[tier == 4 ? SS_T4_N : top ? SS_HINT3_N : SS_OVF3_N], cap);
-  const int h_slot = tier == 4 ? SS_T4_HEAD : top ? SS_HINT3_HEAD : SS_OVF3_HEAD;
+  const int32_t* q = P.queue[R.q];
+  const unsigned long long nt = min(P.stats[R.n_slot], cap);
   while (true) {
     unsigned long long t = 0;
-    if (me == 0) t = atomicAdd(&P.stats[h_slot], 1ull);
+    if (me == 0) t = atomicAdd(&P.stats[R.h_slot], 1ull);
     t = g.broadcast(t);
     if (t >= nt) break;
     if (clear) {
@@ -945,59 +950,68 @@ __device__ void run_tasks(const G& g, const Prog& P, const Arch& A, const Arena&
       g.sync();
       clear = false;
     }
-    const int e = q[top ? cap - 1 - t : t];
-    const int2 packed = P.tasks[e];
-    const int4 task = make_int4(packed.x, packed.y & 0x1FF, (int)((uint32_t)packed.y >> 9 & 0xFFFFu), e);
+    const int e = q[R.top ? cap - 1 - t : t];
+    const int2 task = P.tasks[e];
+    const int r = task.y & 0x1FF;
     const int f = P.block_func[P.instr_block[task.x]];
     // The coverage count needs every source: no latency bound.
-    const int bound = P.diag ? kInf - 1 : P.res_maxlat[(size_t)f * kNumRes + task.y];
-    const uint16_t live = live_literals(P.res_guards[(size_t)f * kNumRes + task.y], P.guard[task.x]);
-    const bool ok = group_search(g, P, A, a, task.x, task.y, (uint16_t)task.z, bound, live, tier, task.w,
-                                 (packed.y >> 25) & 1);
-    if (ok || me != 0) continue;
-    if (tier == 3 && P.t4_nodes > 0) {
-      if (!P.diag) atomicMax(&P.tier_hint[e], (unsigned)kHintCta);  // later steps queue it there
-      const unsigned long long o = atomicAdd(&P.stats[SS_T4_N], 1ull);
-      if (o < cap) P.queue[4][o] = e; else capacity(P, 8);
-    } else {
-      capacity(P, a.ctr[7] > 0 ? a.ctr[7] : 1);  // the last tier: why it ran out
+    const int bound = P.diag ? kInf - 1 : P.res_maxlat[(size_t)f * kNumRes + r];
+    const uint16_t live = live_literals(P.res_guards[(size_t)f * kNumRes + r], P.guard[task.x]);
+    const bool ok = group_search(g, P, A, a, task.x, r, (uint16_t)((uint32_t)task.y >> 9), bound, live, tier, e,
+                                 (task.y >> 25) & 1);
+    if (me != 0) continue;
+    if (ok) {
+      // A search that a full list sent to the warps finds its queue at once.
+      if (tier == 3 && !P.diag) {
+        int c = 0;
+        while (c < kClasses && class_nodes(c, a.N) < ((volatile int*)a.ctr)[0]) ++c;
+        atomicMax(&P.tier_hint[e], (unsigned)(kHintA1 + c));
+      }
+      continue;
     }
+    if (R.next_q < 0) {
+      capacity(P, a.ctr[7] > 0 ? a.ctr[7] : 1);
+      continue;
+    }
+    if (!P.diag) atomicMax(&P.tier_hint[e], R.next_hint);  // later steps queue it there
+    const unsigned long long o = atomicAdd(&P.stats[R.next_slot], 1ull);
+    if (o < cap) P.queue[R.next_q][R.next_top ? cap - 1 - o : o] = e;
+    else capacity(P, 8);
   }
 }
 
-// The third tier: persistent work-stealing warps, one search each, over
-// global-memory arenas, in two parts: part 1 takes the searches queued straight
-// for it and runs beside the other tiers; part 2 takes the shared-memory warps'
-// overflow.
-// Registers: 80 a thread (96 without the bound), so 24 one-warp CTAs fit an SM:
-// the searches are chains of dependent loads, and more warps in flight finish
-// more of them (measured: 40.7 against 41.9 ms a step).
-__global__ void __launch_bounds__(32, 24) k_search_warp(Prog P, Arch A, SearchArena SA, int part) {
+// Persistent work-stealing warps, one search each: what the shared-memory
+// warps' largest classes have beyond three rounds of the chip (part 1), and what
+// overflowed from their CTAs' lists (part 2). 80 registers a thread, so 24 one-warp
+// CTAs fit an SM: the searches are chains of dependent loads, and more warps in
+// flight finish more of them (measured: 40.7 against 41.9 ms a step with 96).
+__global__ void __launch_bounds__(32, 24) k_search_warp(Prog P, Arch A, SearchArena SA, Route R) {
   // The search counters live in shared memory (the arena is in global memory):
   // frontier sizes are read after every round.
   __shared__ int s_ctr[8];
-  // The node hashes lie apart from the arenas (whose pool the fourth tier lays
-  // out anew) and are empty between searches: every search empties the slots
-  // it used, also when it outgrew its arena. They were cleared with the context,
+  // The node hashes lie apart from the arenas (whose pool the largest searches lay
+  // out anew) and are empty between searches: every search empties the slots it
+  // used, also when it outgrew its arena. They were cleared with the context,
   // so a launch clears nothing. (A launch that began by clearing its warps'
   // 256 KB hashes wrote 956 MB and took 145 us with no search to run; the launch
   // appears twice in a step.)
   const Arena a = carve(SA.global + (int64_t)blockIdx.x * SA.bytes, SA.hash + (int64_t)blockIdx.x * 2 * SA.nodes,
                         SA.nodes, SA.src, SA.layers, s_ctr);
-  run_tasks(WarpGroup{}, P, A, a, 3, part, false);
+  run_tasks(WarpGroup{}, P, A, a, R, 3, false);
 }
 
-// The fourth tier: a CTA per search, over a global-memory arena of its own
-// (the searches that outgrow the third tier's arenas have tens of thousands to
-// millions of (block, literal set) nodes: their waves, frontiers and source
-// lists are wide enough for a CTA's threads).
-__global__ void __launch_bounds__(kCtaThreads, 1) k_search_cta(Prog P, Arch A, SearchArena SA) {
+// A CTA per search: the waves, frontiers and source lists of these searches
+// are wide enough for its threads. 128 threads for searches of 5,633 to 32,768
+// nodes (a warp took 31 ms for the largest of them), 512 for larger ones.
+template <int NT>
+__global__ void __launch_bounds__(NT, 512 / NT) k_search_cta(Prog P, Arch A, SearchArena SA, Route R) {
   __shared__ int s_ctr[8];
-  __shared__ int s_red[CtaGroup::kWarps];
+  __shared__ int s_red[CtaGroup<NT>::kWarps];
   __shared__ unsigned long long s_cast;
-  const CtaGroup g{s_red, &s_cast};
-  const Arena a = carve(SA.global + (int64_t)blockIdx.x * SA.bytes, nullptr, SA.nodes, SA.src, SA.layers, s_ctr);
-  run_tasks(g, P, A, a, 4, 0, true);
+  const CtaGroup<NT> g{s_red, &s_cast};
+  int* hash = SA.hash ? SA.hash + (int64_t)blockIdx.x * 2 * SA.nodes : nullptr;
+  const Arena a = carve(SA.global + (int64_t)blockIdx.x * SA.bytes, hash, SA.nodes, SA.src, SA.layers, s_ctr);
+  run_tasks(g, P, A, a, R, 4, hash == nullptr);
 }
 
 }  // namespace
@@ -1019,40 +1033,74 @@ void launch_search(const Prog& P, const Arch& A, const SearchArena* tiers, const
   // waits on another; the joins only order the parts that share arenas or
   // storage after them). They are submitted first, so that the largest searches
   // start first and the first tiers' CTAs fill the SMs as they come free.
-  cudaStream_t s1 = st, s3 = st;
+  cudaStream_t s[4] = {st, st, st, st};
   if (fork) {
     cudaEventRecord(fork->fork, st);
-    s3 = fork->side[0];
-    s1 = fork->side[1];
-    cudaStreamWaitEvent(s3, fork->fork, 0);
-    cudaStreamWaitEvent(s1, fork->fork, 0);
+    for (int k = 0; k < 3; ++k) {
+      s[k] = fork->side[k];
+      cudaStreamWaitEvent(s[k], fork->fork, 0);
+    }
   }
+  // The CTAs of 128 threads take the first of the arenas, the warps the others
+  // (with a single arena they take turns).
+  SearchArena wide = tiers[2], narrow = tiers[2];
+  wide.warps = std::max(1, std::min(tiers[2].warps / 2, 4 * sms));
+  if (tiers[2].warps > 1) {
+    narrow.warps -= wide.warps;
+    narrow.global += (int64_t)wide.warps * narrow.bytes;
+    narrow.hash += (int64_t)wide.warps * 2 * narrow.nodes;
+  } else {
+    s[2] = s[1];
+  }
+  const bool big = P.t4_nodes > 0;
+  const int q4 = big ? 4 : -1;
+  const Route wide1{6, SS_WIDE_N, SS_WIDE_HEAD, false, q4, SS_T4_N, false, kHintCta};
+  const Route wide2{6, SS_WIDE2_N, SS_WIDE2_HEAD, true, q4, SS_T4_N, false, kHintCta};
+  const Route warp1{3, SS_HINT3_N, SS_HINT3_HEAD, true, q4, SS_T4_N, false, kHintCta};
+  const Route warp2{3, SS_OVF3_N, SS_OVF3_HEAD, false, q4, SS_T4_N, false, kHintCta};
   // No launch takes more groups than there can be tasks (one per use entry).
-  const int g3 = (int)std::min<int64_t>(tiers[2].warps, P.queue_cap);
-  launch_search_smem(P, A, tiers[2].nodes, 1, s1, sms, launches);
-  k_search_warp<<<g3, 32, 0, s3>>>(P, A, tiers[2], 1);
+  auto groups = [&](int n) { return (int)std::max<int64_t>(1, std::min<int64_t>(n, P.queue_cap)); };
+  launch_search_smem(P, A, tiers[2].nodes, 1, s[0], sms, launches);
+  k_search_cta<128><<<groups(wide.warps), 128, 0, s[1]>>>(P, A, wide, wide1);
+  k_search_warp<<<groups(narrow.warps), 32, 0, s[2]>>>(P, A, narrow, warp1);
   launch_search_lanes(P, A, tiers[0], 1, st, launches);
   launch_search_lanes(P, A, tiers[1], 2, st, launches);
-  if (fork) {
-    cudaEventRecord(fork->join[0], s3);
-    cudaEventRecord(fork->join[1], s1);
-    cudaStreamWaitEvent(st, fork->join[0], 0);
-    cudaStreamWaitEvent(st, fork->join[1], 0);
-  }
-  launch_search_smem(P, A, tiers[2].nodes, 2, st, sms, launches);
-  k_search_warp<<<g3, 32, 0, st>>>(P, A, tiers[2], 2);
-  *launches += 2;
-  if (P.t4_nodes > 0) {
-    // The fourth tier runs after the third on this stream, so the third tier's
-    // arena pool is free by then: when it holds more fourth-tier arenas than the
-    // program's own, the CTAs carve theirs from it (at most one CTA per SM).
-    SearchArena t4{P.t4_nodes, P.t4_src, kMaxLayers, P.t4_ctas, P.t4_bytes, P.t4_arena, nullptr};
-    const int64_t in_pool = (int64_t)tiers[2].warps * tiers[2].bytes / P.t4_bytes;
-    if (in_pool > t4.warps && tiers[2].global) {
-      t4.warps = (int)std::min<int64_t>(in_pool, std::max(sms, 1));
-      t4.global = tiers[2].global;
+  if (fork)
+    for (int k = 0; k < 3; ++k) {
+      cudaEventRecord(fork->join[k], fork->side[k]);
+      cudaStreamWaitEvent(st, fork->join[k], 0);
     }
-    k_search_cta<<<t4.warps, kCtaThreads, 0, st>>>(P, A, t4);
+  launch_search_smem(P, A, tiers[2].nodes, 2, st, sms, launches);
+  k_search_cta<128><<<groups(wide.warps), 128, 0, st>>>(P, A, wide, wide2);
+  k_search_warp<<<groups(narrow.warps), 32, 0, st>>>(P, A, narrow, warp2);
+  *launches += 4;
+  if (big) {
+    // Larger searches run after the others on this stream, so the third tier's
+    // arena pool is free by then and they carve their arenas from it (at most one
+    // CTA per SM): first those of up to 2^18 nodes (most of them; arenas for the
+    // program's largest function would be so big that the pool holds few), then
+    // the rest in arenas of t4_nodes, from the pool when it holds more of them
+    // than the program's own.
+    const int64_t pool = tiers[2].global ? (int64_t)tiers[2].warps * tiers[2].bytes : 0;
+    SearchArena own{P.t4_nodes, P.t4_src, kMaxLayers, P.t4_ctas, P.t4_bytes, P.t4_arena, nullptr};
+    if (pool / P.t4_bytes > own.warps) {
+      own.warps = (int)std::min<int64_t>(pool / P.t4_bytes, std::max(sms, 1));
+      own.global = tiers[2].global;
+    }
+    const int mid_nodes = 1 << 18;
+    SearchArena mid{mid_nodes, 4096, kMaxLayers, 0, arena_bytes(mid_nodes, 4096, kMaxLayers, true), tiers[2].global,
+                    nullptr};
+    mid.warps = (int)std::min<int64_t>(pool / mid.bytes, std::max(sms, 1));
+    Route r4{4, SS_T4_N, SS_T4_HEAD, false, -1, 0, false, 0};
+    if (P.t4_nodes > mid_nodes && mid.warps > own.warps) {
+      r4.next_q = 7; r4.next_slot = SS_T5_N; r4.next_hint = kHintGiant;
+      k_search_cta<512><<<groups(mid.warps), 512, 0, st>>>(P, A, mid, r4);
+      ++*launches;
+      const Route r5{7, SS_T5_N, SS_T5_HEAD, false, -1, 0, false, 0};
+      k_search_cta<512><<<groups(own.warps), 512, 0, st>>>(P, A, own, r5);
+    } else {
+      k_search_cta<512><<<groups(own.warps), 512, 0, st>>>(P, A, own, r4);
+    }
     ++*launches;
   }
 }

@@ -46,10 +46,6 @@ constexpr uint32_t kNoWall = 0xFFFFu;
 constexpr uint32_t F_EXP = 1u << 24, F_QUE = 1u << 25, F_NEED = 1u << 26, F_BACK = 1u << 27;
 constexpr int kSearchInf = 0x7FFFFFFF;
 
-__host__ __device__ inline int class_nodes(int c, int most) {
-  const int n = c < 4 ? 320 << c : 5632;
-  return n < most ? n : most;
-}
 __host__ __device__ inline int class_warps(int c) { return 16 >> c; }
 __host__ __device__ inline int hash_slots(int n) {  // a power of two, at least 1.4 n
   int h = 16;
@@ -774,8 +770,10 @@ __global__ void __launch_bounds__(768, 1) k_search_smem(Prog P, Arch A, int most
           const int t = atomicAdd(&s_nlocal[next], 1);
           if (t < (next < 2 ? kLocalList : 3 * class_warps(next))) { s_local[next][t] = e; continue; }
         }
-        const unsigned long long o = atomicAdd(&P.stats[SS_OVF3_N], 1ull);
-        if (o < cap) P.queue[3][o] = e; else capacity(P, 8);
+        const bool wide = next == kClasses;  // else a full list
+        const unsigned long long o = atomicAdd(&P.stats[wide ? SS_WIDE2_N : SS_OVF3_N], 1ull);
+        if (o < cap) P.queue[wide ? 6 : 3][wide ? cap - 1 - o : o] = e;
+        else capacity(P, 8);
       }
     }
     __syncthreads();

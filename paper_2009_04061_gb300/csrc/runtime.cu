@@ -337,7 +337,7 @@ gpa_status gpa_create(const gpa_arch_desc* arch, const gpa_options* opts, gpa_ct
   if (!s && cudaEventCreateWithFlags(&c->scratch_ev, cudaEventDisableTiming) != cudaSuccess) s = GPA_ERR_CUDA;
   if (!s && cudaStreamCreateWithFlags(&c->build_stream, cudaStreamNonBlocking) != cudaSuccess) s = GPA_ERR_CUDA;
   if (!s && cudaEventCreateWithFlags(&c->fork.fork, cudaEventDisableTiming) != cudaSuccess) s = GPA_ERR_CUDA;
-  for (int k = 0; k < 2; ++k) {
+  for (int k = 0; k < 3; ++k) {
     if (!s && cudaStreamCreateWithFlags(&c->fork.side[k], cudaStreamNonBlocking) != cudaSuccess) s = GPA_ERR_CUDA;
     if (!s && cudaEventCreateWithFlags(&c->fork.join[k], cudaEventDisableTiming) != cudaSuccess) s = GPA_ERR_CUDA;
   }
@@ -347,7 +347,7 @@ gpa_status gpa_create(const gpa_arch_desc* arch, const gpa_options* opts, gpa_ct
     if (c->scratch_ev) cudaEventDestroy(c->scratch_ev);
     if (c->build_stream) cudaStreamDestroy(c->build_stream);
     if (c->fork.fork) cudaEventDestroy(c->fork.fork);
-    for (int k = 0; k < 2; ++k) {
+    for (int k = 0; k < 3; ++k) {
       if (c->fork.side[k]) cudaStreamDestroy(c->fork.side[k]);
       if (c->fork.join[k]) cudaEventDestroy(c->fork.join[k]);
     }
@@ -374,7 +374,7 @@ gpa_status gpa_destroy(gpa_ctx* ctx) {
   if (ctx->build_stream) cudaStreamDestroy(ctx->build_stream);
   if (ctx->scratch_ev) cudaEventDestroy(ctx->scratch_ev);
   if (ctx->fork.fork) cudaEventDestroy(ctx->fork.fork);
-  for (int k = 0; k < 2; ++k) {
+  for (int k = 0; k < 3; ++k) {
     if (ctx->fork.side[k]) cudaStreamDestroy(ctx->fork.side[k]);
     if (ctx->fork.join[k]) cudaEventDestroy(ctx->fork.join[k]);
   }
@@ -553,7 +553,7 @@ static gpa_status alloc_program(const gpa_program_desc* d, ProgramRec* R, int ti
   P.raw_cap = 2 * (int64_t)d->n_use + 1024;
   TRY(dev_alloc(R, &P.raw, (size_t)P.raw_cap));
   P.queue_cap = (int64_t)d->n_use + 1;
-  for (int k = 0; k < 6; ++k) TRY(dev_alloc(R, &P.queue[k], (size_t)P.queue_cap));
+  for (int k = 0; k < 8; ++k) TRY(dev_alloc(R, &P.queue[k], (size_t)P.queue_cap));
   TRY(dev_alloc(R, &P.tasks, (size_t)std::max<int64_t>(d->n_use, 1)));
   TRY(dev_alloc(R, &P.tier_hint, (size_t)std::max<int64_t>(d->n_use, 1)));
   TRY(dev_alloc(R, &P.cov_cnt, (size_t)std::max<int64_t>(d->n_use, 1)));
@@ -1085,7 +1085,7 @@ gpa_status gpa_sync_status(gpa_ctx* ctx, gpa_pid pid, gpa_stream stream, int64_t
     info[2] = (int64_t)h[SS_MAX_NODES];
     info[3] = (int64_t)h[SS_SWEEPS];
     info[4] = (int64_t)h[SS_OVF_N];
-    info[5] = (int64_t)(h[SS_OVF2_N] + h[SS_HINT3_N]);
+    info[5] = (int64_t)(h[SS_OVF2_N] + h[SS_HINT3_N] + h[SS_WIDE_N]);
     for (int c = 0; c < kClasses; ++c)
       info[5] += (int64_t)std::min<unsigned long long>(h[SS_A1_N + c], (unsigned long long)R->P.class_limit[c]);
     info[6] = (int64_t)(h[SS_MAX_TASK] & 0x7FFFFFFFull);     // use of the largest search
