@@ -1,61 +1,19 @@
 // Layout derivations done once per loaded program (predecessor lists, the
 // block of each instruction, loop depths) and a device exclusive scan.
+#include <algorithm>
+
 #include "gpa_internal.cuh"
+#include "scan_tiles.cuh"
 
 namespace gpa {
 
 namespace {
 
-constexpr int kScanThreads = 1024;
-constexpr int kScanItems = 4;
-constexpr int kScanTile = kScanThreads * kScanItems;
-
-// Block-local exclusive scan of a 4096-element tile; writes the tile total.
-__global__ void k_scan_tiles(int32_t* buf, int n, int32_t* sums) {
-  __shared__ int32_t warp_tot[32];
-  const int base = blockIdx.x * kScanTile + threadIdx.x * kScanItems;
-  int32_t v[kScanItems];
-  int32_t local = 0;
-#pragma unroll
-  for (int t = 0; t < kScanItems; ++t) {
-    v[t] = (base + t < n) ? buf[base + t] : 0;
-    local += v[t];
-  }
-  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-  int32_t incl = local;
-#pragma unroll
-  for (int o = 1; o < 32; o <<= 1) {
-    int32_t y = __shfl_up_sync(0xffffffffu, incl, o);
-    if (lane >= o) incl += y;
-  }
-  if (lane == 31) warp_tot[warp] = incl;
-  __syncthreads();
-  if (warp == 0) {
-    int32_t w = warp_tot[lane];
-    int32_t wi = w;
-#pragma unroll
-    for (int o = 1; o < 32; o <<= 1) {
-      int32_t y = __shfl_up_sync(0xffffffffu, wi, o);
-      if (lane >= o) wi += y;
-    }
-    warp_tot[lane] = wi - w;
-    if (lane == 31) sums[blockIdx.x] = wi;
-  }
-  __syncthreads();
-  int32_t run = warp_tot[warp] + incl - local;
-#pragma unroll
-  for (int t = 0; t < kScanItems; ++t) {
-    if (base + t < n) buf[base + t] = run;
-    run += v[t];
-  }
+__global__ void __launch_bounds__(scan::kThreads) k_scan_sums(const int32_t* buf, int n, int32_t* sums) {
+  scan::tile_sum(buf, n, sums);
 }
-
-__global__ void k_scan_add(int32_t* buf, int n, const int32_t* offs) {
-  const int base = blockIdx.x * kScanTile + threadIdx.x * kScanItems;
-  const int32_t o = offs[blockIdx.x];
-#pragma unroll
-  for (int t = 0; t < kScanItems; ++t)
-    if (base + t < n) buf[base + t] += o;
+__global__ void __launch_bounds__(scan::kThreads) k_scan_tiles(int32_t* buf, int n, const int32_t* sums) {
+  scan::tile_scan(buf, n, sums, buf + n);
 }
 
 __global__ void k_instr_block(Prog P) {
@@ -185,36 +143,18 @@ int grid_for(int64_t n, int threads, int sms) {
   return (int)(g < 1 ? 1 : g);
 }
 
-size_t scan_tmp_ints(int n) {
-  size_t total = 0;
-  int m = n + 1;
-  while (true) {
-    int tiles = (m + kScanTile - 1) / kScanTile;
-    total += (size_t)tiles + 1;
-    if (tiles <= 1) break;
-    m = tiles;
-  }
-  return total + 16;
-}
+size_t scan_tmp_ints(int n) { return (size_t)n / scan::kTile + 16; }
 
 // buf has n + 1 entries; on return buf[k] = sum of the first k inputs and
 // buf[n] = the total (the input buf[n] is ignored).
-static void scan_rec(int32_t* buf, int m, int32_t* tmp, cudaStream_t st, int64_t* launches) {
-  int tiles = (m + kScanTile - 1) / kScanTile;
-  int32_t* sums = tmp;
-  k_scan_tiles<<<tiles, kScanThreads, 0, st>>>(buf, m, sums);
-  ++*launches;
+void scan_exclusive_inplace(int32_t* buf, int n, int32_t* tmp, cudaStream_t st, int64_t* launches) {
+  const int tiles = std::max(1, (n + scan::kTile - 1) / scan::kTile);
   if (tiles > 1) {
-    scan_rec(sums, tiles, tmp + tiles + 1, st, launches);
-    k_scan_add<<<tiles, kScanThreads, 0, st>>>(buf, m, sums);
+    k_scan_sums<<<tiles, scan::kThreads, 0, st>>>(buf, n, tmp);
     ++*launches;
   }
-}
-
-void scan_exclusive_inplace(int32_t* buf, int n, int32_t* tmp, cudaStream_t st, int64_t* launches) {
-  // Scanning n + 1 entries whose last input is 0 puts the total in buf[n].
-  cudaMemsetAsync(buf + n, 0, sizeof(int32_t), st);
-  scan_rec(buf, n + 1, tmp, st, launches);
+  k_scan_tiles<<<tiles, scan::kThreads, 0, st>>>(buf, n, tmp);
+  ++*launches;
 }
 
 void launch_build_layout(const Prog& P, cudaStream_t st, int sms, int64_t* launches) {
