@@ -25,12 +25,9 @@
 //    resource) pairs and explore the (block, literal set) graph.
 //  * k_merge_count / scan / k_apportion: merge sources per use, apportion in
 //    integers, scatter blame with warp-aggregated 64-bit atomics.
-#include <cooperative_groups.h>
-#include <cooperative_groups/reduce.h>
+#include <algorithm>
 
 #include "gpa_internal.cuh"
-
-namespace cg = cooperative_groups;
 
 namespace gpa {
 
@@ -107,16 +104,22 @@ __global__ void k_stalled_list(Prog P) {
   if (s) P.suse[base + __popc(m & ((1u << lane) - 1u))] = j;
 }
 
-// Thread per stalled use (from the stalled-use list).
+// Four threads per stalled use (from the stalled-use list), each taking every
+// fourth resource the use reads: a resource's scans are a chain of dependent
+// loads, so a thread per use ran its two or three of them one after another
+// (55 us for a 200-instruction program).
+constexpr int kLocalLanes = 4;
 __global__ void k_search_local(Prog P, Arch A) {
   const int n_suse = (int)P.stats[SS_SUSE_N];
-  for (int k = blockIdx.x * blockDim.x + threadIdx.x; k < n_suse; k += gridDim.x * blockDim.x) {
-    const int j = P.suse[k];
+  for (int64_t kk = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; kk < (int64_t)n_suse * kLocalLanes;
+       kk += (int64_t)gridDim.x * blockDim.x) {
+    const int j = P.suse[kk / kLocalLanes];
     const int gj = P.guard[j];
     const int b0 = P.instr_block[j];
     const int first = P.block_instr_off[b0];
     const int pj = j - first;
-    for (int e = P.use_off[j]; e < P.use_off[j + 1]; ++e) {
+    const int e_end = P.use_off[j + 1];
+    for (int e = P.use_off[j] + (int)(kk % kLocalLanes); e < e_end; e += kLocalLanes) {
       const int r = P.use_res[e] & 0x1FF;
       const size_t seg = (size_t)b0 * kEvBuckets + ev_bucket(r);  // b0's events of r's bucket
       const int ev0 = P.ev_off[seg], ev1 = P.ev_off[seg + 1];
@@ -221,12 +224,10 @@ __global__ void k_blame_init(Prog P) {
   }
 }
 
-__device__ __forceinline__ void blame_add(unsigned long long* addr, unsigned long long v) {
-  cg::coalesced_group g = cg::coalesced_threads();
-  cg::coalesced_group grp = cg::labeled_partition(g, (unsigned long long)(uintptr_t)addr);
-  const unsigned long long sum = cg::reduce(grp, v, cg::plus<unsigned long long>());
-  if (grp.thread_rank() == 0) atomicAdd(addr, sum);
-}
+// (The lanes of a warp hold neighbouring uses, whose sources are mostly
+// different instructions: partitioning them by address first cost more than the
+// few atomics it saved.)
+__device__ __forceinline__ void blame_add(unsigned long long* addr, unsigned long long v) { atomicAdd(addr, v); }
 
 // Distinct sources of use j over its raw edge list, using ids[cap] as scratch:
 // the count, or -1 if there are more than cap.
@@ -323,13 +324,21 @@ __device__ void apportion_use(const Prog& P, const Arch& A, int j, int off, int 
         blame_add(P.blame + (size_t)j * kCnt + cls * 2 + lat, S);
         continue;
       }
+      if (ns == 1) {  // a single source takes them all, whatever its weight
+        const int t = sel[0];
+        if (P.cnt[(size_t)mi[t] * kCnt] >> 43) set_status(P, ST_OVERFLOW);
+        P.e_share[(int64_t)(off + t) * 8 + ci * 2 + lat] = S;
+        blame_add(P.blame + (size_t)mi[t] * kCnt + cls * 2 + lat, S);
+        continue;
+      }
       // Eq. 1: weight = issued samples / longest path, in units of 2^-20.
       unsigned __int128 W = 0;
       for (int q = 0; q < ns; ++q) {
         const unsigned long long issue = P.cnt[(size_t)mi[sel[q]] * kCnt];
         const unsigned long long len = (unsigned long long)max(ml[sel[q]], 1);
         if (issue >> 43) set_status(P, ST_OVERFLOW);
-        wt[q] = (unsigned long long)(((unsigned __int128)issue << 20) / len);
+        // (len < 2^24, so a 64-bit division does for issue counts below 2^44)
+        wt[q] = issue >> 44 ? (unsigned long long)(((unsigned __int128)issue << 20) / len) : (issue << 20) / len;
         W += wt[q];
       }
       if (W == 0) {
@@ -342,11 +351,19 @@ __device__ void apportion_use(const Prog& P, const Arch& A, int j, int off, int 
         for (int q = 0; q < ns; ++q) wt[q] = 1ull;
         W = (unsigned __int128)ns;
       }
+      // S * wt and W mostly fit 64 bits, whose division is a tenth of the work.
       unsigned long long given = 0;
+      const bool narrow = !(W >> 64);
       for (int q = 0; q < ns; ++q) {
         const unsigned __int128 num = (unsigned __int128)S * wt[q];
-        sh[q] = (unsigned long long)(num / W);
-        rem[q] = num % W;
+        if (narrow && !(num >> 64)) {
+          const unsigned long long a = (unsigned long long)num, b = (unsigned long long)W;
+          sh[q] = a / b;
+          rem[q] = a - sh[q] * b;
+        } else {
+          sh[q] = (unsigned long long)(num / W);
+          rem[q] = num % W;
+        }
         given += sh[q];
       }
       // Largest remainders get the leftover units; ties go to the lower def index.
@@ -455,7 +472,7 @@ void launch_coverage(const Prog& P, const Arch& A, const SearchArena* tiers, con
   // registers allow, each thread taking about one use on the batched workload.
   const int g_use = std::max(1, std::min(grid_for(P.ni, threads, sms) * 4, (P.ni + threads - 1) / threads));
   k_stalled_list<<<std::max(1, (P.ni + 255) / 256), 256, 0, st>>>(P);
-  k_search_local<<<g_use, threads, 0, st>>>(P, A);
+  k_search_local<<<g_use * 2, threads, 0, st>>>(P, A);
   *launches += 2;
   launch_search(P, A, tiers, fork, st, sms, launches);
   k_coverage<<<g_instr, threads, 0, st>>>(P);

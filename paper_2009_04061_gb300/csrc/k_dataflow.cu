@@ -25,7 +25,7 @@ namespace {
 // program, 135 us for 3.3M instructions). The masks stay in registers, each
 // resource's bit added to its word by a compare per word (no indexed register
 // array), then the 9 words of each mask stored.
-__global__ void k_block_masks(Prog P) {
+__global__ void k_block_masks(Prog P, int windowed) {
   for (int b = blockIdx.x * blockDim.x + threadIdx.x; b < P.nb; b += gridDim.x * blockDim.x) {
     uint32_t dm[kWords], um[kWords];
 #pragma unroll
@@ -53,8 +53,10 @@ __global__ void k_block_masks(Prog P) {
       P.def_mask[o + w] = dm[w];
       P.uuse_mask[o + w] = um[w];
       P.touch_mask[o + w] = dm[w] | um[w];
-      P.rin[o + w] = 0u;
-      P.rout[o + w] = dm[w];
+      if (windowed) {  // its fixpoint starts from these; the other kernels write every word
+        P.rin[o + w] = 0u;
+        P.rout[o + w] = dm[w];
+      }
     }
   }
 }
@@ -398,7 +400,7 @@ __global__ void k_reaching(Prog P, int max_sweeps, int all) {
 
 void launch_dataflow(const Prog& P, const Arch& A, int max_sweeps, int schedule, const SearchFork* fork,
                      cudaStream_t st, int sms, int64_t* launches) {
-  k_block_masks<<<grid_for(P.nb, 256, sms), 256, 0, st>>>(P);
+  k_block_masks<<<(P.nb + 127) / 128, 128, 0, st>>>(P, schedule == 1 || P.reach_windowed > 0);
   ++*launches;
   const bool staged = schedule == 0 && P.reach_smem > 0;
   const int n_big = schedule == 0 ? P.reach_cls[0] : P.nf;  // functions beyond the staged kernel
