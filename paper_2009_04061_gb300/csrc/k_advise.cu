@@ -11,7 +11,7 @@
 // reads its instructions' counters and blame and its edges (contiguous, since
 // edges are ordered by use) once: sums, loop and line roll-ups, and all nine
 // optimizers' top five together, each kept by a warp in its first five lanes
-// (a candidate that beats the fifth is inserted by a ballot and a shift). The
+// (candidates that beat the fifth are inserted best first, by a ballot and a shift). The
 // function's last tile to finish merges the tiles' lists and writes its results.
 // What bounds it is the counters' and blame's 384 bytes an instruction.
 #include "gpa_internal.cuh"
@@ -38,15 +38,32 @@ __device__ __forceinline__ Cand shfl_cand(const Cand& c, int src) {
               __shfl_sync(0xffffffffu, c.use, src), __shfl_sync(0xffffffffu, c.dist, src)};
 }
 // A warp's top five, best first, in lanes 0-4 (v == 0: none): takes in every
-// lane's candidate (v == 0: none). Candidates are distinct, so the order is total.
+// lane's candidate (v == 0: none), best first, until one does not make the five
+// (in lane order a warp full of candidates cost 32 insertions). Candidates are
+// distinct, so the order is total.
 __device__ __forceinline__ void top_insert(Cand& top, const Cand& c) {
   const int lane = threadIdx.x & 31;
   const Cand fifth = shfl_cand(top, kHot - 1);
   unsigned m = __ballot_sync(0xffffffffu, c.v != 0ull && better(c, fifth));
   while (m) {
-    const Cand x = shfl_cand(c, __ffs(m) - 1);
-    m &= m - 1;
+    // the best of the lanes in m: largest v, then smallest def, then smallest use
+    unsigned best = m;
+    const uint32_t hi = (uint32_t)(c.v >> 32), lo = (uint32_t)c.v;
+    const uint32_t mh = __reduce_max_sync(0xffffffffu, (m >> lane) & 1u ? hi : 0u);
+    best &= __ballot_sync(0xffffffffu, hi == mh);
+    const uint32_t ml = __reduce_max_sync(0xffffffffu, (best >> lane) & 1u ? lo : 0u);
+    best &= __ballot_sync(0xffffffffu, lo == ml);
+    if (best & (best - 1)) {
+      const int md = __reduce_min_sync(0xffffffffu, (best >> lane) & 1u ? c.def : 0x7FFFFFFF);
+      best &= __ballot_sync(0xffffffffu, c.def == md);
+      const int mu = __reduce_min_sync(0xffffffffu, (best >> lane) & 1u ? c.use : 0x7FFFFFFF);
+      best &= __ballot_sync(0xffffffffu, c.use == mu);
+    }
+    const int src = __ffs(best) - 1;
+    m &= ~(1u << src);
+    const Cand x = shfl_cand(c, src);
     const int rank = __popc(__ballot_sync(0xffffffffu, lane < kHot && better(top, x)));
+    if (rank == kHot) break;  // the others rank below it
     const Cand up{__shfl_up_sync(0xffffffffu, top.v, 1), __shfl_up_sync(0xffffffffu, top.def, 1),
                   __shfl_up_sync(0xffffffffu, top.use, 1), __shfl_up_sync(0xffffffffu, top.dist, 1)};
     if (lane > rank) top = up;  // (lanes past the fifth hold what fell out; they never rank)

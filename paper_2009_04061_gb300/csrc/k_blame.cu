@@ -80,28 +80,43 @@ __device__ bool scan_pred(const Prog& P, const Arch& A, int j, int r, int gj, in
 // The stalled uses (instructions with dependency-class samples), appended a
 // warp at a time: a tenth of the instructions on the batched workload, so the
 // kernels that work per stalled use take them from this list with every lane
-// busy instead of striding over all instructions. One instruction a thread
-// over a grid that covers them all (the loads of many CTAs in flight); the
-// dependency-class counters are words 4-7 and 10-13 of a row, read as four
-// 16-byte pairs.
-__global__ void k_stalled_list(Prog P) {
-  static_assert(2 * GPA_EXEC_DEPENDENCY == 4 && 2 * GPA_MEMORY_DEPENDENCY == 6 && 2 * GPA_SYNC == 10 &&
-                    2 * GPA_CONSTANT_MEMORY_DEPENDENCY == 12,
-                "dependency-class words 4-7 and 10-13");
-  const int lane = threadIdx.x & 31;
-  const int j = blockIdx.x * blockDim.x + threadIdx.x;
-  bool s = false;
-  if (j < P.ni) {
-    const ulonglong2* c = reinterpret_cast<const ulonglong2*>(P.cnt + (size_t)j * kCnt);
-    const ulonglong2 a = c[2], b = c[3], d = c[5], e = c[6];
-    s = (a.x | a.y | b.x | b.y | d.x | d.y | e.x | e.y) != 0ull;
+// busy instead of striding over all instructions. With `init`, the pass also
+// starts the blame: the samples outside the dependency classes stay where they
+// were taken, the others are apportioned later. A warp takes 32 rows of 24
+// counters, 6 KB, as twelve coalesced 16-byte loads a lane (a pair is one class of
+// one row), and marks the rows with stalls in shared memory; reading the rows
+// again for the list alone took 114 us on 3.3M instructions.
+__global__ void __launch_bounds__(256) k_stalled_list(Prog P, int init) {
+  __shared__ int s_row[8][32];
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  const int x0 = (blockIdx.x * 8 + warp) * 32;
+  if (x0 >= P.ni) return;
+  s_row[warp][lane] = 0;
+  __syncwarp();
+  const ulonglong2* c = reinterpret_cast<const ulonglong2*>(P.cnt + (size_t)x0 * kCnt);
+  ulonglong2* b = reinterpret_cast<ulonglong2*>(P.blame + (size_t)x0 * kCnt);
+  const int pairs = min(32, P.ni - x0) * (kCnt / 2);
+#pragma unroll
+  for (int i = 0; i < kCnt / 2; ++i) {
+    const int p = i * 32 + lane;
+    if (p < pairs) {
+      const ulonglong2 v = c[p];
+      const int row = p / (kCnt / 2), cls = p - row * (kCnt / 2);
+      const bool dep = cls == GPA_EXEC_DEPENDENCY || cls == GPA_MEMORY_DEPENDENCY || cls == GPA_SYNC ||
+                       cls == GPA_CONSTANT_MEMORY_DEPENDENCY;
+      if (dep && (v.x | v.y)) s_row[warp][row] = 1;
+      if (init) b[p] = dep ? make_ulonglong2(0ull, 0ull) : v;
+    }
   }
+  if (init && x0 + lane < P.ni) P.head[x0 + lane] = -1;
+  __syncwarp();
+  const bool s = s_row[warp][lane];
   const unsigned m = __ballot_sync(0xffffffffu, s);
   if (!m) return;
   unsigned long long base = 0;
   if (lane == 0) base = atomicAdd(&P.stats[SS_SUSE_N], (unsigned long long)__popc(m));
   base = __shfl_sync(0xffffffffu, base, 0);
-  if (s) P.suse[base + __popc(m & ((1u << lane) - 1u))] = j;
+  if (s) P.suse[base + __popc(m & ((1u << lane) - 1u))] = x0 + lane;
 }
 
 // Four threads per stalled use (from the stalled-use list), each taking every
@@ -214,16 +229,6 @@ __global__ void k_search_local(Prog P, Arch A) {
 }
 
 // ---------------------------------------------------------------- merge and apportion
-__global__ void k_blame_init(Prog P) {
-  const int64_t n = (int64_t)P.ni * kCnt;
-  for (int64_t t = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; t < n; t += (int64_t)gridDim.x * blockDim.x) {
-    const int c = (int)(t % kCnt) >> 1;
-    const bool dep = c == GPA_EXEC_DEPENDENCY || c == GPA_MEMORY_DEPENDENCY || c == GPA_SYNC ||
-                     c == GPA_CONSTANT_MEMORY_DEPENDENCY;
-    P.blame[t] = dep ? 0ull : P.cnt[t];
-  }
-}
-
 // (The lanes of a warp hold neighbouring uses, whose sources are mostly
 // different instructions: partitioning them by address first cost more than the
 // few atomics it saved.)
@@ -467,12 +472,9 @@ void launch_coverage(const Prog& P, const Arch& A, const SearchArena* tiers, con
                      int sms, int64_t* launches) {
   const int threads = 128;
   const int g_instr = grid_for(P.ni, threads, sms);
-  // The per-use kernels take the stalled-use list (its length is known on the
-  // device only): enough CTAs for every SM to hold as many warps as their
-  // registers allow, each thread taking about one use on the batched workload.
-  const int g_use = std::max(1, std::min(grid_for(P.ni, threads, sms) * 4, (P.ni + threads - 1) / threads));
-  k_stalled_list<<<std::max(1, (P.ni + 255) / 256), 256, 0, st>>>(P);
-  k_search_local<<<g_use * 2, threads, 0, st>>>(P, A);
+  const int g_local = std::max(1, std::min(sms * 64, (int)(((int64_t)P.ni * kLocalLanes + threads - 1) / threads)));
+  k_stalled_list<<<(P.ni + 255) / 256, 256, 0, st>>>(P, 0);
+  k_search_local<<<g_local, threads, 0, st>>>(P, A);
   *launches += 2;
   launch_search(P, A, tiers, fork, st, sms, launches);
   k_coverage<<<g_instr, threads, 0, st>>>(P);
@@ -487,11 +489,10 @@ void launch_blame(const Prog& P, const Arch& A, const SearchArena* tiers, const 
   // device only): enough CTAs for every SM to hold as many warps as their
   // registers allow, each thread taking about one use on the batched workload.
   const int g_use = std::max(1, std::min(grid_for(P.ni, threads, sms) * 4, (P.ni + threads - 1) / threads));
-  cudaMemsetAsync(P.head, 0xFF, sizeof(int32_t) * (size_t)P.ni, st);
-  k_blame_init<<<grid_for((int64_t)P.ni * kCnt, 256, sms), 256, 0, st>>>(P);
-  k_stalled_list<<<std::max(1, (P.ni + 255) / 256), 256, 0, st>>>(P);
-  k_search_local<<<g_use, threads, 0, st>>>(P, A);
-  *launches += 3;
+  const int g_local = std::max(1, std::min(sms * 64, (int)(((int64_t)P.ni * kLocalLanes + threads - 1) / threads)));
+  k_stalled_list<<<(P.ni + 255) / 256, 256, 0, st>>>(P, 1);
+  k_search_local<<<g_local, threads, 0, st>>>(P, A);
+  *launches += 2;
   launch_search(P, A, tiers, fork, st, sms, launches);
   k_merge_count<<<g_instr, threads, 0, st>>>(P, max_src);
   k_merge_big<<<sms, 32, 0, st>>>(P, max_src);
