@@ -176,8 +176,10 @@ struct Prog {
   int2* tasks;                    // n_use
   int32_t* queue[8];
   int32_t class_limit[kClasses];  // searches a class takes in a step; the rest go to the global-memory warps
-  uint32_t* tier_hint;            // n_use: the queue known to hold the entry's search (0: none);
-                                  // kept across steps (a search's size depends only on the program)
+  // n_use each: the queue known to hold the entry's search (0: none), kept
+  // across steps (a search's size depends only on the program); [1] of the
+  // diagnostics' searches, which have no latency bound.
+  uint8_t* tier_hint[2];
   int64_t queue_cap;
   int32_t* edge_cnt;              // ni + 1 (exclusive scan in place -> offsets)
   int32_t* big_use;               // ni: uses with more than kMaxSrc sources (SS_BIG_N of them)
@@ -282,13 +284,17 @@ __device__ __forceinline__ bool keeps_any(const Prog& P, const Arch& A, int j, i
          ((c[2 * GPA_CONSTANT_MEMORY_DEPENDENCY] | c[2 * GPA_CONSTANT_MEMORY_DEPENDENCY + 1]) &&
           opcode_keeps(A, GPA_CONSTANT_MEMORY_DEPENDENCY, op));
 }
-// One unpruned edge for the export (GPA_ERR_CAPACITY if the buffer is full).
+// Later steps queue entry e's search for (at least) the queue `hint`. (An entry's
+// search runs in one place at a time.)
+__device__ __forceinline__ void raise_hint(const Prog& P, int e, uint32_t hint) {
+  uint8_t* h = P.tier_hint[P.diag ? 1 : 0] + e;
+  if (*h < hint) *h = (uint8_t)hint;
+}
+// One unpruned edge for the export (counted only when the buffer is full: the
+// host makes it larger and runs the export again).
 __device__ __forceinline__ void xemit(const Prog& P, int j, int i, int r, int dmin, int K, int dlong, bool dom) {
   const unsigned long long k = atomicAdd(&P.stats[SS_XN], 1ull);
-  if (k >= (unsigned long long)P.xcap) {
-    atomicOr(&P.stats[SS_STATUS], (unsigned long long)ST_CAPACITY);
-    return;
-  }
+  if (k >= (unsigned long long)P.xcap) return;
   P.xedges[2 * k] = make_int4(j, i, r, dmin);
   P.xedges[2 * k + 1] = make_int4(K, dlong, dom ? 1 : 0, 0);
 }
@@ -339,6 +345,13 @@ __device__ __forceinline__ void emit_raw(const Prog& P, const Arch& A, int j, in
 
 // ---------------------------------------------------------------- launchers
 int grid_for(int64_t n, int threads, int sms);
+// The exported edges, ordered (launch_order_export): arrays of n entries.
+struct ExportOut {
+  int32_t *use, *def, *res, *dmin, *back, *dlong;
+  uint8_t* dom;
+};
+void launch_order_export(const int4* x, int64_t n, int ni, int32_t* off, int32_t* cursor, int32_t* ids,
+                         const ExportOut& out, int32_t* scan_tmp, cudaStream_t st, int sms, int64_t* launches);
 void launch_build_layout(const Prog& P, cudaStream_t st, int sms, int64_t* launches);
 void launch_store_u64(unsigned long long* p, unsigned long long v, cudaStream_t st, int64_t* launches);
 void launch_build_preds(const Prog& P, int n_succ, int32_t* pred_off, int32_t* cursor, int32_t* tmp, cudaStream_t st,

@@ -202,7 +202,7 @@ __global__ void k_search_local(Prog P, Arch A) {
       if (P.diag) cov_add(P, e, n_all, n_kept);  // the in-block part; the search adds the rest
       // A search known to outgrow the first tier goes straight to the queue
       // that held it before (see Prog::queue).
-      const uint32_t hint = P.tier_hint[e];
+      const uint32_t hint = P.tier_hint[P.diag ? 1 : 0][e];
       P.tasks[e] = make_int2(j, r | ((int)S << 9) | (blocked ? 1 << 25 : 0));
       int slot = SS_QUEUE_N, q = 0;
       bool top = false, placed = false;
@@ -466,7 +466,48 @@ __global__ void k_coverage(Prog P) {
   }
 }
 
+// Ordering the export by (use, resource, def): edges counted per use, scanned,
+// dropped into their use's bucket, and each edge's rank within its bucket taken
+// by comparing it with the others there (a use has a handful).
+__global__ void k_export_count(const int4* x, int64_t n, int32_t* cnt) {
+  for (int64_t k = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; k < n; k += (int64_t)gridDim.x * blockDim.x)
+    atomicAdd(&cnt[x[2 * k].x], 1);
+}
+__global__ void k_export_bucket(const int4* x, int64_t n, const int32_t* off, int32_t* cursor, int32_t* ids) {
+  for (int64_t k = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; k < n; k += (int64_t)gridDim.x * blockDim.x) {
+    const int j = x[2 * k].x;
+    ids[off[j] + atomicAdd(&cursor[j], 1)] = (int32_t)k;
+  }
+}
+__global__ void k_export_order(const int4* x, int64_t n, const int32_t* off, const int32_t* ids, ExportOut out) {
+  for (int64_t k = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; k < n; k += (int64_t)gridDim.x * blockDim.x) {
+    const int4 a = x[2 * k], b = x[2 * k + 1];
+    const int q0 = off[a.x], q1 = off[a.x + 1];
+    int at = q0;
+    for (int q = q0; q < q1; ++q) {
+      const int4 c = x[2 * (int64_t)ids[q]];
+      at += c.z < a.z || (c.z == a.z && c.y < a.y) ? 1 : 0;
+    }
+    out.use[at] = a.x; out.def[at] = a.y; out.res[at] = a.z; out.dmin[at] = a.w;
+    out.back[at] = b.x; out.dlong[at] = b.y; out.dom[at] = (uint8_t)b.z;
+  }
+}
+
 }  // namespace
+
+// off and cursor have ni + 1 and ni entries, ids n.
+void launch_order_export(const int4* x, int64_t n, int ni, int32_t* off, int32_t* cursor, int32_t* ids,
+                         const ExportOut& out, int32_t* scan_tmp, cudaStream_t st, int sms, int64_t* launches) {
+  if (n <= 0) return;
+  cudaMemsetAsync(off, 0, sizeof(int32_t) * (size_t)(ni + 1), st);
+  cudaMemsetAsync(cursor, 0, sizeof(int32_t) * (size_t)ni, st);
+  const int g = grid_for(n, 256, sms);
+  k_export_count<<<g, 256, 0, st>>>(x, n, off);
+  scan_exclusive_inplace(off, ni, scan_tmp, st, launches);
+  k_export_bucket<<<g, 256, 0, st>>>(x, n, off, cursor, ids);
+  k_export_order<<<g, 256, 0, st>>>(x, n, off, ids, out);
+  *launches += 3;
+}
 
 void launch_coverage(const Prog& P, const Arch& A, const SearchArena* tiers, const SearchFork* fork, cudaStream_t st,
                      int sms, int64_t* launches) {

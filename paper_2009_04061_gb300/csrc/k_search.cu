@@ -962,10 +962,10 @@ __device__ void run_tasks(const G& g, const Prog& P, const Arch& A, const Arena&
     if (me != 0) continue;
     if (ok) {
       // A search that a full list sent to the warps finds its queue at once.
-      if (tier == 3 && !P.diag) {
+      if (tier == 3) {
         int c = 0;
         while (c < kClasses && class_nodes(c, a.N) < ((volatile int*)a.ctr)[0]) ++c;
-        atomicMax(&P.tier_hint[e], (unsigned)(kHintA1 + c));
+        raise_hint(P, e, (uint32_t)(kHintA1 + c));
       }
       continue;
     }
@@ -973,7 +973,7 @@ __device__ void run_tasks(const G& g, const Prog& P, const Arch& A, const Arena&
       capacity(P, a.ctr[7] > 0 ? a.ctr[7] : 1);
       continue;
     }
-    if (!P.diag) atomicMax(&P.tier_hint[e], R.next_hint);  // later steps queue it there
+    raise_hint(P, e, R.next_hint);
     const unsigned long long o = atomicAdd(&P.stats[R.next_slot], 1ull);
     if (o < cap) P.queue[R.next_q][R.next_top ? cap - 1 - o : o] = e;
     else capacity(P, 8);

@@ -522,7 +522,7 @@ __global__ void __launch_bounds__(32) k_search_lanes(Prog P, Arch A, int nodes, 
           atomicAdd(&P.stats[SS_SIZES + min(15, 31 - __clz(s.nn))], 1ull);
 #endif
           if (s.over) {
-            if (!P.diag) atomicMax(&P.tier_hint[s.e_use], (unsigned)(tier + 1));  // later steps queue it there
+            raise_hint(P, s.e_use, (uint32_t)(tier + 1));
             // first tier -> bottom of queue 1; second tier -> bottom of queue 0
             const unsigned long long o = atomicAdd(&P.stats[tier == 1 ? SS_OVF_N : SS_OVF2_N], 1ull);
             if (o < cap) P.queue[2 - tier][o] = s.e_use;

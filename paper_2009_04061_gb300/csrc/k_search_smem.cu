@@ -47,6 +47,11 @@ constexpr uint32_t F_EXP = 1u << 24, F_QUE = 1u << 25, F_NEED = 1u << 26, F_BACK
 constexpr int kSearchInf = 0x7FFFFFFF;
 
 __host__ __device__ inline int class_warps(int c) { return 16 >> c; }
+// Searches of class c that a CTA keeps for itself: rounds of the largest
+// classes, bounded so that a list does not outlast the global-memory warps.
+__device__ inline int local_list(int c) {
+  return c < 2 ? kLocalList : (c == 2 ? 8 : c == 3 ? 4 : 3) * class_warps(c);
+}
 __host__ __device__ inline int hash_slots(int n) {  // a power of two, at least 1.4 n
   int h = 16;
   while (5 * h < 7 * n) h <<= 1;
@@ -735,8 +740,7 @@ __global__ void __launch_bounds__(768, 1) k_search_smem(Prog P, Arch A, int most
       const bool top = part == 1 && class_top(c);
       const int head = part == 1 ? SS_A1_HEAD + c : SS_OVF2_HEAD;
       const unsigned long long nt = n_tasks(c);
-      // what a list holds: the largest classes at most three rounds
-      const int list = c < 2 ? kLocalList : 3 * class_warps(c);
+      const int list = local_list(c);
       while (true) {
         int e = -1;
         if (lane == 0) {
@@ -765,10 +769,10 @@ __global__ void __launch_bounds__(768, 1) k_search_smem(Prog P, Arch A, int most
         if (!over) continue;
         int next = c + 1;  // the next class that is larger than this one
         while (next < kClasses && class_nodes(next, most_nodes) == n) ++next;
-        if (!P.diag) atomicMax(&P.tier_hint[e], (unsigned)(kHintA1 + next));
+        raise_hint(P, e, (uint32_t)(kHintA1 + next));
         if (next < kClasses) {
           const int t = atomicAdd(&s_nlocal[next], 1);
-          if (t < (next < 2 ? kLocalList : 3 * class_warps(next))) { s_local[next][t] = e; continue; }
+          if (t < local_list(next)) { s_local[next][t] = e; continue; }
         }
         const bool wide = next == kClasses;  // else a full list
         const unsigned long long o = atomicAdd(&P.stats[wide ? SS_WIDE2_N : SS_OVF3_N], 1ull);

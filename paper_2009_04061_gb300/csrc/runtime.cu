@@ -23,6 +23,8 @@ struct ProgramRec {
   bool dry = false;                     // count bytes only (gpa_program_footprint)
   int4* xbuf = nullptr;                 // export buffer of gpa_export_unpruned_edges (grown on demand)
   int64_t xbuf_cap = 0, x_n = 0;
+  void* xout = nullptr;                 // the ordered export and its scratch, for xout_cap edges
+  int64_t xout_cap = 0;
   cudaStream_t build = nullptr;         // stream of the stream-ordered allocations and copies
   int64_t bytes = 0;                    // device bytes requested for the program
   cudaGraphExec_t step_exec = nullptr;  // captured step (gpa_step_capture)
@@ -96,6 +98,7 @@ gpa_status dev_copy(ProgramRec* R, const T** dst, const T* src, size_t n) {
 void free_program(ProgramRec* R) {
   if (R->step_exec) cudaGraphExecDestroy(R->step_exec);
   if (R->xbuf) cudaFree(R->xbuf);
+  if (R->xout) cudaFree(R->xout);
   if (R->launch) cudaFree(R->launch);
   if (R->build) cudaStreamSynchronize(R->build);
   for (void* p : R->allocs) cudaFree(p);
@@ -555,7 +558,7 @@ static gpa_status alloc_program(const gpa_program_desc* d, ProgramRec* R, int ti
   P.queue_cap = (int64_t)d->n_use + 1;
   for (int k = 0; k < 8; ++k) TRY(dev_alloc(R, &P.queue[k], (size_t)P.queue_cap));
   TRY(dev_alloc(R, &P.tasks, (size_t)std::max<int64_t>(d->n_use, 1)));
-  TRY(dev_alloc(R, &P.tier_hint, (size_t)std::max<int64_t>(d->n_use, 1)));
+  for (int k = 0; k < 2; ++k) TRY(dev_alloc(R, &P.tier_hint[k], (size_t)std::max<int64_t>(d->n_use, 1)));
   TRY(dev_alloc(R, &P.cov_cnt, (size_t)std::max<int64_t>(d->n_use, 1)));
   P.diag = 0;
   TRY(dev_alloc(R, &P.edge_off, ni + 1));
@@ -668,7 +671,8 @@ gpa_status gpa_load_program(gpa_ctx* ctx, const gpa_program_desc* d, gpa_pid* ou
     free_program(R);
     return GPA_ERR_CUDA;
   }
-  if (cudaMemsetAsync(P.tier_hint, 0, sizeof(uint32_t) * (size_t)std::max<int64_t>(R->n_use, 1), st) != cudaSuccess) {
+  if (cudaMemsetAsync(P.tier_hint[0], 0, (size_t)std::max<int64_t>(R->n_use, 1), st) != cudaSuccess ||
+      cudaMemsetAsync(P.tier_hint[1], 0, (size_t)std::max<int64_t>(R->n_use, 1), st) != cudaSuccess) {
     free_program(R);
     return GPA_ERR_CUDA;
   }
@@ -710,6 +714,10 @@ gpa_status gpa_unload_program_async(gpa_ctx* ctx, gpa_pid pid, gpa_stream stream
   for (void* p : R->allocs)
     if (cudaFreeAsync(p, st) != cudaSuccess) s = GPA_ERR_CUDA;
   R->allocs.clear();
+  // not stream-ordered allocations (freeing them waits for the device)
+  if (R->xbuf) cudaFree(R->xbuf);
+  if (R->xout) cudaFree(R->xout);
+  if (R->launch) cudaFree(R->launch);
   delete R;
   ctx->progs.erase(pid);
   return s;
@@ -872,26 +880,70 @@ gpa_status gpa_dependency_coverage(gpa_ctx* ctx, gpa_pid pid, gpa_stream stream,
   return s;
 }
 
+// The ordered export's arrays in xout: seven columns of xout_cap int32 (the
+// last is scratch: ids, then ni + 1 offsets and ni cursors), then the bytes.
+static ExportOut export_out(const ProgramRec* R, int32_t** ids) {
+  int32_t* p = static_cast<int32_t*>(R->xout);
+  const size_t c = (size_t)R->xout_cap;
+  if (ids) *ids = p + 6 * c;
+  return ExportOut{p, p + c, p + 2 * c, p + 3 * c, p + 4 * c, p + 5 * c,
+                   reinterpret_cast<uint8_t*>(p + 7 * c + 2 * (size_t)R->P.ni + 1)};
+}
+
 gpa_status gpa_export_unpruned_edges(gpa_ctx* ctx, gpa_pid pid, gpa_stream stream, int64_t* n_edges) {
   ProgramRec* R = find(ctx, pid);
   if (!R) return GPA_ERR_NO_PROGRAM;
   if (!n_edges) return GPA_ERR_INVALID_ARG;
   cudaStream_t st = (cudaStream_t)stream;
   unsigned long long h[SS_N];
-  gpa_status s = coverage_run(ctx, R, st, 1, h);  // sizes the export
-  if (s) return s;
-  const int64_t need = (int64_t)h[SS_COV_ALL];
-  if (need > R->xbuf_cap) {
+  *n_edges = 0;
+  R->x_n = 0;
+  auto grow = [&](int64_t need) {
     if (R->xbuf) cudaFree(R->xbuf);
     R->xbuf = nullptr;
     R->xbuf_cap = 0;
-    if (cudaMalloc(&R->xbuf, sizeof(int4) * 2 * (size_t)std::max<int64_t>(need, 1)) != cudaSuccess) return GPA_ERR_OOM;
-    R->xbuf_cap = std::max<int64_t>(need, 1);
+    if (cudaMalloc(&R->xbuf, sizeof(int4) * 2 * (size_t)need) != cudaSuccess) {
+      cudaGetLastError();
+      R->xbuf = nullptr;
+      return false;
+    }
+    R->xbuf_cap = need;
+    return true;
+  };
+  // A first buffer of an edge per use entry (32 MB at most) holds most exports;
+  // the run counts every edge, so a buffer that proves too small (or could not be
+  // had) is made to measure and the run repeated. The buffer is kept.
+  if (!R->xbuf) grow(std::min<int64_t>(std::max(R->n_use, 1), (int64_t)1 << 20));
+  gpa_status s = coverage_run(ctx, R, st, 2, h);
+  if (s) return s;
+  if ((int64_t)h[SS_XN] > R->xbuf_cap) {
+    if (!grow((int64_t)h[SS_XN])) return GPA_ERR_OOM;
+    s = coverage_run(ctx, R, st, 2, h);
+    if (s) return s;
   }
-  s = coverage_run(ctx, R, st, 2, h);
-  R->x_n = std::min<int64_t>((int64_t)h[SS_XN], R->xbuf_cap);
-  *n_edges = R->x_n;
-  return s;
+  const int64_t n = std::min<int64_t>((int64_t)h[SS_XN], R->xbuf_cap);
+  if (n > R->xout_cap) {
+    if (R->xout) cudaFree(R->xout);
+    R->xout = nullptr;
+    R->xout_cap = 0;
+    const size_t bytes = (size_t)n * 29 + sizeof(int32_t) * (2 * (size_t)R->P.ni + 1);
+    if (cudaMalloc(&R->xout, bytes) != cudaSuccess) {
+      cudaGetLastError();
+      R->xout = nullptr;
+      return GPA_ERR_OOM;
+    }
+    R->xout_cap = n;
+  }
+  int32_t* ids = nullptr;
+  const ExportOut out = export_out(R, &ids);
+  int32_t* off = ids + R->xout_cap;
+  launch_order_export(R->xbuf, n, R->P.ni, off, off + R->P.ni + 1, ids, out, R->scan_tmp, st, ctx->sms,
+                      &ctx->launches);
+  CK(cudaGetLastError());
+  CK(cudaStreamSynchronize(st));
+  R->x_n = n;
+  *n_edges = n;
+  return GPA_OK;
 }
 
 gpa_status gpa_get_unpruned_edges(gpa_ctx* ctx, gpa_pid pid, int32_t* use, int32_t* def, int32_t* res,
@@ -899,27 +951,14 @@ gpa_status gpa_get_unpruned_edges(gpa_ctx* ctx, gpa_pid pid, int32_t* use, int32
   ProgramRec* R = find(ctx, pid);
   if (!R) return GPA_ERR_NO_PROGRAM;
   CK(cudaStreamSynchronize((cudaStream_t)stream));
-  const int64_t n = R->x_n;
-  std::vector<int4> x(2 * (size_t)n);
-  if (n) CK(cudaMemcpy(x.data(), R->xbuf, sizeof(int4) * 2 * (size_t)n, cudaMemcpyDeviceToHost));
-  std::vector<int64_t> order(n);
-  for (int64_t k = 0; k < n; ++k) order[k] = k;
-  std::sort(order.begin(), order.end(), [&](int64_t a, int64_t b) {
-    const int4 &p = x[2 * a], &q = x[2 * b];
-    if (p.x != q.x) return p.x < q.x;
-    if (p.z != q.z) return p.z < q.z;
-    return p.y < q.y;
-  });
-  for (int64_t t = 0; t < n; ++t) {
-    const int4 a = x[2 * order[t]], b = x[2 * order[t] + 1];
-    if (use) use[t] = a.x;
-    if (def) def[t] = a.y;
-    if (res) res[t] = a.z;
-    if (dmin) dmin[t] = a.w;
-    if (back_edges) back_edges[t] = b.x;
-    if (dlong) dlong[t] = b.y;
-    if (dom) dom[t] = (uint8_t)b.z;
-  }
+  const size_t n = (size_t)R->x_n;
+  if (!n) return GPA_OK;
+  const ExportOut x = export_out(R, nullptr);
+  int32_t* const dst[6] = {use, def, res, dmin, back_edges, dlong};
+  const int32_t* const src[6] = {x.use, x.def, x.res, x.dmin, x.back, x.dlong};
+  for (int k = 0; k < 6; ++k)
+    if (dst[k]) CK(cudaMemcpy(dst[k], src[k], n * sizeof(int32_t), cudaMemcpyDeviceToHost));
+  if (dom) CK(cudaMemcpy(dom, x.dom, n, cudaMemcpyDeviceToHost));
   return GPA_OK;
 }
 
