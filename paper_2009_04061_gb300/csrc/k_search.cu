@@ -1082,7 +1082,7 @@ void launch_search(const Prog& P, const Arch& A, const SearchArena* tiers, const
     // the rest in arenas of t4_nodes, from the pool when it holds more of them
     // than the program's own.
     const int64_t pool = tiers[2].global ? (int64_t)tiers[2].warps * tiers[2].bytes : 0;
-    SearchArena own{P.t4_nodes, P.t4_src, kMaxLayers, P.t4_ctas, P.t4_bytes, P.t4_arena, nullptr};
+    SearchArena own{P.t4_nodes, P.t4_src, kMaxLayers, P.t4_arena ? P.t4_ctas : 0, P.t4_bytes, P.t4_arena, nullptr};
     if (pool / P.t4_bytes > own.warps) {
       own.warps = (int)std::min<int64_t>(pool / P.t4_bytes, std::max(sms, 1));
       own.global = tiers[2].global;

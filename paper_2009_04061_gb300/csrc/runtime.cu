@@ -35,7 +35,23 @@ struct ProgramRec {
   int4* meta = nullptr;
   int n_succ = 0, n_def = 0, n_use = 0;
   int32_t* scan_tmp = nullptr;
-  std::vector<void*> allocs;
+  void* block = nullptr;                // the program's device memory, one allocation
+  size_t zero_at = 0, zero_bytes = 0;   // its part that starts as zeros
+};
+
+// What a load asks for, gathered before anything is allocated: the arrays to
+// copy first, then those that start as zeros, then the rest. The vectors hold
+// derived arrays until they are copied.
+struct Layout {
+  struct Item {
+    void** slot;
+    const void* src;  // host array to copy, or nullptr
+    size_t bytes;
+    bool zero;
+  };
+  std::vector<Item> items;
+  std::vector<int32_t> order, minreach, tile_off, tile_func;
+  std::vector<uint8_t> natural, iflags;
 };
 
 }  // namespace
@@ -56,6 +72,8 @@ struct gpa_ctx {
   cudaStream_t copy_stream = nullptr;
   cudaStream_t capture_stream = nullptr;  // private stream for gpa_step_capture
   cudaStream_t build_stream = nullptr;    // program allocation, copies and layout builds
+  cudaMemPool_t pool = nullptr;           // programs' memory; keeps up to kPoolKeep bytes for the next one
+  char* load_stage = nullptr;             // pinned staging of a load's copies (kLoadStage bytes, on first use)
   cudaEvent_t ev_copied[2] = {nullptr, nullptr}, ev_used[2] = {nullptr, nullptr};
   gpa::SearchFork fork{};  // larger searches beside tiers 1-2
 };
@@ -69,29 +87,36 @@ constexpr size_t kStageSamples = (size_t)64 << 20;  // 64M samples (512 MB) per 
     if ((x) != cudaSuccess) return GPA_ERR_CUDA; \
   } while (0)
 
+constexpr size_t kPoolKeep = (size_t)1 << 30;   // freed program memory a context keeps
+constexpr size_t kLoadStage = (size_t)32 << 20;  // loads with at most this much to copy go through one copy
+
 template <class T>
-gpa_status dev_alloc(ProgramRec* R, T** p, size_t n) {
-  const size_t bytes = std::max<size_t>(n, 1) * sizeof(T);
-  R->bytes += (int64_t)bytes;
-  if (R->dry) {  // counting only: a pointer that is never used
-    *p = nullptr;
-    return GPA_OK;
-  }
-  void* q = nullptr;
-  if (cudaMallocAsync(&q, bytes, R->build) != cudaSuccess) return GPA_ERR_OOM;
-  R->allocs.push_back(q);
-  *p = (T*)q;
-  return GPA_OK;
+void dev_alloc(Layout& L, T** p, size_t n, bool zero = false) {
+  L.items.push_back({(void**)p, nullptr, std::max<size_t>(n, 1) * sizeof(T), zero});
 }
 template <class T>
-gpa_status dev_copy(ProgramRec* R, const T** dst, const T* src, size_t n) {
-  T* p = nullptr;
-  gpa_status s = dev_alloc(R, &p, n);
-  if (s) return s;
-  if (!R->dry && n && cudaMemcpyAsync(p, src, n * sizeof(T), cudaMemcpyHostToDevice, R->build) != cudaSuccess)
-    return GPA_ERR_CUDA;
-  *dst = p;
-  return GPA_OK;
+void dev_copy(Layout& L, const T** dst, const T* src, size_t n) {
+  if (n) L.items.push_back({(void**)dst, src, n * sizeof(T), false});
+  else dev_alloc(L, const_cast<T**>(dst), 1);
+}
+
+// Offsets of the items in the program's one allocation (256-byte aligned).
+size_t lay_out(const Layout& L, ProgramRec* R, std::vector<size_t>* at, size_t* copy_bytes) {
+  at->assign(L.items.size(), 0);
+  size_t off = 0;
+  for (int pass = 0; pass < 3; ++pass) {
+    if (pass == 1) R->zero_at = off;
+    for (size_t k = 0; k < L.items.size(); ++k) {
+      const Layout::Item& it = L.items[k];
+      if ((it.src ? 0 : it.zero ? 1 : 2) != pass) continue;
+      (*at)[k] = off;
+      off += (it.bytes + 255) & ~(size_t)255;
+    }
+    if (pass == 0) *copy_bytes = off;
+    if (pass == 1) R->zero_bytes = off - R->zero_at;
+  }
+  R->bytes = (int64_t)off;
+  return off;
 }
 
 // Frees a program whose work has finished (the callers synchronize first).
@@ -101,8 +126,76 @@ void free_program(ProgramRec* R) {
   if (R->xout) cudaFree(R->xout);
   if (R->launch) cudaFree(R->launch);
   if (R->build) cudaStreamSynchronize(R->build);
-  for (void* p : R->allocs) cudaFree(p);
+  if (R->block) cudaFree(R->block);
   delete R;
+}
+
+// Vectorised sweeps of the validation (no early exit).
+__attribute__((optimize("O3"))) bool any_above(const uint8_t* a, int64_t n, int limit) {
+  int bad = 0;
+  for (int64_t i = 0; i < n; ++i) bad |= a[i] > limit;
+  return bad;
+}
+__attribute__((optimize("O3"))) bool any_above(const uint16_t* a, int64_t n, int limit) {
+  int bad = 0;
+  for (int64_t i = 0; i < n; ++i) bad |= a[i] > limit;
+  return bad;
+}
+__attribute__((optimize("O3"))) bool any_outside(const int32_t* a, int64_t n, int32_t limit) {  // 0 <= a < limit
+  int bad = 0;
+  for (int64_t i = 0; i < n; ++i) bad |= (uint32_t)a[i] >= (uint32_t)limit;
+  return bad;
+}
+__attribute__((optimize("O3"))) bool bad_defs(const uint16_t* a, int64_t n) {
+  int bad = 0;
+  for (int64_t i = 0; i < n; ++i) {
+    const int r = a[i] & 0x1FF, kind = a[i] >> 12;
+    bad |= (r >= kNumRes) | ((a[i] & 0x0E00) != 0) | (kind > 2) | ((kind != 0) & (r < kBarBase));
+  }
+  return bad;
+}
+__attribute__((optimize("O3"))) bool not_ascending(const int32_t* a, int64_t n, int least_step) {
+  int bad = 0;
+  for (int64_t i = 0; i < n; ++i) bad |= (int64_t)a[i + 1] - a[i] < least_step;
+  return bad;
+}
+// Entries of one list that name the same resource `step` apart: apart[e] becomes
+// nonzero once a list starts among the entries e + 1 .. e + step.
+__attribute__((optimize("O3"))) bool repeats_at(const uint16_t* a, const uint8_t* first, uint8_t* apart, int64_t n,
+                                                int step) {
+  uint16_t bad = 0;
+  for (int64_t e = 0; e + step < n; ++e) {
+    const uint8_t s = (uint8_t)(apart[e] | first[e + step]);
+    apart[e] = s;
+    bad |= (uint16_t)((((a[e] ^ a[e + step]) & 0x1FF) == 0) & (s == 0));
+  }
+  return bad;
+}
+// A resource named twice in one of n lists (CSR: off, a). The lists are short and
+// of unpredictable length, so entries are compared with their neighbours in
+// vectorised sweeps, one per distance (list by list it was three quarters of the
+// validation); a list longer than 16 is marked in a bitmap.
+bool any_repeats(const int32_t* off, const uint16_t* a, int n) {
+  int most = 0;
+  for (int x = 0; x < n; ++x) most = std::max(most, off[x + 1] - off[x]);
+  if (most < 2) return false;
+  const int64_t m = off[n];
+  std::vector<uint8_t> first((size_t)m + 1, 0), apart((size_t)m, 0);
+  for (int x = 0; x < n; ++x) first[off[x]] = 1;  // (an empty list marks the next one's start again)
+  for (int step = 1; step < std::min(most, 16); ++step)
+    if (repeats_at(a, first.data(), apart.data(), m, step)) return true;
+  if (most <= 16) return false;
+  for (int x = 0; x < n; ++x) {
+    const int k = off[x + 1] - off[x];
+    if (k <= 16) continue;
+    uint32_t seen[16] = {};
+    for (int i = 0; i < k; ++i) {
+      const unsigned r = a[off[x] + i] & 0x1FFu;
+      if (seen[r >> 5] >> (r & 31) & 1u) return true;
+      seen[r >> 5] |= 1u << (r & 31);
+    }
+  }
+  return false;
 }
 
 ProgramRec* find(gpa_ctx* ctx, gpa_pid pid) {
@@ -134,10 +227,7 @@ gpa_status validate(const gpa_program_desc* d, const Arch& A) {
     if (c && (x < d->call_site[c - 1] || (x >= 0 && x == d->call_site[c - 1]))) return GPA_ERR_INVALID_PROGRAM;
   }
   auto mono = [](const int32_t* a, int n, int last, bool strict) {
-    if (a[0] != 0 || a[n] != last) return false;
-    for (int i = 0; i < n; ++i)
-      if (strict ? a[i + 1] <= a[i] : a[i + 1] < a[i]) return false;
-    return true;
+    return a[0] == 0 && a[n] == last && !not_ascending(a, n, strict ? 1 : 0);
   };
   if (!mono(d->func_instr_off, nf, ni, true) || !mono(d->func_block_off, nf, nb, true) ||
       !mono(d->func_loop_off, nf, nl, false) || !mono(d->block_instr_off, nb, ni, true) ||
@@ -153,25 +243,10 @@ gpa_status validate(const gpa_program_desc* d, const Arch& A) {
     for (int b = d->func_block_off[f]; b < d->func_block_off[f + 1]; ++b) bfunc[b] = f;
     for (int l = d->func_loop_off[f]; l < d->func_loop_off[f + 1]; ++l) lfunc[l] = f;
   }
-  for (int x = 0; x < ni; ++x) {
-    if (d->opclass[x] >= A.n_op || d->guard[x] > 14 || d->line[x] < 0 || d->line[x] >= d->n_lines)
-      return GPA_ERR_INVALID_PROGRAM;
-    uint32_t seen[kWords];
-    std::memset(seen, 0, sizeof seen);
-    for (int e = d->def_off[x]; e < d->def_off[x + 1]; ++e) {
-      const int r = d->def_res[e] & 0x1FF, kind = (d->def_res[e] >> 12) & 0xF;
-      if (r >= kNumRes || (d->def_res[e] & 0x0E00) || kind > 2 || (kind && r < kBarBase)) return GPA_ERR_INVALID_PROGRAM;
-      if (seen[r >> 5] >> (r & 31) & 1) return GPA_ERR_INVALID_PROGRAM;
-      seen[r >> 5] |= 1u << (r & 31);
-    }
-    std::memset(seen, 0, sizeof seen);
-    for (int e = d->use_off[x]; e < d->use_off[x + 1]; ++e) {
-      const int r = d->use_res[e];
-      if (r >= kNumRes) return GPA_ERR_INVALID_PROGRAM;
-      if (seen[r >> 5] >> (r & 31) & 1) return GPA_ERR_INVALID_PROGRAM;
-      seen[r >> 5] |= 1u << (r & 31);
-    }
-  }
+  if (any_above(d->opclass, ni, A.n_op - 1) || any_above(d->guard, ni, 14) || any_outside(d->line, ni, d->n_lines) ||
+      bad_defs(d->def_res, d->n_def) || any_above(d->use_res, d->n_use, kNumRes - 1))
+    return GPA_ERR_INVALID_PROGRAM;
+  if (any_repeats(d->def_off, d->def_res, ni) || any_repeats(d->use_off, d->use_res, ni)) return GPA_ERR_INVALID_PROGRAM;
   for (int l = 0; l < nl; ++l) {
     const int p = d->loop_parent[l], h = d->loop_header[l];
     if (p < -1 || p >= nl || p == l || (p >= 0 && lfunc[p] != lfunc[l])) return GPA_ERR_INVALID_PROGRAM;
@@ -338,6 +413,23 @@ gpa_status gpa_create(const gpa_arch_desc* arch, const gpa_options* opts, gpa_ct
   }
   if (!s && cudaMemset(T[2].hash, 0xFF, hash_bytes) != cudaSuccess) s = GPA_ERR_CUDA;
   if (!s && cudaEventCreateWithFlags(&c->scratch_ev, cudaEventDisableTiming) != cudaSuccess) s = GPA_ERR_CUDA;
+  // Programs' memory comes from a pool of the context's own that keeps up to
+  // kPoolKeep of what unloaded programs gave back (the device's default pool
+  // returns it all at the next synchronization, so every session mapped its memory
+  // anew); gpa_destroy gives it back.
+  if (!s) {
+    cudaMemPoolProps props{};
+    props.allocType = cudaMemAllocationTypePinned;
+    props.location.type = cudaMemLocationTypeDevice;
+    props.location.id = c->device;
+    uint64_t keep = kPoolKeep;
+    if (cudaMemPoolCreate(&c->pool, &props) != cudaSuccess) {
+      cudaGetLastError();
+      c->pool = nullptr;  // (the default pool then)
+    } else if (cudaMemPoolSetAttribute(c->pool, cudaMemPoolAttrReleaseThreshold, &keep) != cudaSuccess) {
+      s = GPA_ERR_CUDA;
+    }
+  }
   if (!s && cudaStreamCreateWithFlags(&c->build_stream, cudaStreamNonBlocking) != cudaSuccess) s = GPA_ERR_CUDA;
   if (!s && cudaEventCreateWithFlags(&c->fork.fork, cudaEventDisableTiming) != cudaSuccess) s = GPA_ERR_CUDA;
   for (int k = 0; k < 3; ++k) {
@@ -348,6 +440,7 @@ gpa_status gpa_create(const gpa_arch_desc* arch, const gpa_options* opts, gpa_ct
     if (c->tier[2].global) cudaFree(c->tier[2].global);
     if (c->tier[2].hash) cudaFree(c->tier[2].hash);
     if (c->scratch_ev) cudaEventDestroy(c->scratch_ev);
+    if (c->pool) cudaMemPoolDestroy(c->pool);
     if (c->build_stream) cudaStreamDestroy(c->build_stream);
     if (c->fork.fork) cudaEventDestroy(c->fork.fork);
     for (int k = 0; k < 3; ++k) {
@@ -365,6 +458,8 @@ gpa_status gpa_destroy(gpa_ctx* ctx) {
   if (!ctx) return GPA_ERR_INVALID_ARG;
   cudaDeviceSynchronize();
   for (auto& kv : ctx->progs) free_program(kv.second);
+  if (ctx->pool) cudaMemPoolDestroy(ctx->pool);
+  if (ctx->load_stage) cudaFreeHost(ctx->load_stage);
   if (ctx->tier[2].global) cudaFree(ctx->tier[2].global);
   if (ctx->tier[2].hash) cudaFree(ctx->tier[2].hash);
   for (int k = 0; k < 2; ++k) {
@@ -385,9 +480,10 @@ gpa_status gpa_destroy(gpa_ctx* ctx) {
   return GPA_OK;
 }
 
-// Allocates (or, with R->dry, only counts) the program's device memory and
-// copies its arrays. On failure the caller frees R.
-static gpa_status alloc_program(const gpa_program_desc* d, ProgramRec* R, int tier3_nodes) {
+// Gathers the program's device arrays and derives those that are computed on
+// the host (with R->dry, only their sizes). pool_bytes: the context's search
+// arenas, which the fourth tier uses when they hold more than its own would.
+static void plan_program(const gpa_program_desc* d, ProgramRec* R, Layout& L, int tier3_nodes, int64_t pool_bytes) {
   Prog& P = R->P;
   P.nf = d->n_functions; P.ni = d->n_instr; P.nb = d->n_blocks; P.nl = d->n_loops; P.n_lines = d->n_lines;
   // Staged fixpoint: the largest per-function need within the cap (edges stay
@@ -407,12 +503,7 @@ static gpa_status alloc_program(const gpa_program_desc* d, ProgramRec* R, int ti
   }
   R->n_succ = d->n_succ; R->n_def = d->n_def; R->n_use = d->n_use;
   const size_t ni = P.ni, nb = P.nb, nl = P.nl, nf = P.nf;
-#define TRY(x)                        \
-  do {                                \
-    gpa_status t_ = (x);              \
-    if (t_) return t_;                \
-  } while (0)
-  TRY(dev_copy(R, &P.func_instr_off, d->func_instr_off, nf + 1));
+  dev_copy(L, &P.func_instr_off, d->func_instr_off, nf + 1);
   {
     // The staged fixpoint takes the functions by shared memory need, largest
     // first, in four launches by size class (kReachClassCap): class c holds the
@@ -420,10 +511,11 @@ static gpa_status alloc_program(const gpa_program_desc* d, ProgramRec* R, int ti
     // largest of them. Functions beyond cap[0] are left to the windowed kernel.
     std::vector<int64_t> need(nf);
     for (size_t f = 0; f < nf; ++f) need[f] = reach_need((int)f);
-    std::vector<int32_t> order(nf);
+    std::vector<int32_t>& order = L.order;
+    order.resize(nf);
     for (size_t f = 0; f < nf; ++f) order[f] = (int32_t)f;
     std::stable_sort(order.begin(), order.end(), [&](int32_t a, int32_t b) { return need[a] > need[b]; });
-    TRY(dev_copy(R, &P.reach_order, order.data(), nf));
+    dev_copy(L, &P.reach_order, order.data(), nf);
     int q = 0;
     while (q < (int)nf && need[order[q]] > kReachClassCap[0]) ++q;
     for (int c = 0; c < 4; ++c) {
@@ -440,7 +532,8 @@ static gpa_status alloc_program(const gpa_program_desc* d, ProgramRec* R, int ti
     // its latches (a body block with an edge to the header) without passing the
     // header. Then every body block reaches every other one, which lets the
     // fixpoint seed a block with the definitions of its enclosing loops.
-    std::vector<uint8_t> natural(nf, 1);
+    std::vector<uint8_t>& natural = L.natural;
+    natural.assign(nf, 1);
     if (!R->dry) {  // (a footprint needs only the sizes)
       std::vector<int32_t> pcnt(nb + 1, 0), pl((size_t)d->n_succ);
       for (size_t u = 0; u < nb; ++u)
@@ -475,7 +568,7 @@ static gpa_status alloc_program(const gpa_program_desc* d, ProgramRec* R, int ti
           if (seen != body_n[l]) natural[f] = 0;
         }
     }
-    TRY(dev_copy(R, &P.func_natural, natural.data(), nf));
+    dev_copy(L, &P.func_natural, natural.data(), nf);
     P.reach_windowed = 0;
     for (int k = 0; k < P.reach_cls[0]; ++k) {
       const int f = order[k];
@@ -486,28 +579,30 @@ static gpa_status alloc_program(const gpa_program_desc* d, ProgramRec* R, int ti
     // Smallest block reachable from each block: a min fixpoint over
     // successors, swept in descending block order (forward edges point up, so
     // each sweep settles every forward path; back edges need a few more).
-    std::vector<int32_t> mr(nb);
+    std::vector<int32_t>& mr = L.minreach;
+    mr.resize(nb);
     for (size_t b = 0; b < nb; ++b) mr[b] = (int32_t)b;
-    for (bool changed = true; changed;) {
+    for (bool changed = !R->dry; changed;) {
       changed = false;
       for (size_t b = nb; b-- > 0;)
         for (int e = d->succ_off[b]; e < d->succ_off[b + 1]; ++e)
           if (mr[d->succ[e]] < mr[b]) { mr[b] = mr[d->succ[e]]; changed = true; }
     }
-    TRY(dev_copy(R, &P.block_minreach, mr.data(), nb));
+    dev_copy(L, &P.block_minreach, mr.data(), nb);
   }
-  TRY(dev_copy(R, &P.func_block_off, d->func_block_off, nf + 1));
-  TRY(dev_copy(R, &P.func_loop_off, d->func_loop_off, nf + 1));
-  TRY(dev_copy(R, &P.block_instr_off, d->block_instr_off, nb + 1));
-  TRY(dev_copy(R, &P.succ_off, d->succ_off, nb + 1));
-  TRY(dev_copy(R, &P.succ, d->succ, (size_t)d->n_succ));
-  TRY(dev_copy(R, &P.opclass, d->opclass, ni));
-  TRY(dev_copy(R, &P.guard, d->guard, ni));
+  dev_copy(L, &P.func_block_off, d->func_block_off, nf + 1);
+  dev_copy(L, &P.func_loop_off, d->func_loop_off, nf + 1);
+  dev_copy(L, &P.block_instr_off, d->block_instr_off, nb + 1);
+  dev_copy(L, &P.succ_off, d->succ_off, nb + 1);
+  dev_copy(L, &P.succ, d->succ, (size_t)d->n_succ);
+  dev_copy(L, &P.opclass, d->opclass, ni);
+  dev_copy(L, &P.guard, d->guard, ni);
   {
     // Instruction flags on the device: bit 0 math-library code (the caller's
     // bit 0), bit 1 call site, bit 2 in a device function (a function some call
     // site calls): Function Inlining matches bits 1-2.
-    std::vector<uint8_t> fl(ni);
+    std::vector<uint8_t>& fl = L.iflags;
+    fl.resize(ni);
     std::vector<char> dev(nf, 0);
     for (int c = 0; c < d->n_calls; ++c)
       if (d->call_callee[c] >= 0) dev[d->call_callee[c]] = 1;
@@ -516,94 +611,81 @@ static gpa_status alloc_program(const gpa_program_desc* d, ProgramRec* R, int ti
         fl[x] = (uint8_t)((d->iflags[x] & 1) | (dev[f] ? 4 : 0));
     for (int c = 0; c < d->n_calls; ++c)
       if (d->call_site[c] >= 0) fl[d->call_site[c]] |= 2;
-    TRY(dev_copy(R, &P.iflags, fl.data(), ni));
+    dev_copy(L, &P.iflags, fl.data(), ni);
   }
-  TRY(dev_copy(R, &P.line, d->line, ni));
-  TRY(dev_copy(R, &P.def_off, d->def_off, ni + 1));
-  TRY(dev_copy(R, &P.def_res, d->def_res, (size_t)d->n_def));
-  TRY(dev_copy(R, &P.use_off, d->use_off, ni + 1));
-  TRY(dev_copy(R, &P.use_res, d->use_res, (size_t)d->n_use));
-  TRY(dev_copy(R, &P.block_loop, d->block_loop, nb));
-  TRY(dev_copy(R, &P.loop_parent, d->loop_parent, nl));
-  TRY(dev_copy(R, &P.loop_header, d->loop_header, nl));
-  int32_t *pred_off = nullptr, *pred = nullptr, *cursor = nullptr, *ldepth = nullptr, *iblock = nullptr,
-          *bfunc = nullptr;
-  TRY(dev_alloc(R, &pred_off, nb + 1));
-  TRY(dev_alloc(R, &pred, (size_t)d->n_succ));
-  TRY(dev_alloc(R, &cursor, nb));
-  TRY(dev_alloc(R, &ldepth, nl));
-  TRY(dev_alloc(R, &iblock, ni));
-  TRY(dev_alloc(R, &bfunc, nb));
-  int32_t* ev_off = nullptr;
-  uint32_t* events = nullptr;
-  TRY(dev_alloc(R, &ev_off, nb * kEvBuckets + 1));
-  TRY(dev_alloc(R, &events, (size_t)d->n_def + (size_t)d->n_use));
-  P.ev_off = ev_off; P.events = events;
-  TRY(dev_alloc(R, &P.res_maxlat, 2 * nf * kNumRes));
-  P.res_guards = reinterpret_cast<uint32_t*>(P.res_maxlat) + nf * kNumRes;
-  P.pred_off = pred_off; P.pred = pred; P.loop_depth = ldepth; P.instr_block = iblock; P.block_func = bfunc;
-  TRY(dev_alloc(R, &R->scan_tmp, scan_tmp_ints((int)std::max(ni, nb * kEvBuckets) + 1)));
-  TRY(dev_alloc(R, &P.cnt, ni * kCnt));
-  TRY(dev_alloc(R, &P.stats, (size_t)SS_N));
-  TRY(dev_alloc(R, &P.def_mask, nb * kWords));
-  TRY(dev_alloc(R, &P.touch_mask, nb * kWords));
-  TRY(dev_alloc(R, &R->meta, 2 * nb));
-  P.block_meta = R->meta;
-  TRY(dev_alloc(R, &P.uuse_mask, nb * kWords));
-  TRY(dev_alloc(R, &P.rin, nb * kWords));
-  TRY(dev_alloc(R, &P.rout, nb * kWords));
-  TRY(dev_alloc(R, &P.head, ni));
+  dev_copy(L, &P.line, d->line, ni);
+  dev_copy(L, &P.def_off, d->def_off, ni + 1);
+  dev_copy(L, &P.def_res, d->def_res, (size_t)d->n_def);
+  dev_copy(L, &P.use_off, d->use_off, ni + 1);
+  dev_copy(L, &P.use_res, d->use_res, (size_t)d->n_use);
+  dev_copy(L, &P.block_loop, d->block_loop, nb);
+  dev_copy(L, &P.loop_parent, d->loop_parent, nl);
+  dev_copy(L, &P.loop_header, d->loop_header, nl);
+  auto alloc_const = [&](const int32_t** q, size_t n) { dev_alloc(L, const_cast<int32_t**>(q), n); };
+  alloc_const(&P.pred_off, nb + 1);
+  alloc_const(&P.pred, (size_t)d->n_succ);
+  dev_alloc(L, &R->cursor, nb);
+  alloc_const(&P.loop_depth, nl);
+  alloc_const(&P.instr_block, ni);
+  alloc_const(&P.block_func, nb);
+  alloc_const(&P.ev_off, nb * kEvBuckets + 1);
+  dev_alloc(L, &R->events, (size_t)d->n_def + (size_t)d->n_use);
+  dev_alloc(L, &P.res_maxlat, 2 * nf * kNumRes);  // and res_guards
+  dev_alloc(L, &R->scan_tmp, scan_tmp_ints((int)std::max(ni, nb * kEvBuckets) + 1));
+  dev_alloc(L, &P.cnt, ni * kCnt, true);
+  dev_alloc(L, &P.stats, (size_t)SS_N, true);
+  dev_alloc(L, &P.def_mask, nb * kWords);
+  dev_alloc(L, &P.touch_mask, nb * kWords);
+  dev_alloc(L, &R->meta, 2 * nb);
+  dev_alloc(L, &P.uuse_mask, nb * kWords);
+  dev_alloc(L, &P.rin, nb * kWords);
+  dev_alloc(L, &P.rout, nb * kWords);
+  dev_alloc(L, &P.head, ni);
   P.raw_cap = 2 * (int64_t)d->n_use + 1024;
-  TRY(dev_alloc(R, &P.raw, (size_t)P.raw_cap));
+  dev_alloc(L, &P.raw, (size_t)P.raw_cap);
   P.queue_cap = (int64_t)d->n_use + 1;
-  for (int k = 0; k < 8; ++k) TRY(dev_alloc(R, &P.queue[k], (size_t)P.queue_cap));
-  TRY(dev_alloc(R, &P.tasks, (size_t)std::max<int64_t>(d->n_use, 1)));
-  for (int k = 0; k < 2; ++k) TRY(dev_alloc(R, &P.tier_hint[k], (size_t)std::max<int64_t>(d->n_use, 1)));
-  TRY(dev_alloc(R, &P.cov_cnt, (size_t)std::max<int64_t>(d->n_use, 1)));
+  for (int k = 0; k < 8; ++k) dev_alloc(L, &P.queue[k], (size_t)P.queue_cap);
+  dev_alloc(L, &P.tasks, (size_t)std::max<int64_t>(d->n_use, 1));
+  for (int k = 0; k < 2; ++k) dev_alloc(L, &P.tier_hint[k], (size_t)std::max<int64_t>(d->n_use, 1), true);
+  dev_alloc(L, &P.cov_cnt, (size_t)std::max<int64_t>(d->n_use, 1));
   P.diag = 0;
-  TRY(dev_alloc(R, &P.edge_off, ni + 1));
-  TRY(dev_alloc(R, &P.big_use, ni));
-  TRY(dev_alloc(R, &P.suse, ni));
-  P.edge_cnt = P.edge_off;
+  dev_alloc(L, &P.edge_off, ni + 1, true);
+  dev_alloc(L, &P.big_use, ni);
+  dev_alloc(L, &P.suse, ni);
   P.edge_cap = P.raw_cap;
-  TRY(dev_alloc(R, &P.e_use, (size_t)P.edge_cap));
-  TRY(dev_alloc(R, &P.e_def, (size_t)P.edge_cap));
-  TRY(dev_alloc(R, &P.e_dmin, (size_t)P.edge_cap));
-  TRY(dev_alloc(R, &P.e_dlong, (size_t)P.edge_cap));
-  TRY(dev_alloc(R, &P.e_flags, (size_t)P.edge_cap));
-  TRY(dev_alloc(R, &P.e_share, (size_t)P.edge_cap * 8));
-  TRY(dev_alloc(R, &P.blame, ni * kCnt));
-  TRY(dev_alloc(R, &P.a_totals, nf * 4));
-  TRY(dev_alloc(R, &P.a_matched, nf * GPA_NUM_OPT));
-  TRY(dev_alloc(R, &P.a_speedup, nf * GPA_NUM_OPT));
-  TRY(dev_alloc(R, &P.a_rank, nf * GPA_NUM_OPT));
-  TRY(dev_alloc(R, &P.a_nhot, nf * GPA_NUM_OPT));
-  TRY(dev_alloc(R, &P.a_hot, nf * GPA_NUM_OPT * 5 * 6));
-  TRY(dev_alloc(R, &P.a_loop_speedup, nl));
+  dev_alloc(L, &P.e_use, (size_t)P.edge_cap);
+  dev_alloc(L, &P.e_def, (size_t)P.edge_cap);
+  dev_alloc(L, &P.e_dmin, (size_t)P.edge_cap);
+  dev_alloc(L, &P.e_dlong, (size_t)P.edge_cap);
+  dev_alloc(L, &P.e_flags, (size_t)P.edge_cap);
+  dev_alloc(L, &P.e_share, (size_t)P.edge_cap * 8);
+  dev_alloc(L, &P.blame, ni * kCnt);
+  dev_alloc(L, &P.a_totals, nf * 4);
+  dev_alloc(L, &P.a_matched, nf * GPA_NUM_OPT);
+  dev_alloc(L, &P.a_speedup, nf * GPA_NUM_OPT);
+  dev_alloc(L, &P.a_rank, nf * GPA_NUM_OPT);
+  dev_alloc(L, &P.a_nhot, nf * GPA_NUM_OPT);
+  dev_alloc(L, &P.a_hot, nf * GPA_NUM_OPT * 5 * 6);
+  dev_alloc(L, &P.a_loop_speedup, nl);
   {
-    std::vector<int32_t> off(nf + 1, 0), func;
+    std::vector<int32_t>&off = L.tile_off, &func = L.tile_func;
+    off.assign(nf + 1, 0);
     for (size_t f = 0; f < nf; ++f) {
       const int n = (d->func_instr_off[f + 1] - d->func_instr_off[f] + kAdvTile - 1) / kAdvTile;
       off[f + 1] = off[f] + n;
       func.insert(func.end(), (size_t)n, (int32_t)f);
     }
     P.adv_tiles = off[nf];
-    TRY(dev_copy(R, &P.adv_tile_off, off.data(), nf + 1));
-    TRY(dev_copy(R, &P.adv_tile_func, func.data(), func.size()));
-    TRY(dev_alloc(R, &P.adv_tops, (size_t)P.adv_tiles * GPA_NUM_OPT * 5));
+    dev_copy(L, &P.adv_tile_off, off.data(), nf + 1);
+    dev_copy(L, &P.adv_tile_func, func.data(), func.size());
+    dev_alloc(L, &P.adv_tops, (size_t)P.adv_tiles * GPA_NUM_OPT * 5);
     P.adv_zero = (int64_t)(nf * kAdvAcc + 4 * nl + 2 * (size_t)P.n_lines);
-    TRY(dev_alloc(R, &P.adv_acc, (size_t)P.adv_zero));
-    P.adv_own_active = P.adv_acc + nf * kAdvAcc;
-    P.adv_own_matched = P.adv_own_active + nl;
-    P.a_loop_active = P.adv_own_matched + nl;
-    P.a_loop_matched = P.a_loop_active + nl;
-    P.a_line_stall = P.a_loop_matched + nl;
-    P.a_line_lat = P.a_line_stall + P.n_lines;
+    dev_alloc(L, &P.adv_acc, (size_t)P.adv_zero);
   }
-  TRY(dev_alloc(R, &P.a_par_match, nf * 2));
-  TRY(dev_alloc(R, &P.a_par_speedup, nf * 2));
-  TRY(dev_alloc(R, &P.a_par_warps, nf * 4));
-  TRY(dev_alloc(R, &P.a_par_limit, nf));
+  dev_alloc(L, &P.a_par_match, nf * 2);
+  dev_alloc(L, &P.a_par_speedup, nf * 2);
+  dev_alloc(L, &P.a_par_warps, nf * 4);
+  dev_alloc(L, &P.a_par_limit, nf);
   P.launch = nullptr;
   P.sm = SmModel{};
   // Fourth search tier: room for 64 literal sets per block of the largest
@@ -620,11 +702,63 @@ static gpa_status alloc_program(const gpa_program_desc* d, ProgramRec* R, int ti
       P.t4_src = (int32_t)std::min<int64_t>(n4, 4096);
       P.t4_ctas = n4 <= ((int64_t)1 << 18) ? 16 : n4 <= ((int64_t)1 << 20) ? 8 : 4;
       P.t4_bytes = search_arena_bytes(P.t4_nodes, P.t4_src, kMaxLayers, true);
-      TRY(dev_alloc(R, &P.t4_arena, (size_t)P.t4_bytes * P.t4_ctas));
+      // arenas of its own only where the context's pool holds no more of them
+      if (pool_bytes / P.t4_bytes <= P.t4_ctas) dev_alloc(L, &P.t4_arena, (size_t)P.t4_bytes * P.t4_ctas);
     }
   }
-#undef TRY
-  R->pred_off = pred_off; R->cursor = cursor; R->ev_off = ev_off; R->events = events;
+}
+
+// Pointers into other allocations, once these have theirs.
+static void derive_pointers(ProgramRec* R) {
+  Prog& P = R->P;
+  R->pred_off = const_cast<int32_t*>(P.pred_off);
+  R->ev_off = const_cast<int32_t*>(P.ev_off);
+  P.events = R->events;
+  P.block_meta = R->meta;
+  P.res_guards = reinterpret_cast<uint32_t*>(P.res_maxlat) + (size_t)P.nf * kNumRes;
+  P.edge_cnt = P.edge_off;
+  P.adv_own_active = P.adv_acc + (size_t)P.nf * kAdvAcc;
+  P.adv_own_matched = P.adv_own_active + P.nl;
+  P.a_loop_active = P.adv_own_matched + P.nl;
+  P.a_loop_matched = P.a_loop_active + P.nl;
+  P.a_line_stall = P.a_loop_matched + P.nl;
+  P.a_line_lat = P.a_line_stall + P.n_lines;
+}
+
+static int64_t arena_pool_bytes(const gpa_ctx* ctx) { return (int64_t)ctx->tier[2].bytes * ctx->tier[2].warps; }
+
+// Allocates the program's memory and queues its copies and clears on the build
+// stream: one allocation (eighty of them, and as many pageable copies, were
+// most of a small program's load), the arrays gathered in pinned memory for one
+// copy unless they are large. On failure the caller frees R.
+static gpa_status place_program(gpa_ctx* ctx, ProgramRec* R, const Layout& L) {
+  std::vector<size_t> at;
+  size_t copy_bytes = 0;
+  const size_t total = lay_out(L, R, &at, &copy_bytes);
+  cudaStream_t st = R->build;
+  if ((ctx->pool ? cudaMallocFromPoolAsync(&R->block, total, ctx->pool, st) : cudaMallocAsync(&R->block, total, st)) !=
+      cudaSuccess) {
+    cudaGetLastError();
+    R->block = nullptr;
+    return GPA_ERR_OOM;
+  }
+  char* base = static_cast<char*>(R->block);
+  for (size_t k = 0; k < L.items.size(); ++k) *L.items[k].slot = base + at[k];
+  derive_pointers(R);
+  if (!ctx->load_stage && cudaMallocHost(&ctx->load_stage, kLoadStage) != cudaSuccess) {
+    cudaGetLastError();
+    ctx->load_stage = nullptr;  // (copied array by array then)
+  }
+  const bool staged = ctx->load_stage && copy_bytes <= kLoadStage;
+  for (size_t k = 0; k < L.items.size(); ++k) {
+    const Layout::Item& it = L.items[k];
+    if (!it.src) continue;
+    if (staged) std::memcpy(ctx->load_stage + at[k], it.src, it.bytes);
+    else if (cudaMemcpyAsync(base + at[k], it.src, it.bytes, cudaMemcpyHostToDevice, st) != cudaSuccess) return GPA_ERR_CUDA;
+  }
+  if (staged && cudaMemcpyAsync(base, ctx->load_stage, copy_bytes, cudaMemcpyHostToDevice, st) != cudaSuccess)
+    return GPA_ERR_CUDA;
+  if (cudaMemsetAsync(base + R->zero_at, 0, R->zero_bytes, st) != cudaSuccess) return GPA_ERR_CUDA;
   return GPA_OK;
 }
 
@@ -634,8 +768,11 @@ gpa_status gpa_program_footprint(gpa_ctx* ctx, const gpa_program_desc* d, int64_
   if (s) return s;
   ProgramRec R;
   R.dry = true;
-  s = alloc_program(d, &R, ctx->tier[2].nodes);
-  if (s) return s;
+  Layout L;
+  plan_program(d, &R, L, ctx->tier[2].nodes, arena_pool_bytes(ctx));
+  std::vector<size_t> at;
+  size_t copy_bytes = 0;
+  lay_out(L, &R, &at, &copy_bytes);
   *bytes = R.bytes;
   return GPA_OK;
 }
@@ -655,34 +792,22 @@ gpa_status gpa_load_program(gpa_ctx* ctx, const gpa_program_desc* d, gpa_pid* ou
   auto* R = new (std::nothrow) ProgramRec();
   if (!R) return GPA_ERR_OOM;
   R->build = ctx->build_stream;
-  s = alloc_program(d, R, ctx->tier[2].nodes);
+  Layout L;
+  plan_program(d, R, L, ctx->tier[2].nodes, arena_pool_bytes(ctx));
+  s = place_program(ctx, R, L);
   if (s) { free_program(R); return s; }
   Prog& P = R->P;
   for (int c = 0; c < kClasses; ++c) P.class_limit[c] = smem_class_limit(c, ctx->sms);
-  const size_t ni = P.ni;
-  int32_t *pred_off = R->pred_off, *cursor = R->cursor, *ev_off = R->ev_off;
-  uint32_t* events = R->events;
   // Everything of the load runs on the context's build stream, which is then
   // synchronized: other streams' work is not waited for.
   cudaStream_t st = R->build;
-  if (cudaMemsetAsync(P.cnt, 0, ni * kCnt * sizeof(unsigned long long), st) != cudaSuccess ||
-      cudaMemsetAsync(P.stats, 0, SS_N * sizeof(unsigned long long), st) != cudaSuccess ||
-      cudaMemsetAsync(P.edge_off, 0, (ni + 1) * sizeof(int32_t), st) != cudaSuccess) {
-    free_program(R);
-    return GPA_ERR_CUDA;
-  }
-  if (cudaMemsetAsync(P.tier_hint[0], 0, (size_t)std::max<int64_t>(R->n_use, 1), st) != cudaSuccess ||
-      cudaMemsetAsync(P.tier_hint[1], 0, (size_t)std::max<int64_t>(R->n_use, 1), st) != cudaSuccess) {
-    free_program(R);
-    return GPA_ERR_CUDA;
-  }
   if (P.t4_arena && cudaMemsetAsync(P.t4_arena, 0, (size_t)P.t4_bytes * P.t4_ctas, st) != cudaSuccess) {
     free_program(R);
     return GPA_ERR_CUDA;
   }
   launch_build_layout(P, st, ctx->sms, &ctx->launches);
-  launch_build_preds(P, R->n_succ, pred_off, cursor, R->scan_tmp, st, ctx->sms, &ctx->launches);
-  launch_build_events(P, ev_off, events, R->scan_tmp, st, ctx->sms, &ctx->launches);
+  launch_build_preds(P, R->n_succ, R->pred_off, R->cursor, R->scan_tmp, st, ctx->sms, &ctx->launches);
+  launch_build_events(P, R->ev_off, R->events, R->scan_tmp, st, ctx->sms, &ctx->launches);
   launch_build_meta(P, R->meta, st, ctx->sms, &ctx->launches);
   if (cudaStreamSynchronize(st) != cudaSuccess || cudaGetLastError() != cudaSuccess) {
     free_program(R);
@@ -711,9 +836,8 @@ gpa_status gpa_unload_program_async(gpa_ctx* ctx, gpa_pid pid, gpa_stream stream
   if (R->step_exec) cudaGraphExecDestroy(R->step_exec);
   R->step_exec = nullptr;
   gpa_status s = GPA_OK;
-  for (void* p : R->allocs)
-    if (cudaFreeAsync(p, st) != cudaSuccess) s = GPA_ERR_CUDA;
-  R->allocs.clear();
+  if (R->block && cudaFreeAsync(R->block, st) != cudaSuccess) s = GPA_ERR_CUDA;
+  R->block = nullptr;
   // not stream-ordered allocations (freeing them waits for the device)
   if (R->xbuf) cudaFree(R->xbuf);
   if (R->xout) cudaFree(R->xout);
