@@ -81,10 +81,10 @@ struct WArena {
                                 // fewest back edges | cut << 31; first occurrence
   uint16_t *l0, *l1, *l2;  // node lists
   uint16_t *ed;    // edges: target | back << 15
-  uint16_t *ht;    // node (or source) hash: 0xFFFF empty, 0xFFFE being filled
+  uint16_t *ht;    // node (or source) hash: 0xFFFF empty, marks while a slot is being filled
   uint16_t *on;    // per occurrence: the next of its source
-  volatile int *ctr;  // 0 nodes, 1 edges, 2 occurrences, 3 unexpanded nodes, 4 too small, 5-6 list lengths, 7 back edges
-  uint16_t *wpos;  // 32 wall positions
+  volatile int *ctr;  // 2 occurrences, 4 too small, 5 sources
+  uint16_t *wpos;  // 32 wall positions (while the graph grows: which edge a lane takes)
 };
 
 __device__ WArena carve(char* base, int n, int* ctr, uint16_t* wpos) {
@@ -112,14 +112,16 @@ __device__ __forceinline__ uint32_t mix(uint32_t k) {
   uint32_t h = (k & 0xFFFFu) * 0x9E3779B1u ^ ((k >> 16) * 0x85EBCA77u);
   return h ^ (h >> 15);
 }
-__device__ __forceinline__ void prefetch_l1(const void* p) {
-  asm volatile("prefetch.global.L1 [%0];" ::"l"(__cvta_generic_to_global(p)));
-}
-
 // One search by one warp. Returns 0 when it is done, else why its arena is too
-// small (nothing was emitted).
+// small (nothing was emitted); *nodes: the nodes met.
+// A warp that has an SM's scheduler to itself is bound by the instructions of a
+// wave, one after another, so list appends are ballots over uniform loops (the
+// counts stay in registers), a wave's edges are spread over the lanes whatever
+// node they belong to, and lanes that look for the same node let one of them
+// probe.
 __device__ int warp_search(const Prog& P, const Arch& A, const WArena& a, int j, int r, uint16_t S0, int e_use,
-                           bool blocked) {
+                           bool blocked, int* nodes) {
+  constexpr unsigned kAll = 0xFFFFFFFFu;
   const int lane = threadIdx.x & 31;
   const unsigned lt = (1u << lane) - 1u;
   volatile int* ctr = a.ctr;
@@ -127,11 +129,8 @@ __device__ int warp_search(const Prog& P, const Arch& A, const WArena& a, int j,
   const int b0 = P.instr_block[j];
   const int f = P.block_func[b0];
   const int fb = P.func_block_off[f];
-  if (P.func_block_off[f + 1] - fb > 0xFFFF) {  // its blocks need more than the arena's 16 bits
-    if (lane == 0) ctr[0] = 0;
-    __syncwarp();
-    return 1;
-  }
+  *nodes = 0;
+  if (P.func_block_off[f + 1] - fb > 0xFFFF) return 1;  // its blocks need more than the arena's 16 bits
   const size_t fr = (size_t)f * kNumRes + r;
   const int bound = P.diag ? kSearchInf : P.res_maxlat[fr];
   const uint16_t live = live_literals(P.res_guards[fr], gj);
@@ -142,70 +141,109 @@ __device__ int warp_search(const Prog& P, const Arch& A, const WArena& a, int j,
     uint32_t* h = reinterpret_cast<uint32_t*>(a.ht);
     for (uint32_t i = lane; i <= a.hmask / 2; i += 32) h[i] = 0xFFFFFFFFu;
   };
-  auto fail = [&](int why) { if (ctr[4] == 0) ctr[4] = why; };
-  // every lane reads the flag before any of them may set it again
-  auto failed = [&]() -> int {
-    __syncwarp();
-    const int x = ctr[4];
-    __syncwarp();
-    return x;
-  };
-  auto dist_of = [&](int u) { return a.dp[u] >> kIdxBits; };
+  auto dist_of = [&](int u) { return *(volatile uint32_t*)&a.dp[u] >> kIdxBits; };
   auto len_of = [&](int u) { return a.wl[u] >> 16; };
   auto wall_of = [&](int u) { return a.wl[u] & 0xFFFFu; };
   auto occ_node = [&](int o) { return (int)((a.oc[o] >> 16) & kIdxMask); };
   auto occ_pos = [&](int o) { return (int)(a.oc[o] & 0xFFFFu); };
+  // An improved distance of an expanded node, which is not queued yet.
+  auto improves = [&](bool has, int v, uint32_t nd) -> bool {
+    return has && nd < *(volatile uint32_t*)&a.dp[v] && atomicMin(&a.dp[v], nd) > nd &&
+           (*(volatile uint32_t*)&a.ef[v] & F_EXP) && !(atomicOr(&a.ef[v], F_QUE) & F_QUE);
+  };
 
+#ifdef GPA_PHASE_TIMING
+  long long t_prev = clock64();
+  auto phase = [&](int i) {  // (the second tier's row of the search profile)
+    if (lane == 0) {
+      const long long t = clock64();
+      atomicAdd(&P.stats[SS_PHASE + 6 + i], (unsigned long long)(t - t_prev));
+      t_prev = t;
+    }
+  };
+#else
+  auto phase = [](int) {};
+#endif
   clear_hash();
   if (lane == 0) {
-    ctr[0] = 1; ctr[1] = 0; ctr[2] = 0; ctr[3] = 1; ctr[4] = 0; ctr[5] = 0; ctr[6] = 0; ctr[7] = 0;
+    ctr[2] = 0; ctr[4] = 0;
     a.key[0] = (uint32_t)(b0 - fb) | ((uint32_t)S0 << 16);
     a.dp[0] = 0u; a.wl[0] = kNoWall; a.ef[0] = 0u;
     a.l0[0] = 0;
   }
   __syncwarp();
-  uint16_t* ub = a.l0;   // unexpanded nodes: ctr[3] of them
+  int nn = 1, ne = 0, nu = 1;   // nodes, edges, unexpanded nodes (all lanes hold the same)
+  bool has_back = false;
+  uint16_t* ub = a.l0;          // the unexpanded nodes
   uint16_t* uk = a.l1;
-  uint16_t* const d0 = reinterpret_cast<uint16_t*>(a.gx);  // nodes to relax from: ctr[5] of them
-  uint16_t* const d1 = d0 + a.n;
+  uint16_t* cur = reinterpret_cast<uint16_t*>(a.gx);  // nodes to relax from
+  uint16_t* nxt = cur + a.n;
 
-  // Expands the nodes of l2, 32 at a time: parallel scans, then linking. With
-  // `only`, the single node dominates everything beyond it and no def was met
-  // yet: returns true when it meets an unguarded reader before any def.
-  auto expand = [&](int cnt, bool only) -> bool {
+  bool cand = false, pass_b = false;
+  int low = 0;
+  while (true) {
+    // A wave: the unexpanded nodes within the bound (pass B: those that can lie
+    // on a path from a source within its latency; the others are dropped).
+    const bool only = nu == 1 && ctr[2] == 0 && !pass_b && !P.diag;
+    int cnt = 0, kept = 0;
+    for (int i0 = 0; i0 < nu; i0 += 32) {
+      const int i = i0 + lane;
+      const int u = i < nu ? ub[i] : 0;
+      const bool now = i < nu && (pass_b ? fb + (int)(a.key[u] & 0xFFFFu) >= low : (int)dist_of(u) <= bound);
+      const bool keep = i < nu && !now && !pass_b;
+      const unsigned mn = __ballot_sync(kAll, now), mk = __ballot_sync(kAll, keep);
+      if (now) a.l2[cnt + __popc(mn & lt)] = (uint16_t)u;
+      if (keep) uk[kept + __popc(mk & lt)] = (uint16_t)u;
+      cnt += __popc(mn);
+      kept += __popc(mk);
+    }
+    __syncwarp();
+    uint16_t* sw = ub; ub = uk; uk = sw;
+    nu = kept;
+    if (cnt == 0) {
+      if (pass_b) break;
+      // End of pass A: a source within its latency? (A source farther than the
+      // bound fails rule 3.)
+      const int no = ctr[2];
+      int lo = kSearchInf;
+      for (int o = lane; o < no; o += 32) {
+        const int u = occ_node(o);
+        const int d = (int)dist_of(u) + (int)len_of(u) - 1 - occ_pos(o);
+        if (d > bound) continue;
+        const int B = fb + (int)(a.key[u] & 0xFFFFu);
+        if (d <= A.lat[P.opclass[P.block_meta[2 * (size_t)B].x + occ_pos(o)]]) lo = min(lo, P.block_minreach[B]);
+      }
+      low = __reduce_min_sync(kAll, lo);
+      cand = low != kSearchInf;
+      if (!cand) break;
+      pass_b = true;
+      continue;
+    }
+    int nq = 0;  // nodes to relax from, in cur
     for (int c0 = 0; c0 < cnt; c0 += 32) {
+      // Expand up to 32 nodes: parallel scans ...
       const bool mine = c0 + lane < cnt;
       const int u = mine ? a.l2[c0 + lane] : 0;
       const uint32_t key = a.key[u];
       const int B = fb + (int)(key & 0xFFFFu);
       uint16_t S = (uint16_t)(key >> 16);
-      int4 pm = make_int4(0, 0, -1, -1);
-      uint32_t ro0 = 0u, ro1 = 0u;
-      bool stop = !mine, cut = false;
-      int len = 0;
+      int deg = 0, pA = 0, pB = 0;  // the first two predecessors that a def of r leaves
+      int q0 = 0;                   // (the predecessor list, for more than two)
+      bool cut = false;
+      uint32_t nd = 0;
       if (mine) {
         const int4 m0 = __ldg(&P.block_meta[2 * (size_t)B]);
-        pm = __ldg(&P.block_meta[2 * (size_t)B + 1]);
+        const int4 pm = __ldg(&P.block_meta[2 * (size_t)B + 1]);
         const uint32_t tw = __ldg(&P.touch_mask[(size_t)B * kWords + w]);
         const size_t seg = (size_t)B * kEvBuckets + ev_bucket(r);
         const int ev_beg = __ldg(&P.ev_off[seg]);
         int ev_end = __ldg(&P.ev_off[seg + 1]);
         if (!(tw & bit) || u == 0) ev_end = ev_beg;
-        if (pm.z >= 0) {
-          ro0 = P.rout[(size_t)pm.z * kWords + w];
-          prefetch_l1(&P.block_meta[2 * (size_t)pm.z]);
-          prefetch_l1(&P.touch_mask[(size_t)pm.z * kWords + w]);
-          prefetch_l1(&P.ev_off[(size_t)pm.z * kEvBuckets + ev_bucket(r)]);
-        }
-        if (pm.w >= 0) {
-          ro1 = P.rout[(size_t)pm.w * kWords + w];
-          prefetch_l1(&P.block_meta[2 * (size_t)pm.w]);
-          prefetch_l1(&P.touch_mask[(size_t)pm.w * kWords + w]);
-          prefetch_l1(&P.ev_off[(size_t)pm.w * kEvBuckets + ev_bucket(r)]);
-        }
+        const uint32_t ro0 = pm.z >= 0 ? P.rout[(size_t)pm.z * kWords + w] & bit : 0u;
+        const uint32_t ro1 = pm.w >= 0 ? P.rout[(size_t)pm.w * kWords + w] & bit : 0u;
         uint32_t wall = kNoWall;
         int last_def = -1;
-        bool any_def = false;
+        bool any_def = false, stop = false;
         for (int e0 = ev_beg; e0 < ev_end && !stop; e0 += 4) {
           uint32_t evs[4];
 #pragma unroll
@@ -221,7 +259,6 @@ __device__ int warp_search(const Prog& P, const Arch& A, const WArena& a, int j,
                 any_def = true;
                 const int o = atomicAdd((int*)&ctr[2], 1);
                 if (o < a.occs) a.oc[o] = (uint32_t)pos | ((uint32_t)u << 16) | (((ev >> 10) & 3u) << 29);
-                else fail(3);
               }
               S = add_literal(S, (int)((ev >> 12) & 0xFu));
               if (contains(S, gj)) stop = true;
@@ -231,231 +268,202 @@ __device__ int warp_search(const Prog& P, const Arch& A, const WArena& a, int j,
             }
           }
         }
-        len = u == 0 ? j - m0.x + 1 : m0.y - m0.x;
-        a.wl[u] = wall | ((uint32_t)len << 16);
-        if (stop) pm = make_int4(0, 0, -1, -1);
-      }
-      if (__any_sync(0xffffffffu, cut)) return true;
-      // Linking: the edge range from a prefix sum, then each lane finds or adds
-      // the nodes of its predecessors that a def of r leaves; a lane claims an
-      // empty slot, fills it in the same round, and lanes that met the claim look
-      // again in the next.
-      auto reaches = [&](int q) -> bool {
-        const int k = q - pm.x;
-        if (k == 0) return ro0 & bit;
-        if (k == 1) return ro1 & bit;
-        return P.rout[(size_t)__ldg(&P.pred[q]) * kWords + w] & bit;
-      };
-      int deg = 0;
-      for (int q = pm.x; q < pm.y; ++q) deg += reaches(q) ? 1 : 0;
-      int incl = deg;
-#pragma unroll
-      for (int o = 1; o < 32; o <<= 1) {
-        const int y = __shfl_up_sync(0xffffffffu, incl, o);
-        if (lane >= o) incl += y;
-      }
-      const int total = __shfl_sync(0xffffffffu, incl, 31);
-      const int maxdeg = __reduce_max_sync(0xffffffffu, deg);
-      const int ne = ctr[1];
-      if (ne + total > a.edges || maxdeg > 255) fail(2);
-      if (failed()) return false;
-      const int at = ne + incl - deg;
-      if (mine) a.ef[u] = (uint32_t)at | ((uint32_t)deg << 16) | F_EXP;
-      __syncwarp();
-      const int Sout = (int)keep_literals(S, live);
-      uint32_t nd = 0xFFFFFFFFu;
-      if (mine) {
-        const uint32_t d = dist_of(u) + (uint32_t)len;
-        if (d >= kFar) fail(1);
-        nd = (d << kIdxBits) | (uint32_t)u;
-      }
-      int qp = pm.x;
-      bool back = false;
-      for (int kk = 0; kk < maxdeg; ++kk) {
-        bool pending = kk < deg;
-        int p = -1;
-        if (pending) {
-          while (!reaches(qp)) ++qp;
-          const int k = qp - pm.x;
-          p = k == 0 ? pm.z : k == 1 ? pm.w : __ldg(&P.pred[qp]);
-          ++qp;
+        const uint32_t len = (uint32_t)(u == 0 ? j - m0.x + 1 : m0.y - m0.x);
+        a.wl[u] = wall | (len << 16);
+        nd = dist_of(u) + len;
+        if (!stop) {
+          deg = (ro0 ? 1 : 0) + (ro1 ? 1 : 0);
+          pA = ro0 ? pm.z : pm.w;
+          pB = pm.w;
+          q0 = pm.x;
+          for (int q = pm.x + 2; q < pm.y; ++q) {
+            const int p = __ldg(&P.pred[q]);
+            if (!(P.rout[(size_t)p * kWords + w] & bit)) continue;
+            if (deg == 0) pA = p;
+            if (deg == 1) pB = p;
+            ++deg;
+          }
         }
-        const uint32_t pk = (uint32_t)(p - fb) | ((uint32_t)Sout << 16);
+      }
+      __syncwarp();
+      // With `only`, the single node dominates everything beyond it: when it meets
+      // an unguarded reader before any def, every source lies beyond that reader.
+      if (__any_sync(kAll, cut)) { *nodes = nn; return 0; }
+      if (ctr[2] > a.occs) { *nodes = nn; return 3; }
+      if (__any_sync(kAll, mine && nd >= kFar)) { *nodes = nn; return 1; }
+      nd = (nd << kIdxBits) | (uint32_t)u;
+      // ... then linking. The edge ranges from a prefix sum of the degrees (two
+      // ballots, as long as none exceeds three).
+      int excl, total;
+      if (__any_sync(kAll, deg > 3)) {
+        int incl = deg;
+#pragma unroll
+        for (int o = 1; o < 32; o <<= 1) {
+          const int y = __shfl_up_sync(kAll, incl, o);
+          if (lane >= o) incl += y;
+        }
+        total = __shfl_sync(kAll, incl, 31);
+        excl = incl - deg;
+        if (__any_sync(kAll, deg > 255)) { *nodes = nn; return 2; }
+      } else {
+        const unsigned m1 = __ballot_sync(kAll, deg & 1), m2 = __ballot_sync(kAll, deg & 2);
+        excl = __popc(m1 & lt) + 2 * __popc(m2 & lt);
+        total = __popc(m1) + 2 * __popc(m2);
+      }
+      if (ne + total > a.edges) { *nodes = nn; return 2; }
+      if (mine) a.ef[u] = (uint32_t)(ne + excl) | ((uint32_t)deg << 16) | F_EXP;
+      const int Sout = (int)keep_literals(S, live);
+      __syncwarp();
+      for (int e0 = 0; e0 < total; e0 += 32) {
+        // lane i takes edge e0 + i: its node's lane and which predecessor it is
+        for (int k = 0; k < deg; ++k) {
+          const int i = excl + k - e0;
+          if (i >= 0 && i < 32) a.wpos[i] = (uint16_t)(lane | (k << 5));
+        }
+        __syncwarp();
+        const bool pend = e0 + lane < total;
+        const int mp = pend ? a.wpos[lane] : 0;
+        const int src = mp & 31, k = mp >> 5;
+        const int p0 = __shfl_sync(kAll, pA, src), p1 = __shfl_sync(kAll, pB, src);
+        const int Bu = __shfl_sync(kAll, B, src), So = __shfl_sync(kAll, Sout, src), qu = __shfl_sync(kAll, q0, src);
+        const uint32_t ndu = __shfl_sync(kAll, nd, src);
+        int p = k == 0 ? p0 : p1;
+        if (pend && k >= 2) {  // the k-th predecessor that a def of r leaves
+          int left = k;
+          for (int q = qu;; ++q) {
+            p = __ldg(&P.pred[q]);
+            if ((P.rout[(size_t)p * kWords + w] & bit) && left-- == 0) break;
+          }
+        }
+        const uint32_t pk = (uint32_t)(p - fb) | ((uint32_t)So << 16);
+        // One lane per node looked for probes the hash. A lane that finds an
+        // empty slot leaves its mark there; the one whose mark stays adds the node.
+        const unsigned pm_ = __ballot_sync(kAll, pend);
+        const unsigned peers = __match_any_sync(kAll, pk) & pm_;
+        const int lead = __ffs(peers) - 1;
+        bool act = pend && lane == lead;
         uint32_t h = mix(pk) & a.hmask;
         int v = -1;
-        for (int round = 0; round < 4 * (int)a.hmask + 64; ++round) {
-          if (!__any_sync(0xffffffffu, pending)) break;
-          if (pending) {
-            const uint32_t c = *(volatile uint16_t*)&a.ht[h];
-            if (c < 0xFFFEu) {
-              if (*(volatile uint32_t*)&a.key[c] == pk) { v = (int)c; pending = false; }
-              else h = (h + 1) & a.hmask;
-            } else if (c == 0xFFFFu) {
-              if (atomicCAS((unsigned short*)&a.ht[h], (unsigned short)0xFFFF, (unsigned short)0xFFFE) == 0xFFFF) {
-                const int nv = atomicAdd((int*)&ctr[0], 1);
-                pending = false;
-                if (nv >= a.n) {
-                  fail(1);
-                  *(volatile uint16_t*)&a.ht[h] = 0xFFFF;
-                } else {
-                  a.key[nv] = pk; a.wl[nv] = kNoWall; a.ef[nv] = 0u;
-                  a.dp[nv] = 0xFFFFFFFFu;
-                  ub[atomicAdd((int*)&ctr[3], 1)] = (uint16_t)nv;
-                  __threadfence_block();
-                  *(volatile uint16_t*)&a.ht[h] = (uint16_t)nv;
-                  v = nv;
-                }
-              }
-            }  // 0xFFFE: another lane is filling this slot
+        while (__any_sync(kAll, act)) {  // ends: the hash has more slots than there can be nodes
+          const uint32_t c = act ? *(volatile uint16_t*)&a.ht[h] : 0u;
+          const bool empty = act && c == 0xFFFFu;
+          if (act && !empty) {
+            if (a.key[c] == pk) { v = (int)c; act = false; }
+            else h = (h + 1) & a.hmask;
+          }
+          __syncwarp();  // every slot is read before any is marked
+          if (empty) *(volatile uint16_t*)&a.ht[h] = (uint16_t)(0x8000 | lane);
+          __syncwarp();
+          const bool won = empty && *(volatile uint16_t*)&a.ht[h] == (0x8000 | lane);
+          const unsigned wm = __ballot_sync(kAll, won);
+          if (wm) {
+            if (nn + __popc(wm) > a.n) { *nodes = a.n; return 1; }
+            if (won) {
+              v = nn + __popc(wm & lt);
+              a.key[v] = pk; a.wl[v] = kNoWall; a.ef[v] = 0u; a.dp[v] = 0xFFFFFFFFu;
+              ub[nu + __popc(wm & lt)] = (uint16_t)v;
+              *(volatile uint16_t*)&a.ht[h] = (uint16_t)v;
+              act = false;
+            }
+            nn += __popc(wm);
+            nu += __popc(wm);
           }
           __syncwarp();
         }
-        if (pending) fail(6);  // the round limit is a bound, not expected to be reached
-        if (kk < deg && v >= 0) {
-          back |= p >= B;
-          a.ed[at + kk] = (uint16_t)(v | (p >= B ? 0x8000 : 0));
-          if (nd < *(volatile uint32_t*)&a.dp[v] && atomicMin(&a.dp[v], nd) > nd &&
-              (*(volatile uint32_t*)&a.ef[v] & F_EXP) && !(atomicOr(&a.ef[v], F_QUE) & F_QUE))
-            d0[atomicAdd((int*)&ctr[5], 1)] = (uint16_t)v;
-        }
+        v = __shfl_sync(kAll, v, lead < 0 ? 0 : lead);
+        const bool back = pend && p >= Bu;
+        has_back |= __any_sync(kAll, back);
+        if (pend) a.ed[ne + e0 + lane] = (uint16_t)(v | (back ? 0x8000 : 0));
+        // The new edges relax their targets; an expanded one that improves is
+        // queued to carry the change on.
+        const bool q = improves(pend, v, ndu);
+        const unsigned qm = __ballot_sync(kAll, q);
+        if (q) cur[nq + __popc(qm & lt)] = (uint16_t)v;
+        nq += __popc(qm);
+        __syncwarp();
       }
-      if (back) ctr[7] = 1;
-      __syncwarp();
-      if (lane == 0) ctr[1] = ne + total;
-      if (failed()) return false;
+      ne += total;
     }
-    return false;
-  };
-
-  // Carries improved distances on from the listed expanded nodes (d0, ctr[5]).
-  auto relax = [&]() {
-    uint16_t* cur = d0;
-    uint16_t* nxt = d1;
-    int fs = ctr[5];
-    __syncwarp();
-    while (fs > 0) {
-      if (lane == 0) ctr[5] = 0;
-      __syncwarp();
-      for (int i = lane; i < fs; i += 32) {
-        const int u = cur[i];
-        const uint32_t ef = atomicAnd(&a.ef[u], ~F_QUE);
-        const uint32_t d = (*(volatile uint32_t*)&a.dp[u] >> kIdxBits) + len_of(u);
-        if (d >= kFar) { fail(1); continue; }
-        const uint32_t nd = (d << kIdxBits) | (uint32_t)u;
-        const int e0 = (int)(ef & 0xFFFFu), e1 = e0 + (int)((ef >> 16) & 0xFFu);
-        for (int e = e0; e < e1; ++e) {
-          const int v = a.ed[e] & 0x7FFF;
-          if (nd < *(volatile uint32_t*)&a.dp[v] && atomicMin(&a.dp[v], nd) > nd &&
-              (*(volatile uint32_t*)&a.ef[v] & F_EXP) && !(atomicOr(&a.ef[v], F_QUE) & F_QUE))
-            nxt[atomicAdd((int*)&ctr[5], 1)] = (uint16_t)v;
+    // Carry improved distances on over the expanded nodes' edges.
+    while (nq > 0) {
+      int nq2 = 0;
+      bool far = false;
+      for (int i0 = 0; i0 < nq; i0 += 32) {
+        const bool in = i0 + lane < nq;
+        const int u = in ? cur[i0 + lane] : 0;
+        const uint32_t ef = in ? atomicAnd(&a.ef[u], ~F_QUE) : 0u;
+        const uint32_t d = dist_of(u) + len_of(u);
+        far |= in && d >= kFar;
+        const uint32_t ndu = (d << kIdxBits) | (uint32_t)u;
+        const int deg = (int)((ef >> 16) & 0xFFu), e0 = (int)(ef & 0xFFFFu);
+        const int md = __reduce_max_sync(kAll, deg);
+        for (int k = 0; k < md; ++k) {
+          const int v = k < deg ? a.ed[e0 + k] & 0x7FFF : 0;
+          const bool q = improves(k < deg && !far, v, ndu);
+          const unsigned qm = __ballot_sync(kAll, q);
+          if (q) nxt[nq2 + __popc(qm & lt)] = (uint16_t)v;
+          nq2 += __popc(qm);
         }
       }
       __syncwarp();
-      fs = ctr[5];
-      uint16_t* sw = cur; cur = nxt; nxt = sw;
-      __syncwarp();
+      if (__any_sync(kAll, far)) { *nodes = nn; return 1; }
+      uint16_t* s2 = cur; cur = nxt; nxt = s2;
+      nq = nq2;
     }
-    if (lane == 0) ctr[5] = 0;
-    __syncwarp();
-  };
-
-  bool cand = false, pass_b = false;
-  int low = 0;
-  while (true) {
-    // A wave: the unexpanded nodes within the bound (pass B: those that can lie
-    // on a path from a source within its latency; the others are dropped).
-    const int m = ctr[3];
-    const bool only = m == 1 && ctr[2] == 0 && !pass_b && !P.diag;
-    int cnt = 0, kept = 0;
-    for (int i0 = 0; i0 < m; i0 += 32) {
-      const int i = i0 + lane;
-      const int u = i < m ? ub[i] : 0;
-      const bool now = i < m && (pass_b ? fb + (int)(a.key[u] & 0xFFFFu) >= low : (int)dist_of(u) <= bound);
-      const bool keep = i < m && !now && !pass_b;
-      const unsigned mn = __ballot_sync(0xffffffffu, now), mk = __ballot_sync(0xffffffffu, keep);
-      if (now) a.l2[cnt + __popc(mn & lt)] = (uint16_t)u;
-      if (keep) uk[kept + __popc(mk & lt)] = (uint16_t)u;
-      cnt += __popc(mn);
-      kept += __popc(mk);
-    }
-    __syncwarp();
-    uint16_t* sw = ub; ub = uk; uk = sw;
-    if (lane == 0) ctr[3] = kept;
-    __syncwarp();
-    if (cnt > 0) {
-      if (expand(cnt, only)) return 0;  // every source lies beyond one unguarded reader
-      if (const int why = failed()) return why;
-      relax();
-      if (const int why = failed()) return why;
-      continue;
-    }
-    if (pass_b) break;
-    // End of pass A: a source within its latency? (A source farther than the
-    // bound fails rule 3.)
-    const int no = ctr[2];
-    int lo = kSearchInf;
-    for (int o = lane; o < no; o += 32) {
-      const int u = occ_node(o);
-      const int d = (int)dist_of(u) + (int)len_of(u) - 1 - occ_pos(o);
-      if (d > bound) continue;
-      const int B = fb + (int)(a.key[u] & 0xFFFFu);
-      if (d <= A.lat[P.opclass[P.block_meta[2 * (size_t)B].x + occ_pos(o)]]) lo = min(lo, P.block_minreach[B]);
-    }
-    low = __reduce_min_sync(0xffffffffu, lo);
-    cand = low != kSearchInf;
-    if (!cand) break;
-    pass_b = true;
   }
+  *nodes = nn;
+  phase(0);
   if (!cand && !P.diag) return 0;
-  const int n = ctr[0], no = ctr[2];
+  const int n = nn, no = ctr[2];
 
   // Fewest back edges from j: layer by layer, forward edges within a layer,
   // back edges into the next (every node is listed once).
-  if (ctr[7]) {
+  if (has_back) {
     for (int u = lane; u < n; u += 32) a.kk[u] = u == 0 ? 0u : 0xFFFFu;
-    if (lane == 0) { a.l0[0] = 0; ctr[5] = 0; ctr[6] = 0; }
+    if (lane == 0) a.l0[0] = 0;
     __syncwarp();
-    int fs = 1;
-    uint16_t* cur = a.l0;
-    uint16_t* nxt = a.l1;
+    int fs = 1, nb = 0;
+    cur = a.l0;
+    nxt = a.l1;
     for (uint32_t k = 0; fs > 0; ++k) {
       while (fs > 0) {
-        for (int i = lane; i < fs; i += 32) {
-          const int u = cur[i];
-          const uint32_t ef = *(volatile uint32_t*)&a.ef[u];
-          const int e0 = (int)(ef & 0xFFFFu), e1 = e0 + (int)((ef >> 16) & 0xFFu);
-          for (int e = e0; e < e1; ++e) {
-            const int ed = a.ed[e], v = ed & 0x7FFF;
-            if (*(volatile uint32_t*)&a.kk[v] <= k) continue;
-            if (ed & 0x8000) {
-              if (!(atomicOr(&a.ef[v], F_BACK) & F_BACK)) a.l2[atomicAdd((int*)&ctr[6], 1)] = (uint16_t)v;
-            } else if (atomicMin(&a.kk[v], k) > k) {
-              nxt[atomicAdd((int*)&ctr[5], 1)] = (uint16_t)v;
-            }
+        int f2 = 0;
+        for (int i0 = 0; i0 < fs; i0 += 32) {
+          const bool in = i0 + lane < fs;
+          const uint32_t ef = in ? *(volatile uint32_t*)&a.ef[cur[i0 + lane]] : 0u;
+          const int deg = (int)((ef >> 16) & 0xFFu), e0 = (int)(ef & 0xFFFFu);
+          const int md = __reduce_max_sync(kAll, deg);
+          for (int q = 0; q < md; ++q) {
+            const int ed = q < deg ? a.ed[e0 + q] : 0, v = ed & 0x7FFF;
+            const bool un = q < deg && *(volatile uint32_t*)&a.kk[v] > k;
+            const bool bk = un && (ed & 0x8000) && !(atomicOr(&a.ef[v], F_BACK) & F_BACK);
+            const bool fw = un && !(ed & 0x8000) && atomicMin(&a.kk[v], k) > k;
+            const unsigned bm = __ballot_sync(kAll, bk), fm = __ballot_sync(kAll, fw);
+            if (bk) a.l2[nb + __popc(bm & lt)] = (uint16_t)v;
+            if (fw) nxt[f2 + __popc(fm & lt)] = (uint16_t)v;
+            nb += __popc(bm);
+            f2 += __popc(fm);
           }
         }
         __syncwarp();
-        fs = ctr[5];
         uint16_t* sw = cur; cur = nxt; nxt = sw;
-        __syncwarp();
-        if (lane == 0) ctr[5] = 0;
-        __syncwarp();
+        fs = f2;
       }
       // the back edges' targets that no fewer back edges reached
-      const int nb = ctr[6];
-      for (int i = lane; i < nb; i += 32) {
-        const int v = a.l2[i];
-        atomicAnd(&a.ef[v], ~F_BACK);
-        if (atomicMin(&a.kk[v], k + 1) > k + 1) cur[atomicAdd((int*)&ctr[5], 1)] = (uint16_t)v;
+      for (int i0 = 0; i0 < nb; i0 += 32) {
+        const bool in = i0 + lane < nb;
+        const int v = in ? a.l2[i0 + lane] : 0;
+        if (in) atomicAnd(&a.ef[v], ~F_BACK);
+        const bool fw = in && atomicMin(&a.kk[v], k + 1) > k + 1;
+        const unsigned fm = __ballot_sync(kAll, fw);
+        if (fw) cur[fs + __popc(fm & lt)] = (uint16_t)v;
+        fs += __popc(fm);
       }
-      __syncwarp();
-      fs = ctr[5];
-      __syncwarp();
-      if (lane == 0) { ctr[5] = 0; ctr[6] = 0; }
+      nb = 0;
       __syncwarp();
     }
   }
-  const bool has_back = ctr[7];
+  phase(1);
 
   // Sources: a hash keyed by (block, position) gives each an index; per source
   // the shortest distance with its occurrence, the fewest back edges, and its
@@ -482,7 +490,7 @@ __device__ int warp_search(const Prog& P, const Arch& A, const WArena& a, int j,
             const int nm = atomicAdd((int*)&ctr[5], 1);
             pending = false;
             if (nm >= a.srcs) {
-              fail(4);
+              ctr[4] = 4;
               *(volatile uint16_t*)&a.ht[h] = 0xFFFF;
             } else {
               a.si[nm] = id; a.sd[nm] = 0xFFFFFFFFu; a.sk[nm] = 0xFFFFu; a.sh[nm] = 0xFFFFu;
@@ -495,7 +503,7 @@ __device__ int warp_search(const Prog& P, const Arch& A, const WArena& a, int j,
       }
       __syncwarp();
     }
-    if (pending) fail(6);
+    if (pending) ctr[4] = 6;
     if (m >= 0) {
       const uint32_t d = dist_of(u) + len_of(u) - 1u - (uint32_t)occ_pos(o);
       atomicMin(&a.sd[m], (d << kIdxBits) | (uint32_t)o);
@@ -504,7 +512,9 @@ __device__ int warp_search(const Prog& P, const Arch& A, const WArena& a, int j,
     }
     __syncwarp();
   }
-  if (const int why = failed()) return why;
+  const int why = ctr[4];
+  __syncwarp();
+  if (why) return why;
   const int nsrc = ctr[5];
   auto src_instr = [&](int m) {
     return P.block_meta[2 * (size_t)(fb + (int)(a.si[m] & 0xFFFFu))].x + (int)(a.si[m] >> 16);
@@ -524,6 +534,7 @@ __device__ int warp_search(const Prog& P, const Arch& A, const WArena& a, int j,
     return 0;
   }
 
+  phase(2);
   // Rule 2. The walls that can cut a source lie on the parent chain of its
   // nearest occurrence: mark their nodes.
   __syncwarp();
@@ -564,37 +575,40 @@ __device__ int warp_search(const Prog& P, const Arch& A, const WArena& a, int j,
     if (ng == 0) break;
     const uint32_t full = ng == 32 ? 0xFFFFFFFFu : (1u << ng) - 1u;
     for (int u = lane; u < n; u += 32) a.dp[u] = u == 0 ? full : 0u;
-    if (lane == 0) { a.l0[0] = 0; ctr[5] = 0; }
+    if (lane == 0) a.l0[0] = 0;
     __syncwarp();
-    uint16_t* cur = a.l0;
-    uint16_t* nxt = a.l1;
+    cur = a.l0;
+    nxt = a.l1;
     int fs = 1;
     while (fs > 0) {
       // The whole frontier's queued flags first: bits that reach a frontier node
       // during this round queue it again.
       for (int i = lane; i < fs; i += 32) atomicAnd(&a.ef[cur[i]], ~F_QUE);
       __syncwarp();
-      for (int i = lane; i < fs; i += 32) {
-        const int u = cur[i];
+      int f2 = 0;
+      for (int i0 = 0; i0 < fs; i0 += 32) {
+        const bool in = i0 + lane < fs;
+        const int u = in ? cur[i0 + lane] : 0;
         const uint32_t g = a.gx[u];
-        const uint32_t mk = *(volatile uint32_t*)&a.dp[u] & (g ? ~(1u << (g - 1)) : 0xFFFFFFFFu);
-        if (!mk) continue;
-        const uint32_t ef = *(volatile uint32_t*)&a.ef[u];
-        const int e0 = (int)(ef & 0xFFFFu), e1 = e0 + (int)((ef >> 16) & 0xFFu);
-        for (int e = e0; e < e1; ++e) {
-          const int v = a.ed[e] & 0x7FFF;
-          if (!(mk & ~*(volatile uint32_t*)&a.dp[v])) continue;
-          const uint32_t old = atomicOr(&a.dp[v], mk);
-          if ((old | mk) != old && !(atomicOr(&a.ef[v], F_QUE) & F_QUE))
-            nxt[atomicAdd((int*)&ctr[5], 1)] = (uint16_t)v;
+        const uint32_t mk = in ? *(volatile uint32_t*)&a.dp[u] & (g ? ~(1u << (g - 1)) : 0xFFFFFFFFu) : 0u;
+        const uint32_t ef = mk ? *(volatile uint32_t*)&a.ef[u] : 0u;
+        const int deg = (int)((ef >> 16) & 0xFFu), e0 = (int)(ef & 0xFFFFu);
+        const int md = __reduce_max_sync(kAll, deg);
+        for (int k = 0; k < md; ++k) {
+          const int v = k < deg ? a.ed[e0 + k] & 0x7FFF : 0;
+          bool q = k < deg && (mk & ~*(volatile uint32_t*)&a.dp[v]);
+          if (q) {
+            const uint32_t old = atomicOr(&a.dp[v], mk);
+            q = (old | mk) != old && !(atomicOr(&a.ef[v], F_QUE) & F_QUE);
+          }
+          const unsigned qm = __ballot_sync(kAll, q);
+          if (q) nxt[f2 + __popc(qm & lt)] = (uint16_t)v;
+          f2 += __popc(qm);
         }
       }
       __syncwarp();
-      fs = ctr[5];
       uint16_t* sw = cur; cur = nxt; nxt = sw;
-      __syncwarp();
-      if (lane == 0) ctr[5] = 0;
-      __syncwarp();
+      fs = f2;
     }
     // A source survives if, for every group, one of its occurrences is reached
     // without passing that group's wall.
@@ -624,6 +638,7 @@ __device__ int warp_search(const Prog& P, const Arch& A, const WArena& a, int j,
   const bool every = P.diag == 2;  // the export keeps every source (the cut is its dom flag)
   if (alive == 0 && !every) return 0;
 
+  phase(3);
   // Longest path with exactly K back edges: one layer per back edge, each a DAG
   // of forward edges processed in Kahn's order; back edges feed the next layer.
   __syncwarp();
@@ -638,7 +653,6 @@ __device__ int warp_search(const Prog& P, const Arch& A, const WArena& a, int j,
     a.gx[u] = 0xFFFFFFFFu;
   }
   __syncwarp();
-  const int ne = ctr[1];
   for (int e = lane; e < ne; e += 32) {
     const int ed = a.ed[e];
     if (!(ed & 0x8000)) atomicAdd(&a.kk[ed], 1u);
@@ -654,33 +668,36 @@ __device__ int warp_search(const Prog& P, const Arch& A, const WArena& a, int j,
       if (in == 0u) a.l0[fs + __popc(z & lt)] = (uint16_t)u;
       fs += __popc(z);
     }
-    uint16_t* cur = a.l0;
-    uint16_t* nxt = a.l1;
-    if (lane == 0) ctr[5] = 0;
+    cur = a.l0;
+    nxt = a.l1;
     __syncwarp();
     while (fs > 0) {
-      for (int i = lane; i < fs; i += 32) {
-        const int u = cur[i];
+      int f2 = 0;
+      for (int i0 = 0; i0 < fs; i0 += 32) {
+        const bool in = i0 + lane < fs;
+        const int u = in ? cur[i0 + lane] : 0;
         const int cv = *(volatile int*)&a.dp[u];
         const int nd = cv + (int)len_of(u);
-        const uint32_t ef = a.ef[u];
-        const int e0 = (int)(ef & 0xFFFFu), e1 = e0 + (int)((ef >> 16) & 0xFFu);
-        for (int e = e0; e < e1; ++e) {
-          const int ed = a.ed[e], v = ed & 0x7FFF;
+        const uint32_t ef = in ? a.ef[u] : 0u;
+        const int deg = (int)((ef >> 16) & 0xFFu), e0 = (int)(ef & 0xFFFFu);
+        const int md = __reduce_max_sync(kAll, deg);
+        for (int k = 0; k < md; ++k) {
+          const int ed = k < deg ? a.ed[e0 + k] : 0x8000, v = ed & 0x7FFF;
+          bool q = false;
           if (ed & 0x8000) {
-            if (cv >= 0 && l < maxk) atomicMax((int*)&a.gx[v], nd);
+            if (k < deg && cv >= 0 && l < maxk) atomicMax((int*)&a.gx[v], nd);
           } else {
             if (cv >= 0) atomicMax((int*)&a.dp[v], nd);
-            if ((atomicSub(&a.kk[v], 1u << 16) >> 16) == 1u) nxt[atomicAdd((int*)&ctr[5], 1)] = (uint16_t)v;
+            q = (atomicSub(&a.kk[v], 1u << 16) >> 16) == 1u;
           }
+          const unsigned qm = __ballot_sync(kAll, q);
+          if (q) nxt[f2 + __popc(qm & lt)] = (uint16_t)v;
+          f2 += __popc(qm);
         }
       }
       __syncwarp();
-      fs = ctr[5];
       uint16_t* sw = cur; cur = nxt; nxt = sw;
-      __syncwarp();
-      if (lane == 0) ctr[5] = 0;
-      __syncwarp();
+      fs = f2;
     }
     for (int m = lane; m < nsrc; m += 32) {
       const bool cut = a.sk[m] >> 31;
@@ -706,6 +723,7 @@ __device__ int warp_search(const Prog& P, const Arch& A, const WArena& a, int j,
       __syncwarp();
     }
   }
+  phase(4);
   return 0;
 }
 
@@ -756,8 +774,9 @@ __global__ void __launch_bounds__(768, 1) k_search_smem(Prog P, Arch A, int most
         if (e < 0) break;
         const int2 task = P.tasks[e];
         const int j = task.x, r = task.y & 0x1FF;
-        const int over = warp_search(P, A, a, j, r, (uint16_t)((uint32_t)task.y >> 9), e, (task.y >> 25) & 1);
-        const unsigned long long nn = (unsigned long long)max(min(s_ctr[warp][0], n), 0);
+        int met = 0;
+        const int over = warp_search(P, A, a, j, r, (uint16_t)((uint32_t)task.y >> 9), e, (task.y >> 25) & 1, &met);
+        const unsigned long long nn = (unsigned long long)met;
         __syncwarp();
         ++runs;
         most = max(most, nn);
