@@ -419,6 +419,16 @@ void launch_build_meta(const Prog& P, int4* meta, cudaStream_t st, int sms, int6
 void launch_build_events(const Prog& P, int32_t* ev_off, uint32_t* events, int32_t* tmp, cudaStream_t st, int sms,
                          int64_t* launches);
 void launch_advise(const Prog& P, const Arch& A, cudaStream_t st, int64_t* launches);
+// Copies up to kOutItems device arrays (4-byte multiples) to memory the device
+// can write, in one launch.
+constexpr int kOutItems = 15;
+struct OutList {
+  const void* src[kOutItems];
+  void* dst[kOutItems];
+  int64_t bytes[kOutItems];
+  int n;
+};
+void launch_copy_out(const OutList& L, cudaStream_t st, int64_t* launches);
 // Exclusive scan of n int32 values in place over buf[0..n], buf[n] receives the total.
 void scan_exclusive_inplace(int32_t* buf, int n, int32_t* tmp, cudaStream_t st, int64_t* launches);
 size_t scan_tmp_ints(int n);

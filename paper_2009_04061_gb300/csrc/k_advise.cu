@@ -400,7 +400,35 @@ __global__ void __launch_bounds__(kThreads) k_advise(Prog P, Arch A) {
     P.a_loop_speedup[lp] = est(T, min(__ldcg(&P.a_loop_active[lp]), __ldcg(&P.a_loop_matched[lp])));
 }
 
+// Results out in one launch: the arrays are cut into pieces of 4 KB, a CTA per
+// piece, written straight into page-locked host memory over the host link (a
+// copy per array was fifteen, a few microseconds each: most of the advice call of
+// a small program).
+constexpr int64_t kOutPiece = 4096;
+__global__ void __launch_bounds__(128) k_copy_out(OutList L) {
+  int64_t piece = blockIdx.x;
+  int k = 0;
+  while (k < L.n - 1 && piece >= (L.bytes[k] + kOutPiece - 1) / kOutPiece) piece -= (L.bytes[k++] + kOutPiece - 1) / kOutPiece;
+  const int64_t at = piece * kOutPiece, n = min(kOutPiece, L.bytes[k] - at);
+  const char* src = static_cast<const char*>(L.src[k]) + at;
+  char* dst = static_cast<char*>(L.dst[k]) + at;
+  const bool vec = ((reinterpret_cast<uintptr_t>(src) | reinterpret_cast<uintptr_t>(dst)) & 15u) == 0;
+  const int64_t nv = vec ? n / 16 : 0;
+  for (int64_t i = threadIdx.x; i < nv; i += blockDim.x)
+    reinterpret_cast<int4*>(dst)[i] = reinterpret_cast<const int4*>(src)[i];
+  for (int64_t i = nv * 4 + threadIdx.x; i < n / 4; i += blockDim.x)
+    reinterpret_cast<int*>(dst)[i] = reinterpret_cast<const int*>(src)[i];
+}
+
 }  // namespace
+
+void launch_copy_out(const OutList& L, cudaStream_t st, int64_t* launches) {
+  int64_t pieces = 0;
+  for (int k = 0; k < L.n; ++k) pieces += (L.bytes[k] + kOutPiece - 1) / kOutPiece;
+  if (pieces == 0) return;
+  k_copy_out<<<(unsigned)pieces, 128, 0, st>>>(L);
+  ++*launches;
+}
 
 void launch_advise(const Prog& P, const Arch& A, cudaStream_t st, int64_t* launches) {
   // every counter that is added to, in one block

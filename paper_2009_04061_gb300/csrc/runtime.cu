@@ -74,6 +74,7 @@ struct gpa_ctx {
   cudaStream_t build_stream = nullptr;    // program allocation, copies and layout builds
   cudaMemPool_t pool = nullptr;           // programs' memory; keeps up to kPoolKeep bytes for the next one
   char* load_stage = nullptr;             // pinned staging of a load's copies (kLoadStage bytes, on first use)
+  char* advice_stage = nullptr;           // and of advice into pageable arrays (kAdviceStage bytes)
   cudaEvent_t ev_copied[2] = {nullptr, nullptr}, ev_used[2] = {nullptr, nullptr};
   gpa::SearchFork fork{};  // larger searches beside tiers 1-2
 };
@@ -89,6 +90,8 @@ constexpr size_t kStageSamples = (size_t)64 << 20;  // 64M samples (512 MB) per 
 
 constexpr size_t kPoolKeep = (size_t)1 << 30;   // freed program memory a context keeps
 constexpr size_t kLoadStage = (size_t)32 << 20;  // loads with at most this much to copy go through one copy
+
+constexpr size_t kAdviceStage = (size_t)4 << 20;
 
 template <class T>
 void dev_alloc(Layout& L, T** p, size_t n, bool zero = false) {
@@ -460,6 +463,7 @@ gpa_status gpa_destroy(gpa_ctx* ctx) {
   for (auto& kv : ctx->progs) free_program(kv.second);
   if (ctx->pool) cudaMemPoolDestroy(ctx->pool);
   if (ctx->load_stage) cudaFreeHost(ctx->load_stage);
+  if (ctx->advice_stage) cudaFreeHost(ctx->advice_stage);
   if (ctx->tier[2].global) cudaFree(ctx->tier[2].global);
   if (ctx->tier[2].hash) cudaFree(ctx->tier[2].hash);
   for (int k = 0; k < 2; ++k) {
@@ -1134,28 +1138,68 @@ gpa_status gpa_step_launch(gpa_ctx* ctx, gpa_pid pid, gpa_stream stream) {
   return GPA_OK;
 }
 
-static gpa_status copy_advice(ProgramRec* R, const gpa_advice* out, cudaStream_t st) {
+static gpa_status copy_advice(gpa_ctx* ctx, ProgramRec* R, const gpa_advice* out, cudaStream_t st) {
   const Prog& P = R->P;
   const size_t nf = P.nf, no = GPA_NUM_OPT;
-  auto cp = [&](void* dst, const void* src, size_t bytes) {
-    return (dst && bytes) ? cudaMemcpyAsync(dst, src, bytes, cudaMemcpyDeviceToHost, st) : cudaSuccess;
+  OutList L{};
+  void* user[kOutItems];
+  size_t total = 0;
+  auto add = [&](void* dst, const void* src, size_t bytes) {
+    if (!dst || !bytes) return;
+    L.src[L.n] = src;
+    L.bytes[L.n] = (int64_t)bytes;
+    user[L.n++] = dst;
+    total += (bytes + 15) & ~(size_t)15;
   };
-  CK(cp(out->totals, P.a_totals, nf * 4 * 8));
-  CK(cp(out->matched, P.a_matched, nf * no * 8));
-  CK(cp(out->speedup, P.a_speedup, nf * no * 8));
-  CK(cp(out->rank, P.a_rank, nf * no * 4));
-  CK(cp(out->n_hot, P.a_nhot, nf * no * 4));
-  CK(cp(out->hot, P.a_hot, nf * no * 5 * 6 * 8));
-  CK(cp(out->loop_active, P.a_loop_active, (size_t)P.nl * 8));
-  CK(cp(out->loop_matched, P.a_loop_matched, (size_t)P.nl * 8));
-  CK(cp(out->loop_speedup, P.a_loop_speedup, (size_t)P.nl * 8));
-  CK(cp(out->line_stall, P.a_line_stall, (size_t)P.n_lines * 8));
-  CK(cp(out->line_latency, P.a_line_lat, (size_t)P.n_lines * 8));
-  CK(cp(out->par_match, P.a_par_match, nf * 2 * 4));
-  CK(cp(out->par_speedup, P.a_par_speedup, nf * 2 * 8));
-  CK(cp(out->par_warps, P.a_par_warps, nf * 4 * 8));
-  CK(cp(out->par_limit, P.a_par_limit, nf * 4));
+  add(out->totals, P.a_totals, nf * 4 * 8);
+  add(out->matched, P.a_matched, nf * no * 8);
+  add(out->speedup, P.a_speedup, nf * no * 8);
+  add(out->rank, P.a_rank, nf * no * 4);
+  add(out->n_hot, P.a_nhot, nf * no * 4);
+  add(out->hot, P.a_hot, nf * no * 5 * 6 * 8);
+  add(out->loop_active, P.a_loop_active, (size_t)P.nl * 8);
+  add(out->loop_matched, P.a_loop_matched, (size_t)P.nl * 8);
+  add(out->loop_speedup, P.a_loop_speedup, (size_t)P.nl * 8);
+  add(out->line_stall, P.a_line_stall, (size_t)P.n_lines * 8);
+  add(out->line_latency, P.a_line_lat, (size_t)P.n_lines * 8);
+  add(out->par_match, P.a_par_match, nf * 2 * 4);
+  add(out->par_speedup, P.a_par_speedup, nf * 2 * 8);
+  add(out->par_warps, P.a_par_warps, nf * 4 * 8);
+  add(out->par_limit, P.a_par_limit, nf * 4);
+  // Page-locked destinations that this device can address are written by one
+  // kernel; others of up to kAdviceStage in all through page-locked staging, and
+  // larger ones array by array.
+  bool direct = true;
+  for (int k = 0; k < L.n && direct; ++k) {
+    cudaPointerAttributes at{};
+    direct = cudaPointerGetAttributes(&at, user[k]) == cudaSuccess && at.type == cudaMemoryTypeHost &&
+             at.devicePointer && (reinterpret_cast<uintptr_t>(at.devicePointer) & 3u) == 0;
+    L.dst[k] = at.devicePointer;
+  }
+  cudaGetLastError();  // a failed query is not an error here
+  bool staged = false;
+  if (!direct && total <= kAdviceStage) {
+    if (!ctx->advice_stage && cudaMallocHost(&ctx->advice_stage, kAdviceStage) != cudaSuccess) {
+      cudaGetLastError();
+      ctx->advice_stage = nullptr;
+    }
+    staged = ctx->advice_stage != nullptr;
+    size_t off = 0;
+    for (int k = 0; k < L.n && staged; ++k) {
+      L.dst[k] = ctx->advice_stage + off;
+      off += ((size_t)L.bytes[k] + 15) & ~(size_t)15;
+    }
+  }
+  if (direct || staged) {
+    launch_copy_out(L, st, &ctx->launches);
+    CK(cudaGetLastError());
+  } else {
+    for (int k = 0; k < L.n; ++k)
+      CK(cudaMemcpyAsync(user[k], L.src[k], (size_t)L.bytes[k], cudaMemcpyDeviceToHost, st));
+  }
   CK(cudaStreamSynchronize(st));
+  if (staged)
+    for (int k = 0; k < L.n; ++k) std::memcpy(user[k], L.dst[k], (size_t)L.bytes[k]);
   return GPA_OK;
 }
 
@@ -1224,7 +1268,7 @@ gpa_status gpa_advise(gpa_ctx* ctx, gpa_pid pid, const gpa_advice* out, gpa_stre
   cudaStream_t st = (cudaStream_t)stream;
   launch_advise(R->P, ctx->arch, st, &ctx->launches);
   CK(cudaGetLastError());
-  if (out) return copy_advice(R, out, st);
+  if (out) return copy_advice(ctx, R, out, st);
   return GPA_OK;
 }
 
@@ -1232,7 +1276,7 @@ gpa_status gpa_get_advice(gpa_ctx* ctx, gpa_pid pid, const gpa_advice* out, gpa_
   ProgramRec* R = find(ctx, pid);
   if (!R) return GPA_ERR_NO_PROGRAM;
   if (!out) return GPA_ERR_INVALID_ARG;
-  return copy_advice(R, out, (cudaStream_t)stream);
+  return copy_advice(ctx, R, out, (cudaStream_t)stream);
 }
 
 gpa_status gpa_sync_status(gpa_ctx* ctx, gpa_pid pid, gpa_stream stream, int64_t* info) {
