@@ -90,7 +90,11 @@ struct LaunchRec {
   long long blocks;
   int32_t threads, regs, smem, reserved;
 };
-constexpr int kAdvTile = 1024;  // instructions of an advice tile
+// Instructions of an advice tile: 1,024, or 256 for programs of fewer tiles than
+// the chip has SMs (a tile is a chain of its warps' passes: Rodinia-shaped step
+// 520 us with tiles of 1,024, 497 with 256; thousand-function step 6.63 and
+// 6.73 ms, advice over 301 functions 318 and 337 us).
+inline int adv_tile_size(int64_t n_instr, int sms) { return n_instr <= 1024ll * sms ? 256 : 1024; }
 constexpr int kAdvAcc = 14;     // per-function sums of the advice kernel, and its tiles that are done
 // A hotspot candidate of a tile.
 struct AdvCand {
@@ -193,8 +197,8 @@ struct Prog {
   unsigned long long* e_share;    // edges * 8
   int64_t edge_cap;
   unsigned long long* blame;      // ni * 24
-  // advice: tiles of at most kAdvTile instructions of one function
-  int32_t adv_tiles;
+  // advice: tiles of at most adv_tile instructions of one function
+  int32_t adv_tile, adv_tiles;
   const int32_t* adv_tile_off;    // nf + 1: first tile of each function
   const int32_t* adv_tile_func;   // adv_tiles
   AdvCand* adv_tops;              // adv_tiles * 9 * 5

@@ -5,7 +5,7 @@
 // pick each optimizer's top five hotspots (def, use, distance); with launch
 // statistics, the parallel optimizers (Eqs. 6-10).
 //
-// One CTA per tile of 1,024 instructions of one function, so that a large
+// One CTA per tile of 1,024 (or 256) instructions of one function, so that a large
 // function is spread over the chip (one CTA a function left a 20,000-instruction
 // function 880 us behind the others and a 120,000-instruction one 4.3 ms). A tile
 // reads its instructions' counters and blame and its edges (contiguous, since
@@ -208,7 +208,7 @@ __global__ void __launch_bounds__(kThreads) k_advise(Prog P, Arch A) {
   const int f = P.adv_tile_func[blockIdx.x];
   const int t0 = P.adv_tile_off[f], nt = P.adv_tile_off[f + 1] - t0;
   const int i0 = P.func_instr_off[f];
-  const int x0 = i0 + ((int)blockIdx.x - t0) * kAdvTile, x1 = min(P.func_instr_off[f + 1], x0 + kAdvTile);
+  const int x0 = i0 + ((int)blockIdx.x - t0) * P.adv_tile, x1 = min(P.func_instr_off[f + 1], x0 + P.adv_tile);
   // Edge ranges are clamped to the edge capacity (overflow is reported in the status word).
   const int64_t e0 = min((int64_t)P.edge_off[x0], P.edge_cap), e1 = min((int64_t)P.edge_off[x1], P.edge_cap);
   unsigned long long acc[kAcc];

@@ -284,9 +284,15 @@ __global__ void k_merge_big(Prog P, int max_src) {
 // Merged edges of use j (ascending def index) and Eq. 1 shares of each of its
 // dependency classes and latency flags, with arrays of capacity cap.
 __device__ void apportion_use(const Prog& P, const Arch& A, int j, int off, int c, int* mi, int* md, int* ml,
-                              uint32_t* mf, int* sel, unsigned long long* wt, unsigned __int128* rem,
-                              unsigned long long* sh) {
-  const unsigned long long* cj = P.cnt + (size_t)j * kCnt;
+                              uint32_t* mf, uint32_t* mo, unsigned long long* mc, int* sel,
+                              unsigned long long* wt, unsigned __int128* rem, unsigned long long* sh) {
+  // the eight dependency counters of j, and of each source its opcode's flags
+  // and issue count: loaded once, the sources' while the list is walked
+  static_assert(2 * GPA_EXEC_DEPENDENCY == 4 && 2 * GPA_MEMORY_DEPENDENCY == 6 && 2 * GPA_SYNC == 10 &&
+                    2 * GPA_CONSTANT_MEMORY_DEPENDENCY == 12,
+                "dependency-class words 4-7 and 10-13");
+  const ulonglong2* cj2 = reinterpret_cast<const ulonglong2*>(P.cnt + (size_t)j * kCnt);
+  const ulonglong2 cj[4] = {cj2[2], cj2[3], cj2[5], cj2[6]};
   int m = 0;
   if (c > 0) {
     for (int t = P.head[j]; t >= 0; t = P.raw[t].y) {
@@ -297,7 +303,10 @@ __device__ void apportion_use(const Prog& P, const Arch& A, int j, int off, int 
       while (q < m && mi[q] != R.x) ++q;
       if (q == m) {
         if (m >= c) continue;  // capacity already reported by the count pass
-        mi[m] = R.x; md[m] = R.z; ml[m] = dl; mf[m] = fl; ++m;
+        mi[m] = R.x; md[m] = R.z; ml[m] = dl; mf[m] = fl;
+        mo[m] = A.flags[P.opclass[R.x]];
+        mc[m] = P.cnt[(size_t)R.x * kCnt];
+        ++m;
       } else {
         md[q] = min(md[q], R.z); ml[q] = max(ml[q], dl); mf[q] |= fl;
       }
@@ -305,10 +314,14 @@ __device__ void apportion_use(const Prog& P, const Arch& A, int j, int off, int 
     // ascending def index
     for (int a = 1; a < m; ++a) {
       const int xi = mi[a], xd = md[a], xl = ml[a];
-      const uint32_t xf = mf[a];
+      const uint32_t xf = mf[a], xo = mo[a];
+      const unsigned long long xc = mc[a];
       int b = a - 1;
-      while (b >= 0 && mi[b] > xi) { mi[b + 1] = mi[b]; md[b + 1] = md[b]; ml[b + 1] = ml[b]; mf[b + 1] = mf[b]; --b; }
-      mi[b + 1] = xi; md[b + 1] = xd; ml[b + 1] = xl; mf[b + 1] = xf;
+      while (b >= 0 && mi[b] > xi) {
+        mi[b + 1] = mi[b]; md[b + 1] = md[b]; ml[b + 1] = ml[b]; mf[b + 1] = mf[b]; mo[b + 1] = mo[b]; mc[b + 1] = mc[b];
+        --b;
+      }
+      mi[b + 1] = xi; md[b + 1] = xd; ml[b + 1] = xl; mf[b + 1] = xf; mo[b + 1] = xo; mc[b + 1] = xc;
     }
     for (int t = 0; t < m; ++t) {
       const int64_t e = off + t;
@@ -319,19 +332,21 @@ __device__ void apportion_use(const Prog& P, const Arch& A, int j, int off, int 
   }
   for (int ci = 0; ci < 4; ++ci) {
     const int cls = dep_class(ci);
+    // rule 1 (opcode_keeps): the flag a source of this class carries
+    const uint32_t keeps = ci == 1 || ci == 3 ? (uint32_t)GPA_F_MEM : ci == 2 ? (uint32_t)GPA_F_SYNC : 0u;
     for (int lat = 0; lat < 2; ++lat) {
-      const unsigned long long S = cj[cls * 2 + lat];
+      const unsigned long long S = lat ? cj[ci].y : cj[ci].x;
       if (!S) continue;
       int ns = 0;
       for (int t = 0; t < m; ++t)
-        if (opcode_keeps(A, cls, P.opclass[mi[t]])) sel[ns++] = t;
+        if (!keeps || (mo[t] & keeps)) sel[ns++] = t;
       if (ns == 0) {  // no surviving source: the samples stay on j
         blame_add(P.blame + (size_t)j * kCnt + cls * 2 + lat, S);
         continue;
       }
       if (ns == 1) {  // a single source takes them all, whatever its weight
         const int t = sel[0];
-        if (P.cnt[(size_t)mi[t] * kCnt] >> 43) set_status(P, ST_OVERFLOW);
+        if (mc[t] >> 43) set_status(P, ST_OVERFLOW);
         P.e_share[(int64_t)(off + t) * 8 + ci * 2 + lat] = S;
         blame_add(P.blame + (size_t)mi[t] * kCnt + cls * 2 + lat, S);
         continue;
@@ -339,7 +354,7 @@ __device__ void apportion_use(const Prog& P, const Arch& A, int j, int off, int 
       // Eq. 1: weight = issued samples / longest path, in units of 2^-20.
       unsigned __int128 W = 0;
       for (int q = 0; q < ns; ++q) {
-        const unsigned long long issue = P.cnt[(size_t)mi[sel[q]] * kCnt];
+        const unsigned long long issue = mc[sel[q]];
         const unsigned long long len = (unsigned long long)max(ml[sel[q]], 1);
         if (issue >> 43) set_status(P, ST_OVERFLOW);
         // (len < 2^24, so a 64-bit division does for issue counts below 2^44)
@@ -404,10 +419,10 @@ __global__ void k_apportion(Prog P, Arch A, int max_src) {
     if (c > kMaxSrc) continue;  // k_apportion_big
     if (off + c > P.edge_cap) { capacity(P, 10); c = 0; }
     int mi[kMaxSrc], md[kMaxSrc], ml[kMaxSrc], sel[kMaxSrc];
-    uint32_t mf[kMaxSrc];
-    unsigned long long wt[kMaxSrc], sh[kMaxSrc];
+    uint32_t mf[kMaxSrc], mo[kMaxSrc];
+    unsigned long long mc[kMaxSrc], wt[kMaxSrc], sh[kMaxSrc];
     unsigned __int128 rem[kMaxSrc];
-    apportion_use(P, A, j, off, c, mi, md, ml, mf, sel, wt, rem, sh);
+    apportion_use(P, A, j, off, c, mi, md, ml, mf, mo, mc, sel, wt, rem, sh);
   }
 }
 
@@ -421,6 +436,8 @@ __global__ void k_apportion_big(Prog P, Arch A) {
   int* ml = md + kBigSrc;
   int* sel = ml + kBigSrc;
   uint32_t* mf = reinterpret_cast<uint32_t*>(sel + kBigSrc);
+  uint32_t* mo = mf + kBigSrc;
+  unsigned long long* mc = reinterpret_cast<unsigned long long*>(mo + kBigSrc);
   const unsigned long long nbig = P.stats[SS_BIG_N];
   for (unsigned long long k = blockIdx.x; k < nbig; k += gridDim.x) {
     if (threadIdx.x == 0) {
@@ -428,7 +445,7 @@ __global__ void k_apportion_big(Prog P, Arch A) {
       const int off = P.edge_off[j];
       int c = P.edge_off[j + 1] - off;
       if (off + c > P.edge_cap) { capacity(P, 10); c = 0; }
-      if (c > kMaxSrc) apportion_use(P, A, j, off, c, mi, md, ml, mf, sel, wt, rem, sh);
+      if (c > kMaxSrc) apportion_use(P, A, j, off, c, mi, md, ml, mf, mo, mc, sel, wt, rem, sh);
     }
     __syncthreads();
   }
@@ -540,7 +557,7 @@ void launch_blame(const Prog& P, const Arch& A, const SearchArena* tiers, const 
   *launches += 2;
   scan_exclusive_inplace(P.edge_off, P.ni, scan_tmp, st, launches);
   k_apportion<<<g_use, threads, 0, st>>>(P, A, max_src);
-  const size_t big_smem = (size_t)kBigSrc * (16 + 8 + 8 + 4 * 5);
+  const size_t big_smem = (size_t)kBigSrc * (16 + 8 + 8 + 4 * 6 + 8);
   allow_max_smem(k_apportion_big);
   k_apportion_big<<<sms, 32, big_smem, st>>>(P, A);
   *launches += 2;

@@ -743,9 +743,12 @@ __global__ void __launch_bounds__(768, 1) k_search_smem(Prog P, Arch A, int most
     if (part == 1) return min(P.stats[SS_A1_N + c], min(cap, (unsigned long long)P.class_limit[c]));
     return c == 0 ? min(P.stats[SS_OVF2_N], cap) : 0ull;
   };
-  unsigned long long any = 0;
-  for (int c = 0; c < kClasses; ++c) any |= n_tasks(c);
-  if (!any) return;
+  // Beside tiers 1 and 2 (part 1) no more SMs are taken than give every search a
+  // warp at once: a CTA holds its SM's shared memory, which those tiers need too
+  // (259 searches spread over all SMs kept them waiting).
+  unsigned long long need = 0;
+  for (int c = 0; c < kClasses; ++c) need += (n_tasks(c) + class_warps(c) - 1) / class_warps(c);
+  if (need == 0 || (part == 1 && blockIdx.x >= need)) return;
   if (threadIdx.x < kClasses) { s_nlocal[threadIdx.x] = 0; s_hlocal[threadIdx.x] = 0; }
   __syncthreads();
   unsigned long long runs = 0, most = 0, most_task = 0;

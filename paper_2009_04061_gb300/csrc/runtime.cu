@@ -487,7 +487,8 @@ gpa_status gpa_destroy(gpa_ctx* ctx) {
 // Gathers the program's device arrays and derives those that are computed on
 // the host (with R->dry, only their sizes). pool_bytes: the context's search
 // arenas, which the fourth tier uses when they hold more than its own would.
-static void plan_program(const gpa_program_desc* d, ProgramRec* R, Layout& L, int tier3_nodes, int64_t pool_bytes) {
+static void plan_program(const gpa_program_desc* d, ProgramRec* R, Layout& L, int tier3_nodes, int64_t pool_bytes,
+                         int sms) {
   Prog& P = R->P;
   P.nf = d->n_functions; P.ni = d->n_instr; P.nb = d->n_blocks; P.nl = d->n_loops; P.n_lines = d->n_lines;
   // Staged fixpoint: the largest per-function need within the cap (edges stay
@@ -672,10 +673,11 @@ static void plan_program(const gpa_program_desc* d, ProgramRec* R, Layout& L, in
   dev_alloc(L, &P.a_hot, nf * GPA_NUM_OPT * 5 * 6);
   dev_alloc(L, &P.a_loop_speedup, nl);
   {
+    P.adv_tile = adv_tile_size(P.ni, sms);
     std::vector<int32_t>&off = L.tile_off, &func = L.tile_func;
     off.assign(nf + 1, 0);
     for (size_t f = 0; f < nf; ++f) {
-      const int n = (d->func_instr_off[f + 1] - d->func_instr_off[f] + kAdvTile - 1) / kAdvTile;
+      const int n = (d->func_instr_off[f + 1] - d->func_instr_off[f] + P.adv_tile - 1) / P.adv_tile;
       off[f + 1] = off[f] + n;
       func.insert(func.end(), (size_t)n, (int32_t)f);
     }
@@ -773,7 +775,7 @@ gpa_status gpa_program_footprint(gpa_ctx* ctx, const gpa_program_desc* d, int64_
   ProgramRec R;
   R.dry = true;
   Layout L;
-  plan_program(d, &R, L, ctx->tier[2].nodes, arena_pool_bytes(ctx));
+  plan_program(d, &R, L, ctx->tier[2].nodes, arena_pool_bytes(ctx), ctx->sms);
   std::vector<size_t> at;
   size_t copy_bytes = 0;
   lay_out(L, &R, &at, &copy_bytes);
@@ -797,7 +799,7 @@ gpa_status gpa_load_program(gpa_ctx* ctx, const gpa_program_desc* d, gpa_pid* ou
   if (!R) return GPA_ERR_OOM;
   R->build = ctx->build_stream;
   Layout L;
-  plan_program(d, R, L, ctx->tier[2].nodes, arena_pool_bytes(ctx));
+  plan_program(d, R, L, ctx->tier[2].nodes, arena_pool_bytes(ctx), ctx->sms);
   s = place_program(ctx, R, L);
   if (s) { free_program(R); return s; }
   Prog& P = R->P;
