@@ -1171,16 +1171,22 @@ static gpa_status copy_advice(gpa_ctx* ctx, ProgramRec* R, const gpa_advice* out
   // Page-locked destinations that this device can address are written by one
   // kernel; others of up to kAdviceStage in all through page-locked staging, and
   // larger ones array by array.
-  bool direct = true;
-  for (int k = 0; k < L.n && direct; ++k) {
-    cudaPointerAttributes at{};
-    direct = cudaPointerGetAttributes(&at, user[k]) == cudaSuccess && at.type == cudaMemoryTypeHost &&
-             at.devicePointer && (reinterpret_cast<uintptr_t>(at.devicePointer) & 3u) == 0;
+  bool direct = true, on_host = true;
+  for (int k = 0; k < L.n; ++k) {
+    // (the last byte too: a caller may have registered only part of an array)
+    cudaPointerAttributes at{}, end{};
+    const bool known = cudaPointerGetAttributes(&at, user[k]) == cudaSuccess;
+    direct = direct && known && at.type == cudaMemoryTypeHost && at.devicePointer &&
+             (reinterpret_cast<uintptr_t>(at.devicePointer) & 3u) == 0 &&
+             cudaPointerGetAttributes(&end, static_cast<const char*>(user[k]) + L.bytes[k] - 1) == cudaSuccess &&
+             end.type == cudaMemoryTypeHost &&
+             end.devicePointer == static_cast<char*>(at.devicePointer) + L.bytes[k] - 1;
+    on_host = on_host && known && at.type != cudaMemoryTypeDevice;
     L.dst[k] = at.devicePointer;
   }
   cudaGetLastError();  // a failed query is not an error here
   bool staged = false;
-  if (!direct && total <= kAdviceStage) {
+  if (!direct && on_host && total <= kAdviceStage) {
     if (!ctx->advice_stage && cudaMallocHost(&ctx->advice_stage, kAdviceStage) != cudaSuccess) {
       cudaGetLastError();
       ctx->advice_stage = nullptr;
