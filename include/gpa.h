@@ -101,16 +101,17 @@ typedef struct {
 typedef struct {
   int32_t max_fixpoint_sweeps;  /* reaching-definitions sweep limit; 0 = 64 */
   int32_t max_search_nodes;     /* (block, predicate-set) nodes of the largest general search; 0 = 32768 */
-  int32_t search_slots;         /* warps with a max_search_nodes global-memory arena; 0 = as many as the
-                                   search kernel keeps resident (24 per SM on GB300, about 16 GB of arenas
-                                   at the default max_search_nodes) */
+  int32_t search_slots;         /* global-memory arenas of max_search_nodes; 0 = as many as one-warp search
+                                   CTAs stay resident (24 per SM on GB300, about 16 GB of arenas at the
+                                   default max_search_nodes) */
   int32_t max_sources_per_use;  /* distinct sources merged per stalled use; 0 = 2048 (max 2048) */
-  int32_t small_search_nodes;   /* nodes of the shared-memory arena of a first-tier search warp; 0 = 64
-                                   (max 1024). A search that outgrows it is redone in the next tier */
-  int32_t mid_search_nodes;     /* nodes of the second tier's shared-memory arenas (three warps per SM
-                                   up to 512 nodes, one up to 1024); 0 = small_search_nodes (searches that
-                                   outgrow the first tier go on to the global-memory warps, which are
-                                   faster than few large shared-memory arenas) */
+  int32_t small_search_nodes;   /* nodes of a first-tier search, one search a lane in shared memory;
+                                   0 = 16 (max 1024; values over 128 count as 128). A search that
+                                   outgrows it is redone in the next tier */
+  int32_t mid_search_nodes;     /* nodes of a second-tier search, one search a lane too; 0 = 64 (at least
+                                   small_search_nodes; values over 128 count as 128). Larger searches
+                                   run one to a warp in shared memory (up to 5,632 nodes) and beyond
+                                   that one to a CTA in global memory */
   int32_t hist_variant;         /* aggregation kernel: 0 (default) = one CTA per SM taking chunks of
                                    tiles of 8,192 samples from a counter, shared memory used per
                                    2,048-sample segment as a direct-indexed window over up to 1,558
@@ -118,17 +119,17 @@ typedef struct {
                                    grid-strided with a shared-memory hash: 1 = 8,192 entries, 512
                                    threads, 2 CTAs per SM; 2 = 16,384 entries, 1,024 threads, 1 CTA
                                    per SM; 3 = 8,192 entries, 256 threads, 3 CTAs per SM */
-  int32_t large_search_nodes;   /* a global-memory search that reached this many nodes is started
-                                   before the others on later steps of its program; 0 = 1024 */
-  int32_t hist_chunk;           /* aggregation variant 0: tiles per claimed chunk, 0 = 24 (max 4096) */
+  int32_t large_search_nodes;   /* accepted (>= 0) and without effect: searches are queued by size class,
+                                   the largest first */
+  int32_t hist_chunk;           /* aggregation variant 0: tiles per claimed chunk (max 4096); 0 = sized to
+                                   the stream, about six chunks an SM, at most 24 tiles */
   int32_t reach_schedule;       /* reaching-definitions fixpoint: 0 (default) = a CTA per function staged
-                                   in shared memory (launches by size class; functions beyond 200 KB of
-                                   stage take the windowed kernel); 1 = the windowed kernel for every
-                                   function (a lane per basic block, windows of 32 blocks in global
-                                   memory) */
-  int32_t small_search_warps;   /* first-tier search warps per SM (a multiple of 4, at most 32); 0 = 24.
-                                   The first tier shares the SMs with the third tier's searches known
-                                   from earlier steps, which take the registers it leaves */
+                                   in shared memory (launches by size class), or a CTA per function and
+                                   mask word for larger functions of natural loops; 1 = the windowed
+                                   kernel for every function (a lane per basic block, windows of 32
+                                   blocks in global memory) */
+  int32_t small_search_warps;   /* first-tier search warps per SM (a multiple of 4, at most 32), as far as
+                                   their arenas fit; 0 = 24 */
 } gpa_options;
 
 /* A program: n_functions functions laid out one after another. All arrays are
@@ -353,9 +354,9 @@ gpa_status gpa_advise(gpa_ctx* ctx, gpa_pid pid, const gpa_advice* out, gpa_stre
  * not NULL it must have room for 8 values: info[0] = invalid samples,
  * info[1] = general (multi-block) searches run, info[2] = largest search in
  * nodes, info[3] = fixpoint sweeps, info[4] and info[5] = searches run by the
- * second and third search tiers in the last gpa_blame (handed on by a smaller
- * tier, or queued there directly because an earlier step of the program found
- * them that large), info[6] and
+ * second search tier and by the larger ones in the last gpa_blame (handed on by
+ * a smaller tier, or queued there directly because an earlier step of the program
+ * found them that large), info[6] and
  * info[7] = the stalled use (global instruction index) and the resource of
  * the largest search. */
 gpa_status gpa_sync_status(gpa_ctx* ctx, gpa_pid pid, gpa_stream stream, int64_t* info);
@@ -379,8 +380,9 @@ gpa_status gpa_dependency_coverage(gpa_ctx* ctx, gpa_pid pid, gpa_stream stream,
  * distance with exactly that many back edges, and whether the dominator rule
  * cuts it (an unguarded reader of the resource on all its source paths; the
  * latency and opcode rules are left to the caller, from dmin and the def's
- * opcode class). Runs the unbounded searches twice (a counting pass sizes the
- * program-owned export buffer); *n_edges receives the edge count. Blame, edges
+ * opcode class). Runs the unbounded searches once, and again into a larger buffer
+ * when there are more edges than the program-owned one holds (it is kept);
+ * *n_edges receives the edge count. Blame, edges
  * and advice stay as they were. Synchronizes stream. */
 gpa_status gpa_export_unpruned_edges(gpa_ctx* ctx, gpa_pid pid, gpa_stream stream, int64_t* n_edges);
 
@@ -405,8 +407,9 @@ gpa_status gpa_step_capture(gpa_ctx* ctx, gpa_pid pid, const uint64_t* dev_sampl
  * context's search scratch. GPA_ERR_INVALID_ARG if nothing was captured. */
 gpa_status gpa_step_launch(gpa_ctx* ctx, gpa_pid pid, gpa_stream stream);
 
-/* Diagnostic: per search tier (3) the SM cycles summed over the searches of the
- * last gpa_blame in six phases: building the graph, shortest distances and
+/* Diagnostic: the SM cycles summed over the searches of the last gpa_blame (row
+ * 0 unused, row 1 the shared-memory warps, row 2 the global-memory searches; the
+ * one-lane searches are not timed) in six phases: building the graph, shortest distances and
  * fewest back edges, sources and rule 3, rule 2, longest paths and emission,
  * and (not cycles) the number of rule-2 reachability runs; out[0..17],
  * tier-major. Then out[18..33] = searches by floor(log2(nodes)) (the last

@@ -12,8 +12,8 @@ tried with the best values found so far for the others):
 - reaching-definitions schedule: a CTA per function staged in shared memory
   (launched by size class) against the windowed kernel, a lane per basic block
   in windows of 32 blocks, for every function;
-- search tiers: the node capacity of the first tier's shared-memory arenas, the
-  first tier's warps per SM, and the number of global-memory search warps per SM.
+- search tiers: the node capacity of the first tier's shared-memory arenas (one
+  search a lane), the first tier's warps per SM, and the number of global-memory search warps per SM.
 
 A dimension's values are compared by the time of the phase it schedules
 (ingest for the aggregation options, blame for the others). Every candidate
@@ -23,13 +23,13 @@ from __future__ import annotations
 
 from . import gpa
 
-# Candidate values per dimension (the first is the library default) and the
+# Candidate values per dimension (the first is where the search starts) and the
 # phase of the step the dimension schedules, by whose time it is judged.
 DIMENSIONS = [
     ("hist_variant", (0, 1, 2, 3)),
-    ("hist_chunk", (24, 8, 16, 32, 48)),
+    ("hist_chunk", (24, 8, 16, 32, 48, 0)),
     ("reach_schedule", (0, 1)),
-    ("small_search_nodes", (64, 128, 32)),
+    ("small_search_nodes", (64, 16, 32, 128)),
     ("small_search_warps", (24, 16, 20)),
     ("search_slots_per_sm", (0, 12, 16)),
 ]

@@ -13,7 +13,7 @@
 // (rule 1) match the class's opcode rule.
 //
 // Work split:
-//  * k_search_local: one thread per stalled use, one linear scan per
+//  * k_search_local: four threads per stalled use, one linear scan per
 //    resource inside j's block. It settles every source of that block
 //    (their only path is the straight segment) and stops at coverage or at
 //    the first unguarded reader of r (that reader lies on every path beyond,
@@ -21,10 +21,11 @@
 //    through which a def of r arrives covers j's guard, those predecessors
 //    are settled here too (one path per source); otherwise the (use,
 //    resource) pair is queued.
-//  * k_search_warp (k_search.cu): persistent warps pull queued (use,
-//    resource) pairs and explore the (block, literal set) graph.
+//  * k_search_lanes, k_search_smem, k_search_warp, k_search_cta: persistent
+//    lanes, warps and CTAs pull queued (use, resource) pairs and explore the
+//    (block, literal set) graph, by its size.
 //  * k_merge_count / scan / k_apportion: merge sources per use, apportion in
-//    integers, scatter blame with warp-aggregated 64-bit atomics.
+//    integers, scatter blame with 64-bit atomics.
 #include <algorithm>
 
 #include "gpa_internal.cuh"
