@@ -22,7 +22,8 @@
 // source farther than that fails rule 3 whatever the rest of the graph holds.
 // Only if some source is within its latency does pass B complete the graph,
 // which rule 2 and the longest paths need; when pass B adds no node, pass A's
-// distances are already those of the whole graph.
+// distances are already those of the whole graph. A CTA's search mostly gets by
+// with a part of it (kLayers below).
 #include <algorithm>
 
 #include "gpa_internal.cuh"
@@ -206,6 +207,94 @@ struct CtaGroup {
     return v;
   }
 };
+
+// Rule 2 on the function's blocks alone, for the sources within their latency
+// (sp 2): bit b of reach[B] says block B is reached
+// from the root's predecessors without passing the wall of the batch's b-th
+// needed group (ord holds the nl groups). A block whose own defs of r cover j's
+// guard passes nothing on, whatever literal set comes in. Every path of the graph
+// is such a path of blocks, so a source whose block is not reached past some
+// wall is cut (sp 3). Returns how many were. A function has tens of thousands of blocks where the
+// graph has hundreds of thousands of nodes. Uses dl's second and third layer, q
+// and tmp.
+template <class G>
+__device__ int cut_by_blocks(const G& g, const Prog& P, const Arena& a, int b0, int r, int gj, int nsrc, int nl,
+                             int undecided) {
+  const int me = g.rank();
+  const int f = P.block_func[b0], fb = P.func_block_off[f], nblk = P.func_block_off[f + 1] - fb;
+  if (nblk > a.N || a.L < 4) return 0;
+  volatile int* ctr = a.ctr;
+  int* reach = a.dl + a.N;
+  int* mark = a.dl + 2 * (int64_t)a.N;  // the batch's bit + 1 of the block's group; 64: queued; 128: covers
+  const int w = r >> 5;
+  const uint32_t bit = 1u << (r & 31);
+  auto offer = [&](int p, unsigned m, int* nxt) {
+    if (!(P.rout[(size_t)p * kWords + w] & bit)) return;
+    const unsigned add = m & ~(unsigned)reach[p - fb];
+    if (!add) return;
+    const unsigned old = (unsigned)atomicOr(&reach[p - fb], (int)add);
+    if ((old | add) != old && !(atomicOr(&mark[p - fb], 64) & 64)) nxt[atomicAdd((int*)&ctr[5], 1)] = p - fb;
+  };
+  for (int t = me; t < nblk; t += G::kSize) {
+    const size_t B = fb + t;
+    uint16_t S = 0;
+    if (P.touch_mask[B * kWords + w] & bit) {
+      const size_t seg = B * kEvBuckets + ev_bucket(r);
+      for (int e = P.ev_off[seg]; e < P.ev_off[seg + 1]; ++e) {
+        const uint32_t ev = P.events[e];
+        if ((int)(ev & 0x1FFu) == r && (ev & 0x200u)) S = add_literal(S, (int)((ev >> 12) & 0xFu));
+      }
+    }
+    mark[t] = contains(S, gj) ? 128 : 0;
+  }
+  int cut = 0;
+  for (int w0 = 0; w0 < nl && cut < undecided; w0 += 32) {
+    const int nbits = min(32, nl - w0);
+    const unsigned full = nbits == 32 ? 0xFFFFFFFFu : ((1u << nbits) - 1u);
+    for (int t = me; t < nblk; t += G::kSize) reach[t] = 0;
+    if (me == 0) ctr[5] = 0;
+    g.sync();
+    if (me < nbits) mark[a.wblk[a.ord[w0 + me]] - fb] |= me + 1;
+    g.sync();
+    int* cur = a.q;
+    int* nxt = a.tmp;
+    const int4 pm0 = P.block_meta[2 * (size_t)b0 + 1];
+    for (int q = pm0.x + me; q < pm0.y; q += G::kSize) offer(P.pred[q], full, cur);
+    g.sync();
+    int fsize = g.read(&ctr[5]);
+    while (fsize > 0) {
+      if (me == 0) ctr[5] = 0;
+      for (int t = me; t < fsize; t += G::kSize) atomicAnd(&mark[cur[t]], ~64);
+      g.sync();
+      for (int t = me; t < fsize; t += G::kSize) {
+        const int B = cur[t];
+        unsigned m = (unsigned)atomicOr(&reach[B], 0);
+        const int mk = mark[B], wb = mk & 63;
+        if (mk & 128) continue;
+        if (wb) m &= ~(1u << (wb - 1));
+        if (!m) continue;
+        const int4 pm = P.block_meta[2 * (size_t)(fb + B) + 1];
+        for (int q = pm.x; q < pm.y; ++q) offer(P.pred[q], m, nxt);
+      }
+      g.sync();
+      fsize = g.read(&ctr[5]);
+      int* sw = cur; cur = nxt; nxt = sw;
+    }
+    int now = 0;
+    for (int m = me; m < nsrc; m += G::kSize) {
+      if (a.sp[m] != 2) continue;
+      const int x = a.si[m], B = P.instr_block[x] - fb;
+      unsigned ok = (unsigned)reach[B];
+      const int wb = mark[B] & 63;
+      if (wb && x < a.wpos[a.ord[w0 + wb - 1]]) ok &= ~(1u << (wb - 1));
+      if ((ok & full) != full) { a.sp[m] = 3; ++now; }
+    }
+    cut += g.sum(now);
+    if (me < nbits) mark[a.wblk[a.ord[w0 + me]] - fb] &= 128;
+    g.sync();
+  }
+  return cut;
+}
 
 // Returns false when the search outgrew the arena (nothing emitted).
 // With P.diag, the search counts the sources of (j, r) before and after
@@ -519,68 +608,129 @@ __device__ bool group_search(const G& g, const Prog& P, const Arch& A, const Are
   int cand_low = 0;
   auto relevant = [&](int u) { return a.blk[u] >= cand_low; };
 
-  // Split the unexpanded list: nodes to expand now (into list) and the rest,
-  // which stay unexpanded (all of them when bound < 0; in pass B, nodes off
-  // every candidate's paths are dropped from the list for good).
+  // How the graph grows. kNear (pass A): the nodes within the bound. kLayers:
+  // those that paths of at most k_max back edges to a live candidate can pass,
+  // where k_max is the most that the candidates' occurrences in pass A need:
+  // nodes of fewer back edges, and of k_max where the block is not above every
+  // candidate's (from there on only forward edges are left, and block indices
+  // fall along them). kAll (pass B): every node on a path to a candidate.
+  enum { kNear, kLayers, kAll };
+  constexpr bool kParts = G::kSize > 32;
+  int k_max = 0, blk_low = 0;
+  auto in_layers = [&](int u) { return a.k[u] < k_max || (a.k[u] == k_max && a.blk[u] >= blk_low); };
+
+  // Split unexpanded nodes: those to expand now (into list) and the rest, which
+  // stay unexpanded (beyond pass A, nodes off every candidate's paths are
+  // dropped for good). kLayers sets the rest aside in `defer` (the layers of
+  // the longest paths are free until then), so its waves do not read them again.
   int* list = a.q;
-  auto take_wave = [&](int lim) {
-    const int m = ctr[6];
+  int* const defer = a.dl;
+  int n_defer = 0;
+  auto split = [&](const int* from, int m, int* rest, int grow, int* kept_out) {
     int cnt = 0, kept = 0;
     for (int i0 = 0; i0 < m; i0 += G::kSize) {
       const int i = i0 + me;
-      const int u = i < m ? ubuf[i] : 0;
-      const bool now = i < m && (lim < 0 ? relevant(u) : dist_of(a, u) <= lim);
-      const bool keep = i < m && !now && lim >= 0;
+      const int u = i < m ? from[i] : 0;
+      const bool now = i < m && (grow == kNear ? dist_of(a, u) <= bound : relevant(u) && (!kParts || grow == kAll || in_layers(u)));
+      const bool keep = i < m && !now && (grow == kNear || (kParts && grow == kLayers && relevant(u)));
       int tot_now, tot_keep;
       const int at_now = g.slot(now, &tot_now);
       const int at_keep = g.slot(keep, &tot_keep);
       if (now) list[cnt + at_now] = u;
-      if (keep) ukeep[kept + at_keep] = u;
+      if (keep) rest[kept + at_keep] = u;
       cnt += tot_now;
       kept += tot_keep;
     }
     g.sync();
+    *kept_out = kept;
+    return cnt;
+  };
+  auto take_wave = [&](int grow) {
+    int kept;
+    int cnt = split(ubuf, g.read(&ctr[6]), kParts && grow == kLayers ? defer + n_defer : ukeep, grow, &kept);
     int* sw = ubuf; ubuf = ukeep; ukeep = sw;
+    if (kParts && grow == kLayers) {
+      n_defer += kept;
+      kept = 0;
+      // nodes whose fewest back edges fell meanwhile (compacted in place: a
+      // chunk is read before any of it is written, and writes stay below it)
+      if (cnt == 0) cnt = split(defer, n_defer, defer, grow, &n_defer);
+    }
     if (me == 0) ctr[6] = kept;
     g.sync();
     return cnt;
   };
 
   // Pass A expands in waves the nodes within the bound, relaxing as they
-  // link; pass B, only if some source is within its
-  // latency, completes the graph. Both run in this one loop, so the wave code
-  // exists once in the kernel (the search kernel is bound by instruction fetch
-  // when its warps spread over a larger body).
-  bool cand = false, pass_b = false, grew_b = false;
+  // link. Only if some source is within its latency does the graph grow on.
+  // A CTA's searches then first drop the sources that rule 2 cuts on the
+  // function's blocks already (cut_by_blocks), and grow the layers of what is
+  // left: the longest paths need no more, and a source that reaches past every
+  // wall there survives. Only where some does not is the graph completed
+  // (`whole`). Counted on kernels of 45,000 to 200,000 instructions: six in ten
+  // sources go on the blocks, a search is left with one wall to test on the graph
+  // instead of dozens, and one or no search in 2,000 needs the whole graph.
+  // Blame with 5M samples of 120,000 instructions: 480 -> 330 ms; 60,000: 54 ->
+  // 46 ms; 200,000 (20M samples): 340 -> 250 ms. The warps' searches, whose size
+  // tells later steps their shared-memory class, take the whole graph at once.
+  // All growth runs in this one loop, so the wave code exists once in the kernel.
+  bool cand = false, grew_b = false, whole = !kParts || P.diag, again = false;
+  int grow = kNear;
+  int nsrc, nl, alive, n_cut = 0;
+  int* const cut_list = a.dl + 3 * (int64_t)a.N;  // sources cut on the blocks
+  auto candidate = [&](int o) {
+    const int u = a.on[o];
+    return dist_of(a, u) + (last_of(u) - a.ox[o]) <= A.lat[P.opclass[a.ox[o]]];
+  };
+  // Puts the nodes back into the hash and the list in `defer` back into ubuf.
+  auto resume = [&](int n) {
+    for (int u = 1 + me; u < n; u += G::kSize) {
+      uint32_t h = node_hash(a.blk[u], a.S[u] & 0xFFFF) & hmask;
+      for (uint32_t t = 0; t <= hmask && atomicCAS(&a.ht[h], -1, u) != -1; ++t) h = (h + 1) & hmask;
+      a.hused[u - 1] = (int)h;
+    }
+    for (int t = me; t < n_defer; t += G::kSize) a.seen[t] = defer[t];
+    ubuf = a.seen;
+    ukeep = a.tmp;
+    if (me == 0) { ctr[3] = n - 1; ctr[5] = 0; ctr[6] = n_defer; }
+    g.sync();
+    n_defer = 0;
+    again = true;
+  };
+  while (true) {  // once; a CTA's search: pass A, the layers, and the whole graph if need be
   while (!ctr[4]) {
-    const int cnt = take_wave(pass_b ? -1 : bound);
+    const int cnt = take_wave(grow);
     if (cnt > 0) {
-      grew_b |= pass_b;
-      expand_list(list, cnt, !pass_b);
+      grew_b |= grow != kNear;
+      expand_list(list, cnt, grow == kNear);
       if (ctr[4]) break;
       // pass A relaxed the wave's edges as they were linked; carry on from the
       // expanded nodes that improved (queued in ord, counted in ctr[5])
       // (every thread reads the count before relax_from's rank 0 clears it)
-      const int n_dirty = pass_b ? 0 : g.read(&ctr[5]);
-      if (n_dirty > 0) relax_from(a.ord, n_dirty, 0);
+      if (grow == kNear) {
+        const int n_dirty = g.read(&ctr[5]);
+        if (n_dirty > 0) relax_from(a.ord, n_dirty, 0);
+      } else if (kParts && grow == kLayers) {
+        relax_from(list, cnt, 1);
+      }
       continue;
     }
-    if (pass_b) break;
+    if (grow != kNear) break;
     // End of pass A. A source within its latency? (Every candidate is found
     // by pass A: a source farther than the bound fails rule 3.)
     const int no = min(ctr[2], a.O);
     int low = 0x7FFFFFFF;
     for (int o = me; o < no; o += G::kSize) {
-      const int u = a.on[o];
-      if (dist_of(a, u) + (last_of(u) - a.ox[o]) <= A.lat[P.opclass[a.ox[o]]]) {
+      if (candidate(o)) {
         cand = true;
-        low = min(low, P.block_minreach[a.blk[u]]);
+        low = min(low, P.block_minreach[a.blk[a.on[o]]]);
       }
     }
     cand = g.any(cand);
     cand_low = g.min(low);
     if (!cand) break;
-    pass_b = true;
+    if (kParts && !whole) break;
+    grow = kAll;
   }
   // Clear the hash slots this search used.
   const int nh = ctr[3];
@@ -588,7 +738,7 @@ __device__ bool group_search(const G& g, const Prog& P, const Arch& A, const Are
   g.sync();
   const int n = ctr[0];
   if (me == 0) {
-    atomicAdd(&P.stats[SS_GENERAL], 1ull);
+    if (!again) atomicAdd(&P.stats[SS_GENERAL], 1ull);
     atomicMax(&P.stats[SS_MAX_NODES], (unsigned long long)n);
     atomicMax(&P.stats[SS_MAX_TASK], ((unsigned long long)n << 40) | ((unsigned long long)r << 31) | (unsigned)j);
 #ifdef GPA_PHASE_TIMING
@@ -607,17 +757,22 @@ __device__ bool group_search(const G& g, const Prog& P, const Arch& A, const Are
   // Shortest distance with parents, and fewest back edges, over the whole
   // graph. When pass B expanded no node, every edge of the graph was relaxed
   // to the fixpoint in pass A, whose (distance, parent) minimum over the same
-  // edges is this one.
-  const bool fresh_d = grew_b;
-  for (int u = me; u < n; u += G::kSize) {
-    if (fresh_d) a.dpk[u] = u == 0 ? 0ull : (((unsigned long long)kInf << 32) | 0xFFFFFFFFull);
-    a.k[u] = u == 0 ? 0 : kInf;
-    a.fl[u] &= ~8;
-  }
-  if (me == 0) a.q[0] = 0;
-  g.sync();
+  // edges is this one. On the layers both are there already: the back edges
+  // were relaxed as they grew, and the distances of pass A's nodes are final
+  // (any path within the bound stays in them; a node beyond it keeps a distance
+  // beyond it, so its occurrences fail rule 3 as they should).
+  const bool fresh_d = (!kParts || whole) && grew_b;
+  if (!kParts || whole) {
+    for (int u = me; u < n; u += G::kSize) {
+      if (fresh_d) a.dpk[u] = u == 0 ? 0ull : (((unsigned long long)kInf << 32) | 0xFFFFFFFFull);
+      a.k[u] = u == 0 ? 0 : kInf;
+      a.fl[u] &= ~8;
+    }
+    if (me == 0) a.q[0] = 0;
+    g.sync();
 #pragma unroll 1
-  for (int mode = fresh_d ? 0 : 1; mode < 2; ++mode) relax_from(a.q, 1, mode);
+    for (int mode = fresh_d ? 0 : 1; mode < 2; ++mode) relax_from(a.q, 1, mode);
+  }
   phase(1);
 
   // Sources: a warp-synchronous hash keyed by instruction gives each source an
@@ -678,12 +833,15 @@ __device__ bool group_search(const G& g, const Prog& P, const Arch& A, const Are
     g.sync();
     return false;
   }
-  const int nsrc = ctr[5];
-  int alive = 0;
+  nsrc = g.read(&ctr[5]);
+  alive = 0;
   for (int m = me; m < nsrc; m += G::kSize) {
     a.sp[m] = (int)(a.sdb[m] >> 32) > A.lat[P.opclass[a.si[m]]] ? 1 : 0;  // rule 3
     if (P.diag == 1 && (blocked || !keeps_any(P, A, j, P.opclass[a.si[m]]))) a.sp[m] = 1;  // rule 2 above j, rule 1
     if (P.diag == 2) a.sp[m] = 0;  // export: rule 2 for every source
+    if (kParts && !a.sp[m])
+      for (int t = 0; t < n_cut; ++t)
+        if (cut_list[t] == a.si[m]) { a.sp[m] = 1; break; }
     alive += a.sp[m] ? 0 : 1;
   }
   alive = g.sum(alive);
@@ -749,7 +907,7 @@ __device__ bool group_search(const G& g, const Prog& P, const Arch& A, const Are
   }
   g.sync();
   // The needed groups, compacted into ord (free until the longest paths).
-  int nl = 0;
+  nl = 0;
   for (int t0 = 0; t0 < nw; t0 += G::kSize) {
     const bool need = t0 + me < nw && a.wneed[t0 + me];
     int tot;
@@ -759,20 +917,54 @@ __device__ bool group_search(const G& g, const Prog& P, const Arch& A, const Are
   }
   for (int t = me; t < nw; t += G::kSize) a.wneed[t] = 0;
   g.sync();
+  if (kParts && grow == kNear && !whole) {
+    // Pass A is done: rule 2 on the blocks, then the layers of the survivors.
+    n_defer = g.read(&ctr[6]);
+    for (int t = me; t < n_defer; t += G::kSize) defer[t] = ubuf[t];
+    for (int m = me; m < nsrc; m += G::kSize) if (!a.sp[m]) a.sp[m] = 2;
+    g.sync();
+    alive -= cut_by_blocks(g, P, a, b0, r, gj, nsrc, nl, alive);
+    phase(3);
+    if (alive == 0) return true;
+    if (me == 0) { ctr[5] = 0; a.q[0] = 0; }
+    g.sync();
+    for (int m = me; m < nsrc; m += G::kSize)
+      if (a.sp[m] == 3) cut_list[atomicAdd((int*)&a.ctr[5], 1)] = a.si[m];
+    g.sync();
+    n_cut = g.read(&ctr[5]);
+    relax_from(a.q, 1, 1);
+    int most = 0, low_blk = 0x7FFFFFFF, low_reach = 0x7FFFFFFF;
+    for (int m = me; m < nsrc; m += G::kSize) {
+      if (a.sp[m] != 2) continue;
+      const int B = P.instr_block[a.si[m]];
+      low_blk = min(low_blk, B);
+      low_reach = min(low_reach, P.block_minreach[B]);
+      for (int o = a.shead[m]; o >= 0; o = a.onext[o])
+        if (candidate(o)) most = max(most, a.k[a.on[o]]);
+    }
+    k_max = g.max(most);
+    blk_low = g.min(low_blk);
+    cand_low = g.min(low_reach);
+    whole = k_max >= a.L;
+    grow = whole ? kAll : kLayers;
+    resume(n);
+    continue;
+  }
   // Bit-parallel reachability over up to 32 groups at a time: bit b of
   // reach[u] (kept in seen) says u is reachable from the root without passing
   // the wall of the batch's b-th group. A node truncated by a group (each node
   // of its block that has a wall) passes every bit on but that group's.
   // wneed[g] holds g's bit + 1 while g is in the batch.
   int* reach = a.seen;
-  for (int b0 = 0; b0 < nl && alive > 0; b0 += 32) {
-    const int nbits = min(32, nl - b0);
+  const int undecided = alive;
+  for (int w0 = 0; w0 < nl && alive > 0; w0 += 32) {
+    const int nbits = min(32, nl - w0);
     const unsigned full = nbits == 32 ? 0xFFFFFFFFu : ((1u << nbits) - 1u);
 #ifdef GPA_PHASE_TIMING
     if (me == 0) atomicAdd(&P.stats[SS_PHASE + (min(tier, 3) - 1) * 6 + 5], 1ull);
     ++r2runs;
 #endif
-    if (me < nbits) a.wneed[a.ord[b0 + me]] = me + 1;
+    if (me < nbits) a.wneed[a.ord[w0 + me]] = me + 1;
     for (int u = me; u < n; u += G::kSize) reach[u] = u == 0 ? (int)full : 0;
     g.sync();
     auto pass_mask = [&](int u) {
@@ -826,14 +1018,29 @@ __device__ bool group_search(const G& g, const Prog& P, const Arch& A, const Are
         if (wg >= 0 && a.wneed[wg] && a.ox[o] < a.wpos[wg]) r &= ~(1u << (a.wneed[wg] - 1));
         ok |= r;
       }
-      if ((ok & full) != full) { a.sp[m] = 1; ++dropped; }
+      if ((ok & full) != full) { a.sp[m] = !kParts || whole ? 1 : 2; ++dropped; }
     }
     alive -= g.sum(dropped);
     g.sync();
-    if (me < nbits) a.wneed[a.ord[b0 + me]] = 0;
+    if (me < nbits) a.wneed[a.ord[w0 + me]] = 0;
     g.sync();
   }
   phase(3);
+  // A path found on the layers is a path of the whole graph, so a source that
+  // survived there survives. Where one did not, the whole graph decides.
+  if (kParts && !whole && undecided > alive) {
+    if (n_defer > 0) {
+      whole = true;
+      grow = kAll;
+      resume(n);
+      continue;
+    }
+    for (int m = me; m < nsrc; m += G::kSize) if (a.sp[m] == 2) a.sp[m] = 1;  // the layers are the whole graph
+    g.sync();
+  }
+  break;
+  }
+  const int n = g.read(&ctr[0]);
   if (P.diag == 1) {
     if (me == 0) cov_add(P, e, nsrc, alive);
     return true;

@@ -92,6 +92,19 @@ def test_search_arena_sizes(small, mid, most):
             prog.unload()
 
 
+@pytest.mark.parametrize("seed", [71, 72, 73])
+def test_searches_of_a_cta(seed):
+    """Every search of more than 16 nodes by a CTA: sources cut on the function's blocks,
+    the layers of back edges that the others need, and the whole graph where those do
+    not decide; several back edges and guarded defs."""
+    import paper_2009_04061_gb300 as g
+    rng = np.random.default_rng(seed)
+    P = synth.make_program(synth.batched_params(16, rng, seed), 1.0)
+    s = P.samples(900_000, seed=seed)
+    with g.Context(ARCH, dict(small_search_nodes=4, mid_search_nodes=8, max_search_nodes=16, search_slots=16)) as c:
+        assert_full_parity(gpu_run(c, P, dev(s)), oracle_run(P, s))
+
+
 def test_one_search_slot():
     """A context with a single global-memory arena: the CTAs and the warps take turns with it."""
     import paper_2009_04061_gb300 as g
