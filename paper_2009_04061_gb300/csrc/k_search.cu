@@ -1209,9 +1209,16 @@ __global__ void __launch_bounds__(32, 24) k_search_warp(Prog P, Arch A, SearchAr
 
 // A CTA per search: the waves, frontiers and source lists of these searches
 // are wide enough for its threads. 128 threads for searches of 5,633 to 32,768
-// nodes (a warp took 31 ms for the largest of them), 512 for larger ones.
+// nodes (a warp took 31 ms for the largest of them), 512 for larger ones, two of
+// these CTAs on an SM (64 registers), 1,024 for those beyond 2^18 nodes, whose
+// arenas are too large for a CTA on every SM. Both are chains of barriers and
+// arena latency, so what counts is threads in flight: on the 120,000-instruction
+// kernel 330 ms of blame with one CTA of 512 an SM for both, 298 with two,
+// 247 with 1,024 threads for the largest. (256 threads, three CTAs: 233 there, but
+// 31.6 against 28.1 ms at 45,000 instructions, where the searches do not fill
+// the chip; 128 threads, six CTAs: slower everywhere.)
 template <int NT>
-__global__ void __launch_bounds__(NT, 512 / NT) k_search_cta(Prog P, Arch A, SearchArena SA, Route R) {
+__global__ void __launch_bounds__(NT, NT == 128 ? 4 : 1024 / NT) k_search_cta(Prog P, Arch A, SearchArena SA, Route R) {
   __shared__ int s_ctr[8];
   __shared__ int s_red[CtaGroup<NT>::kWarps];
   __shared__ unsigned long long s_cast;
@@ -1283,8 +1290,8 @@ void launch_search(const Prog& P, const Arch& A, const SearchArena* tiers, const
   *launches += 4;
   if (big) {
     // Larger searches run after the others on this stream, so the third tier's
-    // arena pool is free by then and they carve their arenas from it (at most one
-    // CTA per SM): first those of up to 2^18 nodes (most of them; arenas for the
+    // arena pool is free by then and they carve their arenas from it (at most two
+    // CTAs per SM): first those of up to 2^18 nodes (most of them; arenas for the
     // program's largest function would be so big that the pool holds few), then
     // the rest in arenas of t4_nodes, from the pool when it holds more of them
     // than the program's own.
@@ -1297,14 +1304,14 @@ void launch_search(const Prog& P, const Arch& A, const SearchArena* tiers, const
     const int mid_nodes = 1 << 18;
     SearchArena mid{mid_nodes, 4096, kMaxLayers, 0, arena_bytes(mid_nodes, 4096, kMaxLayers, true), tiers[2].global,
                     nullptr};
-    mid.warps = (int)std::min<int64_t>(pool / mid.bytes, std::max(sms, 1));
+    mid.warps = (int)std::min<int64_t>(pool / mid.bytes, 2 * std::max(sms, 1));
     Route r4{4, SS_T4_N, SS_T4_HEAD, false, -1, 0, false, 0};
     if (P.t4_nodes > mid_nodes && mid.warps > own.warps) {
       r4.next_q = 7; r4.next_slot = SS_T5_N; r4.next_hint = kHintGiant;
       k_search_cta<512><<<groups(mid.warps), 512, 0, st>>>(P, A, mid, r4);
       ++*launches;
       const Route r5{7, SS_T5_N, SS_T5_HEAD, false, -1, 0, false, 0};
-      k_search_cta<512><<<groups(own.warps), 512, 0, st>>>(P, A, own, r5);
+      k_search_cta<1024><<<groups(own.warps), 1024, 0, st>>>(P, A, own, r5);
     } else {
       k_search_cta<512><<<groups(own.warps), 512, 0, st>>>(P, A, own, r4);
     }
