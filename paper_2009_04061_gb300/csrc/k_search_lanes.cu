@@ -8,9 +8,10 @@
 // lies at w * LPW + lane), so whatever nodes the lanes are at, a warp's access
 // touches one bank per lane. What bounds the kernel is the chain of dependent
 // loads of each search (a block's record, then its events and its predecessors'
-// reach words), so what counts is how many searches an SM has in flight: 192 of
-// 32 nodes (six warps of 32 lanes) or 48 of 128 nodes (six warps of 8 lanes), as
-// many as their arenas fit in shared memory.
+// reach words), so what counts is how many searches an SM has in flight: 352 of
+// 16 nodes (eleven warps of 32 lanes) or 96 of 64 nodes (twelve warps of 8 lanes),
+// as many as their arenas fit in shared memory. Searches of up to 64 nodes of the
+// thousand-function step: 3.88 ms with a warp each, 0.42 + 1.01 ms in these two.
 //
 // The lanes of a warp are kept together by state, not by search: a step
 // expands one node of every lane that is building its graph; lanes whose graph
