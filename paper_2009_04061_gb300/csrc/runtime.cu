@@ -21,6 +21,7 @@ namespace {
 struct ProgramRec {
   Prog P{};
   bool dry = false;                     // count bytes only (gpa_program_footprint)
+  // Like the program's block, these come from the pool in stream order.
   int4* xbuf = nullptr;                 // export buffer of gpa_export_unpruned_edges (grown on demand)
   int64_t xbuf_cap = 0, x_n = 0;
   void* xout = nullptr;                 // the ordered export and its scratch, for xout_cap edges
@@ -120,6 +121,15 @@ size_t lay_out(const Layout& L, ProgramRec* R, std::vector<size_t>* at, size_t* 
   }
   R->bytes = (int64_t)off;
   return off;
+}
+
+// Stream-ordered memory from the context's pool, nullptr if there is none.
+void* pool_alloc(const gpa_ctx* ctx, size_t bytes, cudaStream_t st) {
+  void* p = nullptr;
+  if ((ctx->pool ? cudaMallocFromPoolAsync(&p, bytes, ctx->pool, st) : cudaMallocAsync(&p, bytes, st)) == cudaSuccess)
+    return p;
+  cudaGetLastError();
+  return nullptr;
 }
 
 // Frees a program whose work has finished (the callers synchronize first).
@@ -742,12 +752,8 @@ static gpa_status place_program(gpa_ctx* ctx, ProgramRec* R, const Layout& L) {
   size_t copy_bytes = 0;
   const size_t total = lay_out(L, R, &at, &copy_bytes);
   cudaStream_t st = R->build;
-  if ((ctx->pool ? cudaMallocFromPoolAsync(&R->block, total, ctx->pool, st) : cudaMallocAsync(&R->block, total, st)) !=
-      cudaSuccess) {
-    cudaGetLastError();
-    R->block = nullptr;
-    return GPA_ERR_OOM;
-  }
+  R->block = pool_alloc(ctx, total, st);
+  if (!R->block) return GPA_ERR_OOM;
   char* base = static_cast<char*>(R->block);
   for (size_t k = 0; k < L.items.size(); ++k) *L.items[k].slot = base + at[k];
   derive_pointers(R);
@@ -842,12 +848,8 @@ gpa_status gpa_unload_program_async(gpa_ctx* ctx, gpa_pid pid, gpa_stream stream
   if (R->step_exec) cudaGraphExecDestroy(R->step_exec);
   R->step_exec = nullptr;
   gpa_status s = GPA_OK;
-  if (R->block && cudaFreeAsync(R->block, st) != cudaSuccess) s = GPA_ERR_CUDA;
-  R->block = nullptr;
-  // not stream-ordered allocations (freeing them waits for the device)
-  if (R->xbuf) cudaFree(R->xbuf);
-  if (R->xout) cudaFree(R->xout);
-  if (R->launch) cudaFree(R->launch);
+  for (void* p : {R->block, (void*)R->xbuf, R->xout, (void*)R->launch})
+    if (p && cudaFreeAsync(p, st) != cudaSuccess) s = GPA_ERR_CUDA;
   delete R;
   ctx->progs.erase(pid);
   return s;
@@ -1029,16 +1031,10 @@ gpa_status gpa_export_unpruned_edges(gpa_ctx* ctx, gpa_pid pid, gpa_stream strea
   *n_edges = 0;
   R->x_n = 0;
   auto grow = [&](int64_t need) {
-    if (R->xbuf) cudaFree(R->xbuf);
-    R->xbuf = nullptr;
-    R->xbuf_cap = 0;
-    if (cudaMalloc(&R->xbuf, sizeof(int4) * 2 * (size_t)need) != cudaSuccess) {
-      cudaGetLastError();
-      R->xbuf = nullptr;
-      return false;
-    }
-    R->xbuf_cap = need;
-    return true;
+    if (R->xbuf) cudaFreeAsync(R->xbuf, st);
+    R->xbuf = static_cast<int4*>(pool_alloc(ctx, sizeof(int4) * 2 * (size_t)need, st));
+    R->xbuf_cap = R->xbuf ? need : 0;
+    return R->xbuf != nullptr;
   };
   // A first buffer of an edge per use entry (32 MB at most) holds most exports;
   // the run counts every edge, so a buffer that proves too small (or could not be
@@ -1053,16 +1049,10 @@ gpa_status gpa_export_unpruned_edges(gpa_ctx* ctx, gpa_pid pid, gpa_stream strea
   }
   const int64_t n = std::min<int64_t>((int64_t)h[SS_XN], R->xbuf_cap);
   if (n > R->xout_cap) {
-    if (R->xout) cudaFree(R->xout);
-    R->xout = nullptr;
-    R->xout_cap = 0;
-    const size_t bytes = (size_t)n * 29 + sizeof(int32_t) * (2 * (size_t)R->P.ni + 1);
-    if (cudaMalloc(&R->xout, bytes) != cudaSuccess) {
-      cudaGetLastError();
-      R->xout = nullptr;
-      return GPA_ERR_OOM;
-    }
-    R->xout_cap = n;
+    if (R->xout) cudaFreeAsync(R->xout, st);
+    R->xout = pool_alloc(ctx, (size_t)n * 29 + sizeof(int32_t) * (2 * (size_t)R->P.ni + 1), st);
+    R->xout_cap = R->xout ? n : 0;
+    if (!R->xout) return GPA_ERR_OOM;
   }
   int32_t* ids = nullptr;
   const ExportOut out = export_out(R, &ids);
@@ -1243,11 +1233,11 @@ gpa_status gpa_set_launch_stats(gpa_ctx* ctx, gpa_pid pid, const gpa_launch_stat
     P.launch = nullptr;
     return GPA_OK;
   }
-  if (!R->launch && cudaMalloc(&R->launch, sizeof(LaunchRec) * (size_t)std::max(P.nf, 1)) != cudaSuccess) {
-    R->launch = nullptr;
-    return GPA_ERR_OOM;
-  }
-  CK(cudaMemcpy(R->launch, stats, sizeof(LaunchRec) * (size_t)P.nf, cudaMemcpyHostToDevice));
+  const size_t bytes = sizeof(LaunchRec) * (size_t)std::max(P.nf, 1);
+  if (!R->launch) R->launch = static_cast<LaunchRec*>(pool_alloc(ctx, bytes, ctx->build_stream));
+  if (!R->launch) return GPA_ERR_OOM;
+  CK(cudaMemcpyAsync(R->launch, stats, sizeof(LaunchRec) * (size_t)P.nf, cudaMemcpyHostToDevice, ctx->build_stream));
+  CK(cudaStreamSynchronize(ctx->build_stream));
   P.launch = R->launch;
   P.sm = SmModel{sm->n_sms, sm->schedulers_per_sm, sm->max_warps_per_sm, sm->max_blocks_per_sm, sm->regs_per_sm,
                  sm->reg_alloc_unit, sm->smem_per_sm, sm->smem_alloc_unit, sm->smem_reserved_per_block};
