@@ -276,7 +276,11 @@ gpa_status gpa_destroy(gpa_ctx* ctx);
 
 /* Validates and copies a program to the device and allocates its counters
  * and result buffers (stream-ordered allocations on the context's own build
- * stream; returns when they are done, without waiting for other streams).
+ * stream; returns when they are done, without waiting for other streams, unless
+ * the device has no memory left but what their work has yet to release).
+ * Programs' memory comes from a pool that the process's contexts on a device
+ * share: what unloaded programs gave back stays there for the next loads while
+ * the pool holds no more than 1 GB in all, until the last context is destroyed.
  * The program is what the paper's static analyzer provides to the dynamic one
  * (Sec. 3: control flow graphs, loop nests, line maps; Sec. 2.2 and Sec. 4:
  * per-instruction operands, virtual barrier registers, predicates).

@@ -9,6 +9,7 @@
 #include <cstdio>
 #include <cstring>
 #include <map>
+#include <mutex>
 #include <new>
 #include <vector>
 
@@ -73,7 +74,7 @@ struct gpa_ctx {
   cudaStream_t copy_stream = nullptr;
   cudaStream_t capture_stream = nullptr;  // private stream for gpa_step_capture
   cudaStream_t build_stream = nullptr;    // program allocation, copies and layout builds
-  cudaMemPool_t pool = nullptr;           // programs' memory; keeps up to kPoolKeep bytes for the next one
+  cudaMemPool_t pool = nullptr;           // programs' memory, shared by the device's contexts (take_pool)
   char* load_stage = nullptr;             // pinned staging of a load's copies (kLoadStage bytes, on first use)
   char* advice_stage = nullptr;           // and of advice into pageable arrays (kAdviceStage bytes)
   cudaEvent_t ev_copied[2] = {nullptr, nullptr}, ev_used[2] = {nullptr, nullptr};
@@ -89,7 +90,7 @@ constexpr size_t kStageSamples = (size_t)64 << 20;  // 64M samples (512 MB) per 
     if ((x) != cudaSuccess) return GPA_ERR_CUDA; \
   } while (0)
 
-constexpr size_t kPoolKeep = (size_t)1 << 30;   // freed program memory a context keeps
+constexpr size_t kPoolKeep = (size_t)1 << 30;   // program memory a device's pool holds on to
 constexpr size_t kLoadStage = (size_t)32 << 20;  // loads with at most this much to copy go through one copy
 
 constexpr size_t kAdviceStage = (size_t)4 << 20;
@@ -123,7 +124,52 @@ size_t lay_out(const Layout& L, ProgramRec* R, std::vector<size_t>* at, size_t* 
   return off;
 }
 
-// Stream-ordered memory from the context's pool, nullptr if there is none.
+// Programs' memory comes from a pool of the library's own, one a device for all of
+// the process's contexts, that holds on to up to kPoolKeep of it (the device's
+// default pool returns all that unloaded programs gave back at the next
+// synchronization, so every session mapped its memory anew). With a pool for each
+// context, a server's eight slots could hold 8 GB that only they could reuse. The
+// first context creates the pool, the last one gives it back.
+struct DevicePool {
+  cudaMemPool_t pool = nullptr;
+  int users = 0;
+};
+std::mutex g_pool_mu;
+std::map<int, DevicePool>& device_pools() {
+  static auto* pools = new std::map<int, DevicePool>();  // (contexts may outlive the program's static objects)
+  return *pools;
+}
+// The device's pool, nullptr if it cannot be had (programs take the default pool then).
+cudaMemPool_t take_pool(int device) {
+  std::lock_guard<std::mutex> lock(g_pool_mu);
+  DevicePool& d = device_pools()[device];
+  if (d.users == 0) {
+    cudaMemPoolProps props{};
+    props.allocType = cudaMemAllocationTypePinned;
+    props.location.type = cudaMemLocationTypeDevice;
+    props.location.id = device;
+    uint64_t keep = kPoolKeep;
+    if (cudaMemPoolCreate(&d.pool, &props) != cudaSuccess) {
+      cudaGetLastError();
+      return nullptr;
+    }
+    if (cudaMemPoolSetAttribute(d.pool, cudaMemPoolAttrReleaseThreshold, &keep) != cudaSuccess) {
+      cudaGetLastError();
+      cudaMemPoolDestroy(d.pool);
+      return nullptr;
+    }
+  }
+  ++d.users;
+  return d.pool;
+}
+void drop_pool(int device, cudaMemPool_t pool) {
+  if (!pool) return;
+  std::lock_guard<std::mutex> lock(g_pool_mu);
+  DevicePool& d = device_pools()[device];
+  if (--d.users == 0) cudaMemPoolDestroy(d.pool);
+}
+
+// Stream-ordered memory from the pool, nullptr if there is none.
 void* pool_alloc(const gpa_ctx* ctx, size_t bytes, cudaStream_t st) {
   void* p = nullptr;
   if ((ctx->pool ? cudaMallocFromPoolAsync(&p, bytes, ctx->pool, st) : cudaMallocAsync(&p, bytes, st)) == cudaSuccess)
@@ -426,23 +472,7 @@ gpa_status gpa_create(const gpa_arch_desc* arch, const gpa_options* opts, gpa_ct
   }
   if (!s && cudaMemset(T[2].hash, 0xFF, hash_bytes) != cudaSuccess) s = GPA_ERR_CUDA;
   if (!s && cudaEventCreateWithFlags(&c->scratch_ev, cudaEventDisableTiming) != cudaSuccess) s = GPA_ERR_CUDA;
-  // Programs' memory comes from a pool of the context's own that keeps up to
-  // kPoolKeep of what unloaded programs gave back (the device's default pool
-  // returns it all at the next synchronization, so every session mapped its memory
-  // anew); gpa_destroy gives it back.
-  if (!s) {
-    cudaMemPoolProps props{};
-    props.allocType = cudaMemAllocationTypePinned;
-    props.location.type = cudaMemLocationTypeDevice;
-    props.location.id = c->device;
-    uint64_t keep = kPoolKeep;
-    if (cudaMemPoolCreate(&c->pool, &props) != cudaSuccess) {
-      cudaGetLastError();
-      c->pool = nullptr;  // (the default pool then)
-    } else if (cudaMemPoolSetAttribute(c->pool, cudaMemPoolAttrReleaseThreshold, &keep) != cudaSuccess) {
-      s = GPA_ERR_CUDA;
-    }
-  }
+  if (!s) c->pool = take_pool(c->device);
   if (!s && cudaStreamCreateWithFlags(&c->build_stream, cudaStreamNonBlocking) != cudaSuccess) s = GPA_ERR_CUDA;
   if (!s && cudaEventCreateWithFlags(&c->fork.fork, cudaEventDisableTiming) != cudaSuccess) s = GPA_ERR_CUDA;
   for (int k = 0; k < 3; ++k) {
@@ -453,7 +483,7 @@ gpa_status gpa_create(const gpa_arch_desc* arch, const gpa_options* opts, gpa_ct
     if (c->tier[2].global) cudaFree(c->tier[2].global);
     if (c->tier[2].hash) cudaFree(c->tier[2].hash);
     if (c->scratch_ev) cudaEventDestroy(c->scratch_ev);
-    if (c->pool) cudaMemPoolDestroy(c->pool);
+    drop_pool(c->device, c->pool);
     if (c->build_stream) cudaStreamDestroy(c->build_stream);
     if (c->fork.fork) cudaEventDestroy(c->fork.fork);
     for (int k = 0; k < 3; ++k) {
@@ -471,7 +501,7 @@ gpa_status gpa_destroy(gpa_ctx* ctx) {
   if (!ctx) return GPA_ERR_INVALID_ARG;
   cudaDeviceSynchronize();
   for (auto& kv : ctx->progs) free_program(kv.second);
-  if (ctx->pool) cudaMemPoolDestroy(ctx->pool);
+  drop_pool(ctx->device, ctx->pool);
   if (ctx->load_stage) cudaFreeHost(ctx->load_stage);
   if (ctx->advice_stage) cudaFreeHost(ctx->advice_stage);
   if (ctx->tier[2].global) cudaFree(ctx->tier[2].global);

@@ -67,7 +67,9 @@ class _Slot:
 
 class Server:
     """slots: concurrent sessions; budget_bytes: device memory the admitted
-    sessions' programs may hold together; keep_results: also return counts,
+    sessions' programs may hold together (what finished sessions give back is kept
+    for the next ones up to 1 GB on the device, whatever the number of slots);
+    keep_results: also return counts,
     blame and edges (for checking results against the session run alone and
     against the oracle)."""
 

@@ -1,5 +1,5 @@
 """Device memory of programs and contexts: what is freed in stream order waits for no
-other work, and a load takes memory without waiting for the streams that gave it back."""
+other work, and what is kept for later loads is bounded over all contexts."""
 import numpy as np
 import pytest
 
@@ -62,3 +62,31 @@ def test_unload_async_waits_for_no_other_stream(what):
         own.synchronize()
         assert other.running()
         other.stream.synchronize()
+
+
+def test_memory_kept_is_bounded_over_contexts():
+    """What unloaded programs gave back is kept once for all contexts of a device, not by
+    each of them, is there for every context, and is given back with the last one."""
+    import torch
+    import paper_2009_04061_gb300 as g
+    P = synth.make_program(synth.batched_params(60, np.random.default_rng(3), 3), 1.0)
+    with g.Context(ARCH, SLOTS) as first:     # (what a process's first context leaves for good)
+        first.load_program(P).unload()
+    torch.cuda.synchronize()
+    base = torch.cuda.mem_get_info()[0]
+    ctxs = [g.Context(ARCH, SLOTS) for _ in range(5)]
+    try:
+        need = ctxs[0].footprint(P)
+        assert 100 << 20 < need < 512 << 20
+        torch.cuda.synchronize()
+        before = torch.cuda.mem_get_info()[0]
+        for c in ctxs:
+            c.load_program(P).unload()
+        torch.cuda.synchronize()
+        kept = before - torch.cuda.mem_get_info()[0]
+        assert kept < 2 * need, (kept, need)
+    finally:
+        for c in ctxs:
+            c.close()
+    torch.cuda.synchronize()
+    assert base - torch.cuda.mem_get_info()[0] < 64 << 20
