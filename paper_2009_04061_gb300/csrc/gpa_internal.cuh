@@ -40,7 +40,7 @@ enum {
   // And the slowest search: (cycles << 20 | nodes), its rule-2 runs and the
   // cycles of its five phases.
   SS_PHASE = 13, SS_SIZES = 31, SS_PASSB = 47, SS_SLOW = 48,
-  // 55: unused
+  SS_DIRECT_N = 55,  // searches queued straight for the CTAs beyond max_search_nodes (queues 4 and 7)
   SS_OVF3_N = 56, SS_OVF3_HEAD = 57,  // searches of full lists of the shared-memory warps (bottom of queue[3])
   SS_SIZE_CYC = 58,  // with -DGPA_PHASE_TIMING: cycles of the searches by log2 of their node count (16)
   SS_HINT3_N = 74,   // searches beyond a class's limit (from the top of queue[3])

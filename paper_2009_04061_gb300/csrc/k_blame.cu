@@ -212,6 +212,7 @@ __global__ void k_search_local(Prog P, Arch A) {
         const bool giant = hint >= kHintGiant;
         slot = giant ? SS_T5_N : SS_T4_N;
         q = giant ? 7 : 4;
+        atomicAdd(&P.stats[SS_DIRECT_N], 1ull);
       } else if (hint >= kHintWide) { slot = SS_WIDE_N; q = 6; }
       else if (hint >= kHintA1) {
         const int c = (int)hint - kHintA1;

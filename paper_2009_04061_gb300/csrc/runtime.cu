@@ -1320,7 +1320,8 @@ gpa_status gpa_sync_status(gpa_ctx* ctx, gpa_pid pid, gpa_stream stream, int64_t
     info[2] = (int64_t)h[SS_MAX_NODES];
     info[3] = (int64_t)h[SS_SWEEPS];
     info[4] = (int64_t)h[SS_OVF_N];
-    info[5] = (int64_t)(h[SS_OVF2_N] + h[SS_HINT3_N] + h[SS_WIDE_N]);
+    // each search once: handed on by the lanes, or queued straight for a larger tier
+    info[5] = (int64_t)(h[SS_OVF2_N] + h[SS_HINT3_N] + h[SS_WIDE_N] + h[SS_DIRECT_N]);
     for (int c = 0; c < kClasses; ++c)
       info[5] += (int64_t)std::min<unsigned long long>(h[SS_A1_N + c], (unsigned long long)R->P.class_limit[c]);
     info[6] = (int64_t)(h[SS_MAX_TASK] & 0x7FFFFFFFull);     // use of the largest search
