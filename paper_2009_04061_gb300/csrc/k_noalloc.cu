@@ -13,7 +13,7 @@ namespace {
 
 using gpa::scan::kThreads;
 using gpa::scan::kTile;                         // 4096 values per tile
-constexpr int kMaxTiles = 4096;                 // so n <= 16,777,216
+constexpr int kMaxTiles = gpa::scan::kDirectTiles;  // so n <= 16,777,216
 constexpr int kMaxDevices = 64;
 
 // Tile sums of the last call. Every call writes each entry it reads before
@@ -28,7 +28,7 @@ __global__ void __launch_bounds__(kThreads) k_na_scan_sums(const int32_t* buf, i
 }
 __global__ void __launch_bounds__(kThreads) k_na_scan_tiles(int32_t* buf, int n, const int32_t* scratch,
                                                             int32_t* total) {
-  gpa::scan::tile_scan(buf, n, scratch, total);
+  gpa::scan::tile_scan(buf, n, scratch, false, total);
 }
 
 // Device address of the scratch array on the current device, resolved once per
@@ -61,7 +61,7 @@ extern "C" gpa_status gpa_exclusive_scan_noalloc(int32_t* dev_buf, int64_t n, in
   if (cudaPeekAtLastError() != cudaSuccess) return GPA_ERR_CUDA;
   cudaStream_t st = (cudaStream_t)stream;
   if (n == 0) return cudaMemsetAsync(dev_total, 0, sizeof(int32_t), st) == cudaSuccess ? GPA_OK : GPA_ERR_CUDA;
-  const int tiles = (int)((n + kTile - 1) / kTile);
+  const int tiles = gpa::scan::tiles_of(n);
   if (tiles > 1) {  // (a single tile has nothing before it)
     k_na_scan_sums<<<tiles, kThreads, 0, st>>>(dev_buf, (int)n, scratch);
     if (cudaGetLastError() != cudaSuccess) return GPA_ERR_CUDA;

@@ -12,8 +12,8 @@ namespace {
 __global__ void __launch_bounds__(scan::kThreads) k_scan_sums(const int32_t* buf, int n, int32_t* sums) {
   scan::tile_sum(buf, n, sums);
 }
-__global__ void __launch_bounds__(scan::kThreads) k_scan_tiles(int32_t* buf, int n, const int32_t* sums) {
-  scan::tile_scan(buf, n, sums, buf + n);
+__global__ void __launch_bounds__(scan::kThreads) k_scan_tiles(int32_t* buf, int n, const int32_t* sums, bool scanned) {
+  scan::tile_scan(buf, n, sums, scanned, buf + n);
 }
 
 __global__ void k_instr_block(Prog P) {
@@ -179,17 +179,20 @@ int grid_for(int64_t n, int threads, int sms) {
   return (int)(g < 1 ? 1 : g);
 }
 
-size_t scan_tmp_ints(int n) { return (size_t)n / scan::kTile + 16; }
+// The tiles' sums and their total, and the same again for those beyond kDirectTiles.
+size_t scan_tmp_ints(int n) { return (size_t)scan::tiles_of(n) + scan::tiles_of(scan::tiles_of(n)) + 16; }
 
 // buf has n + 1 entries; on return buf[k] = sum of the first k inputs and
 // buf[n] = the total (the input buf[n] is ignored).
 void scan_exclusive_inplace(int32_t* buf, int n, int32_t* tmp, cudaStream_t st, int64_t* launches) {
-  const int tiles = std::max(1, (n + scan::kTile - 1) / scan::kTile);
+  const int tiles = scan::tiles_of(n);
+  const bool many = tiles > scan::kDirectTiles;
   if (tiles > 1) {
     k_scan_sums<<<tiles, scan::kThreads, 0, st>>>(buf, n, tmp);
     ++*launches;
   }
-  k_scan_tiles<<<tiles, scan::kThreads, 0, st>>>(buf, n, tmp);
+  if (many) scan_exclusive_inplace(tmp, tiles, tmp + tiles + 1, st, launches);
+  k_scan_tiles<<<tiles, scan::kThreads, 0, st>>>(buf, n, tmp, many);
   ++*launches;
 }
 

@@ -1,10 +1,14 @@
 // Exclusive scan of int32 values in two launches, shared by the library's own
 // offsets (k_util.cu) and the scan for callers that may not allocate
 // (k_noalloc.cu). The first launch only reads: it sums tiles of 4,096 values. In
-// the second, each CTA adds up the sums of the tiles before its own (at most a few
-// thousand values out of L2) and scans its tile from there, so the values are
+// the second, each CTA adds up the sums of the tiles before its own (at most
+// kDirectTiles of them, out of L2) and scans its tile from there, so the values are
 // read twice and written once, and no launch scans the sums or adds them in a
-// pass of its own (3,000,001 values: 10.7 + 2.7 + 8.9 us in three launches).
+// pass of its own (3,000,001 values: 10.7 + 2.7 + 8.9 us in three launches). Of more
+// tiles the sums are scanned first, by the same two launches: adding them up in
+// every CTA grows with the square of their number (2,048 tiles 26 us against 27
+// with the sums scanned first, 4,096 42 against 40, 16,384 168 against 149, 524,288
+// 22.7 against 4.0 ms).
 // What bounds it is memory; values move as 16-byte vectors where the buffer
 // allows.
 #pragma once
@@ -18,6 +22,12 @@ namespace scan {
 constexpr int kThreads = 512;
 constexpr int kItems = 8;                 // two 16-byte vectors a thread
 constexpr int kTile = kThreads * kItems;  // 4,096 values
+constexpr int kDirectTiles = 4096;
+
+// Tiles of n values (0 <= n <= INT32_MAX), at least one.
+constexpr int tiles_of(int64_t n) { return n <= kTile ? 1 : (int)((n + kTile - 1) / kTile); }
+static_assert(tiles_of(0) == 1 && tiles_of(kTile) == 1 && tiles_of(kTile + 1) == 2 && tiles_of(INT32_MAX) == 524288,
+              "up to the largest count");
 
 // Loads this thread's kItems values of the tile at `off` (0 past n).
 __device__ __forceinline__ void load_items(const int32_t* buf, int64_t off, int64_t n, bool vec, int32_t* v) {
@@ -58,9 +68,10 @@ __device__ __forceinline__ void tile_sum(const int32_t* buf, int64_t n, int32_t*
   if (threadIdx.x == 0) sums[blockIdx.x] = s;
 }
 
-// Scans the tile in place from the sum of sums[0, blockIdx.x); the last tile's
-// CTA writes the total (total may be null).
-__device__ __forceinline__ void tile_scan(int32_t* buf, int64_t n, const int32_t* sums, int32_t* total) {
+// Scans the tile in place from the sum of sums[0, blockIdx.x), or from
+// sums[blockIdx.x] where they are scanned already; the last tile's CTA writes the
+// total (total may be null).
+__device__ __forceinline__ void tile_scan(int32_t* buf, int64_t n, const int32_t* sums, bool scanned, int32_t* total) {
   __shared__ int32_t red[kThreads / 32];
   __shared__ int32_t warp_off[kThreads / 32];
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
@@ -69,8 +80,12 @@ __device__ __forceinline__ void tile_scan(int32_t* buf, int64_t n, const int32_t
   int32_t v[kItems], local = 0;
   load_items(buf, off, n, vec, v);
   int32_t before = 0;
-  for (unsigned t = threadIdx.x; t < blockIdx.x; t += kThreads) before += sums[t];
-  before = cta_sum(before, red);
+  if (scanned) {
+    before = sums[blockIdx.x];
+  } else {
+    for (unsigned t = threadIdx.x; t < blockIdx.x; t += kThreads) before += sums[t];
+    before = cta_sum(before, red);
+  }
 #pragma unroll
   for (int t = 0; t < kItems; ++t) local += v[t];
   int32_t incl = local;
