@@ -41,7 +41,7 @@ enum {
   // cycles of its five phases.
   SS_PHASE = 13, SS_SIZES = 31, SS_PASSB = 47, SS_SLOW = 48,
   SS_DIRECT_N = 55,  // searches queued straight for the CTAs beyond max_search_nodes (queues 4 and 7)
-  SS_OVF3_N = 56, SS_OVF3_HEAD = 57,  // searches of full lists of the shared-memory warps (bottom of queue[3])
+  // 56, 57: unused
   SS_SIZE_CYC = 58,  // with -DGPA_PHASE_TIMING: cycles of the searches by log2 of their node count (16)
   SS_HINT3_N = 74,   // searches beyond a class's limit (from the top of queue[3])
   SS_FAILBITS = 75,  // why a step reported GPA_ERR_CAPACITY: the last search tier ran out of
@@ -61,7 +61,7 @@ enum {
   // searches queued straight for a size class of the shared-memory warps
   SS_A1_N = 92, SS_A1_HEAD = 97,  // kClasses of each
   SS_WIDE_N = 102, SS_WIDE_HEAD = 103,    // searches for the CTAs of 128 threads: known ones (bottom of queue[6])
-  SS_WIDE2_N = 104, SS_WIDE2_HEAD = 105,  // and those that outgrew the shared-memory warps (its top)
+  SS_WIDE2_N = 104, SS_WIDE2_HEAD = 105,  // and what the shared-memory warps hand on (its top)
   SS_T5_N = 106, SS_T5_HEAD = 107,        // searches beyond 2^18 nodes (queue[7])
   SS_N = 108
 };
@@ -172,10 +172,9 @@ struct Prog {
   // resource | start literal set << 9 | blocked << 25}. Each queue has queue_cap
   // entries: 0 first tier from the bottom (after it the second tier's overflow),
   // first size class of the shared-memory warps from the top; 1 second tier,
-  // second class; 2 third class, fourth class; 3 full lists' overflow to the
-  // global-memory warps, what is beyond a class's limit; 4 CTAs of 512 threads; 5
-  // fifth class; 6 CTAs of 128 threads, the last class's overflow; 7 beyond 2^18
-  // nodes. An entry is in one region of a
+  // second class; 2 third class, fourth class; 3 (top) what is beyond a class's limit;
+  // 4 CTAs of 512 threads; 5 fifth class; 6 CTAs of 128 threads, what the
+  // shared-memory warps hand on; 7 beyond 2^18 nodes. An entry is in one region of a
   // queue at a time, so the two regions never meet.
   int2* tasks;                    // n_use
   int32_t* queue[8];

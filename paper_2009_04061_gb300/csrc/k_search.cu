@@ -299,10 +299,11 @@ __device__ int cut_by_blocks(const G& g, const Prog& P, const Arena& a, int b0, 
 // Returns false when the search outgrew the arena (nothing emitted).
 // With P.diag, the search counts the sources of (j, r) before and after
 // pruning into use entry e (`blocked`: an unguarded reader above j in its
-// block prunes them all by rule 2) and emits nothing.
+// block prunes them all by rule 2) and emits nothing. `unsized`: the search takes
+// its whole graph, whose size tells later steps its shared-memory class.
 template <class G>
 __device__ bool group_search(const G& g, const Prog& P, const Arch& A, const Arena& a, int j, int r, uint16_t S0,
-                             int bound, uint16_t live, int tier, int e = 0, bool blocked = false) {
+                             int bound, uint16_t live, int tier, int e, bool blocked, bool unsized) {
   const int me = g.rank();
 #ifdef GPA_PHASE_TIMING
   long long t_prev = clock64();
@@ -674,7 +675,7 @@ __device__ bool group_search(const G& g, const Prog& P, const Arch& A, const Are
   // 46 ms; 200,000 (20M samples): 340 -> 250 ms. The warps' searches, whose size
   // tells later steps their shared-memory class, take the whole graph at once.
   // All growth runs in this one loop, so the wave code exists once in the kernel.
-  bool cand = false, grew_b = false, whole = !kParts || P.diag, again = false;
+  bool cand = false, grew_b = false, whole = !kParts || P.diag || unsized, again = false;
   int grow = kNear;
   int nsrc, nl, alive, n_cut = 0;
   int* const cut_list = a.dl + 3 * (int64_t)a.N;  // sources cut on the blocks
@@ -1164,12 +1165,15 @@ __device__ void run_tasks(const G& g, const Prog& P, const Arch& A, const Arena&
     // The coverage count needs every source: no latency bound.
     const int bound = P.diag ? kInf - 1 : P.res_maxlat[(size_t)f * kNumRes + r];
     const uint16_t live = live_literals(P.res_guards[(size_t)f * kNumRes + r], P.guard[task.x]);
+    // What a CTA gets from a full list may be of any class yet. (Every thread reads
+    // the hint before rank 0 raises it: the search's barriers lie between.)
+    const bool unsized = G::kSize > 32 && P.tier_hint[P.diag ? 1 : 0][e] < kHintWide;
     const bool ok = group_search(g, P, A, a, task.x, r, (uint16_t)((uint32_t)task.y >> 9), bound, live, tier, e,
-                                 (task.y >> 25) & 1);
+                                 (task.y >> 25) & 1, unsized);
     if (me != 0) continue;
     if (ok) {
-      // A search that a full list sent to the warps finds its queue at once.
-      if (tier == 3) {
+      // Later steps queue the search for the class of its graph.
+      if (tier == 3 || unsized) {
         int c = 0;
         while (c < kClasses && class_nodes(c, a.N) < ((volatile int*)a.ctr)[0]) ++c;
         raise_hint(P, e, (uint32_t)(kHintA1 + c));
@@ -1188,10 +1192,11 @@ __device__ void run_tasks(const G& g, const Prog& P, const Arch& A, const Arena&
 }
 
 // Persistent work-stealing warps, one search each: what the shared-memory
-// warps' largest classes have beyond three rounds of the chip (part 1), and what
-// overflowed from their CTAs' lists (part 2). 80 registers a thread, so 24 one-warp
-// CTAs fit an SM: the searches are chains of dependent loads, and more warps in
-// flight finish more of them (measured: 40.7 against 41.9 ms a step with 96).
+// warps' largest classes are known to have beyond three rounds of the chip. (Of
+// unknown size, searches of up to 32,768 nodes would come here: those go to the CTAs.)
+// 80 registers a thread, so 24 one-warp CTAs fit an SM: the searches are chains of
+// dependent loads, and more warps in flight finish more of them (measured: 40.7
+// against 41.9 ms a step with 96).
 __global__ void __launch_bounds__(32, 24) k_search_warp(Prog P, Arch A, SearchArena SA, Route R) {
   // The search counters live in shared memory (the arena is in global memory):
   // frontier sizes are read after every round.
@@ -1200,8 +1205,7 @@ __global__ void __launch_bounds__(32, 24) k_search_warp(Prog P, Arch A, SearchAr
   // out anew) and are empty between searches: every search empties the slots it
   // used, also when it outgrew its arena. They were cleared with the context,
   // so a launch clears nothing. (A launch that began by clearing its warps'
-  // 256 KB hashes wrote 956 MB and took 145 us with no search to run; the launch
-  // appears twice in a step.)
+  // 256 KB hashes wrote 956 MB and took 145 us with no search to run.)
   const Arena a = carve(SA.global + (int64_t)blockIdx.x * SA.bytes, SA.hash + (int64_t)blockIdx.x * 2 * SA.nodes,
                         SA.nodes, SA.src, SA.layers, s_ctr);
   run_tasks(WarpGroup{}, P, A, a, R, 3, false);
@@ -1209,7 +1213,10 @@ __global__ void __launch_bounds__(32, 24) k_search_warp(Prog P, Arch A, SearchAr
 
 // A CTA per search: the waves, frontiers and source lists of these searches
 // are wide enough for its threads. 128 threads for searches of 5,633 to 32,768
-// nodes (a warp took 31 ms for the largest of them), 512 for larger ones, two of
+// nodes (a warp took 31 ms for the largest of them) and for what the shared-memory
+// warps' full lists hand on, whose size is not known yet (first step of 20,000, 30,000
+// and 45,000 instructions: 26, 35 and 70 ms of blame with those by the warps, 16, 18
+// and 41 by CTAs); 512 for larger ones, two of
 // these CTAs on an SM (64 registers), 1,024 for those beyond 2^18 nodes, whose
 // arenas are too large for a CTA on every SM. Both are chains of barriers and
 // arena latency, so what counts is threads in flight: on the 120,000-instruction
@@ -1271,7 +1278,6 @@ void launch_search(const Prog& P, const Arch& A, const SearchArena* tiers, const
   const Route wide1{6, SS_WIDE_N, SS_WIDE_HEAD, false, q4, SS_T4_N, false, kHintCta};
   const Route wide2{6, SS_WIDE2_N, SS_WIDE2_HEAD, true, q4, SS_T4_N, false, kHintCta};
   const Route warp1{3, SS_HINT3_N, SS_HINT3_HEAD, true, q4, SS_T4_N, false, kHintCta};
-  const Route warp2{3, SS_OVF3_N, SS_OVF3_HEAD, false, q4, SS_T4_N, false, kHintCta};
   // No launch takes more groups than there can be tasks (one per use entry).
   auto groups = [&](int n) { return (int)std::max<int64_t>(1, std::min<int64_t>(n, P.queue_cap)); };
   launch_search_smem(P, A, tiers[2].nodes, 1, s[0], sms, launches);
@@ -1286,8 +1292,7 @@ void launch_search(const Prog& P, const Arch& A, const SearchArena* tiers, const
     }
   launch_search_smem(P, A, tiers[2].nodes, 2, st, sms, launches);
   k_search_cta<128><<<groups(wide.warps), 128, 0, st>>>(P, A, wide, wide2);
-  k_search_warp<<<groups(narrow.warps), 32, 0, st>>>(P, A, narrow, warp2);
-  *launches += 4;
+  *launches += 3;
   if (big) {
     // Larger searches run after the others on this stream, so the third tier's
     // arena pool is free by then and they carve their arenas from it (at most two

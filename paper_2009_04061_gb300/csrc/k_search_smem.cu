@@ -19,9 +19,10 @@
 // that an earlier step of the program found to be of a class are queued for it
 // and run largest class first; a search that outgrows its class goes on a list of
 // its CTA, which works off its lists in ascending order at the end. Beyond the
-// last class the global-memory tier takes over. It also takes what the three
-// largest classes have beyond three rounds of the chip: there a search takes three
-// times as long, but 3,648 run at once (see smem_class_limit).
+// last class, and where a list is full, CTAs of 128 threads over global memory take
+// over. One-warp searches there take what the three largest classes are known to have
+// beyond three rounds of the chip: a search takes three times as long, but 3,648 run
+// at once (see smem_class_limit).
 // Registers: 80 a thread, so that global-memory searches (which use no shared
 // memory) find room beside this CTA.
 //
@@ -48,7 +49,7 @@ constexpr int kSearchInf = 0x7FFFFFFF;
 
 __host__ __device__ inline int class_warps(int c) { return 16 >> c; }
 // Searches of class c that a CTA keeps for itself: rounds of the largest
-// classes, bounded so that a list does not outlast the global-memory warps.
+// classes, bounded so that a list does not outlast the CTAs that take the rest.
 __device__ inline int local_list(int c) {
   return c < 2 ? kLocalList : (c == 2 ? 8 : c == 3 ? 4 : 3) * class_warps(c);
 }
@@ -796,9 +797,9 @@ __global__ void __launch_bounds__(768, 1) k_search_smem(Prog P, Arch A, int most
           const int t = atomicAdd(&s_nlocal[next], 1);
           if (t < local_list(next)) { s_local[next][t] = e; continue; }
         }
-        const bool wide = next == kClasses;  // else a full list
-        const unsigned long long o = atomicAdd(&P.stats[wide ? SS_WIDE2_N : SS_OVF3_N], 1ull);
-        if (o < cap) P.queue[wide ? 6 : 3][wide ? cap - 1 - o : o] = e;
+        // beyond the last class, or the CTA's list is full
+        const unsigned long long o = atomicAdd(&P.stats[SS_WIDE2_N], 1ull);
+        if (o < cap) P.queue[6][cap - 1 - o] = e;
         else capacity(P, 8);
       }
     }

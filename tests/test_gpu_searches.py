@@ -54,3 +54,38 @@ def test_larger_searches_are_counted_on_every_step():
     n = [info["tier3_searches"] for info, _ in out]
     assert out[0][0]["max_nodes"] > 16 and n[0] > 0
     assert n == n[:1] * 3, n
+
+
+def test_first_step_of_a_large_kernel():
+    """On a first step no search's size is known: the thousands that fill the
+    shared-memory warps' lists go to CTAs, and the step takes at most three times as long
+    as one that knows them (two is what it measures, four with those searches a warp each).
+    Both give the same edges."""
+    import torch
+    import paper_2009_04061_gb300 as g
+    P = synth.make_program([dict(n_instr=30_000, n_loops=6, max_depth=4, n_regs=255, ldg_pct=30, zipf_s=1.1,
+                                 seed=1_000_003)], 1.0)
+    d = dev(P.samples(2_000_000, seed=5))
+    times, edges = [], []
+    with g.Context(ARCH) as c:
+        for _ in range(3):
+            prog = c.load_program(P)
+            for k in range(3):
+                prog.reset()
+                prog.ingest(d)
+                a, b = torch.cuda.Event(enable_timing=True), torch.cuda.Event(enable_timing=True)
+                torch.cuda.synchronize()
+                a.record()
+                prog.blame()
+                b.record()
+                torch.cuda.synchronize()
+                times.append(a.elapsed_time(b))
+                if len(times) <= 3:
+                    edges.append(prog.edges())
+            assert prog.status()[0] == 0
+            prog.unload()
+    for e in edges[1:]:
+        assert_edges_equal(e, edges[0])
+    first, second, later = (min(times[k::3]) for k in range(3))
+    print(f"first {first:.2f} ms, second {second:.2f}, third {later:.2f}")
+    assert first < 3 * later and second < 1.5 * later
