@@ -353,7 +353,9 @@ struct ExportOut {
   int32_t *use, *def, *res, *dmin, *back, *dlong;
   uint8_t* dom;
 };
-void launch_order_export(const int4* x, int64_t n, int ni, int32_t* off, int32_t* cursor, int32_t* ids,
+constexpr int kExportRank = 1024;  // most edges of a use that are ordered by comparing each with all
+inline int64_t export_big_ints(int64_t n) { return n / kExportRank + 2; }  // the uses with more, and their number
+void launch_order_export(const int4* x, int64_t n, int ni, int32_t* off, int32_t* cursor, int32_t* ids, int32_t* big,
                          const ExportOut& out, int32_t* scan_tmp, cudaStream_t st, int sms, int64_t* launches);
 void launch_build_layout(const Prog& P, cudaStream_t st, int sms, int64_t* launches);
 void launch_store_u64(unsigned long long* p, unsigned long long v, cudaStream_t st, int64_t* launches);

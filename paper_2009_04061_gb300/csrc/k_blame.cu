@@ -487,21 +487,29 @@ __global__ void k_coverage(Prog P) {
 
 // Ordering the export by (use, resource, def): edges counted per use, scanned,
 // dropped into their use's bucket, and each edge's rank within its bucket taken
-// by comparing it with the others there (a use has a handful).
+// by comparing it with the others there (a use has a handful). Buckets of more than
+// kExportRank edges (guarded defs can give a use tens of thousands) are listed and
+// merge-sorted instead, a CTA each: comparing is quadratic (60 uses of 32,001 sources:
+// the export and its copy out 203 ms by comparing, 53 ms sorted; 2,050 sources 2.0 and
+// 1.8 ms, 1,025 the same).
 __global__ void k_export_count(const int4* x, int64_t n, int32_t* cnt) {
   for (int64_t k = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; k < n; k += (int64_t)gridDim.x * blockDim.x)
     atomicAdd(&cnt[x[2 * k].x], 1);
 }
-__global__ void k_export_bucket(const int4* x, int64_t n, const int32_t* off, int32_t* cursor, int32_t* ids) {
+__global__ void k_export_bucket(const int4* x, int64_t n, const int32_t* off, int32_t* cursor, int32_t* ids,
+                                int32_t* big) {
   for (int64_t k = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; k < n; k += (int64_t)gridDim.x * blockDim.x) {
     const int j = x[2 * k].x;
-    ids[off[j] + atomicAdd(&cursor[j], 1)] = (int32_t)k;
+    const int at = atomicAdd(&cursor[j], 1);
+    ids[off[j] + at] = (int32_t)k;
+    if (at == 0 && off[j + 1] - off[j] > kExportRank) big[1 + atomicAdd(&big[0], 1)] = j;
   }
 }
 __global__ void k_export_order(const int4* x, int64_t n, const int32_t* off, const int32_t* ids, ExportOut out) {
   for (int64_t k = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; k < n; k += (int64_t)gridDim.x * blockDim.x) {
     const int4 a = x[2 * k], b = x[2 * k + 1];
     const int q0 = off[a.x], q1 = off[a.x + 1];
+    if (q1 - q0 > kExportRank) continue;  // k_export_sort
     int at = q0;
     for (int q = q0; q < q1; ++q) {
       const int4 c = x[2 * (int64_t)ids[q]];
@@ -511,21 +519,64 @@ __global__ void k_export_order(const int4* x, int64_t n, const int32_t* off, con
     out.back[at] = b.x; out.dlong[at] = b.y; out.dom[at] = (uint8_t)b.z;
   }
 }
+// The listed buckets: runs of 1, 2, 4, ... merged pairwise, each element placed by a
+// binary search in the run beside its own (an earlier run's elements come first among
+// equals). The use column serves as the other buffer until it is written.
+__global__ void __launch_bounds__(1024) k_export_sort(const int4* x, const int32_t* off, int32_t* ids,
+                                                      const int32_t* big, ExportOut out) {
+  for (int t = blockIdx.x; t < big[0]; t += gridDim.x) {
+    const int j = big[1 + t], q0 = off[j], m = off[j + 1] - q0;
+    int32_t *a = ids + q0, *b = out.use + q0;
+    for (int64_t w = 1; w < m; w *= 2) {
+      for (int i = threadIdx.x; i < m; i += blockDim.x) {
+        const int id = a[i];
+        const int4 v = x[2 * (int64_t)id];
+        const bool right = (i / w) & 1;
+        const int64_t base = i / w * w, other = right ? base - w : base + w;
+        int64_t lo = min(other, (int64_t)m), hi = min(other + w, (int64_t)m);
+        const int64_t first = lo;
+        while (lo < hi) {
+          const int64_t mid = (lo + hi) / 2;
+          const int4 c = x[2 * (int64_t)a[mid]];
+          const bool before = c.z != v.z ? c.z < v.z : c.y < v.y || (right && c.y == v.y);
+          if (before) lo = mid + 1;
+          else hi = mid;
+        }
+        b[min(base, other) + (i - base) + (lo - first)] = id;
+      }
+      __syncthreads();
+      int32_t* sw = a; a = b; b = sw;
+    }
+    for (int i = threadIdx.x; i < m; i += blockDim.x) {
+      const int64_t id = a[i];
+      const int4 v = x[2 * id], u = x[2 * id + 1];
+      const int at = q0 + i;
+      out.use[at] = v.x; out.def[at] = v.y; out.res[at] = v.z; out.dmin[at] = v.w;
+      out.back[at] = u.x; out.dlong[at] = u.y; out.dom[at] = (uint8_t)u.z;
+    }
+    __syncthreads();
+  }
+}
 
 }  // namespace
 
-// off and cursor have ni + 1 and ni entries, ids n.
-void launch_order_export(const int4* x, int64_t n, int ni, int32_t* off, int32_t* cursor, int32_t* ids,
+// n <= INT32_MAX; off and cursor have ni + 1 and ni entries, ids n, big export_big_ints(n).
+void launch_order_export(const int4* x, int64_t n, int ni, int32_t* off, int32_t* cursor, int32_t* ids, int32_t* big,
                          const ExportOut& out, int32_t* scan_tmp, cudaStream_t st, int sms, int64_t* launches) {
   if (n <= 0) return;
   cudaMemsetAsync(off, 0, sizeof(int32_t) * (size_t)(ni + 1), st);
   cudaMemsetAsync(cursor, 0, sizeof(int32_t) * (size_t)ni, st);
+  cudaMemsetAsync(big, 0, sizeof(int32_t), st);
   const int g = grid_for(n, 256, sms);
   k_export_count<<<g, 256, 0, st>>>(x, n, off);
   scan_exclusive_inplace(off, ni, scan_tmp, st, launches);
-  k_export_bucket<<<g, 256, 0, st>>>(x, n, off, cursor, ids);
+  k_export_bucket<<<g, 256, 0, st>>>(x, n, off, cursor, ids, big);
   k_export_order<<<g, 256, 0, st>>>(x, n, off, ids, out);
   *launches += 3;
+  if (n > kExportRank) {
+    k_export_sort<<<sms, 1024, 0, st>>>(x, off, ids, big, out);
+    ++*launches;
+  }
 }
 
 void launch_coverage(const Prog& P, const Arch& A, const SearchArena* tiers, const SearchFork* fork, cudaStream_t st,

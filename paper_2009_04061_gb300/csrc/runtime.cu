@@ -1042,14 +1042,15 @@ gpa_status gpa_dependency_coverage(gpa_ctx* ctx, gpa_pid pid, gpa_stream stream,
   return s;
 }
 
-// The ordered export's arrays in xout: seven columns of xout_cap int32 (the
-// last is scratch: ids, then ni + 1 offsets and ni cursors), then the bytes.
+// The ordered export's arrays in xout: seven columns of xout_cap int32 (the last is
+// scratch: ids, then ni + 1 offsets, ni cursors and the list of large buckets), then
+// the bytes.
 static ExportOut export_out(const ProgramRec* R, int32_t** ids) {
   int32_t* p = static_cast<int32_t*>(R->xout);
   const size_t c = (size_t)R->xout_cap;
   if (ids) *ids = p + 6 * c;
   return ExportOut{p, p + c, p + 2 * c, p + 3 * c, p + 4 * c, p + 5 * c,
-                   reinterpret_cast<uint8_t*>(p + 7 * c + 2 * (size_t)R->P.ni + 1)};
+                   reinterpret_cast<uint8_t*>(p + 7 * c + 2 * (size_t)R->P.ni + 1 + export_big_ints(R->xout_cap))};
 }
 
 gpa_status gpa_export_unpruned_edges(gpa_ctx* ctx, gpa_pid pid, gpa_stream stream, int64_t* n_edges) {
@@ -1078,16 +1079,22 @@ gpa_status gpa_export_unpruned_edges(gpa_ctx* ctx, gpa_pid pid, gpa_stream strea
     if (s) return s;
   }
   const int64_t n = std::min<int64_t>((int64_t)h[SS_XN], R->xbuf_cap);
+  if (n > INT32_MAX) {  // beyond the device's 32-bit offsets: ordered on the host (gpa_get_unpruned_edges)
+    R->x_n = *n_edges = n;
+    return GPA_OK;
+  }
   if (n > R->xout_cap) {
     if (R->xout) cudaFreeAsync(R->xout, st);
-    R->xout = pool_alloc(ctx, (size_t)n * 29 + sizeof(int32_t) * (2 * (size_t)R->P.ni + 1), st);
+    R->xout = pool_alloc(
+        ctx, (size_t)n * 29 + sizeof(int32_t) * (2 * (size_t)R->P.ni + 1 + (size_t)export_big_ints(n)), st);
     R->xout_cap = R->xout ? n : 0;
     if (!R->xout) return GPA_ERR_OOM;
   }
   int32_t* ids = nullptr;
   const ExportOut out = export_out(R, &ids);
   int32_t* off = ids + R->xout_cap;
-  launch_order_export(R->xbuf, n, R->P.ni, off, off + R->P.ni + 1, ids, out, R->scan_tmp, st, ctx->sms,
+  int32_t* cursor = off + R->P.ni + 1;
+  launch_order_export(R->xbuf, n, R->P.ni, off, cursor, ids, cursor + R->P.ni, out, R->scan_tmp, st, ctx->sms,
                       &ctx->launches);
   CK(cudaGetLastError());
   CK(cudaStreamSynchronize(st));
@@ -1103,6 +1110,27 @@ gpa_status gpa_get_unpruned_edges(gpa_ctx* ctx, gpa_pid pid, int32_t* use, int32
   CK(cudaStreamSynchronize((cudaStream_t)stream));
   const size_t n = (size_t)R->x_n;
   if (!n) return GPA_OK;
+  if (n > INT32_MAX) {
+    std::vector<int4> x(2 * n);
+    CK(cudaMemcpy(x.data(), R->xbuf, sizeof(int4) * x.size(), cudaMemcpyDeviceToHost));
+    std::vector<size_t> order(n);
+    for (size_t k = 0; k < n; ++k) order[k] = k;
+    std::sort(order.begin(), order.end(), [&](size_t a, size_t b) {
+      const int4 &p = x[2 * a], &q = x[2 * b];
+      return p.x != q.x ? p.x < q.x : p.z != q.z ? p.z < q.z : p.y < q.y;
+    });
+    for (size_t t = 0; t < n; ++t) {
+      const int4 a = x[2 * order[t]], b = x[2 * order[t] + 1];
+      if (use) use[t] = a.x;
+      if (def) def[t] = a.y;
+      if (res) res[t] = a.z;
+      if (dmin) dmin[t] = a.w;
+      if (back_edges) back_edges[t] = b.x;
+      if (dlong) dlong[t] = b.y;
+      if (dom) dom[t] = (uint8_t)b.z;
+    }
+    return GPA_OK;
+  }
   const ExportOut x = export_out(R, nullptr);
   int32_t* const dst[6] = {use, def, res, dmin, back_edges, dlong};
   const int32_t* const src[6] = {x.use, x.def, x.res, x.dmin, x.back, x.dlong};
