@@ -28,7 +28,7 @@ __global__ void __launch_bounds__(kThreads) k_na_scan_sums(const int32_t* buf, i
 }
 __global__ void __launch_bounds__(kThreads) k_na_scan_tiles(int32_t* buf, int n, const int32_t* scratch,
                                                             int32_t* total) {
-  gpa::scan::tile_scan(buf, n, scratch, false, total);
+  gpa::scan::tile_scan<false>(buf, n, scratch, total);
 }
 
 // Device address of the scratch array on the current device, resolved once per

@@ -12,8 +12,9 @@ namespace {
 __global__ void __launch_bounds__(scan::kThreads) k_scan_sums(const int32_t* buf, int n, int32_t* sums) {
   scan::tile_sum(buf, n, sums);
 }
-__global__ void __launch_bounds__(scan::kThreads) k_scan_tiles(int32_t* buf, int n, const int32_t* sums, bool scanned) {
-  scan::tile_scan(buf, n, sums, scanned, buf + n);
+template <bool kScanned>
+__global__ void __launch_bounds__(scan::kThreads) k_scan_tiles(int32_t* buf, int n, const int32_t* sums) {
+  scan::tile_scan<kScanned>(buf, n, sums, buf + n);
 }
 
 __global__ void k_instr_block(Prog P) {
@@ -186,13 +187,16 @@ size_t scan_tmp_ints(int n) { return (size_t)scan::tiles_of(n) + scan::tiles_of(
 // buf[n] = the total (the input buf[n] is ignored).
 void scan_exclusive_inplace(int32_t* buf, int n, int32_t* tmp, cudaStream_t st, int64_t* launches) {
   const int tiles = scan::tiles_of(n);
-  const bool many = tiles > scan::kDirectTiles;
   if (tiles > 1) {
     k_scan_sums<<<tiles, scan::kThreads, 0, st>>>(buf, n, tmp);
     ++*launches;
   }
-  if (many) scan_exclusive_inplace(tmp, tiles, tmp + tiles + 1, st, launches);
-  k_scan_tiles<<<tiles, scan::kThreads, 0, st>>>(buf, n, tmp, many);
+  if (tiles > scan::kDirectTiles) {
+    scan_exclusive_inplace(tmp, tiles, tmp + tiles + 1, st, launches);
+    k_scan_tiles<true><<<tiles, scan::kThreads, 0, st>>>(buf, n, tmp);
+  } else {
+    k_scan_tiles<false><<<tiles, scan::kThreads, 0, st>>>(buf, n, tmp);
+  }
   ++*launches;
 }
 

@@ -69,9 +69,10 @@ __device__ __forceinline__ void tile_sum(const int32_t* buf, int64_t n, int32_t*
 }
 
 // Scans the tile in place from the sum of sums[0, blockIdx.x), or from
-// sums[blockIdx.x] where they are scanned already; the last tile's CTA writes the
-// total (total may be null).
-__device__ __forceinline__ void tile_scan(int32_t* buf, int64_t n, const int32_t* sums, bool scanned, int32_t* total) {
+// sums[blockIdx.x] where they are scanned already (kScanned); the last tile's CTA
+// writes the total (total may be null).
+template <bool kScanned>
+__device__ __forceinline__ void tile_scan(int32_t* buf, int64_t n, const int32_t* sums, int32_t* total) {
   __shared__ int32_t red[kThreads / 32];
   __shared__ int32_t warp_off[kThreads / 32];
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
@@ -80,7 +81,7 @@ __device__ __forceinline__ void tile_scan(int32_t* buf, int64_t n, const int32_t
   int32_t v[kItems], local = 0;
   load_items(buf, off, n, vec, v);
   int32_t before = 0;
-  if (scanned) {
+  if (kScanned) {
     before = sums[blockIdx.x];
   } else {
     for (unsigned t = threadIdx.x; t < blockIdx.x; t += kThreads) before += sums[t];
