@@ -50,7 +50,7 @@ enum {
                      // 11 distance range, 12 raw edges, 13 no path length
   SS_BIG_N = 76,     // uses with more than kMaxSrc distinct sources (listed in big_use)
   SS_COV = 77,       // gpa_dependency_coverage: stalled uses, single before, single after pruning
-  SS_COV_ALL = 80,   // the counting pass's total of sources before pruning
+  // 80: unused
   SS_XN = 81,        // unpruned edges written by the export pass
   SS_HIST_HEAD = 82, // next chunk of the run-aware aggregation kernel (reset before each launch)
   SS_HINT3_HEAD = 83,  // next of them
@@ -159,8 +159,8 @@ struct Prog {
   unsigned long long* cnt;        // ni * 24
   unsigned long long* stats;      // SS_N
   uint32_t* def_mask;             // nb * 9: resources defined in the block
-  uint32_t* uuse_mask;            // nb * 9: resources read by an unguarded instruction
-  uint32_t* touch_mask;           // nb * 9: DEF | UUSE (blocks a search must scan)
+  uint32_t* touch_mask;           // nb * 9: resources defined or read by an unguarded instruction (blocks a search
+                                  // must scan)
   int32_t* res_maxlat;            // nf * 268: largest latency of any def of the resource in the function
   uint32_t* res_guards;           // nf * 268, right behind res_maxlat: guard literals of the resource's defs in the function
   uint32_t* rin;                  // nb * 9
@@ -184,10 +184,9 @@ struct Prog {
   // diagnostics' searches, which have no latency bound.
   uint8_t* tier_hint[2];
   int64_t queue_cap;
-  int32_t* edge_cnt;              // ni + 1 (exclusive scan in place -> offsets)
   int32_t* big_use;               // ni: uses with more than kMaxSrc sources (SS_BIG_N of them)
   int32_t* suse;                  // ni: the stalled uses of this step, SS_SUSE_N of them (any order)
-  int32_t* edge_off;              // ni + 1
+  int32_t* edge_off;              // ni + 1: edges per use, scanned in place
   int32_t* e_use;
   int32_t* e_def;
   int32_t* e_dmin;
@@ -301,8 +300,9 @@ __device__ __forceinline__ void xemit(const Prog& P, int j, int i, int r, int dm
   P.xedges[2 * k] = make_int4(j, i, r, dmin);
   P.xedges[2 * k + 1] = make_int4(K, dlong, dom ? 1 : 0, 0);
 }
-// Adds a (use entry) contribution to the coverage count.
+// Adds a (use entry) contribution to the coverage count (the export has none).
 __device__ __forceinline__ void cov_add(const Prog& P, int e, int n_all, int n_kept) {
+  if (P.diag != 1) return;
   atomicAdd(&P.cov_cnt[e], (uint32_t)min(n_all, 0xFFFF) | ((uint32_t)min(n_kept, 0xFFFF) << 16));
 }
 

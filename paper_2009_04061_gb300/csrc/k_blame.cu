@@ -457,7 +457,7 @@ __global__ void k_apportion_big(Prog P, Arch A) {
 // no resource it reads has more than one source (before pruning) or more than
 // one kept source (after).
 __global__ void k_coverage(Prog P) {
-  unsigned long long nodes = 0, before = 0, after = 0, total = 0;
+  unsigned long long nodes = 0, before = 0, after = 0;
   for (int j = blockIdx.x * blockDim.x + threadIdx.x; j < P.ni; j += gridDim.x * blockDim.x) {
     if (!stalled(P, j)) continue;
     uint32_t most_all = 0, most_kept = 0;
@@ -465,7 +465,6 @@ __global__ void k_coverage(Prog P) {
       const uint32_t c = P.cov_cnt[e];
       most_all = max(most_all, c & 0xFFFFu);
       most_kept = max(most_kept, c >> 16);
-      total += c & 0xFFFFu;
     }
     ++nodes;
     before += most_all <= 1u;
@@ -475,13 +474,11 @@ __global__ void k_coverage(Prog P) {
     nodes += __shfl_xor_sync(0xffffffffu, nodes, o);
     before += __shfl_xor_sync(0xffffffffu, before, o);
     after += __shfl_xor_sync(0xffffffffu, after, o);
-    total += __shfl_xor_sync(0xffffffffu, total, o);
   }
   if ((threadIdx.x & 31) == 0 && nodes) {
     atomicAdd(&P.stats[SS_COV], nodes);
     atomicAdd(&P.stats[SS_COV + 1], before);
     atomicAdd(&P.stats[SS_COV + 2], after);
-    atomicAdd(&P.stats[SS_COV_ALL], total);
   }
 }
 
@@ -582,13 +579,13 @@ void launch_order_export(const int4* x, int64_t n, int ni, int32_t* off, int32_t
 void launch_coverage(const Prog& P, const Arch& A, const SearchArena* tiers, const SearchFork* fork, cudaStream_t st,
                      int sms, int64_t* launches) {
   const int threads = 128;
-  const int g_instr = grid_for(P.ni, threads, sms);
   const int g_local = std::max(1, std::min(sms * 64, (int)(((int64_t)P.ni * kLocalLanes + threads - 1) / threads)));
   k_stalled_list<<<(P.ni + 255) / 256, 256, 0, st>>>(P, 0);
   k_search_local<<<g_local, threads, 0, st>>>(P, A);
   *launches += 2;
   launch_search(P, A, tiers, fork, st, sms, launches);
-  k_coverage<<<g_instr, threads, 0, st>>>(P);
+  if (P.diag != 1) return;
+  k_coverage<<<grid_for(P.ni, threads, sms), threads, 0, st>>>(P);
   ++*launches;
 }
 

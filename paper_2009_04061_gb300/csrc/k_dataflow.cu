@@ -51,7 +51,6 @@ __global__ void k_block_masks(Prog P, int windowed) {
 #pragma unroll
     for (int w = 0; w < kWords; ++w) {
       P.def_mask[o + w] = dm[w];
-      P.uuse_mask[o + w] = um[w];
       P.touch_mask[o + w] = dm[w] | um[w];
       if (windowed) {  // its fixpoint starts from these; the other kernels write every word
         P.rin[o + w] = 0u;

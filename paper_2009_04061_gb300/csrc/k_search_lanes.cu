@@ -48,7 +48,7 @@ enum {
   W_NEXT = 5,  // the next layer's longest distance
   kNodeWords = 6
 };
-enum { F_EXPANDED = 1, F_QUEUED = 2 };
+enum { F_QUEUED = 1 };
 constexpr uint32_t kFar = 0xFFFFFFu;  // no distance yet (distances are below 128 * 65,535)
 constexpr int kOccWords = 3;          // position | node << 16 | def kind << 24; distance << 8 | nearest
                                       // occurrence; source | back edges << 8 | within latency << 16 | kept << 17
@@ -188,7 +188,6 @@ struct LaneSearch {
     if (cut) { no = 0; pass_b = true; state = L_FINISH; return; }  // nothing survives: see finish()
     const int len = u == 0 ? j - m0.x + 1 : m0.y - m0.x;
     a.half(u, W_INFO, 0) = (uint16_t)wall;
-    a.byte(u, W_INFO, 3) |= F_EXPANDED;
     a.half(u, W_LEN, 0) = (uint16_t)len;
     a.byte(u, W_EDGE, 0) = (uint8_t)ne;
     const int Sout = (int)keep_literals(S, live);

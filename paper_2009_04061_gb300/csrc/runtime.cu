@@ -682,7 +682,6 @@ static void plan_program(const gpa_program_desc* d, ProgramRec* R, Layout& L, in
   dev_alloc(L, &P.def_mask, nb * kWords);
   dev_alloc(L, &P.touch_mask, nb * kWords);
   dev_alloc(L, &R->meta, 2 * nb);
-  dev_alloc(L, &P.uuse_mask, nb * kWords);
   dev_alloc(L, &P.rin, nb * kWords);
   dev_alloc(L, &P.rout, nb * kWords);
   dev_alloc(L, &P.head, ni);
@@ -762,7 +761,6 @@ static void derive_pointers(ProgramRec* R) {
   P.events = R->events;
   P.block_meta = R->meta;
   P.res_guards = reinterpret_cast<uint32_t*>(P.res_maxlat) + (size_t)P.nf * kNumRes;
-  P.edge_cnt = P.edge_off;
   P.adv_own_active = P.adv_acc + (size_t)P.nf * kAdvAcc;
   P.adv_own_matched = P.adv_own_active + P.nl;
   P.a_loop_active = P.adv_own_matched + P.nl;
@@ -843,10 +841,6 @@ gpa_status gpa_load_program(gpa_ctx* ctx, const gpa_program_desc* d, gpa_pid* ou
   // Everything of the load runs on the context's build stream, which is then
   // synchronized: other streams' work is not waited for.
   cudaStream_t st = R->build;
-  if (P.t4_arena && cudaMemsetAsync(P.t4_arena, 0, (size_t)P.t4_bytes * P.t4_ctas, st) != cudaSuccess) {
-    free_program(R);
-    return GPA_ERR_CUDA;
-  }
   launch_build_layout(P, st, ctx->sms, &ctx->launches);
   launch_build_preds(P, R->n_succ, R->pred_off, R->cursor, R->scan_tmp, st, ctx->sms, &ctx->launches);
   launch_build_events(P, R->ev_off, R->events, R->scan_tmp, st, ctx->sms, &ctx->launches);
@@ -1016,7 +1010,7 @@ static gpa_status coverage_run(gpa_ctx* ctx, ProgramRec* R, cudaStream_t st, int
   D.diag = diag;
   D.xedges = R->xbuf;
   D.xcap = diag == 2 ? R->xbuf_cap : 0;
-  CK(cudaMemsetAsync(D.cov_cnt, 0, sizeof(uint32_t) * (size_t)std::max(R->n_use, 1), st));
+  if (diag == 1) CK(cudaMemsetAsync(D.cov_cnt, 0, sizeof(uint32_t) * (size_t)std::max(R->n_use, 1), st));
   CK(cudaMemsetAsync(D.stats + SS_GENERAL, 0, sizeof(unsigned long long) * 3, st));
   CK(cudaMemsetAsync(D.stats + SS_RAW_N, 0, sizeof(unsigned long long) * (SS_N - SS_RAW_N), st));
   CK(cudaStreamWaitEvent(st, ctx->scratch_ev, 0));
