@@ -300,7 +300,8 @@ __device__ int cut_by_blocks(const G& g, const Prog& P, const Arena& a, int b0, 
 // With P.diag, the search counts the sources of (j, r) before and after
 // pruning into use entry e (`blocked`: an unguarded reader above j in its
 // block prunes them all by rule 2) and emits nothing. `unsized`: the search takes
-// its whole graph, whose size tells later steps its shared-memory class.
+// its whole graph, whose size tells later steps its shared-memory class, unless that
+// turns out larger than the last of them.
 template <class G>
 __device__ bool group_search(const G& g, const Prog& P, const Arch& A, const Arena& a, int j, int r, uint16_t S0,
                              int bound, uint16_t live, int tier, int e, bool blocked, bool unsized) {
@@ -676,6 +677,7 @@ __device__ bool group_search(const G& g, const Prog& P, const Arch& A, const Are
   // tells later steps their shared-memory class, take the whole graph at once.
   // All growth runs in this one loop, so the wave code exists once in the kernel.
   bool cand = false, grew_b = false, whole = !kParts || P.diag || unsized, again = false;
+  bool sizing = kParts && unsized && !P.diag;
   int grow = kNear;
   int nsrc, nl, alive, n_cut = 0;
   int* const cut_list = a.dl + 3 * (int64_t)a.N;  // sources cut on the blocks
@@ -713,6 +715,12 @@ __device__ bool group_search(const G& g, const Prog& P, const Arch& A, const Are
         if (n_dirty > 0) relax_from(a.ord, n_dirty, 0);
       } else if (kParts && grow == kLayers) {
         relax_from(list, cnt, 1);
+      } else if (kParts && sizing && g.read(&ctr[0]) > class_nodes(kClasses - 1, a.N)) {
+        // Of no class: on with the parts, from a graph that is pass A's and some more
+        // (which adds only paths of the whole graph; k is not set yet, like after pass A).
+        sizing = whole = false;
+        grow = kNear;
+        break;
       }
       continue;
     }
@@ -1215,8 +1223,9 @@ __global__ void __launch_bounds__(32, 24) k_search_warp(Prog P, Arch A, SearchAr
 // are wide enough for its threads. 128 threads for searches of 5,633 to 32,768
 // nodes (a warp took 31 ms for the largest of them) and for what the shared-memory
 // warps' full lists hand on, whose size is not known yet (first step of 20,000, 30,000
-// and 45,000 instructions: 26, 35 and 70 ms of blame with those by the warps, 16, 18
-// and 41 by CTAs); 512 for larger ones, two of
+// and 45,000 instructions: 26, 35 and 70 ms of blame with those by the warps, 16, 17
+// and 41 by CTAs; 200,000 with 20M samples 194 and 184, with 300M, where most of them
+// outgrow these arenas too, 266 and 271); 512 for larger ones, two of
 // these CTAs on an SM (64 registers), 1,024 for those beyond 2^18 nodes, whose
 // arenas are too large for a CTA on every SM. Both are chains of barriers and
 // arena latency, so what counts is threads in flight: on the 120,000-instruction
