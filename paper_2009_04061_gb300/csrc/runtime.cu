@@ -540,7 +540,8 @@ static void plan_program(const gpa_program_desc* d, ProgramRec* R, Layout& L, in
                            (int64_t)d->func_loop_off[f + 1] - d->func_loop_off[f]);
   };
   // Staged fixpoint: functions needing at most this much shared memory (the
-  // others take the windowed global-memory kernel).
+  // others go by mask words where their loops are natural ones and a word a block
+  // fits, else to the windowed global-memory kernel).
   P.reach_smem = 0;
   for (int f = 0; f < d->n_functions; ++f) {
     const int64_t need = reach_need(f);
@@ -553,7 +554,8 @@ static void plan_program(const gpa_program_desc* d, ProgramRec* R, Layout& L, in
     // The staged fixpoint takes the functions by shared memory need, largest
     // first, in four launches by size class (kReachClassCap): class c holds the
     // needs in (cap[c + 1], cap[c]], and its launch sizes its stage for the
-    // largest of them. Functions beyond cap[0] are left to the windowed kernel.
+    // largest of them. Functions beyond cap[0] are left to the kernels by mask words
+    // and by windows (reach_windowed of them).
     std::vector<int64_t> need(nf);
     for (size_t f = 0; f < nf; ++f) need[f] = reach_need((int)f);
     std::vector<int32_t>& order = L.order;
